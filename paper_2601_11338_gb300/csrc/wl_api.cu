@@ -2437,18 +2437,18 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       // Y = phi Omega by the solve of the handle's form (FP64 n x K), Gram in FP64
       if (e == cudaSuccess && (rc = ensure(h->packV, nk * 8)) != WL_OK) break;
       if (e == cudaSuccess && (rc = ensure(h->packX, nk * 8)) != WL_OK) break;
-      if (e == cudaSuccess && (rc = ensure(h->gram, (size_t)Gg * 2 * kMaxSketch * kMaxSketch * 8 +
-                                                     2 * kMaxSketch * kMaxSketch * 8 + 128 * 8)) != WL_OK) break;
+      if (e == cudaSuccess && (rc = ensure(h->gram, (gram_f64_partial_doubles(n, M) + 2 * kMaxSketch * kMaxSketch +
+                                                      128) * 8)) != WL_OK) break;
       counted(h);
       if (e == cudaSuccess) e = launch_sketch_block_f64(om_int, n, M, K, (double*)h->packV.p, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "sketch"); break; }
       if ((rc = phi_apply(h, (const double*)h->packV.p, (double*)h->packX.p, K, info)) != WL_OK) break;
       if (info.status != WL_OK) break;
       double* part64 = (double*)h->gram.p;
-      gout = part64 + (size_t)Gg * 2 * kMaxSketch * kMaxSketch;
+      gout = part64 + gram_f64_partial_doubles(n, M);
       core = gout + 2 * kMaxSketch * kMaxSketch;
       counted(h, 3);
-      e = launch_gram_f64(om_int, (const double*)h->packX.p, n, M, K, part64, Gg, gout, S(h));
+      e = launch_gram_f64(om_int, (const double*)h->packX.p, n, M, K, part64, gout, S(h));
       if (e == cudaSuccess) e = launch_nys_core(gout, M, core, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "gram/core"); break; }
       double* hp = h->h_pin;
@@ -2533,7 +2533,7 @@ int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt,
     if ((rc = ensure(h->ybig, (size_t)kMaxTau * nk * 8)) != WL_OK) break;
     const int Gg = gram_grid(n);
     const bool sketch = h->prm.prec == WL_SKETCH;  // FP32 Gram on the tensor cores; else FP64
-    const size_t pbytes = (size_t)Gg * 2 * kMaxSketch * kMaxSketch * (sketch ? 4 : 8);
+    const size_t pbytes = sketch ? (size_t)Gg * 2 * kMaxSketch * kMaxSketch * 4 : gram_f64_partial_doubles(n, M) * 8;
     if ((rc = ensure(h->gram, pbytes + 2 * kMaxSketch * kMaxSketch * 8 + 128 * 8)) != WL_OK) break;
     uint16_t* omega = (uint16_t*)h->omega.p;
     float* partial = (float*)h->gram.p;
@@ -2569,7 +2569,7 @@ int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt,
         e = cudaMemsetAsync(gerr, 0, sizeof(int), S(h));
         if (!sketch) {
           if (e == cudaSuccess)
-            e = launch_gram_f64(om_int, Y + (size_t)i * nk, n, M, K, (double*)h->gram.p, Gg, gout, S(h));
+            e = launch_gram_f64(om_int, Y + (size_t)i * nk, n, M, K, (double*)h->gram.p, gout, S(h));
         } else {
           if (e == cudaSuccess) e = launch_to_f32(Y + (size_t)i * nk, (int64_t)nk, (float*)h->x.p, S(h));
           if (e == cudaSuccess)

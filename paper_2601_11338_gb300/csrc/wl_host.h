@@ -203,7 +203,9 @@ cudaError_t launch_gram(const uint16_t* omega, const float* Y, int64_t n, int M,
 // out[0] estimate, out[1] error estimate, out[2] status, out[8 + i] = t_i
 cudaError_t launch_nys_core(const double* gram, int M, double* out, cudaStream_t s);
 // [Omega Y]^T Y from an FP64 Y (n x K, first M columns), FP64 throughout; partial: G x 2 x 64 x 64 doubles
-cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K, double* partial, int G,
+int gram_grid_f64(int64_t n);
+size_t gram_f64_partial_doubles(int64_t n, int M);
+cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K, double* partial,
                             double* out, cudaStream_t s);
 
 // cooperative launch helper (all CTAs co-resident; required by grid_sync)

@@ -2,6 +2,8 @@
 #define WL_TRACE_KERNELS
 #include <string.h>
 
+#include <algorithm>
+
 #include "wl.h"
 #include "wl_gram_tc.cuh"
 #include "wl_host.h"
@@ -82,11 +84,22 @@ cudaError_t launch_gram(const uint16_t* omega, const float* Y, int64_t n, int M,
   return cudaGetLastError();
 }
 
-cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K, double* partial, int G,
+// one CTA per SM: the FP64 pipe is saturated by the 8 to 16 warps of one
+int gram_grid_f64(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(152, (n + kGramRows64 - 1) / kGramRows64));
+}
+
+size_t gram_f64_partial_doubles(int64_t n, int M) { return (size_t)gram_grid_f64(n) * gram64_tiles(M) * 16; }
+
+cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K, double* partial,
                             double* out, cudaStream_t s) {
+  const int G = gram_grid_f64(n), nt = gram64_tiles(M);
   const int64_t chunk = (n + G - 1) / G;
-  gram_f64<<<G, 256, 0, s>>>(omega, Y, n, M, K, chunk, partial);
-  gram_reduce_f64<<<(2 * kMaxSketch * kMaxSketch + 255) / 256, 256, 0, s>>>(partial, G, out);
+  cudaError_t e = cudaMemsetAsync(out, 0, 2 * kMaxSketch * kMaxSketch * sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  const int threads = (nt * gram64_groups(M) + 31) / 32 * 32;
+  gram_f64<<<G, threads, 0, s>>>(omega, Y, n, M, K, chunk, partial);
+  gram_reduce_f64<<<(nt * 16 + 31) / 32, 256, 0, s>>>(partial, G, M, out);
   return cudaGetLastError();
 }
 

@@ -203,27 +203,68 @@ __global__ void gram_reduce(const float* partial, int G, double* out) {
 
 // ---------------------------------------------------------------- Gram in FP64 (CUDA cores)
 // The same block [Omega Y]^T Y from an FP64 Y (the FP64 and refined forms of
-// the estimators): FP64 products and sums throughout, partial per CTA in
-// the layout of gram_cc (doubles), summed by gram_reduce_f64.
-constexpr int kGramRows64 = 16;  // rows staged per tile
+// the estimators), FP64 products and sums throughout. Bound by the FP64 pipe
+// (2 lanes per clock and SM: a warp's DFMA holds its scheduler's pipe for 64
+// cycles, so shared-memory reads and loads hide behind it). So the work is
+// cut to what the M columns need: 4 x 4 output tiles of H = Omega^T Y (all)
+// and of G = Y^T Y (the upper triangle), one tile per thread, and the rows of
+// a staged tile dealt to `groups` copies of the tile set where it is small.
+// One CTA per SM over the whole chip, however few the rows. Measured with 131072 x 64:
+// 1550 us (a fixed 128 x 64 block per CTA of 4096 rows, 32 CTAs: 8766 us);
+// with 62500 x 30: 195 us (16 CTAs and the block padded to 64 columns: 8283 us).
+constexpr int kGramRows64 = 32;       // rows staged per tile
+constexpr int kGramThreads64 = 512;   // most threads of a CTA
+constexpr int kGramGroups64 = 16;     // most copies of the tile set in a CTA
+__host__ __device__ constexpr int gram64_tiles(int M) {  // 4 x 4 tiles of H and of G's upper triangle
+  const int nb = (M + 3) / 4;
+  return nb * nb + nb * (nb + 1) / 2;
+}
+__host__ __device__ constexpr int gram64_groups(int M) {
+  const int g = kGramThreads64 / gram64_tiles(M);
+  return g < 1 ? 1 : (g > kGramGroups64 ? kGramGroups64 : g);
+}
+// tile t -> (ti, tj): H tiles row by row, then G tiles with ti <= tj
+__device__ __forceinline__ void gram64_tile(int t, int nb, bool* is_g, int* ti, int* tj) {
+  *is_g = t >= nb * nb;
+  if (!*is_g) {
+    *ti = t / nb;
+    *tj = t % nb;
+    return;
+  }
+  int q = t - nb * nb, r = 0;
+  while (q >= nb - r) {
+    q -= nb - r;
+    ++r;
+  }
+  *ti = r;
+  *tj = r + q;
+}
 
-__global__ void __launch_bounds__(256) gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K,
-                                                int64_t chunk, double* partial /* G x 2M x M */) {
-  __shared__ double sX[kGramRows64][2 * kMaxSketch];  // [Omega_i, Y_i]
-  const int tid = threadIdx.x;
-  const int rt = tid / 16, ct = tid % 16;
+// partial: gridDim.x blocks of gram64_tiles(M) x 16 doubles
+__global__ void __launch_bounds__(kGramThreads64) gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M,
+                                                           int K, int64_t chunk, double* partial) {
+  // [Omega_i, Y_i] of the staged rows; the groups' accumulators at the end
+  __shared__ __align__(16) double sX[kGramRows64][2 * kMaxSketch];
+  const int nb = (M + 3) / 4, W = 4 * nb, nt = gram64_tiles(M), groups = gram64_groups(M);
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int grp = tid / nt, t = tid % nt;
+  const bool live = grp < groups;
+  bool is_g;
+  int ti, tj;
+  gram64_tile(t, nb, &is_g, &ti, &tj);
+  const int xo = (is_g ? kMaxSketch : 0) + 4 * ti, yo = kMaxSketch + 4 * tj;
   const int64_t r0 = (int64_t)blockIdx.x * chunk;
   const int64_t r1 = min(n, r0 + chunk);
-  double acc[8][4];
+  double acc[4][4];
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
   for (int64_t base = r0; base < r1; base += kGramRows64) {
     const int rows = (int)min((int64_t)kGramRows64, r1 - base);
     __syncthreads();
-    for (int e = tid; e < kGramRows64 * kMaxSketch; e += 256) {
-      const int i = e / kMaxSketch, j = e % kMaxSketch;
+    for (int e = tid; e < kGramRows64 * W; e += nthr) {
+      const int i = e / W, j = e % W;
       double om = 0.0, y = 0.0;
       if (i < rows && j < M) {
         om = (double)bf16_to_f32(omega[(base + i) * M + j]);
@@ -233,31 +274,75 @@ __global__ void __launch_bounds__(256) gram_f64(const uint16_t* omega, const dou
       sX[i][kMaxSketch + j] = y;
     }
     __syncthreads();
-    for (int i = 0; i < rows; ++i) {
-      double xv[8], yv[4];
+    if (live) {
+      for (int i = grp; i < rows; i += groups) {
+        const double2 x01 = *reinterpret_cast<const double2*>(&sX[i][xo]);
+        const double2 x23 = *reinterpret_cast<const double2*>(&sX[i][xo + 2]);
+        const double2 y01 = *reinterpret_cast<const double2*>(&sX[i][yo]);
+        const double2 y23 = *reinterpret_cast<const double2*>(&sX[i][yo + 2]);
+        const double xv[4] = {x01.x, x01.y, x23.x, x23.y};
+        const double yv[4] = {y01.x, y01.y, y23.x, y23.y};
 #pragma unroll
-      for (int a = 0; a < 8; ++a) xv[a] = sX[i][rt + 16 * a];
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) yv[b] = sX[i][kMaxSketch + ct + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(xv[a], yv[b], acc[a][b]);
+          for (int b = 0; b < 4; ++b) acc[a][b] = fma(xv[a], yv[b], acc[a][b]);
+      }
     }
   }
-  double* out = partial + (size_t)blockIdx.x * (2 * kMaxSketch) * kMaxSketch;
+  double* out = partial + ((size_t)blockIdx.x * nt + t) * 16;
+  if (groups > 1) {  // the groups' sums added in order, 16 doubles per tile at a time
+    // sX holds 4096 doubles: nt * 16 <= 512 / 2 * 16 of them, as groups > 1
+    double* s = &sX[0][0];
+    for (int g = 0; g < groups; ++g) {
+      __syncthreads();
+      if (live && grp == g) {
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) out[(rt + 16 * a) * kMaxSketch + (ct + 16 * b)] = acc[a][b];
+          for (int b = 0; b < 4; ++b) {
+            if (g > 0) acc[a][b] += s[t * 16 + a * 4 + b];
+            s[t * 16 + a * 4 + b] = acc[a][b];
+          }
+      }
+    }
+    if (!live || grp != groups - 1) return;
+  } else if (!live) {
+    return;
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) out[a * 4 + b] = acc[a][b];
 }
 
-__global__ void gram_reduce_f64(const double* partial, int G, double* out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= 2 * kMaxSketch * kMaxSketch) return;
-  double s = 0.0;
-  for (int g = 0; g < G; ++g) s += partial[(size_t)g * 2 * kMaxSketch * kMaxSketch + e];
-  out[e] = s;
+// out (128 x 64, zeroed): H in rows 0..63, G in rows 64..127, both triangles;
+// 8 threads per entry add the CTAs' partials in a fixed order
+__global__ void __launch_bounds__(256) gram_reduce_f64(const double* partial, int G, int M, double* out) {
+  __shared__ double s[8][32];
+  const int nb = (M + 3) / 4, nt = gram64_tiles(M);
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  double v = 0.0;
+  if (e < nt * 16) {
+#pragma unroll 4
+    for (int g = sl; g < G; g += 8) v += partial[(size_t)g * nt * 16 + e];
+  }
+  s[sl][lane] = v;
+  __syncthreads();
+  if (sl != 0 || e >= nt * 16) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) v += s[q][lane];
+  bool is_g;
+  int ti, tj;
+  gram64_tile(e / 16, nb, &is_g, &ti, &tj);
+  const int r = 4 * ti + (e % 16) / 4, c = 4 * tj + e % 4;
+  if (r >= M || c >= M) return;
+  if (!is_g) {
+    out[r * kMaxSketch + c] = v;
+  } else {
+    out[(kMaxSketch + r) * kMaxSketch + c] = v;
+    if (ti != tj) out[(kMaxSketch + c) * kMaxSketch + r] = v;
+  }
 }
 
 // ---------------------------------------------------------------- FP64 leave-one-out core

@@ -1,0 +1,35 @@
+"""Kernels at the sizes where their work split changes: tile edges, remainders,
+and the smallest and largest members of each range. Every result is compared
+with the oracle, or with a closed form where the graph has one, at the
+tolerance of the quantity's own parity test."""
+import numpy as np
+import pytest
+
+import wlgen
+from oracle import graph, philox, walks, xnys
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def WL(g, **kw):
+    from paper_2601_11338_gb300.api import WalkLaplacian
+    return WalkLaplacian(g.row_ptr.astype(np.int32), g.col_idx, g.n, **kw)
+
+
+# FP64 Gram: 4 x 4 tiles (M = 3, 4, 5), many copies of the tile set in a CTA
+# (M = 2), the last M with two copies and the first with one (M = 48, 52), all
+# tiles (M = 64); row counts below, at and above a 32-row stage
+@pytest.mark.parametrize("M,n", [(2, 97), (3, 97), (4, 128), (5, 97), (31, 300), (48, 700), (52, 704), (61, 700),
+                                 (64, 801)])
+def test_trace_fp64_gram_tiles(M, n):
+    g = wlgen.erdos_renyi(n, 8, 4)
+    w = WL(g, variant="nbt", alpha_rel=0.5, tol=1e-13, prec="fp64")
+    A = graph.dense_adjacency(g.row_ptr, g.col_idx, g.n)
+    phi = walks.phi_resolvent_closed(A, 1.0, w.info["alpha"])
+    est, err = w.trace(M, 900 + M)
+    Om, _ = philox.gaussian_sketch(g.n, M, 900 + M)
+    e_o, r_o, _ = xnys.xnystrace(phi, Om)
+    assert abs(est - e_o) <= 1e-10 * abs(e_o), (est, e_o)
+    assert abs(err - r_o) <= 1e-6 * r_o, (err, r_o)
+    w.close()
