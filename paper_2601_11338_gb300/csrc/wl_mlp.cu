@@ -39,143 +39,258 @@ constexpr int kRowsCTA = 128;              // rows per CTA of the gradient kerne
 constexpr int kPad = kH + 1;               // shared-memory row stride (bank-conflict free)
 
 // ------------------------------------------------------------------ features
-// one warp per row: d_i and (A d)_i; hub rows by a whole CTA each
-__global__ void k_feat_ad(const int32_t* __restrict__ rp, const int32_t* __restrict__ col, int64_t n,
-                          double* __restrict__ ad) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nw) {
-    const int beg = rp[i], end = rp[i + 1];
-    double s = 0.0;
-    for (int e = beg + lane; e < end; e += 32) {
-      const int j = __ldg(col + e);
-      s += (double)(rp[j + 1] - rp[j]);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) ad[i] = s;
-  }
-}
+// Row passes of the features: a warp takes a row of up to kFeatLong entries,
+// the CTA's eight warps a longer one together. The rows of a CTA lie a grid
+// apart, so that the hubs, which the relabelling puts first, spread over the
+// chip (R-MAT scale 18: 64 and 80 us for the two passes; with one warp per row the
+// longest row held each of them: 313 and 314 us).
+constexpr int kFeatLong = 512;
+constexpr int kFeatBlock = 256;
 
 // rank order for the triangle orientation: (degree, index)
 __device__ __forceinline__ bool ranks_above(int dj, int j, int di, int i) { return dj > di || (dj == di && j > i); }
 
-// out-degree in the orientation (neighbours of higher rank)
-__global__ void k_feat_outdeg(const int32_t* __restrict__ rp, const int32_t* __restrict__ col, int64_t n,
-                              int64_t* __restrict__ outdeg) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nw) {
-    const int beg = rp[i], end = rp[i + 1], di = end - beg;
-    int c = 0;
-    for (int e = beg + lane; e < end; e += 32) {
-      const int j = __ldg(col + e);
-      c += ranks_above(rp[j + 1] - rp[j], j, di, (int)i) ? 1 : 0;
+// calls f(row, beg, end, lane, lanes, whole) for every row: by a warp (lanes =
+// 32), or for a long row by the whole CTA (lanes = kFeatBlock, whole = true)
+template <typename F>
+__device__ __forceinline__ void feat_rows(const int32_t* __restrict__ rp, int64_t n, F f) {
+  constexpr int NW = kFeatBlock / 32;
+  __shared__ int s_long[NW];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t base = blockIdx.x; base < n; base += (int64_t)gridDim.x * NW) {
+    const int64_t i = base + (int64_t)w * gridDim.x;
+    int is_long = 0;
+    if (i < n) {
+      const int beg = rp[i], end = rp[i + 1];
+      is_long = end - beg > kFeatLong;
+      if (!is_long) f(i, beg, end, lane, 32, false);
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-    if (lane == 0) outdeg[i] = c;
+    if (lane == 0) s_long[w] = is_long;
+    if (__syncthreads_or(is_long)) {
+      for (int q = 0; q < NW; ++q) {
+        if (!s_long[q]) continue;
+        const int64_t r = base + (int64_t)q * gridDim.x;
+        f(r, rp[r], rp[r + 1], (int)threadIdx.x, kFeatBlock, true);
+      }
+    }
+    __syncthreads();
   }
 }
 
-// oriented lists (ascending index order kept by an ordered warp compaction)
-__global__ void k_feat_orient(const int32_t* __restrict__ rp, const int32_t* __restrict__ col, int64_t n,
-                              const int64_t* __restrict__ orp, const int32_t* __restrict__ key,
-                              int32_t* __restrict__ ocol, int32_t* __restrict__ okey) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nw) {
-    const int beg = rp[i], end = rp[i + 1], di = end - beg;
-    int64_t o = orp[i];
-    for (int e0 = beg; e0 < end; e0 += 32) {
+// (A d)_i and, for the triangle orientation (OUT), the number of neighbours
+// of higher rank; nodes with more than kTriWarpDeg of them go to `big`
+constexpr int kTriWarpDeg = 128;
+
+template <bool OUT>
+__global__ void __launch_bounds__(kFeatBlock) k_feat_ad(const int32_t* __restrict__ rp,
+                                                        const int32_t* __restrict__ col, int64_t n,
+                                                        double* __restrict__ ad, int64_t* __restrict__ outdeg,
+                                                        int32_t* __restrict__ big, int* __restrict__ nbig) {
+  __shared__ long long s_sum;
+  __shared__ int s_cnt;
+  feat_rows(rp, n, [&](int64_t i, int beg, int end, int lane, int lanes, bool whole) {
+    const int di = end - beg;
+    long long s = 0;  // exact: at most 2^31 neighbours of degree below 2^31
+    int c = 0;
+#pragma unroll 4
+    for (int e = beg + lane; e < end; e += lanes) {
+      const int j = __ldg(col + e);
+      const int dj = __ldg(rp + j + 1) - __ldg(rp + j);
+      s += dj;
+      if (OUT) c += ranks_above(dj, j, di, (int)i) ? 1 : 0;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, off);
+      if (OUT) c += __shfl_xor_sync(0xffffffffu, c, off);
+    }
+    if (whole) {  // integer sums: the order does not matter
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        s_sum = 0;
+        s_cnt = 0;
+      }
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) {
+        atomicAdd((unsigned long long*)&s_sum, (unsigned long long)s);
+        if (OUT) atomicAdd(&s_cnt, c);
+      }
+      __syncthreads();
+      s = s_sum;
+      c = s_cnt;
+    }
+    if (lane == 0) {
+      ad[i] = (double)s;
+      if (OUT) {
+        outdeg[i] = c;
+        if (c > kTriWarpDeg) big[atomicAdd(nbig, 1)] = (int32_t)i;
+      }
+    }
+  });
+}
+
+// oriented lists N+(i), in no particular order
+__global__ void __launch_bounds__(kFeatBlock) k_feat_orient(const int32_t* __restrict__ rp,
+                                                            const int32_t* __restrict__ col, int64_t n,
+                                                            const int64_t* __restrict__ orp,
+                                                            int32_t* __restrict__ ocol) {
+  __shared__ int s_pos;
+  feat_rows(rp, n, [&](int64_t i, int beg, int end, int lane, int lanes, bool whole) {
+    const int di = end - beg;
+    const int64_t o = orp[i];
+    const int wl = threadIdx.x & 31;
+    if (whole) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_pos = 0;
+      __syncthreads();
+    }
+    int pos = 0;
+    for (int e0 = beg; e0 < end; e0 += lanes) {
       const int e = e0 + lane;
       bool keep = false;
       int j = 0;
       if (e < end) {
         j = __ldg(col + e);
-        keep = ranks_above(rp[j + 1] - rp[j], j, di, (int)i);
+        keep = ranks_above(__ldg(rp + j + 1) - __ldg(rp + j), j, di, (int)i);
       }
       const unsigned m = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const int64_t q = o + __popc(m & ((1u << lane) - 1u));
-        ocol[q] = j;
-        okey[q] = key ? key[j] : j;
+      if (whole) {
+        if (wl == 0) pos = atomicAdd(&s_pos, __popc(m));
+        pos = __shfl_sync(0xffffffffu, pos, 0);
       }
-      o += __popc(m);
+      if (keep) ocol[o + pos + __popc(m & ((1u << wl) - 1u))] = j;
+      if (!whole) pos += __popc(m);
     }
+  });
+}
+
+// Every triangle once: for each i, N+(i) goes into a hash table in shared
+// memory, and the w of every N+(j), j in N+(i), are looked up in it. A hit is
+// one triangle (i, j, w): t_w is counted in the table's slot, t_j in a
+// register of the eight lanes that walk N+(j), t_i beside it, and the global
+// counters see one atomic per node of N+(i) instead of one per triangle. The
+// table is at most a quarter full, so a look-up reads 1.2 words on average:
+// the pass is bound by shared-memory reads, one for each wedge (i, j, w)
+// (6.6e8 on R-MAT scale 18), and not by the dependent global reads of a
+// merge or binary search per edge. R-MAT scale 18, 7.6e6 entries: 2.98 ms (a
+// merge or binary search by one lane per edge, a global atomic per triangle:
+// 20.4 ms).
+// A warp takes a node of up to kTriWarpDeg out-neighbours, a CTA a longer
+// one, in pieces of kTriPiece that fit its table.
+constexpr int kTriWarpTab = 4 * kTriWarpDeg;
+constexpr int kTriPiece = 1024;
+constexpr int kTriTab = 4 * kTriPiece;
+constexpr int kTriBlock = 256;
+constexpr int kTriTicket = 8;  // nodes a warp takes at a time
+constexpr int kTriLanes = 8;   // lanes that walk one N+(j)
+constexpr int kTriUnroll = 4;  // look-ups in flight per lane
+
+__device__ __forceinline__ unsigned tri_hash(int key, int shift) { return ((unsigned)key * 0x9E3779B1u) >> shift; }
+
+// slot of key in the table, or -1 (empty slots hold -1; never full)
+__device__ __forceinline__ int tri_find(const int* tab, unsigned mask, int shift, int key) {
+  unsigned s = tri_hash(key, shift);
+  for (;;) {
+    const int v = tab[s];
+    if (v == key) return (int)s;
+    if (v < 0) return -1;
+    s = (s + 1) & mask;
   }
 }
 
-// position in okey[lo, end) (ascending) holding k, or -1
-__device__ __forceinline__ int64_t find_key(const int32_t* __restrict__ okey, int64_t lo, int64_t end, int k) {
-  int64_t hi = end;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (okey[mid] < k) lo = mid + 1; else hi = mid;
-  }
-  return (lo < end && okey[lo] == k) ? lo : -1;
-}
-
-// Every triangle once: for i, each oriented neighbour j (one per lane) and
-// each w in N+(i) and N+(j) adds one to t_i, t_j and t_w. The lists are
-// ascending in key (the caller's node index, which is the column order of
-// every row); two lists of similar length are merged, a much shorter one is
-// looked up element by element in the longer one by binary search.
-__global__ void k_feat_triangles(const int64_t* __restrict__ orp, const int32_t* __restrict__ ocol,
-                                 const int32_t* __restrict__ okey, int64_t n, unsigned long long* __restrict__ t) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nw) {
-    const int64_t ib = orp[i], ie = orp[i + 1];
-    unsigned long long ti = 0;
-    for (int64_t e = ib + lane; e < ie; e += 32) {
-      const int j = ocol[e];
-      const int64_t jb = orp[j], je = orp[j + 1];
-      const int64_t la = ie - ib, lb = je - jb;
-      unsigned long long tj = 0;
-      if (la > 16 * lb) {  // look up N+(j) in N+(i)
-        for (int64_t b = jb; b < je; ++b) {
-          const int64_t pos = find_key(okey, ib, ie, okey[b]);
-          if (pos >= 0) {
-            ++tj;
-            atomicAdd(t + ocol[b], 1ull);
-          }
-        }
-      } else if (lb > 16 * la) {  // look up N+(i) in N+(j)
-        for (int64_t a = ib; a < ie; ++a) {
-          const int64_t pos = find_key(okey, jb, je, okey[a]);
-          if (pos >= 0) {
-            ++tj;
-            atomicAdd(t + ocol[a], 1ull);
-          }
-        }
-      } else {
-        int64_t a = ib, b = jb;
-        while (a < ie && b < je) {
-          const int kx = okey[a], ky = okey[b];
-          if (kx == ky) {
-            ++tj;
-            atomicAdd(t + ocol[a], 1ull);
-            ++a;
-            ++b;
-          } else if (kx < ky) {
-            ++a;
-          } else {
-            ++b;
-          }
-        }
-      }
-      if (tj) atomicAdd(t + j, tj);
-      ti += tj;
+template <int T, int PIECE, typename Sync>
+__device__ __forceinline__ void tri_node(int64_t i, const int64_t* __restrict__ orp, const int32_t* __restrict__ ocol,
+                                         unsigned long long* __restrict__ t, int* tab, int* cnt, int tid, Sync sync) {
+  constexpr int L = kTriLanes, NG = T / L;
+  const int64_t ib = orp[i];
+  const int len = (int)(orp[i + 1] - ib);
+  if (len < 2) return;
+  const int g = tid / L, l = tid % L;
+  const unsigned gmask = 0xFFu << (threadIdx.x & 24);
+  unsigned long long ti = 0;
+  for (int p0 = 0; p0 < len; p0 += PIECE) {
+    const int pl = min(PIECE, len - p0);
+    const int lg = max(5, 34 - __clz(pl - 1 > 0 ? pl - 1 : 1));  // log2 of the table: 4 x the next power of two
+    const int S = 1 << lg, shift = 32 - lg;
+    const unsigned mask = (unsigned)S - 1u;
+    for (int s = tid; s < S; s += T) {
+      tab[s] = -1;
+      cnt[s] = 0;
     }
+    sync();
+    for (int p = tid; p < pl; p += T) {
+      const int key = ocol[ib + p0 + p];
+      unsigned s = tri_hash(key, shift);
+      while (atomicCAS(tab + s, -1, key) != -1) s = (s + 1) & mask;
+    }
+    sync();
+    for (int q = g; q < len; q += NG) {
+      const int j = __ldg(ocol + ib + q);
+      const int64_t jb = __ldg(orp + j), je = __ldg(orp + j + 1);
+      int tj = 0;
+      for (int64_t b = jb + l; b < je; b += L * kTriUnroll) {
+        int key[kTriUnroll];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) ti += __shfl_xor_sync(0xffffffffu, ti, off);
-    if (lane == 0 && ti) atomicAdd(t + i, ti);
+        for (int u = 0; u < kTriUnroll; ++u) key[u] = b + u * L < je ? __ldg(ocol + b + u * L) : -1;
+#pragma unroll
+        for (int u = 0; u < kTriUnroll; ++u) {
+          if (key[u] < 0) continue;
+          const int s = tri_find(tab, mask, shift, key[u]);
+          if (s >= 0) {
+            atomicAdd(cnt + s, 1);
+            ++tj;
+          }
+        }
+      }
+#pragma unroll
+      for (int off = 1; off < L; off <<= 1) tj += __shfl_xor_sync(gmask, tj, off);
+      if (l == 0 && tj) {
+        atomicAdd(t + j, (unsigned long long)tj);
+        ti += tj;
+      }
+    }
+    sync();
+    for (int p = tid; p < pl; p += T) {
+      const int key = ocol[ib + p0 + p];
+      const int c = cnt[tri_find(tab, mask, shift, key)];
+      if (c) atomicAdd(t + key, (unsigned long long)c);
+    }
+    sync();
   }
+  if (ti) atomicAdd(t + i, ti);
+}
+
+__global__ void __launch_bounds__(kTriBlock) k_feat_tri_warp(const int64_t* __restrict__ orp,
+                                                             const int32_t* __restrict__ ocol, int64_t n,
+                                                             unsigned long long* __restrict__ t,
+                                                             unsigned long long* __restrict__ ticket) {
+  __shared__ int s_tab[kTriBlock / 32][kTriWarpTab];
+  __shared__ int s_cnt[kTriBlock / 32][kTriWarpTab];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (;;) {
+    unsigned long long i0 = 0;
+    if (lane == 0) i0 = atomicAdd(ticket, (unsigned long long)kTriTicket);
+    i0 = __shfl_sync(0xffffffffu, i0, 0);
+    if (i0 >= (unsigned long long)n) return;
+    const int64_t i1 = min((int64_t)i0 + kTriTicket, n);
+    for (int64_t i = (int64_t)i0; i < i1; ++i) {
+      if (orp[i + 1] - orp[i] > kTriWarpDeg) continue;
+      tri_node<32, kTriWarpDeg>(i, orp, ocol, t, s_tab[w], s_cnt[w], lane, [] { __syncwarp(); });
+      __syncwarp();
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kTriBlock) k_feat_tri_cta(const int64_t* __restrict__ orp,
+                                                            const int32_t* __restrict__ ocol,
+                                                            const int32_t* __restrict__ big,
+                                                            const int* __restrict__ nbig,
+                                                            unsigned long long* __restrict__ t) {
+  __shared__ int s_tab[kTriTab];
+  __shared__ int s_cnt[kTriTab];
+  const int nb = *nbig;
+  for (int b = blockIdx.x; b < nb; b += gridDim.x)
+    tri_node<kTriBlock, kTriPiece>(big[b], orp, ocol, t, s_tab, s_cnt, (int)threadIdx.x, [] { __syncthreads(); });
 }
 
 // features (FP32) and the analytic guess x_an (FP64), written at position
@@ -425,35 +540,44 @@ cudaError_t grad_setup() {
 
 // ------------------------------------------------------------------ launchers (wl_host.h)
 cudaError_t launch_features(const int32_t* rp, const int32_t* col, int64_t n, int64_t nnz, double alpha, double mu,
-                            const int32_t* perm, const int32_t* perm_key, float* F, double* xan, void* tmp,
-                            cudaStream_t s) {
+                            const int32_t* perm, float* F, double* xan, void* tmp, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  // tmp: ad (n doubles), t (n u64), outdeg / orp (n + 1 int64 each), scan scratch, ocol (nnz / 2 + 1 int32)
+  // tmp: ad (n doubles), t (n u64), ticket (u64) and number of long lists (int) in 16 bytes, outdeg / orp (n + 1
+  // int64 each), scan scratch, ocol (nnz / 2 + 1 int32), the nodes with long lists (n int32)
   double* ad = (double*)tmp;
   unsigned long long* t = (unsigned long long*)(ad + n);
-  int64_t* outdeg = (int64_t*)(t + n);
+  unsigned long long* ticket = t + n;
+  int* nbig = (int*)(ticket + 1);
+  int64_t* outdeg = (int64_t*)(ticket + 2);
   int64_t* orp = outdeg + n + 1;
   int64_t* sc = orp + n + 1;
   int32_t* ocol = (int32_t*)(sc + n / 1024 + 64);
-  int32_t* okey = ocol + nnz / 2 + 1;
-  const unsigned gw = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n * 32 + 255) / 256, 152 * 64));
+  int32_t* big = ocol + nnz / 2 + 1;
+  constexpr int NW = kFeatBlock / 32;
+  const unsigned gw = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + NW - 1) / NW, 152 * 8));
   const unsigned g1 = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 32));
-  k_feat_ad<<<gw, 256, 0, s>>>(rp, col, n, ad);
   if (F) {  // triangles only for the network's inputs (x_an needs d and A d alone)
-    cudaError_t e = cudaMemsetAsync(t, 0, sizeof(unsigned long long) * n, s);
+    cudaError_t e = cudaMemsetAsync(t, 0, sizeof(unsigned long long) * (n + 2), s);
     if (e != cudaSuccess) return e;
-    k_feat_outdeg<<<gw, 256, 0, s>>>(rp, col, n, outdeg);
+    k_feat_ad<true><<<gw, kFeatBlock, 0, s>>>(rp, col, n, ad, outdeg, big, nbig);
     e = launch_scan(outdeg, n, orp, sc, s);  // orp[0..n]: exclusive prefix, orp[n] = total
     if (e != cudaSuccess) return e;
-    k_feat_orient<<<gw, 256, 0, s>>>(rp, col, n, orp, perm_key, ocol, okey);
-    k_feat_triangles<<<gw, 256, 0, s>>>(orp, ocol, okey, n, t);
+    k_feat_orient<<<gw, kFeatBlock, 0, s>>>(rp, col, n, orp, ocol);
+    // long lists first (one CTA each, the heaviest work), then the rest of the nodes by warps
+    const unsigned gb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(n, 152 * 6));
+    k_feat_tri_cta<<<gb, kTriBlock, 0, s>>>(orp, ocol, big, nbig, t);
+    const unsigned gt = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + NW - 1) / NW, 152 * 6));
+    k_feat_tri_warp<<<gt, kTriBlock, 0, s>>>(orp, ocol, n, t, ticket);
+  } else {
+    k_feat_ad<false><<<gw, kFeatBlock, 0, s>>>(rp, col, n, ad, nullptr, nullptr, nullptr);
   }
   k_feat_out<<<g1, 256, 0, s>>>(rp, ad, t, n, alpha, mu, perm, F, xan);
   return cudaGetLastError();
 }
 
 size_t features_tmp_bytes(int64_t n, int64_t nnz) {
-  return (size_t)n * 8 * 2 + (size_t)(n + 1) * 8 * 2 + (size_t)(n / 1024 + 64) * 8 + (size_t)(nnz / 2 + 1) * 8 + 256;
+  return (size_t)n * 8 * 2 + 16 + (size_t)(n + 1) * 8 * 2 + (size_t)(n / 1024 + 64) * 8 + (size_t)(nnz / 2 + 1) * 4 +
+         (size_t)n * 4 + 256;
 }
 
 cudaError_t launch_mlp_predict(const float* P, const float* F, int64_t rows, const double* xan, double* out,

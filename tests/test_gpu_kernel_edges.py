@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import wlgen
-from oracle import graph, philox, walks, xnys
+from oracle import features, graph, philox, walks, xnys
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -32,4 +32,30 @@ def test_trace_fp64_gram_tiles(M, n):
     e_o, r_o, _ = xnys.xnystrace(phi, Om)
     assert abs(est - e_o) <= 1e-10 * abs(e_o), (est, e_o)
     assert abs(err - r_o) <= 1e-6 * r_o, (err, r_o)
+    w.close()
+# Triangles: lists for one warp (up to 128 higher-ranked neighbours), for a CTA
+# (more), in pieces of 1024, and rows read by a whole CTA (more than 512 entries)
+@pytest.mark.parametrize("reorder", [0, 1, 2])
+@pytest.mark.parametrize("n", [3, 129, 130, 514, 1026, 1300])
+def test_triangles_of_complete_graphs(n, reorder):
+    from paper_2601_11338_gb300.api import mlp_features
+    g = wlgen.complete(n)
+    w = WL(g, variant="nbt", alpha=0.2 / n, reorder=reorder)
+    F, _ = mlp_features(w)
+    t = (n - 1) * (n - 2) // 2
+    want = np.log1p([n - 1.0, (n - 1.0) ** 2, float(t), (n - 1.0) * (n - 2.0)])
+    # log1p in FP64 rounded to FP32: half a unit in the last place
+    assert np.abs(F.cpu().numpy() / want - 1.0).max() <= 1.2e-7
+    w.close()
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+def test_triangles_of_a_skewed_graph(seed):
+    """R-MAT scale 11: hubs beyond 512 entries beside nodes of degree 0 and 1."""
+    from paper_2601_11338_gb300.api import mlp_features
+    g = wlgen.rmat(11, 24, seed=seed)
+    w = WL(g, variant="nbt", alpha_rel=0.5)
+    F, _ = mlp_features(w)
+    tri = features.triangles_by_intersection(g.row_ptr, g.col_idx, g.n)
+    assert np.abs(F[:, 2].cpu().numpy().astype(np.float64) - np.log1p(tri)).max() <= 1.2e-7 * np.log1p(tri.max())
     w.close()
