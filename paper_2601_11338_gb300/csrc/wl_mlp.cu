@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "wl.h"
+#include "wl_df.cuh"
 #include "wl_host.h"
 
 namespace wl {
@@ -35,8 +36,7 @@ constexpr int kOffMean = 0, kOffStd = 4, kOffW1 = 8, kOffB1 = kOffW1 + kH * kIn,
               kOffB2 = kOffW2 + kH * kH, kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH;
 constexpr int kParams = kOffB3 + 1;        // 4553
 constexpr int kTrain = kParams - kOffW1;   // 4545 trainable values (after the standardisation)
-constexpr int kRowsCTA = 128;              // rows per CTA of the gradient kernel
-constexpr int kPad = kH + 1;               // shared-memory row stride (bank-conflict free)
+constexpr int kRowsCTA = 128;              // rows per tile of the network kernels
 
 // ------------------------------------------------------------------ features
 // Row passes of the features: a warp takes a row of up to kFeatLong entries,
@@ -315,160 +315,364 @@ __global__ void k_feat_out(const int32_t* __restrict__ rp, const double* __restr
 }
 
 // ------------------------------------------------------------------ network
-__device__ __forceinline__ void load_params(const float* __restrict__ P, float* s) {
-  for (int i = threadIdx.x; i < kParams; i += blockDim.x) s[i] = P[i];
+// Both network kernels take kRowsCTA rows at a time as small matrix products
+// in shared memory (rows x 64 by 64 x 64) with eight rows and four units per
+// thread in packed FP32 pairs (fma.rn.f32x2: two IEEE fused multiply-adds an
+// instruction), so that a k step costs 16 packed products for three vector
+// reads; the FP32 pipe bounds them. FP32 throughout, as the parity tests ask
+// (TF32 tensor cores would drop 13 bits).
+constexpr int kMlpThreads = 256;
+constexpr int kMlpPitch = kRowsCTA + 4;  // unit-major tiles [64][kMlpPitch]: 16-byte rows, distinct banks
+constexpr int kWPitch = kH + 4;
+
+typedef unsigned long long f2x;  // two FP32 values, the lower address in the lower half
+__device__ __forceinline__ f2x f2_pack(float lo, float hi) {
+  f2x r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(f2x v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
+  f2x d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+struct alignas(16) MlpTile {
+  float h1[kH * kMlpPitch];   // tanh of layer 1, [unit][row]
+  float w2t[kH * kWPitch];    // W2 transposed, [k][j]
+  float x[kRowsCTA * kIn];    // standardised inputs
+  float head[kOffW2 + 8];     // mean, std, W1, b1
+  float b2[kH], w3[kH];
+  float b3;
+};
+static_assert(sizeof(MlpTile) % 16 == 0, "vector access to what follows it");
+
+__device__ __forceinline__ void mlp_load(const float* __restrict__ P, MlpTile& t) {
+  for (int i = threadIdx.x; i < kOffW2; i += kMlpThreads) t.head[i] = P[i];
+  for (int i = threadIdx.x; i < kH * kH; i += kMlpThreads) t.w2t[(i % kH) * kWPitch + i / kH] = P[kOffW2 + i];
+  if (threadIdx.x < kH) {
+    t.b2[threadIdx.x] = P[kOffB2 + threadIdx.x];
+    t.w3[threadIdx.x] = P[kOffW3 + threadIdx.x];
+  }
+  if (threadIdx.x == 0) t.b3 = P[kOffB3];
   __syncthreads();
 }
 
-// y (per row) of the perceptron; x0 = exp(y) * xan (xan may be NULL: x0 = y)
-__global__ void __launch_bounds__(128) k_mlp_predict(const float* __restrict__ P, const float* __restrict__ F,
-                                                      int64_t rows, const double* __restrict__ xan,
-                                                      double* __restrict__ out) {
-  __shared__ float s[kParams];
-  load_params(P, s);
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
-    float x[kIn];
+// Forward pass of rows [r0, r0 + kRowsCTA) below `rows`: thread (ty, tx) =
+// (tid / 16, tid % 16) gets h2 of rows 8 ty .. 8 ty + 7 and units 4 tx .. 4 tx
+// + 3. Rows past the end are computed on zero inputs.
+__device__ __forceinline__ void mlp_forward(const float* __restrict__ F, int64_t r0, int64_t rows, MlpTile& t,
+                                            float (&h2)[8][4]) {
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  {
+    // layer 1: two threads per row, 32 units each
+    const int rr = tid & (kRowsCTA - 1), half = tid / kRowsCTA;
+    float x[kIn] = {0.f, 0.f, 0.f, 0.f};
+    if (r0 + rr < rows) {
 #pragma unroll
-    for (int c = 0; c < kIn; ++c) x[c] = (F[r * 4 + c] - s[kOffMean + c]) / s[kOffStd + c];
-    // z2 accumulated over the hidden units of layer 1, each computed once
-    float z2[kH];
-#pragma unroll
-    for (int j = 0; j < kH; ++j) z2[j] = s[kOffB2 + j];
-#pragma unroll 1
-    for (int k = 0; k < kH; ++k) {
-      float z = s[kOffB1 + k];
-#pragma unroll
-      for (int c = 0; c < kIn; ++c) z = fmaf(s[kOffW1 + k * kIn + c], x[c], z);
-      const float h = tanhf(z);
-#pragma unroll
-      for (int j = 0; j < kH; ++j) z2[j] = fmaf(s[kOffW2 + j * kH + k], h, z2[j]);
+      for (int c = 0; c < kIn; ++c) x[c] = (F[(r0 + rr) * 4 + c] - t.head[kOffMean + c]) / t.head[kOffStd + c];
     }
-    float y = s[kOffB3];
+    if (half == 0)
 #pragma unroll
-    for (int j = 0; j < kH; ++j) y = fmaf(s[kOffW3 + j], tanhf(z2[j]), y);
-    out[r] = xan ? xan[r] * exp((double)y) : (double)y;
+      for (int c = 0; c < kIn; ++c) t.x[rr * kIn + c] = x[c];
+#pragma unroll 4
+    for (int k = half * (kH / 2); k < (half + 1) * (kH / 2); ++k) {
+      float z = t.head[kOffB1 + k];
+#pragma unroll
+      for (int c = 0; c < kIn; ++c) z = fmaf(t.head[kOffW1 + k * kIn + c], x[c], z);
+      t.h1[k * kMlpPitch + rr] = tanhf(z);
+    }
+  }
+  __syncthreads();
+  f2x acc[4][4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float b = t.b2[4 * tx + c];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) acc[p][c] = f2_pack(b, b);
+  }
+#pragma unroll 4
+  for (int k = 0; k < kH; ++k) {
+    const ulonglong2 a01 = *reinterpret_cast<const ulonglong2*>(&t.h1[k * kMlpPitch + 8 * ty]);
+    const ulonglong2 a23 = *reinterpret_cast<const ulonglong2*>(&t.h1[k * kMlpPitch + 8 * ty + 4]);
+    const float4 w = *reinterpret_cast<const float4*>(&t.w2t[k * kWPitch + 4 * tx]);
+    const f2x av[4] = {a01.x, a01.y, a23.x, a23.y};
+    const f2x wv[4] = {f2_pack(w.x, w.x), f2_pack(w.y, w.y), f2_pack(w.z, w.z), f2_pack(w.w, w.w)};
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[p][c] = f2_fma(av[p], wv[c], acc[p][c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const float2 z = f2_unpack(acc[p][c]);
+      h2[2 * p][c] = tanhf(z.x);
+      h2[2 * p + 1][c] = tanhf(z.y);
+    }
+}
+
+// h2 into a unit-major tile
+__device__ __forceinline__ void mlp_store_h2(const float (&h2)[8][4], float* tile) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float4* o = reinterpret_cast<float4*>(tile + (4 * tx + c) * kMlpPitch + 8 * ty);
+    o[0] = make_float4(h2[0][c], h2[1][c], h2[2][c], h2[3][c]);
+    o[1] = make_float4(h2[4][c], h2[5][c], h2[6][c], h2[7][c]);
   }
 }
 
-// Forward and backward over kRowsCTA rows of [row0, row0 + rows); writes the
-// CTA's gradient partial (kTrain values, layout of the trainable parameters)
-// and its sum of squared errors to part[blockIdx.x * (kTrain + 1) ...].
+// y of one row from the h2 tile, the units in order
+__device__ __forceinline__ float mlp_output(const MlpTile& t, const float* tile, int row) {
+  float y = t.b3;
+#pragma unroll 16
+  for (int j = 0; j < kH; ++j) y = fmaf(t.w3[j], tile[j * kMlpPitch + row], y);
+  return y;
+}
+
+// y (per row) of the perceptron; x0 = exp(y) * xan (xan may be NULL: x0 = y).
+// 200003 rows: 57 us (a thread per row reading one weight per product
+// from shared memory: 112 us).
+__global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_predict(const float* __restrict__ P,
+                                                                const float* __restrict__ F, int64_t rows,
+                                                                const double* __restrict__ xan,
+                                                                double* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MlpTile& t = *reinterpret_cast<MlpTile*>(smem_raw);
+  mlp_load(P, t);
+  for (int64_t r0 = (int64_t)blockIdx.x * kRowsCTA; r0 < rows; r0 += (int64_t)gridDim.x * kRowsCTA) {
+    float h2[8][4];
+    mlp_forward(F, r0, rows, t, h2);
+    __syncthreads();  // h1 has been read
+    mlp_store_h2(h2, t.h1);
+    __syncthreads();
+    const int64_t r = r0 + threadIdx.x;
+    if (threadIdx.x < kRowsCTA && r < rows) {
+      const double v = (double)mlp_output(t, t.h1, threadIdx.x);
+      out[r] = xan ? xan[r] * exp(v) : v;
+    }
+    __syncthreads();  // h1 is rewritten by the next tile
+  }
+}
+
+// Forward and backward over the rows [row0, row0 + rows) in tiles of
+// kRowsCTA, `tiles` consecutive tiles per CTA (at most kGradTiles); writes
+// the CTA's gradient (kTrain values, layout of the trainable parameters) and
+// its sum of squared errors, FP64, to part[blockIdx.x * (kTrain + 1) ...].
 // Loss L = (1/B) sum (y - t)^2 over the B rows of the batch.
-__global__ void __launch_bounds__(kRowsCTA) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ F,
-                                                        const float* __restrict__ T, int64_t row0, int64_t rows,
-                                                        double inv_b, float* __restrict__ part) {
-  extern __shared__ float sm[];
-  float* s = sm;                            // parameters
-  float* s_h1 = s + kParams + 3;            // [kRowsCTA][kPad]
-  float* s_h2 = s_h1 + kRowsCTA * kPad;     // [kRowsCTA][kPad]
-  float* s_g2 = s_h2 + kRowsCTA * kPad;     // dL/dz2
-  float* s_g1 = s_g2 + kRowsCTA * kPad;     // dL/dz1
-  float* s_x = s_g1 + kRowsCTA * kPad;      // [kRowsCTA][4] standardised inputs
-  float* s_gy = s_x + kRowsCTA * kIn;       // [kRowsCTA]
-  load_params(P, s);
-  const int tid = threadIdx.x;
-  const int64_t r = row0 + (int64_t)blockIdx.x * kRowsCTA + tid;
-  const bool live = (int64_t)blockIdx.x * kRowsCTA + tid < rows;
-  float* h1r = s_h1 + tid * kPad;
-  float* h2r = s_h2 + tid * kPad;
-  float* g2r = s_g2 + tid * kPad;
-  float* g1r = s_g1 + tid * kPad;
-  float gy = 0.f, sq = 0.f;
-  if (live) {
-    float x[kIn];
+// Three products per tile: z2 = h1 W2^T, dL/dh1 = g2 W2 and dW2 = g2^T h1 (g2 =
+// dL/dz2). dW2 is summed in FP32 over a tile and in double-float across the
+// CTA's tiles; the other gradients are summed per thread in FP32 over its 8
+// rows of each tile (at most 128 rows) and in double-float over the threads.
+// 200003 rows: 172 us for this and the reduction (a thread per row with
+// its activations in shared memory, four warps per SM, and a partial per 128
+// rows: 602 us and 224 us for the reduction of the partials).
+constexpr int kGradTiles = 16;
+
+struct alignas(16) MlpGradSmem {
+  MlpTile t;
+  float g2[kH * kMlpPitch];  // dL/dz2, [unit][row]
+  float w2[kH * kWPitch];    // [j][k]
+  float sq[kRowsCTA], gy[kRowsCTA];
+};
+
+__global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ F,
+                                                             const float* __restrict__ T, int64_t row0, int64_t rows,
+                                                             int tiles, double inv_b, double* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MlpGradSmem& s = *reinterpret_cast<MlpGradSmem*>(smem_raw);
+  MlpTile& t = s.t;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  for (int i = tid; i < kH * kH; i += kMlpThreads) s.w2[(i / kH) * kWPitch + i % kH] = P[kOffW2 + i];
+  mlp_load(P, t);
+  F += row0 * 4;
+  T += row0;
+  float dw2h[4][4], dw2l[4][4];  // j = ty + 16 a, k = tx + 16 b
+  float dw1[4][4], db1[4];       // k = 4 tx + a, input b
+  float db2[4], dw3[4];          // unit 4 tx + a
+  float db3 = 0.f;
+  double sq = 0.0;               // thread 0
 #pragma unroll
-    for (int c = 0; c < kIn; ++c) {
-      x[c] = (F[r * 4 + c] - s[kOffMean + c]) / s[kOffStd + c];
-      s_x[tid * kIn + c] = x[c];
-    }
-#pragma unroll 8
-    for (int k = 0; k < kH; ++k) {
-      float z = s[kOffB1 + k];
+  for (int a = 0; a < 4; ++a) {
+    db1[a] = db2[a] = dw3[a] = 0.f;
 #pragma unroll
-      for (int c = 0; c < kIn; ++c) z = fmaf(s[kOffW1 + k * kIn + c], x[c], z);
-      h1r[k] = tanhf(z);
-    }
-    float y = s[kOffB3];
-    for (int j = 0; j < kH; ++j) {
-      float z = s[kOffB2 + j];
-      for (int k = 0; k < kH; ++k) z = fmaf(s[kOffW2 + j * kH + k], h1r[k], z);
-      const float h = tanhf(z);
-      h2r[j] = h;
-      y = fmaf(s[kOffW3 + j], h, y);
-    }
-    const float e = y - T[r];
-    sq = e * e;
-    gy = (float)(2.0 * inv_b) * e;
-    for (int j = 0; j < kH; ++j) g2r[j] = gy * s[kOffW3 + j] * (1.f - h2r[j] * h2r[j]);
-    for (int k = 0; k < kH; ++k) {
-      float gh = 0.f;
-      for (int j = 0; j < kH; ++j) gh = fmaf(g2r[j], s[kOffW2 + j * kH + k], gh);
-      g1r[k] = gh * (1.f - h1r[k] * h1r[k]);
-    }
-  } else {
-    for (int k = 0; k < kH; ++k) {
-      h1r[k] = h2r[k] = g2r[k] = g1r[k] = 0.f;
-    }
-#pragma unroll
-    for (int c = 0; c < kIn; ++c) s_x[tid * kIn + c] = 0.f;
+    for (int b = 0; b < 4; ++b) dw2h[a][b] = dw2l[a][b] = dw1[a][b] = 0.f;
   }
-  s_gy[tid] = gy;
-  // squared error of the CTA (fixed order)
-  __shared__ float s_sq[kRowsCTA];
-  s_sq[tid] = sq;
+  const int64_t tile0 = (int64_t)blockIdx.x * tiles;
+  for (int q = 0; q < tiles; ++q) {
+    const int64_t r0 = (tile0 + q) * kRowsCTA;
+    if (r0 >= rows) break;
+    {
+      float h2[8][4];
+      mlp_forward(F, r0, rows, t, h2);
+      mlp_store_h2(h2, s.g2);
+      __syncthreads();
+      if (tid < kRowsCTA) {
+        const float e = r0 + tid < rows ? mlp_output(t, s.g2, tid) - T[r0 + tid] : 0.f;
+        s.sq[tid] = e * e;
+        s.gy[tid] = (float)(2.0 * inv_b) * e;
+      }
+      __syncthreads();
+      if (tid == 0) {  // the tile's squared error, its rows in order
+        float v = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < kRowsCTA; ++r) v += s.sq[r];
+        sq += (double)v;
+      }
+      float gy[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        gy[r] = s.gy[8 * ty + r];
+        db3 += gy[r];
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float w = t.w3[4 * tx + c];
+        float g[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          dw3[c] = fmaf(gy[r], h2[r][c], dw3[c]);
+          g[r] = gy[r] * w * (1.f - h2[r][c] * h2[r][c]);
+          db2[c] += g[r];
+        }
+        float4* o = reinterpret_cast<float4*>(&s.g2[(4 * tx + c) * kMlpPitch + 8 * ty]);
+        o[0] = make_float4(g[0], g[1], g[2], g[3]);
+        o[1] = make_float4(g[4], g[5], g[6], g[7]);
+      }
+    }
+    __syncthreads();
+    {  // dL/dh1 = g2 W2, then dL/dz1, dW1 and db1
+      f2x acc[4][4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[p][c] = 0ull;
+#pragma unroll 4
+      for (int j = 0; j < kH; ++j) {
+        const ulonglong2 a01 = *reinterpret_cast<const ulonglong2*>(&s.g2[j * kMlpPitch + 8 * ty]);
+        const ulonglong2 a23 = *reinterpret_cast<const ulonglong2*>(&s.g2[j * kMlpPitch + 8 * ty + 4]);
+        const float4 w = *reinterpret_cast<const float4*>(&s.w2[j * kWPitch + 4 * tx]);
+        const f2x av[4] = {a01.x, a01.y, a23.x, a23.y};
+        const f2x wv[4] = {f2_pack(w.x, w.x), f2_pack(w.y, w.y), f2_pack(w.z, w.z), f2_pack(w.w, w.w)};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[p][c] = f2_fma(av[p], wv[c], acc[p][c]);
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const float4 x0 = *reinterpret_cast<const float4*>(&t.x[(8 * ty + 2 * p) * kIn]);
+        const float4 x1 = *reinterpret_cast<const float4*>(&t.x[(8 * ty + 2 * p + 1) * kIn]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float2 gh = f2_unpack(acc[p][c]);
+          const float2 h = *reinterpret_cast<const float2*>(&t.h1[(4 * tx + c) * kMlpPitch + 8 * ty + 2 * p]);
+          const float g0 = gh.x * (1.f - h.x * h.x), g1 = gh.y * (1.f - h.y * h.y);
+          db1[c] += g0 + g1;
+          dw1[c][0] = fmaf(g1, x1.x, fmaf(g0, x0.x, dw1[c][0]));
+          dw1[c][1] = fmaf(g1, x1.y, fmaf(g0, x0.y, dw1[c][1]));
+          dw1[c][2] = fmaf(g1, x1.z, fmaf(g0, x0.z, dw1[c][2]));
+          dw1[c][3] = fmaf(g1, x1.w, fmaf(g0, x0.w, dw1[c][3]));
+        }
+      }
+    }
+    {  // dW2 = g2^T h1: even and odd rows in the halves of each pair
+      f2x acc[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0ull;
+#pragma unroll 2
+      for (int r = 0; r < kRowsCTA; r += 4) {
+        ulonglong2 g[4], hh[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          g[a] = *reinterpret_cast<const ulonglong2*>(&s.g2[(ty + 16 * a) * kMlpPitch + r]);
+          hh[a] = *reinterpret_cast<const ulonglong2*>(&t.h1[(tx + 16 * a) * kMlpPitch + r]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[a][b] = f2_fma(g[a].y, hh[b].y, f2_fma(g[a].x, hh[b].x, acc[a][b]));
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float2 v = f2_unpack(acc[a][b]);
+          df_acc(dw2h[a][b], dw2l[a][b], v.x + v.y);
+        }
+    }
+    __syncthreads();  // h1, g2 and x are rewritten by the next tile
+  }
+  double* out = part + (size_t)blockIdx.x * (kTrain + 1);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      out[kOffW2 - kOffW1 + (ty + 16 * a) * kH + tx + 16 * b] = (double)dw2h[a][b] + (double)dw2l[a][b];
+  // the other gradients: 16 threads (ty) hold parts of each; red[v][ty][tx]
+  float* red = s.g2;
+  constexpr int NV = 29;
+  static_assert(NV * kMlpThreads <= kH * kMlpPitch, "reduction fits in g2");
+  auto put = [&](int v, float x) { red[v * kMlpThreads + tid] = x; };
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) put(a * 4 + b, dw1[a][b]);
+    put(16 + a, db1[a]);
+    put(20 + a, db2[a]);
+    put(24 + a, dw3[a]);
+  }
+  put(28, db3);
   __syncthreads();
-  float* out = part + (size_t)blockIdx.x * (kTrain + 1);
-  const int nr = kRowsCTA;
-  // W1 (256) and b1 (64): entries j*4 + c and j
-  for (int q = tid; q < kH * kIn + kH; q += blockDim.x) {
-    float acc = 0.f;
-    if (q < kH * kIn) {
-      const int j = q / kIn, c = q % kIn;
-      for (int rr = 0; rr < nr; ++rr) acc = fmaf(s_g1[rr * kPad + j], s_x[rr * kIn + c], acc);
-    } else {
-      const int j = q - kH * kIn;
-      for (int rr = 0; rr < nr; ++rr) acc += s_g1[rr * kPad + j];
-    }
-    out[q] = acc;
+  for (int e = tid; e < NV * 16; e += kMlpThreads) {
+    const int v = e / 16, u = e % 16;  // u: tx
+    float h = 0.f, l = 0.f;
+    for (int g = 0; g < 16; ++g) df_acc(h, l, red[v * kMlpThreads + g * 16 + u]);
+    const double d = (double)h + (double)l;
+    if (v < 16)
+      out[(4 * u + v / 4) * kIn + v % 4] = d;
+    else if (v < 20)
+      out[kOffB1 - kOffW1 + 4 * u + v - 16] = d;
+    else if (v < 24)
+      out[kOffB2 - kOffW1 + 4 * u + v - 20] = d;
+    else if (v < 28)
+      out[kOffW3 - kOffW1 + 4 * u + v - 24] = d;
+    else if (u == 0)  // every tx holds the same rows
+      out[kOffB3 - kOffW1] = d;
   }
-  // W2 (4096): entry j*64 + k = sum_r g2[r][j] h1[r][k]
-  for (int q = tid; q < kH * kH; q += blockDim.x) {
-    const int j = q / kH, k = q % kH;
-    float acc = 0.f;
-    for (int rr = 0; rr < nr; ++rr) acc = fmaf(s_g2[rr * kPad + j], s_h1[rr * kPad + k], acc);
-    out[kOffW2 - kOffW1 + q] = acc;
-  }
-  // b2, W3, b3
-  for (int q = tid; q < 2 * kH + 1; q += blockDim.x) {
-    float acc = 0.f;
-    if (q < kH) {
-      for (int rr = 0; rr < nr; ++rr) acc += s_g2[rr * kPad + q];
-      out[kOffB2 - kOffW1 + q] = acc;
-    } else if (q < 2 * kH) {
-      const int j = q - kH;
-      for (int rr = 0; rr < nr; ++rr) acc = fmaf(s_gy[rr], s_h2[rr * kPad + j], acc);
-      out[kOffW3 - kOffW1 + j] = acc;
-    } else {
-      for (int rr = 0; rr < nr; ++rr) acc += s_gy[rr];
-      out[kOffB3 - kOffW1] = acc;
-    }
-  }
-  if (tid == 0) {
-    float t = 0.f;
-    for (int rr = 0; rr < nr; ++rr) t += s_sq[rr];
-    out[kTrain] = t;
-  }
+  if (tid == 0) out[kTrain] = sq;
 }
 
-// Sums the CTA partials in a fixed order (FP64). mode 0: write the gradient
-// and loss; mode 1: Adam update of the trainable parameters (m, v state).
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, double inv_b, float* __restrict__ P,
-                             float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
-                             double bc1, double bc2, int mode, float* __restrict__ grad, double* __restrict__ loss) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q > kTrain) return;
+// Sums the CTA partials in a fixed order (FP64), eight threads per value. mode
+// 0: write the gradient and loss; mode 1: Adam update of the trainable
+// parameters (m, v state).
+__global__ void __launch_bounds__(256) k_mlp_reduce(const double* __restrict__ part, int nblk, double inv_b,
+                                                    float* __restrict__ P, float* __restrict__ m,
+                                                    float* __restrict__ v, float lr, float b1, float b2, float eps,
+                                                    double bc1, double bc2, int mode, float* __restrict__ grad,
+                                                    double* __restrict__ loss) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + lane;
   double g = 0.0;
-  for (int c = 0; c < nblk; ++c) g += (double)part[(size_t)c * (kTrain + 1) + q];
+  if (q <= kTrain) {
+#pragma unroll 4
+    for (int c = sl; c < nblk; c += 8) g += part[(size_t)c * (kTrain + 1) + q];
+  }
+  red[sl][lane] = g;
+  __syncthreads();
+  if (sl != 0 || q > kTrain) return;
+#pragma unroll
+  for (int c = 1; c < 8; ++c) g += red[c][lane];
   if (q == kTrain) {
     if (loss) *loss = g * inv_b;
     return;
@@ -485,6 +689,7 @@ __global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, double in
   const double mh = (double)mm / bc1, vh = (double)vv / bc2;
   P[kOffW1 + q] = (float)((double)P[kOffW1 + q] - (double)lr * mh / (sqrt(vh) + (double)eps));
 }
+constexpr int kReduceBlocks = (kTrain + 1 + 31) / 32;
 
 // feature means and standard deviations (FP64 partial sums per CTA)
 __global__ void k_mlp_stats_part(const float* __restrict__ F, int64_t rows, double* __restrict__ part) {
@@ -528,14 +733,25 @@ __global__ void k_log_ratio(const double* __restrict__ Df, const double* __restr
     t[r] = (float)log(Df[r] / xan[r]);
 }
 
-size_t grad_smem() { return sizeof(float) * (kParams + 3 + 4 * kRowsCTA * kPad + kRowsCTA * kIn + kRowsCTA); }
-
-cudaError_t grad_setup() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem());
-  if (e == cudaSuccess) done = true;
+cudaError_t mlp_setup() {
+  static const cudaError_t e = [] {
+    cudaError_t r = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(MlpGradSmem));
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(k_mlp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
+    return r;
+  }();
   return e;
+}
+
+// CTAs of a gradient pass: up to two per SM, each with at most kGradTiles tiles
+int grad_tiles(int64_t rows) {
+  const int64_t tiles = (rows + kRowsCTA - 1) / kRowsCTA;
+  return (int)std::min<int64_t>(kGradTiles, std::max<int64_t>(1, (tiles + 2 * 152 - 1) / (2 * 152)));
+}
+int grad_blocks(int64_t rows) {
+  const int64_t tiles = (rows + kRowsCTA - 1) / kRowsCTA;
+  return (int)((tiles + grad_tiles(rows) - 1) / grad_tiles(rows));
 }
 
 // ------------------------------------------------------------------ launchers (wl_host.h)
@@ -583,8 +799,10 @@ size_t features_tmp_bytes(int64_t n, int64_t nnz) {
 cudaError_t launch_mlp_predict(const float* P, const float* F, int64_t rows, const double* xan, double* out,
                                cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
-  const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, 152 * 16));
-  k_mlp_predict<<<g, 128, 0, s>>>(P, F, rows, xan, out);
+  const cudaError_t e = mlp_setup();
+  if (e != cudaSuccess) return e;
+  const unsigned g = (unsigned)std::min<int64_t>((rows + kRowsCTA - 1) / kRowsCTA, 152 * 3);
+  k_mlp_predict<<<g, kMlpThreads, sizeof(MlpTile), s>>>(P, F, rows, xan, out);
   return cudaGetLastError();
 }
 
@@ -637,11 +855,11 @@ int stage(const void* src, size_t bytes, DevBuf& own, const void** dev, cudaStre
 }
 
 // gradient partials over rows [row0, row0 + rows)
-int grad_pass(const float* P, const float* F, const float* T, int64_t row0, int64_t rows, float* part,
+int grad_pass(const float* P, const float* F, const float* T, int64_t row0, int64_t rows, double* part,
               cudaStream_t s) {
-  ML_CU(grad_setup());
-  const int nb = (int)((rows + kRowsCTA - 1) / kRowsCTA);
-  k_mlp_grad<<<nb, kRowsCTA, grad_smem(), s>>>(P, F, T, row0, rows, 1.0 / (double)rows, part);
+  ML_CU(mlp_setup());
+  k_mlp_grad<<<grad_blocks(rows), kMlpThreads, sizeof(MlpGradSmem), s>>>(P, F, T, row0, rows, grad_tiles(rows),
+                                                                       1.0 / (double)rows, part);
   ML_CU(cudaGetLastError());
   return WL_OK;
 }
@@ -660,13 +878,13 @@ int wl_mlp_loss_grad(const float* params, const float* feats, const float* targe
   if ((rc = stage(params, sizeof(float) * kParams, bp, &P, s)) != WL_OK) return rc;
   if ((rc = stage(feats, sizeof(float) * 4 * rows, bf, &F, s)) != WL_OK) return rc;
   if ((rc = stage(target, sizeof(float) * rows, bt, &T, s)) != WL_OK) return rc;
-  const int nb = (int)((rows + kRowsCTA - 1) / kRowsCTA);
-  ML_CU(bpart.alloc(sizeof(float) * (size_t)nb * (kTrain + 1)));
+  const int nb = grad_blocks(rows);
+  ML_CU(bpart.alloc(sizeof(double) * (size_t)nb * (kTrain + 1)));
   ML_CU(bg.alloc(sizeof(float) * kTrain));
   ML_CU(bl.alloc(sizeof(double)));
-  if ((rc = grad_pass((const float*)P, (const float*)F, (const float*)T, 0, rows, (float*)bpart.p, s)) != WL_OK)
+  if ((rc = grad_pass((const float*)P, (const float*)F, (const float*)T, 0, rows, (double*)bpart.p, s)) != WL_OK)
     return rc;
-  k_mlp_reduce<<<(kTrain + 1 + 255) / 256, 256, 0, s>>>((const float*)bpart.p, nb, 1.0 / (double)rows, nullptr,
+  k_mlp_reduce<<<kReduceBlocks, 256, 0, s>>>((const double*)bpart.p, nb, 1.0 / (double)rows, nullptr,
                                                        nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 1.0, 1.0, 0,
                                                        (float*)bg.p, (double*)bl.p);
   ML_CU(cudaGetLastError());
@@ -701,8 +919,7 @@ int wl_mlp_train(float* params, const float* feats, const float* target, int64_t
     k_mlp_stats_fin<<<1, 32, 0, s>>>((const double*)bst.p, sb, rows, P);
     ML_CU(cudaGetLastError());
   }
-  const int nb_max = (int)((batch + kRowsCTA - 1) / kRowsCTA);
-  ML_CU(bpart.alloc(sizeof(float) * (size_t)std::max(nb_max, (int)((rows + kRowsCTA - 1) / kRowsCTA)) * (kTrain + 1)));
+  ML_CU(bpart.alloc(sizeof(double) * (size_t)std::max(grad_blocks(batch), grad_blocks(rows)) * (kTrain + 1)));
   ML_CU(bm.alloc(sizeof(float) * kTrain));
   ML_CU(bv.alloc(sizeof(float) * kTrain));
   ML_CU(bl.alloc(sizeof(double)));
@@ -712,9 +929,9 @@ int wl_mlp_train(float* params, const float* feats, const float* target, int64_t
   int64_t off = 0;
   for (int it = 1; it <= steps; ++it) {
     if (off + batch > rows) off = 0;
-    if ((rc = grad_pass(P, (const float*)F, (const float*)T, off, batch, (float*)bpart.p, s)) != WL_OK) return rc;
-    const int nb = (int)((batch + kRowsCTA - 1) / kRowsCTA);
-    k_mlp_reduce<<<(kTrain + 1 + 255) / 256, 256, 0, s>>>((const float*)bpart.p, nb, 1.0 / (double)batch, P,
+    if ((rc = grad_pass(P, (const float*)F, (const float*)T, off, batch, (double*)bpart.p, s)) != WL_OK) return rc;
+    const int nb = grad_blocks(batch);
+    k_mlp_reduce<<<kReduceBlocks, 256, 0, s>>>((const double*)bpart.p, nb, 1.0 / (double)batch, P,
                                                          (float*)bm.p, (float*)bv.p, lr, b1, b2, eps,
                                                          1.0 - std::pow((double)b1, it), 1.0 - std::pow((double)b2, it),
                                                          1, nullptr, (double*)bl.p);
@@ -722,8 +939,8 @@ int wl_mlp_train(float* params, const float* feats, const float* target, int64_t
     off += batch;
   }
   // loss of the trained network over all rows
-  if ((rc = grad_pass(P, (const float*)F, (const float*)T, 0, rows, (float*)bpart.p, s)) != WL_OK) return rc;
-  k_mlp_reduce<<<(kTrain + 1 + 255) / 256, 256, 0, s>>>((const float*)bpart.p, (int)((rows + kRowsCTA - 1) / kRowsCTA),
+  if ((rc = grad_pass(P, (const float*)F, (const float*)T, 0, rows, (double*)bpart.p, s)) != WL_OK) return rc;
+  k_mlp_reduce<<<kReduceBlocks, 256, 0, s>>>((const double*)bpart.p, grad_blocks(rows),
                                                        1.0 / (double)rows, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f,
                                                        0.f, 1.0, 1.0, 0, (float*)bm.p, (double*)bl.p);
   ML_CU(cudaGetLastError());

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import wlgen
-from oracle import features, graph, philox, walks, xnys
+from oracle import features, graph, mlp, philox, walks, xnys
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -59,3 +59,33 @@ def test_triangles_of_a_skewed_graph(seed):
     tri = features.triangles_by_intersection(g.row_ptr, g.col_idx, g.n)
     assert np.abs(F[:, 2].cpu().numpy().astype(np.float64) - np.log1p(tri)).max() <= 1.2e-7 * np.log1p(tri.max())
     w.close()
+
+
+# Network: tiles of 128 rows, one tile a CTA up to 304 tiles, then several
+@pytest.mark.parametrize("rows", [1, 127, 128, 129, 304 * 128, 304 * 128 + 1, 3 * 304 * 128 + 77])
+def test_network_gradient_and_prediction_tiles(rows):
+    from paper_2601_11338_gb300 import wl
+    rng = np.random.default_rng(rows)
+    p = mlp.init_params(64, 4, seed=5)
+    for k in ("b1", "b2", "b3"):
+        p[k] = 0.1 * rng.standard_normal(p[k].shape)
+    v = np.concatenate([rng.normal(size=4), rng.uniform(0.5, 2, 4)] +
+                       [p[k].ravel() for k in ("W1", "b1", "W2", "b2", "W3", "b3")]).astype(np.float32)
+    F = rng.normal(size=(rows, 4)).astype(np.float32)
+    T = rng.normal(size=rows).astype(np.float32)
+    xan = rng.uniform(1, 2, rows)
+    w = v.astype(np.float64)
+    X = (F.astype(np.float64) - w[0:4]) / w[4:8]
+    q = {"W1": w[8:264].reshape(64, 4), "b1": w[264:328], "W2": w[328:4424].reshape(64, 64), "b2": w[4424:4488],
+         "W3": w[4488:4552].reshape(1, 64), "b3": w[4552:]}
+    g = mlp.backward(q, X, T.astype(np.float64))
+    want = np.concatenate([g[k].ravel() for k in ("W1", "b1", "W2", "b2", "W3", "b3")])
+    grad = np.zeros(v.size, dtype=np.float32)
+    loss = wl.wl_mlp_loss_grad(v, F, T, rows, grad)
+    assert np.linalg.norm(grad[8:] - want) <= 1e-5 * np.linalg.norm(want)
+    assert not grad[:8].any()
+    y, _ = mlp.forward(q, X)
+    assert abs(loss - np.mean((y - T) ** 2)) <= 1e-5 * np.mean((y - T) ** 2)
+    out = torch.full((rows,), float("nan"), dtype=torch.float64, device="cuda")
+    wl.wl_mlp_predict(torch.as_tensor(v).cuda(), torch.as_tensor(F).cuda(), rows, torch.as_tensor(xan).cuda(), out)
+    assert np.abs(out.cpu().numpy() / (xan * np.exp(y)) - 1.0).max() <= 1e-5
