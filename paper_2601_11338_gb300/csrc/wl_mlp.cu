@@ -167,12 +167,13 @@ __global__ void __launch_bounds__(kFeatBlock) k_feat_orient(const int32_t* __res
 // Every triangle once: for each i, N+(i) goes into a hash table in shared
 // memory, and the w of every N+(j), j in N+(i), are looked up in it. A hit is
 // one triangle (i, j, w): t_w is counted in the table's slot, t_j in a
-// register of the eight lanes that walk N+(j), t_i beside it, and the global
+// register of the warp that walks N+(j), t_i beside it, and the global
 // counters see one atomic per node of N+(i) instead of one per triangle. The
 // table is at most a quarter full, so a look-up reads 1.2 words on average:
 // the pass is bound by shared-memory reads, one for each wedge (i, j, w)
 // (6.6e8 on R-MAT scale 18), and not by the dependent global reads of a
-// merge or binary search per edge. R-MAT scale 18, 7.6e6 entries: 2.98 ms (a
+// merge or binary search per edge. R-MAT scale 18, 7.6e6 entries: 2.19 ms (eight lanes to a
+// list, four lists a warp: 2.98 ms; a
 // merge or binary search by one lane per edge, a global atomic per triangle:
 // 20.4 ms).
 // A warp takes a node of up to kTriWarpDeg out-neighbours, a CTA a longer
@@ -182,7 +183,6 @@ constexpr int kTriPiece = 1024;
 constexpr int kTriTab = 4 * kTriPiece;
 constexpr int kTriBlock = 256;
 constexpr int kTriTicket = 8;  // nodes a warp takes at a time
-constexpr int kTriLanes = 8;   // lanes that walk one N+(j)
 constexpr int kTriUnroll = 4;  // look-ups in flight per lane
 
 __device__ __forceinline__ unsigned tri_hash(int key, int shift) { return ((unsigned)key * 0x9E3779B1u) >> shift; }
@@ -201,12 +201,11 @@ __device__ __forceinline__ int tri_find(const int* tab, unsigned mask, int shift
 template <int T, int PIECE, typename Sync>
 __device__ __forceinline__ void tri_node(int64_t i, const int64_t* __restrict__ orp, const int32_t* __restrict__ ocol,
                                          unsigned long long* __restrict__ t, int* tab, int* cnt, int tid, Sync sync) {
-  constexpr int L = kTriLanes, NG = T / L;
-  const int64_t ib = orp[i];
+  constexpr int NW = T / 32;
+  const int ib = (int)orp[i];  // at most 2^30 oriented entries
   const int len = (int)(orp[i + 1] - ib);
   if (len < 2) return;
-  const int g = tid / L, l = tid % L;
-  const unsigned gmask = 0xFFu << (threadIdx.x & 24);
+  const int w = tid / 32, lane = tid & 31;
   unsigned long long ti = 0;
   for (int p0 = 0; p0 < len; p0 += PIECE) {
     const int pl = min(PIECE, len - p0);
@@ -224,29 +223,41 @@ __device__ __forceinline__ void tri_node(int64_t i, const int64_t* __restrict__ 
       while (atomicCAS(tab + s, -1, key) != -1) s = (s + 1) & mask;
     }
     sync();
-    for (int q = g; q < len; q += NG) {
-      const int j = __ldg(ocol + ib + q);
-      const int64_t jb = __ldg(orp + j), je = __ldg(orp + j + 1);
-      int tj = 0;
-      for (int64_t b = jb + l; b < je; b += L * kTriUnroll) {
-        int key[kTriUnroll];
+    // 32 members j of N+(i) at a time, their list bounds one per lane; then the
+    // warp walks one N+(j) after the other
+    for (int q0 = w; q0 < len; q0 += 32 * NW) {
+      const int q = q0 + lane * NW;
+      int j = 0, jb = 0, je = 0;
+      if (q < len) {
+        j = __ldg(ocol + ib + q);
+        jb = (int)__ldg(orp + j);
+        je = (int)__ldg(orp + j + 1);
+      }
+      const int nj = min(32, (len - q0 + NW - 1) / NW);
+      int mine = 0;  // triangles with this lane's j
+      for (int u = 0; u < nj; ++u) {
+        const int b0 = __shfl_sync(0xffffffffu, jb, u), b1 = __shfl_sync(0xffffffffu, je, u);
+        int tj = 0;
+        for (int b = b0 + lane; b - lane < b1; b += 32 * kTriUnroll) {
+          int key[kTriUnroll];
 #pragma unroll
-        for (int u = 0; u < kTriUnroll; ++u) key[u] = b + u * L < je ? __ldg(ocol + b + u * L) : -1;
+          for (int v = 0; v < kTriUnroll; ++v) key[v] = b + 32 * v < b1 ? __ldg(ocol + b + 32 * v) : -1;
 #pragma unroll
-        for (int u = 0; u < kTriUnroll; ++u) {
-          if (key[u] < 0) continue;
-          const int s = tri_find(tab, mask, shift, key[u]);
-          if (s >= 0) {
-            atomicAdd(cnt + s, 1);
-            ++tj;
+          for (int v = 0; v < kTriUnroll; ++v) {
+            if (key[v] < 0) continue;
+            const int s = tri_find(tab, mask, shift, key[v]);
+            if (s >= 0) {
+              atomicAdd(cnt + s, 1);
+              ++tj;
+            }
           }
         }
+        tj = __reduce_add_sync(0xffffffffu, tj);
+        if (lane == u) mine = tj;
       }
-#pragma unroll
-      for (int off = 1; off < L; off <<= 1) tj += __shfl_xor_sync(gmask, tj, off);
-      if (l == 0 && tj) {
-        atomicAdd(t + j, (unsigned long long)tj);
-        ti += tj;
+      if (mine) {
+        atomicAdd(t + j, (unsigned long long)mine);
+        ti += mine;
       }
     }
     sync();
@@ -257,7 +268,9 @@ __device__ __forceinline__ void tri_node(int64_t i, const int64_t* __restrict__ 
     }
     sync();
   }
-  if (ti) atomicAdd(t + i, ti);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) ti += __shfl_xor_sync(0xffffffffu, ti, off);
+  if (lane == 0 && ti) atomicAdd(t + i, ti);
 }
 
 __global__ void __launch_bounds__(kTriBlock) k_feat_tri_warp(const int64_t* __restrict__ orp,
