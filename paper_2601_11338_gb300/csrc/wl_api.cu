@@ -317,6 +317,15 @@ void sp_batch_free(SpBatch* b) {
 
 }  // namespace wl
 
+// State of a solve. The cooperative CG kernel's barrier follows the norms of
+// the refinement residual, so that clearing those before each residual also
+// readies it for the next solve.
+struct CgBlock {
+  CgState st;
+  CgState res;  // norms of the refinement residual that follows a cooperative solve
+  CoopBar bar;
+};
+
 struct wl_handle {
   int64_t n = 0, nnz = 0;
   Graph g{};
@@ -366,7 +375,7 @@ struct wl_handle {
   Buf hubs;               // rows with more than kHubDeg entries (internal order)
   int nhub = 0;
   std::vector<void*> retired;  // blocks released during calls, returned to the allocator at destroy
-  Buf cgstate;            // CgState of the running solve
+  Buf cgstate;            // CgBlock of the running solve
   Buf spV, spW;           // spectral-scale Lanczos: basis (double-float, float2 per node) and raw w vectors
   Buf spstate;            // SpState of the spectral-scale Lanczos
   Buf mid;                // rows with kSpWarpDeg < deg <= kHubDeg (a warp each in the spectral Lanczos)
@@ -379,7 +388,11 @@ struct wl_handle {
   int cg_hint = 7;          // CG iterations of the handle's last solve (sizes the first launch chunk)
   int cg_hint_ref[2] = {7, 7};  // the same for the first and the later corrections of a refined solve
   bool gram_tc = false;     // XNysTrace Gram of the sketch form on the tensor cores (tcgen05); false: CUDA cores
-  CgState* cgst() { return (CgState*)cgstate.p; }
+  CgState* cgst() { return &((CgBlock*)cgstate.p)->st; }
+  CgState* cgres() { return &((CgBlock*)cgstate.p)->res; }
+  CoopBar* cgbar() { return &((CgBlock*)cgstate.p)->bar; }
+  int sms = 0;              // SMs of the device
+  bool bar_clean = false;   // the cooperative kernel's barrier is cleared for the next launch
   double* h_pin = nullptr;  // pinned host scratch (4096 doubles)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // per-call kernel timing: event pairs recorded on the stream around launches
@@ -419,6 +432,15 @@ int prof_begin(wl_handle* h, int cat) {
 
 void prof_end(wl_handle* h, int i) {
   if (i >= 0) cudaEventRecord(h->ev_pool[h->recs[i].b], h->stream);
+}
+
+// the record opened last, for a launch that did not happen
+void prof_cancel(wl_handle* h, int i) {
+  h->launches--;
+  if (i >= 0) {
+    h->recs.pop_back();
+    h->ev_used -= 2;
+  }
 }
 
 void prof_reset(wl_handle* h) {
@@ -504,6 +526,14 @@ double alg_bytes_per_iter(wl_handle* h, int K, int s) {
   return 4.0 * (double)h->nnz + 4.0 * (double)(h->n + 1) + 6.0 * (double)h->n * K * s;
 }
 
+// CTAs of a phase kernel: those that are resident at once, but no more than
+// have a lane unit (a row's 16 bytes of K columns) per thread; every CTA adds
+// to the last one's sum (the double-float residual of 20000 x 8: 13.4 -> 10.4 us)
+int phase_grid(wl_handle* h, int resident, int K, int val_bytes) {
+  const int lanes = std::max(1, K * val_bytes / 16);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(resident, (h->n * lanes + kPhaseBlock - 1) / kPhaseBlock));
+}
+
 PhaseGraph phase_graph(wl_handle* h) {
   return PhaseGraph{h->g.row_ptr, h->g.col, h->n, (const int32_t*)h->hubs.p, h->nhub};
 }
@@ -526,6 +556,86 @@ PhaseGraph phase_graph_mid(wl_handle* h, int grid_u) {
 constexpr double kInner0C = 0.5;
 constexpr int kChunk = 8;      // CG iterations launched between two reads of the device flag (cap: 2 kChunk)
 constexpr int kChunkMore = 4;  // iterations of every chunk after the first
+
+// The outcome of a CG solve from its state on the host (h_pin)
+void cg_outcome(wl_handle* h, int K, int val_bytes, SolveInfo& info) {
+  const CgState* hs = &reinterpret_cast<CgBlock*>(h->h_pin)->st;
+  const int it = hs->iters;
+  h->cg_hint = it;
+  int cs[64];
+  for (int c = 0; c < K; ++c) {  // iteration cap reached with a column still iterating
+    cs[c] = hs->status[c];
+    if (!hs->done[c] && cs[c] == 0) cs[c] = WL_ERR_NO_CONVERGENCE;
+  }
+  info.iters += it;
+  info.cg_iters += it;
+  info.nnz_rhs += (double)it * h->nnz * K;
+  info.bytes += (double)it * alg_bytes_per_iter(h, K, val_bytes);
+  info.last_rel = 0.0;
+  for (int c = 0; c < K; ++c) {
+    if (cs[c] != 0 && info.status == WL_OK) info.status = cs[c];
+    if (hs->b2[c] > 0) info.last_rel = std::max(info.last_rel, std::sqrt(hs->gamma[c] / hs->b2[c]));
+  }
+}
+
+// Reads the solve's block back (st, res, the barrier) and waits for it.
+int cg_block_to_host(wl_handle* h) {
+  CgBlock* hb = reinterpret_cast<CgBlock*>(h->h_pin);
+  WL_CU(cudaMemcpyAsync(hb, h->cgstate.p, sizeof(CgBlock), cudaMemcpyDeviceToHost, S(h)));
+  WL_CU(cudaStreamSynchronize(S(h)));
+  if (hb->bar.err != 0) {  // a wait of the cooperative kernel gave up
+    const int err = hb->bar.err;
+    h->bar_clean = false;
+    return err;
+  }
+  return WL_OK;
+}
+
+// Starting residual of a solve: r0 with its column norms gamma0 (NULL: a.r,
+// norms computed by the solve); add_x: x holds a start value, else it is zero.
+template <typename T>
+struct CgStart {
+  const T* r0 = nullptr;
+  const double* gamma0 = nullptr;
+  bool add_x = false;
+};
+
+// Launches a solve as one cooperative kernel; false where its vectors don't
+// fit in shared memory (nothing launched).
+template <typename T>
+bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& start, cudaError_t* e) {
+  CoopArgs<T> co{a, h->cgbar(), 0, start.r0 ? start.r0 : a.r, start.gamma0, start.add_x ? 1 : 0};
+  if (!h->bar_clean) {
+    *e = cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h));
+    if (*e != cudaSuccess) return true;
+  }
+  h->bar_clean = true;
+  const int fault = fault_mode();
+  if (fault == kFaultNoconv) co.a.max_iter = 1;
+  if (fault == kFaultNan) {
+    static const T nan_v = (T)NAN;
+    *e = cudaMemcpyAsync(const_cast<T*>(co.r0), &nan_v, sizeof(T), cudaMemcpyHostToDevice, S(h));
+    if (*e != cudaSuccess) return true;
+  }
+  if (fault == kFaultTimeout) {
+    static const int gave_up = WL_ERR_TIMEOUT;
+    *e = cudaMemcpyAsync(&h->cgbar()->err, &gave_up, sizeof(int), cudaMemcpyHostToDevice, S(h));
+    if (*e != cudaSuccess) return true;
+  }
+  const int pc = prof_begin(h, kCatCG);
+  bool coop;
+  if constexpr (sizeof(T) == 4)
+    coop = launch_cg_coop_f32(K, co, h->nnz, h->sms, S(h), e);
+  else
+    coop = launch_cg_coop_f64(K, co, h->nnz, h->sms, S(h), e);
+  if (coop) {
+    prof_end(h, pc);
+    h->bar_clean = false;
+  } else {
+    prof_cancel(h, pc);
+  }
+  return coop;
+}
 
 // Runs the CG iterations of an initialised solve state to completion (or the
 // iteration cap), reading back one flag per chunk, then the final x update.
@@ -553,8 +663,8 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, int grid_s, int grid_u
   // the whole CG state comes back after every chunk: the check of the last
   // chunk also carries the per-column results (the deferred x update launched
   // after it changes none of them), so the solve ends without another wait
-  CgState* hs = reinterpret_cast<CgState*>(h->h_pin);
-  static_assert(sizeof(CgState) <= 4096 * sizeof(double), "pinned staging holds the CG state");
+  CgState* hs = &reinterpret_cast<CgBlock*>(h->h_pin)->st;
+  static_assert(sizeof(CgBlock) <= 4096 * sizeof(double), "pinned staging holds the CG state");
   // first chunk: one more iteration than the handle's previous solve took (a
   // launch that finds the solve finished returns at once, but still costs a
   // grid); later chunks of kChunkMore iterations
@@ -570,53 +680,39 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, int grid_s, int grid_u
   counted(h, 1);
   WL_CU(launch(2, 0));
   prof_end(h, pc);
-  // per-column results
-  const int it = hs->iters;
-  h->cg_hint = it;
-  int cs[64];
-  for (int c = 0; c < K; ++c) {  // iteration cap reached with a column still iterating
-    cs[c] = hs->status[c];
-    if (!hs->done[c] && cs[c] == 0) cs[c] = WL_ERR_NO_CONVERGENCE;
-  }
-  info.iters += it;
-  info.cg_iters += it;
-  info.nnz_rhs += (double)it * h->nnz * K;
-  info.bytes += (double)it * alg_bytes_per_iter(h, K, cat_bytes);
-  info.last_rel = 0.0;
-  for (int c = 0; c < K; ++c) {
-    if (cs[c] != 0 && info.status == WL_OK) info.status = cs[c];
-    if (hs->b2[c] > 0) info.last_rel = std::max(info.last_rel, std::sqrt(hs->gamma[c] / hs->b2[c]));
-  }
+  cg_outcome(h, K, cat_bytes, info);
   return WL_OK;
 }
 
 int ensure_phase_buffers(wl_handle* h, int grid) {
   WL_TRY(ensure(h->part, (size_t)grid * 64 * 2 * 8 + 1024));
-  WL_TRY(ensure(h->cgstate, sizeof(CgState)));
+  if (!h->cgstate.p) {
+    WL_TRY(ensure(h->cgstate, sizeof(CgBlock)));
+    WL_CU(cudaMemsetAsync(h->cgstate.p, 0, sizeof(CgBlock), S(h)));
+  }
   return WL_OK;
 }
 
 // FP64 lockstep CG on M x = b for K columns (b, x contiguous n x K doubles).
-// x holds the starting guess on entry (zero unless a warm start is given).
+// x holds the starting guess on entry, or, x_is_zero, nothing yet.
 int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool x_is_zero, SolveInfo& info) {
   NvtxRange nvtx__("fp64 solve");
-  const int grid_u = phase_blocks_f64(K), grid_s = grid_u + h->nhub;
+  const int grid_u = phase_grid(h, phase_blocks_f64(K), K, 8), grid_s = grid_u + h->nhub;
+  const int grid_w = phase_grid(h, res_blocks(K), K, 8) + h->nhub;
   const size_t nk = (size_t)h->n * K;
   WL_TRY(ensure(h->r, nk * 8));
   WL_TRY(ensure(h->p, nk * 8));
   WL_TRY(ensure(h->q, nk * 8));
-  WL_TRY(ensure_phase_buffers(h, std::max(grid_s, res_blocks(K) + h->nhub)));
+  WL_TRY(ensure_phase_buffers(h, std::max({grid_s, grid_w, h->sms})));
   CgState* st = h->cgst();
-  WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
+  WL_CU(cudaMemsetAsync(st, 0, sizeof(CgBlock), S(h)));  // the cooperative kernel's barrier too
+  h->bar_clean = true;
   const double* bn2 = nullptr;
-  if (x_is_zero) {
-    WL_CU(cudaMemcpyAsync(h->r.p, b, nk * 8, cudaMemcpyDeviceToDevice, S(h)));
-  } else {
-    const int gr = res_blocks(K) + h->nhub;
+  if (!x_is_zero) {
     ResPhaseArgs ra{phase_graph(h), x, b, (double*)h->r.p, h->ca, h->cA, h->cD, (double*)h->part.p, st};
     const int pi = prof_begin(h, kCatRes);
     counted(h);
-    WL_CU(launch_res_phases(K, ra, gr, S(h)));
+    WL_CU(launch_res_phases(K, ra, grid_w, S(h)));
     prof_end(h, pi);
     bn2 = st->b2;
     info.nnz_rhs += (double)h->nnz * K;
@@ -624,7 +720,23 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
   PhaseArgs<double> a{phase_graph_mid(h, grid_u), x, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
                       bn2, nullptr, (double*)h->part.p, st, h->prm.max_iter, tol * tol};
   a.dshift = h->si_dsh64;  // shifted solve of the shift-and-invert Lanczos (else NULL)
-  WL_TRY(run_cg<double>(h, K, a, grid_s, grid_u, info, 8));
+  {
+    CgStart<double> start;
+    start.r0 = x_is_zero ? b : nullptr;
+    start.add_x = !x_is_zero;
+    cudaError_t ce = cudaSuccess;
+    if (cg_coop_try<double>(h, K, a, start, &ce)) {
+      WL_CU(ce);
+      WL_TRY(cg_block_to_host(h));
+      cg_outcome(h, K, 8, info);
+    } else {
+      if (x_is_zero) {
+        WL_CU(cudaMemsetAsync(x, 0, nk * 8, S(h)));
+        WL_CU(cudaMemcpyAsync(h->r.p, b, nk * 8, cudaMemcpyDeviceToDevice, S(h)));
+      }
+      WL_TRY(run_cg<double>(h, K, a, grid_s, grid_u, info, 8));
+    }
+  }
   info.max_rel = std::max(info.max_rel, info.last_rel);
   return WL_OK;
 }
@@ -638,8 +750,8 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
 int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const double* bn2, float* xh, float* xl,
                      const double* x0, int K, double tol, SolveInfo& info) {
   NvtxRange nvtx__("refined solve");
-  const int grid_u = phase_blocks_f32(K), grid_s = grid_u + h->nhub;
-  const int grid_r = df_res_blocks(K) + h->nhub;
+  const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4), grid_s = grid_u + h->nhub;
+  const int grid_r = phase_grid(h, df_res_blocks(K), K, 4) + h->nhub;
   const size_t nk = (size_t)h->n * K;
   WL_TRY(ensure(h->p, nk * 4));
   WL_TRY(ensure(h->q, nk * 4));
@@ -648,7 +760,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   WL_TRY(ensure(h->r32, nk * 4));
   WL_TRY(ensure(h->rh, nk * 4));
   WL_TRY(ensure(h->rl, nk * 4));
-  WL_TRY(ensure_phase_buffers(h, std::max(grid_s, grid_r)));
+  WL_TRY(ensure_phase_buffers(h, std::max({grid_s, grid_r, h->sms})));
   CgState* st = h->cgst();
   float* rh = (float*)h->rh.p;
   float* rl = (float*)h->rl.p;
@@ -656,21 +768,28 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   float* dnext = (float*)h->d32b.p;
   const df ca = df_from_double(h->ca), cA = df_from_double(h->cA), cD = df_from_double(h->cD);
   double* hp = h->h_pin;
+  double* hbn2 = h->h_pin + 2048;  // beyond the solve's block
+  static_assert(sizeof(CgBlock) <= 2048 * sizeof(double), "room for the solve's block");
+  int* dskip = (int*)((double*)h->small.p + 256);
   // current residual: B itself while X = 0
   const float* rch = bh;
   const float* rcl = bl;
   bool x_zero = (x0 == nullptr);
-  WL_CU(cudaMemsetAsync(dcur, 0, nk * 4, S(h)));
-  WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
-  if (x_zero) {
-    WL_CU(cudaMemcpyAsync(h->r32.p, bh, nk * 4, cudaMemcpyDeviceToDevice, S(h)));
-    WL_CU(cudaMemcpyAsync(st->gamma, bn2, K * 8, cudaMemcpyDeviceToDevice, S(h)));
-  } else {
+  // Small solves run each correction as one cooperative kernel. It starts from
+  // B's or the residual's leading terms where they are and writes d whole, so
+  // nothing is staged for it, and the residual that follows it keeps its norms
+  // in a state of its own: both are launched before one wait for their outcome.
+  PhaseArgs<float> a{phase_graph_mid(h, grid_u), dcur, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
+                     h->ca, h->cA, h->cD, nullptr, dskip, (double*)h->part.p, st, h->prm.max_iter, 0.0};
+  a.dshift = h->si_dsh_h;
+  const bool coop = cg_coop_fits_f32(K, a.g, h->nnz, h->sms);
+  CgState* rst = coop ? h->cgres() : st;  // the residual's norms
+  if (!x_zero) {
     // r = B - M x0 (x0 split into two FP32 terms and gathered whole)
     counted(h, 2);
     WL_CU(launch_split_x(x0, (int64_t)nk, xh, xl, false, nullptr, S(h)));
     DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), xh, xl, bh, bl, rh, rl, (float*)h->r32.p, nullptr, nullptr, nullptr,
-                 ca, cA, cD, (double*)h->part.p, st, 0};
+                 ca, cA, cD, (double*)h->part.p, rst, 0};
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
     const int pi = prof_begin(h, kCatRes);
@@ -686,30 +805,40 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // rel, with the same floor)
   const double inner0 = std::min(1e-3, std::max(h->inner_tol, kInner0C * std::sqrt(tol)));
   const int max_ref = 12;
-  int ndf = 0;
-  int* dskip = (int*)((double*)h->small.p + 256);
   // r32 (the next inner solve's right-hand side) and dcur (its zero start)
   // are ready: the residual after the first correction writes them, later
   // ones do not (the solve almost always ends there), and a further
   // correction stages them itself
   bool staged = true;
+  if (!coop) {
+    WL_CU(cudaMemsetAsync(dcur, 0, nk * 4, S(h)));
+    if (x_zero) {
+      WL_CU(cudaMemcpyAsync(h->r32.p, bh, nk * 4, cudaMemcpyDeviceToDevice, S(h)));
+      WL_CU(cudaMemcpyAsync(st->gamma, bn2, K * 8, cudaMemcpyDeviceToDevice, S(h)));
+    }
+  }
+  const double* hgamma = nullptr;  // residual norms on the host, when the last wait brought them
   for (int ref = 0;; ++ref) {
     info.refinements++;
     double mx = 1.0;
-    if (ref == 0 && x_zero) {
+    const bool from_b = ref == 0 && x_zero;
+    if (from_b) {
       // the residual is B itself: every column with B != 0 still needs its
       // first correction (rel = 1), and the inner solve's start marks a zero
       // column done by itself, so no host check (and no wait) is needed
-      WL_CU(cudaMemsetAsync(dskip, 0, K * sizeof(int), S(h)));
+      if (!coop) WL_CU(cudaMemsetAsync(dskip, 0, K * sizeof(int), S(h)));
     } else {
-      WL_CU(cudaMemcpyAsync(hp, st->gamma, K * 8, cudaMemcpyDeviceToHost, S(h)));
-      WL_CU(cudaMemcpyAsync(hp + 64, bn2, K * 8, cudaMemcpyDeviceToHost, S(h)));
-      WL_CU(cudaStreamSynchronize(S(h)));
+      if (!hgamma) {
+        WL_CU(cudaMemcpyAsync(hp, rst->gamma, K * 8, cudaMemcpyDeviceToHost, S(h)));
+        WL_CU(cudaMemcpyAsync(hbn2, bn2, K * 8, cudaMemcpyDeviceToHost, S(h)));
+        WL_CU(cudaStreamSynchronize(S(h)));
+        hgamma = hp;
+      }
       bool all = true;
       mx = 0.0;
       int skip[64];
       for (int c = 0; c < K; ++c) {
-        const double rr = hp[c], bb = hp[64 + c];
+        const double rr = hgamma[c], bb = hbn2[c];
         if (!std::isfinite(rr)) info.status = WL_ERR_NONFINITE;
         const double rel = bb > 0 ? std::sqrt(rr / bb) : 0.0;
         mx = std::max(mx, rel);
@@ -723,50 +852,68 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
         break;
       }
       WL_CU(cudaMemcpyAsync(dskip, skip, K * sizeof(int), cudaMemcpyHostToDevice, S(h)));
-      if (!staged) {
+      if (!coop && !staged) {
         WL_CU(cudaMemcpyAsync(h->r32.p, rh, nk * 4, cudaMemcpyDeviceToDevice, S(h)));
         WL_CU(cudaMemsetAsync(dcur, 0, nk * 4, S(h)));
         staged = true;
       }
     }
-    const double inner_tol = ref == 0 && x_zero ? inner0 : std::min(1e-3, std::max(h->inner_tol, 0.5 * tol / mx));
-    // the inner solve starts from the residual norms in st->gamma (from the
-    // double-float residual, or B's norms): no pass over r32 to recompute them
-    counted(h);
-    WL_CU(launch_cg_state_restart(st, dskip, K, S(h)));
-    PhaseArgs<float> a{phase_graph_mid(h, grid_u), dcur, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
-                       h->ca, h->cA, h->cD, nullptr, dskip, (double*)h->part.p, st, h->prm.max_iter,
-                       inner_tol * inner_tol};
-    a.dshift = h->si_dsh_h;
+    const double inner_tol = from_b ? inner0 : std::min(1e-3, std::max(h->inner_tol, 0.5 * tol / mx));
+    a.x = dcur;
+    a.tol2 = inner_tol * inner_tol;
+    a.skip = coop && from_b ? nullptr : dskip;
     SolveInfo inner;
-    // the first correction and the later ones go to different depths: each
-    // sizes its first launch chunk from the previous solve of its kind
-    int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
-    h->cg_hint = hint;
-    WL_TRY(run_cg<float>(h, K, a, grid_s, grid_u, inner, 4, false));
-    hint = h->cg_hint;
-    if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
-      info.status = inner.status;
-      break;
+    if (coop) {
+      CgStart<float> start;
+      start.r0 = rch;
+      start.gamma0 = from_b ? bn2 : rst->gamma;
+      cudaError_t ce = cudaSuccess;
+      if (!cg_coop_try<float>(h, K, a, start, &ce)) return WL_ERR_UNSUPPORTED;  // fits: checked above
+      WL_CU(ce);
+    } else {
+      // the inner solve starts from the residual norms in st->gamma (from the
+      // double-float residual, or B's norms): no pass over r32 to recompute them
+      counted(h);
+      WL_CU(launch_cg_state_restart(st, dskip, K, S(h)));
+      // the first correction and the later ones go to different depths: each
+      // sizes its first launch chunk from the previous solve of its kind
+      int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
+      h->cg_hint = hint;
+      WL_TRY(run_cg<float>(h, K, a, grid_s, grid_u, inner, 4, false));
+      hint = h->cg_hint;
+      if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
+        info.status = inner.status;
+        break;
+      }
+    }
+    // r <- r - M d, x <- x + d, next correction buffer zeroed
+    WL_CU(cudaMemsetAsync(rst, 0, coop ? sizeof(CgState) + sizeof(CoopBar) : sizeof(CgState), S(h)));
+    if (coop) h->bar_clean = true;
+    const bool stage_next = (ref == 0) && !coop;
+    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), dcur, nullptr, rch, rcl, rh, rl,
+                 stage_next ? (float*)h->r32.p : nullptr, xh, xl, stage_next ? dnext : nullptr,
+                 ca, cA, cD, (double*)h->part.p, rst, x_zero ? 1 : 0};
+    ra.dsh_h = h->si_dsh_h;
+    ra.dsh_l = h->si_dsh_l;
+    const int pi = prof_begin(h, kCatRes);
+    WL_CU(launch_df_res(K, ra, grid_r, false, S(h)));
+    prof_end(h, pi);
+    hgamma = nullptr;
+    if (coop) {
+      WL_CU(cudaMemcpyAsync(hbn2, bn2, K * 8, cudaMemcpyDeviceToHost, S(h)));
+      WL_TRY(cg_block_to_host(h));
+      cg_outcome(h, K, 4, inner);
+      hgamma = reinterpret_cast<CgBlock*>(h->h_pin)->res.gamma;
+      if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
+        info.status = inner.status;
+        break;
+      }
     }
     info.iters += inner.iters;
     info.cg_iters += inner.cg_iters;
     info.nnz_rhs += inner.nnz_rhs;
     info.bytes += inner.bytes;
-    // r <- r - M d, x <- x + d, next correction buffer zeroed
-    WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
-    const bool stage_next = (ref == 0);
-    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), dcur, nullptr, rch, rcl, rh, rl,
-                 stage_next ? (float*)h->r32.p : nullptr, xh, xl, stage_next ? dnext : nullptr,
-                 ca, cA, cD, (double*)h->part.p, st, x_zero ? 1 : 0};
-    ra.dsh_h = h->si_dsh_h;
-    ra.dsh_l = h->si_dsh_l;
-    const int pi = prof_begin(h, kCatRes);
-    counted(h);
-    WL_CU(launch_df_res(K, ra, grid_r, false, S(h)));
-    prof_end(h, pi);
     info.nnz_rhs += (double)h->nnz * K;
-    ++ndf;
     x_zero = false;
     staged = stage_next;
     rch = rh;
@@ -783,7 +930,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
 // Refined solve with FP64 B and X: B -> double-float once, X back to FP64.
 int solve_refined(wl_handle* h, const double* b, double* x, int K, double tol, bool x_is_zero, SolveInfo& info) {
   const size_t nk = (size_t)h->n * K;
-  const int grid_u = phase_blocks_f32(K);
+  const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4);
   WL_TRY(ensure(h->bh, nk * 4));
   WL_TRY(ensure(h->bl, nk * 4));
   WL_TRY(ensure(h->xh, nk * 4));
@@ -806,7 +953,6 @@ int solve_refined(wl_handle* h, const double* b, double* x, int K, double tol, b
 int solve(wl_handle* h, const double* b, double* x, int K, bool x_is_zero, SolveInfo& info) {
   const double tol = h->prm.tol;
   if (h->prm.prec != WL_FP64) return solve_refined(h, b, x, K, tol, x_is_zero, info);
-  if (x_is_zero) WL_CU(cudaMemsetAsync(x, 0, (size_t)h->n * K * 8, S(h)));
   return solve_fp64(h, b, x, K, tol, x_is_zero, info);
 }
 
@@ -1404,7 +1550,6 @@ int si_apply(wl_handle* h, bool dfp, int K, int j, size_t blk, SolveInfo& info) 
     WL_TRY(ensure(h->x, blk * 8));
     counted(h);
     WL_CU(launch_si_rhs64(vj, d64 + n, n, K, (double*)h->b64.p, S(h)));
-    WL_CU(cudaMemsetAsync(h->x.p, 0, blk * 8, S(h)));
     {
       SiScope sc(h, false);
       WL_TRY(solve_fp64(h, (const double*)h->b64.p, (double*)h->x.p, K, h->prm.tol, true, info));
@@ -1862,6 +2007,10 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
   };
   if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess)
     return fail(set_cuda_error(cudaGetLastError(), "cudaEventCreate"));
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return fail(set_cuda_error(cudaGetLastError(), "cudaDeviceGetAttribute"));
   if (pool_malloc_host((void**)&h->h_pin, 4096 * sizeof(double)) != cudaSuccess)
     return fail(set_cuda_error(cudaGetLastError(), "cudaMallocHost"));
   if (pool_malloc((void**)&h->bar, sizeof(GridBar)) != cudaSuccess)
@@ -2467,8 +2616,8 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
     if (e == cudaSuccess) e = cudaMemsetAsync(h->x.p, 0, nk * 4, S(h));
     if (e != cudaSuccess) { rc = set_cuda_error(e, "sketch"); break; }
     // Y = M^{-1} (a Omega) in FP32 lockstep CG
-    const int grid_u = phase_blocks_f32(K), grid_s = grid_u + h->nhub;
-    if ((rc = ensure_phase_buffers(h, grid_s)) != WL_OK) break;
+    const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4), grid_s = grid_u + h->nhub;
+    if ((rc = ensure_phase_buffers(h, std::max(grid_s, h->sms))) != WL_OK) break;
     Smalls sm = smalls(h);
     CgState* st = h->cgst();
     WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
@@ -2476,7 +2625,13 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
     PhaseArgs<float> a{phase_graph_mid(h, grid_u), (float*)h->x.p, (float*)h->r32.p, (float*)h->p.p,
                        (float*)h->q.p, h->ca, h->cA, h->cD, nullptr, nullptr, (double*)h->part.p, st,
                        h->prm.max_iter, tol * tol};
-    if ((rc = run_cg<float>(h, K, a, grid_s, grid_u, info, 4)) != WL_OK) break;
+    if (cg_coop_try<float>(h, K, a, CgStart<float>{}, &e)) {
+      if (e != cudaSuccess) { rc = set_cuda_error(e, "cooperative CG"); break; }
+      if ((rc = cg_block_to_host(h)) != WL_OK) break;
+      cg_outcome(h, K, 4, info);
+    } else if ((rc = run_cg<float>(h, K, a, grid_s, grid_u, info, 4)) != WL_OK) {
+      break;
+    }
     (void)sm;
     counted(h, 3);
     int* gerr = (int*)((double*)h->small.p + 1000);

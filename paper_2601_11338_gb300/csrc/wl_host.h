@@ -10,6 +10,7 @@
 #include <string>
 
 #include "wl_cg2.cuh"
+#include "wl_coop.cuh"
 #include "wl_common.cuh"
 #include "wl_lanczos.cuh"
 #include "wl_expdf.cuh"
@@ -98,6 +99,11 @@ cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, i
                                  cudaStream_t s);
 cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, int mode, int chunk,
                                  cudaStream_t s);
+// ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the
+// solve's vectors don't fit in shared memory
+bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
+bool cg_coop_fits_f32(int K, const PhaseGraph& g, int64_t nnz, int sms);
+bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
 // one CTA waiting in the bounded grid barrier for nblocks CTAs (failure-detection self-test)
 cudaError_t launch_selftest_wait(GridBar* bar, unsigned nblocks, cudaStream_t s);
 // FP64 residual r = b - M x of a warm start, norms into st->gamma / st->b2

@@ -1,0 +1,30 @@
+// FP64 instances of the cooperative CG kernel, K = 1, 2, 4, ..., 64 columns.
+#include <algorithm>
+
+#include "wl_coop.cuh"
+#include "wl_host.h"
+
+namespace wl {
+
+template <int K>
+static bool run(const CoopArgs<double>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e) {
+  CoopShape sh;
+  if (!cgc_shape<double, K>(a.a.g, nnz, sms, &sh)) return false;
+  *e = a.a.dshift ? cgc_launch<double, K, true>(a, sh, s) : cgc_launch<double, K, false>(a, sh, s);
+  return true;
+}
+
+bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e) {
+  switch (K) {
+    case 1: return run<1>(a, nnz, sms, s, e);
+    case 2: return run<2>(a, nnz, sms, s, e);
+    case 4: return run<4>(a, nnz, sms, s, e);
+    case 8: return run<8>(a, nnz, sms, s, e);
+    case 16: return run<16>(a, nnz, sms, s, e);
+    case 32: return run<32>(a, nnz, sms, s, e);
+    case 64: return run<64>(a, nnz, sms, s, e);
+  }
+  return false;
+}
+
+}  // namespace wl

@@ -89,3 +89,39 @@ def test_network_gradient_and_prediction_tiles(rows):
     out = torch.full((rows,), float("nan"), dtype=torch.float64, device="cuda")
     wl.wl_mlp_predict(torch.as_tensor(v).cuda(), torch.as_tensor(F).cuda(), rows, torch.as_tensor(xan).cuda(), out)
     assert np.abs(out.cpu().numpy() / (xan * np.exp(y)) - 1.0).max() <= 1e-5
+
+
+# Cooperative CG: one row, rows below and above a pass of the CTAs, K on both
+# sides of every lane width, long hub rows (a whole CTA), hub and mid rows (a
+# warp), against the oracle's dense phi at the form's parity tolerance
+def _solve_graphs():
+    yield wlgen.path(2)
+    yield wlgen.erdos_renyi(257, 6.0, 7)
+    yield wlgen.star(2500)                      # one hub of 2500 entries
+    yield wlgen.barabasi_albert(1500, 20, 3)    # mid and hub rows
+    yield wlgen.erdos_renyi(1900, 90.0, 5)      # only mid rows
+
+
+@pytest.mark.parametrize("reorder", [0, 1])
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)])
+def test_small_solves(prec, tol, bound, reorder):
+    for g in _solve_graphs():
+        A = graph.dense_adjacency(g.row_ptr, g.col_idx, g.n)
+        w = WL(g, variant="btdw", mu=0.4, alpha_rel=0.5, prec=prec, tol=tol, reorder=reorder)
+        phi = walks.phi_resolvent_closed(A, 0.4, w.info["alpha"])
+        D = walks.walk_degrees(phi)
+        L = walks.walk_laplacian(phi)
+        Df = w.degrees().cpu().numpy()
+        assert np.abs(Df - D).max() <= bound * np.abs(D).max(), g.name
+        for k in (1, 2, 3, 4, 8, 16, 32, 64):
+            V = np.random.default_rng(k).standard_normal((g.n, k))
+            V[:, k // 2] = 0.0 if k > 1 else V[:, 0]  # a zero column takes no part
+            W = w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy()
+            want = L @ V
+            assert np.abs(W - want).max() <= bound * np.abs(want).max(), (g.name, k)
+        # a warm start away from the solution
+        x0 = D * (1.0 + 0.3 * np.cos(np.arange(g.n)))
+        w.warm_start(torch.as_tensor(x0, device="cuda"))
+        Df = w.degrees().cpu().numpy()
+        assert np.abs(Df - D).max() <= bound * np.abs(D).max(), g.name
+        w.close()
