@@ -1880,7 +1880,7 @@ int outer_combine(wl_handle* h, const OuterRun& o, int t0, int nt, double* out, 
     WL_TRY(ensure(h->ydf, ny * 8));
     counted(h, 2);
     e = launch_df_split((const double*)h->ybuf.p, ny, (float*)h->ydf.p, (float*)h->ydf.p + ny, S(h));
-    DfCombineArgs ca{(const float*)h->basis.p, (const float*)h->ydf.p, (const float*)h->ydf.p + ny, mcol, nrm, out,
+    DfCombineArgs ca{(const float*)h->basis.p, (const float*)h->ydf.p, (const float*)h->ydf.p + ny, o.m, nrm, out,
                      n, ld, tstride, c0, ldT, nt, perm};
     if (e == cudaSuccess) e = launch_df_combine(K, ca, S(h));
   } else {

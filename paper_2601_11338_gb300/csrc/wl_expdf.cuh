@@ -66,7 +66,7 @@ struct DfCombineArgs {
   const float* basis;  // block j: hi at basis + 2 j n K, lo at basis + (2 j + 1) n K
   const float* yh;
   const float* yl;
-  const int* mcol;
+  int m;               // Lanczos steps
   const double* nrm;
   double* out;
   int64_t n, ld, tstride;
@@ -188,67 +188,71 @@ __global__ void __launch_bounds__(kBlock) df_lanczos_step(DfLanczosArgs a) {
 
 // U(tau) = |u0| V_m y(tau) over a double-float basis, all tau from one read
 // of the basis; y in double-float (yh, yl: K x ntau x ldT), output FP64.
-// The coefficients of the CTA's columns are staged in shared memory (layout
-// [j][tau][c]) when they fit; four basis blocks are read per round so that
-// eight independent loads are in flight per thread.
-constexpr int kCombSmemFloats = 10240;  // 40 KB of staged coefficients
+// Bound by the basis read (8 bytes per step and entry) and by the 15 FP32
+// operations per step, tau and entry. A CTA works on CS <= K columns whose
+// coefficients for all steps and tau fit in shared memory as (hi, lo) pairs,
+// [j][tau][c] (one 8-byte read per product, consecutive columns in consecutive
+// banks); four basis blocks are read per round so that eight independent loads
+// are in flight per thread. 62500 x 32, 44 steps, 8 tau: 625 us
+// (coefficients in shared memory only up to 40 KB, else read from L2: 4790 us).
+constexpr size_t kCombSmem = 100 * 1024;     // two CTAs per SM
+constexpr size_t kCombSmemMax = 200 * 1024;  // fewer columns than 8 would break the 32-byte sectors instead
 
-template <int K>
-__global__ void __launch_bounds__(kBlock) df_combine(DfCombineArgs a) {
-  __shared__ float s_y[kCombSmemFloats];
+template <int K, int NT, bool STAGED>
+__global__ void __launch_bounds__(kBlock) df_combine(DfCombineArgs a, int CS) {
+  extern __shared__ __align__(16) float2 s_y[];
   const size_t total = (size_t)a.n * K;
-  int mmax = 0;
-  for (int c = 0; c < K; ++c) mmax = max(mmax, a.mcol[c]);
-  const bool staged = (size_t)mmax * a.ntau * K * 2 <= (size_t)kCombSmemFloats;
-  if (staged) {
-    const int cnt = mmax * a.ntau * K;
-    for (int q = threadIdx.x; q < cnt; q += kBlock) {
-      const int c = q % K, t = (q / K) % a.ntau, j = q / (K * a.ntau);
-      const size_t src = ((size_t)c * a.ntau + t) * a.ldT + j;
-      s_y[2 * q] = __ldg(a.yh + src);
-      s_y[2 * q + 1] = __ldg(a.yl + src);
+  const int tid = threadIdx.x, cl = tid % CS, c0 = (int)blockIdx.y * CS, c = c0 + cl;
+  if constexpr (STAGED) {
+    const int cnt = a.m * a.ntau * CS;
+    for (int q = tid; q < cnt; q += kBlock) {  // consecutive threads: consecutive steps of one (c, tau)
+      const int j = q % a.m, t = (q / a.m) % a.ntau, cc = q / (a.m * a.ntau);
+      const size_t src = ((size_t)(c0 + cc) * a.ntau + t) * a.ldT + j;
+      s_y[(j * a.ntau + t) * CS + cc] = make_float2(__ldg(a.yh + src), __ldg(a.yl + src));
     }
+    __syncthreads();
   }
-  __syncthreads();
-  for (size_t e = (size_t)blockIdx.x * kBlock + threadIdx.x; e < total; e += (size_t)gridDim.x * kBlock) {
-    const int c = (int)(e % K);
-    const size_t i = e / K;
-    const int m = a.mcol[c];
-    float S[kMaxTau], Cc[kMaxTau];
-#pragma unroll
-    for (int t = 0; t < kMaxTau; ++t) S[t] = Cc[t] = 0.f;
-    auto ycoef = [&](int j, int t) -> df {
-      if (staged) {
-        const int q = (j * a.ntau + t) * K + c;
-        return df{s_y[2 * q], s_y[2 * q + 1]};
-      }
+  auto ycoef = [&](int j, int t) -> df {
+    if constexpr (STAGED) {
+      const float2 y = s_y[(j * a.ntau + t) * CS + cl];
+      return df{y.x, y.y};
+    } else {
       const size_t src = ((size_t)c * a.ntau + t) * a.ldT + j;
       return df{__ldg(a.yh + src), __ldg(a.yl + src)};
-    };
+    }
+  };
+  const df sc = df_from_double(a.nrm[c]);
+  const int rpb = kBlock / CS;
+  for (int64_t i = (int64_t)blockIdx.x * rpb + tid / CS; i < a.n; i += (int64_t)gridDim.x * rpb) {
+    const size_t e = (size_t)i * K + c;
+    float S[NT], Cc[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) S[t] = Cc[t] = 0.f;
     int j = 0;
-    for (; j + 3 < m; j += 4) {
+    for (; j + 3 < a.m; j += 4) {
       df v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         v[u] = df{__ldcs(a.basis + (size_t)(2 * (j + u)) * total + e),
                   __ldcs(a.basis + (size_t)(2 * (j + u) + 1) * total + e)};
 #pragma unroll
-      for (int t = 0; t < kMaxTau; ++t)
+      for (int t = 0; t < NT; ++t)
         if (t < a.ntau) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) df_acc2(S[t], Cc[t], df_mul(v[u], ycoef(j + u, t)));
         }
     }
-    for (; j < m; ++j) {
+    for (; j < a.m; ++j) {
       const df v{__ldcs(a.basis + (size_t)(2 * j) * total + e), __ldcs(a.basis + (size_t)(2 * j + 1) * total + e)};
 #pragma unroll
-      for (int t = 0; t < kMaxTau; ++t)
+      for (int t = 0; t < NT; ++t)
         if (t < a.ntau) df_acc2(S[t], Cc[t], df_mul(v, ycoef(j, t)));
     }
-    const double sc = a.nrm[c];
-    const size_t io = a.perm ? (size_t)a.perm[i] : i;
-    for (int t = 0; t < a.ntau; ++t)
-      a.out[(size_t)t * a.tstride + io * a.ld + a.c0 + c] = sc * ((double)S[t] + (double)Cc[t]);
+    const size_t io = a.perm ? (size_t)a.perm[i] : (size_t)i;
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+      if (t < a.ntau)
+        a.out[(size_t)t * a.tstride + io * a.ld + a.c0 + c] = df_to_double(df_mul(sc, two_sum(S[t], Cc[t])));
   }
 }
 

@@ -84,13 +84,34 @@ cudaError_t launch_df_lanczos_step(int K, const DfLanczosArgs& a, int G, cudaStr
   return coop_launch(f, G, a, s);
 }
 
+template <int K, int NT>
+static cudaError_t run_combine(const DfCombineArgs& a, cudaStream_t s) {
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(df_combine<K, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCombSmemMax);
+  if (attr != cudaSuccess) return attr;
+  const size_t per_col = (size_t)a.m * a.ntau * sizeof(float2);
+  int CS = K;
+  while (CS > 8 && per_col * CS > kCombSmem) CS /= 2;
+  const bool staged = per_col * CS <= kCombSmemMax;
+  if (!staged) CS = K;
+  const int rpb = kBlock / CS;
+  // CTAs that fill the chip at the shared memory each takes, so that the coefficients are staged once
+  const int per_sm = staged ? (int)std::max<size_t>(1, std::min<size_t>(6, 220 * 1024 / (per_col * CS + 1024))) : 6;
+  const int64_t gx = std::max<int64_t>(1, std::min<int64_t>((a.n + rpb - 1) / rpb, 152 * per_sm * CS / K));
+  const dim3 grid((unsigned)gx, K / CS);
+  if (staged)
+    df_combine<K, NT, true><<<grid, kBlock, per_col * CS, s>>>(a, CS);
+  else
+    df_combine<K, NT, false><<<grid, kBlock, 0, s>>>(a, CS);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_df_combine(int K, const DfCombineArgs& a, cudaStream_t s) {
-  const int64_t blocks = std::min<int64_t>(((int64_t)a.n * K + kBlock - 1) / kBlock, 152 * 16);
+  if (a.ntau > kMaxTau || a.n <= 0) return a.n <= 0 ? cudaSuccess : cudaErrorInvalidValue;
   switch (K) {
-#define CB(k)                                                                  \
-  case k:                                                                      \
-    df_combine<k><<<(unsigned)std::max<int64_t>(blocks, 1), kBlock, 0, s>>>(a); \
-    return cudaGetLastError();
+#define CB(k) \
+  case k:     \
+    return a.ntau <= 4 ? run_combine<k, 4>(a, s) : run_combine<k, kMaxTau>(a, s);
     WL_FOR_K(CB)
 #undef CB
   }
