@@ -2568,7 +2568,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
     if ((rc = ensure(h->q, nk * 4)) != WL_OK) break;
     const int Gg = gram_grid(n);
     if ((rc = ensure(h->gram, (size_t)Gg * 2 * kMaxSketch * kMaxSketch * 4 + 2 * kMaxSketch * kMaxSketch * 8 +
-                                 128 * 8)) != WL_OK) break;
+                                 kCoreDoubles * 8)) != WL_OK) break;
     uint16_t* omega = (uint16_t*)h->omega.p;
     float* partial = (float*)h->gram.p;
     double* gout = (double*)((char*)h->gram.p + (size_t)Gg * 2 * kMaxSketch * kMaxSketch * 4);
@@ -2587,7 +2587,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       if (e == cudaSuccess && (rc = ensure(h->packV, nk * 8)) != WL_OK) break;
       if (e == cudaSuccess && (rc = ensure(h->packX, nk * 8)) != WL_OK) break;
       if (e == cudaSuccess && (rc = ensure(h->gram, (gram_f64_partial_doubles(n, M) + 2 * kMaxSketch * kMaxSketch +
-                                                      128) * 8)) != WL_OK) break;
+                                                      kCoreDoubles) * 8)) != WL_OK) break;
       counted(h);
       if (e == cudaSuccess) e = launch_sketch_block_f64(om_int, n, M, K, (double*)h->packV.p, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "sketch"); break; }
@@ -2689,7 +2689,7 @@ int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt,
     const int Gg = gram_grid(n);
     const bool sketch = h->prm.prec == WL_SKETCH;  // FP32 Gram on the tensor cores; else FP64
     const size_t pbytes = sketch ? (size_t)Gg * 2 * kMaxSketch * kMaxSketch * 4 : gram_f64_partial_doubles(n, M) * 8;
-    if ((rc = ensure(h->gram, pbytes + 2 * kMaxSketch * kMaxSketch * 8 + 128 * 8)) != WL_OK) break;
+    if ((rc = ensure(h->gram, pbytes + 2 * kMaxSketch * kMaxSketch * 8 + kCoreDoubles * 8)) != WL_OK) break;
     uint16_t* omega = (uint16_t*)h->omega.p;
     float* partial = (float*)h->gram.p;
     double* gout = (double*)((char*)h->gram.p + pbytes);

@@ -207,7 +207,8 @@ int gram_grid(int64_t n);
 cudaError_t launch_gram(const uint16_t* omega, const float* Y, int64_t n, int M, int K, float* partial, int G,
                         double* out, bool tensor_cores, int* err, cudaStream_t s);
 // out[0] estimate, out[1] error estimate, out[2] status, out[8 + i] = t_i
-cudaError_t launch_nys_core(const double* gram, int M, double* out, cudaStream_t s);
+// gram (128 x 64) is used as scratch; out: kCoreDoubles
+cudaError_t launch_nys_core(double* gram, int M, double* out, cudaStream_t s);
 // [Omega Y]^T Y from an FP64 Y (n x K, first M columns), FP64 throughout; partial: G x 2 x 64 x 64 doubles
 int gram_grid_f64(int64_t n);
 size_t gram_f64_partial_doubles(int64_t n, int M);

@@ -11,7 +11,7 @@
 //  gram_cc       : per-CTA partial Grams H = Omega^T Y and G = Y^T Y over a
 //                  contiguous row chunk (FP32 products and sums inside a
 //                  chunk, FP64 across chunks in gram_reduce).
-//  nys_core      : with P = H^{-1} (Cholesky, FP64), the leave-one-out
+//  nys_factor, nys_core : with P = H^{-1} (LDL^T, FP64), the leave-one-out
 //                  estimates t_i = tr(P G) + (1 - (P G P)_ii) / P_ii, which
 //                  equal tr(A_hat_(i)) + w_i^T (A - A_hat_(i)) w_i for the
 //                  Nystrom approximation A_hat_(i) = Y_-i (Omega_-i^T Y_-i)^{-1}
@@ -25,6 +25,7 @@
 namespace wl {
 
 constexpr int kMaxSketch = 64;
+constexpr int kCoreDoubles = 512;  // results and scratch of the leave-one-out core
 
 __device__ __forceinline__ void philox4x32_10(uint32_t (&c)[4], uint32_t k0, uint32_t k1) {
 #pragma unroll
@@ -347,85 +348,139 @@ __global__ void __launch_bounds__(256) gram_reduce_f64(const double* partial, in
 
 // ---------------------------------------------------------------- FP64 leave-one-out core
 // gram: 128 x 64 doubles, rows 0..63 = Omega^T Y (H), rows 64..127 = Y^T Y (G).
-// out[0] = estimate, out[1] = error estimate, out[2] = status (0 ok, 1 not PD), out[8 + i] = t_i
-__global__ void __launch_bounds__(256) nys_core(const double* gram, int M, double* out) {
+// out[0] = estimate, out[1] = error estimate, out[2] = status (0 ok, 1 not PD), out[8 + i] = t_i;
+// out holds kCoreDoubles, the rest is scratch.
+//
+// An FP64 operation waits about a hundred clocks for the one before it, and
+// one SM does two a clock, so the core is split: nys_factor (one CTA)
+// brings H = L D L^T and L^{-1} out of the same M elimination steps, all
+// rows at once with one reciprocal per step; nys_core (one CTA per column i
+// of P = H^{-1}) then needs two products with M terms a thread. Measured at
+// M = 64: 97 + 33 us (one CTA for all of it, a thread per column of P and two
+// triangular solves in sequence: 440 us).
+constexpr int kFactorThreads = 512;
+constexpr int kCoreAux = 8 + kMaxSketch;  // out[kCoreAux + 3 i ..]: (G P)_ii, (P G P)_ii, P_ii; then the ticket
+
+// gram rows 0..63 become L^{-1} (unit lower triangle) with 1 / D_j on the diagonal
+__global__ void __launch_bounds__(kFactorThreads) nys_factor(double* gram, int M, double* out) {
   extern __shared__ double sm[];
-  double* H = sm;                        // M x M (Cholesky factor in the lower triangle)
-  double* Gm = H + kMaxSketch * kMaxSketch;  // M x M
-  double* P = Gm + kMaxSketch * kMaxSketch;  // M x M inverse
-  double* W = P + kMaxSketch * kMaxSketch;   // M x M
-  __shared__ double s_t[kMaxSketch];
-  __shared__ int s_bad;
+  constexpr int LD = kMaxSketch + 1;
+  double* H = sm;                          // lower triangle, eliminated in place
+  double* R = H + kMaxSketch * LD;         // L^{-1}
+  double* s_l = R + kMaxSketch * LD;       // column k of L
+  double* s_rd = s_l + kMaxSketch;         // 1 / D_k
   const int tid = threadIdx.x;
-  constexpr int LD = kMaxSketch;
-  if (tid == 0) s_bad = 0;
-  for (int e = tid; e < M * M; e += 256) {
+  for (int e = tid; e < M * M; e += kFactorThreads) {
     const int r = e / M, c = e % M;
-    H[r * LD + c] = 0.5 * (gram[r * kMaxSketch + c] + gram[c * kMaxSketch + r]);
-    Gm[r * LD + c] = 0.5 * (gram[(kMaxSketch + r) * kMaxSketch + c] + gram[(kMaxSketch + c) * kMaxSketch + r]);
+    if (c <= r) H[r * LD + c] = 0.5 * (gram[r * kMaxSketch + c] + gram[c * kMaxSketch + r]);
+    R[r * LD + c] = r == c ? 1.0 : 0.0;
   }
+  int bad = 0;
   __syncthreads();
-  // right-looking Cholesky H = L L^T (lower triangle)
   for (int k = 0; k < M; ++k) {
-    if (tid == 0) {
+    if (tid < kMaxSketch) {
       const double d = H[k * LD + k];
-      if (!(d > 0.0)) s_bad = 1;
-      H[k * LD + k] = sqrt(fmax(d, 1e-300));
+      if (!(d > 0.0)) bad = 1;
+      const double rd = 1.0 / fmax(d, 1e-300);
+      if (tid == 0) s_rd[k] = rd;
+      if (tid > k && tid < M) s_l[tid] = H[tid * LD + k] * rd;
     }
     __syncthreads();
-    const double dk = H[k * LD + k];
-    for (int i = k + 1 + tid; i < M; i += 256) H[i * LD + k] /= dk;
-    __syncthreads();
-    for (int e = tid; e < (M - k - 1) * (M - k - 1); e += 256) {
-      const int i = k + 1 + e / (M - k - 1), j = k + 1 + e % (M - k - 1);
-      if (j <= i) H[i * LD + j] -= H[i * LD + k] * H[j * LD + k];
+    // row i loses l_ik times row k: columns 0..k of L^{-1}, columns k + 1..i of H
+    for (int i = k + 1 + (tid >> 4); i < M; i += kFactorThreads / 16) {
+      const double l = s_l[i];
+      for (int c = tid & 15; c <= i; c += 16) {
+        if (c <= k)
+          R[i * LD + c] = fma(-l, R[k * LD + c], R[i * LD + c]);
+        else
+          H[i * LD + c] = fma(-l, H[c * LD + k], H[i * LD + c]);
+      }
     }
     __syncthreads();
   }
-  // P = H^{-1}: thread c solves L L^T p = e_c
-  for (int c = tid; c < M; c += 256) {
-    for (int i = 0; i < M; ++i) {  // forward: L z = e_c, z stored in P[i][c]
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int k = 0; k < i; ++k) s -= H[i * LD + k] * P[k * LD + c];
-      P[i * LD + c] = s / H[i * LD + i];
-    }
-    for (int i = M - 1; i >= 0; --i) {  // backward: L^T p = z
-      double s = P[i * LD + c];
-      for (int k = i + 1; k < M; ++k) s -= H[k * LD + i] * P[k * LD + c];
-      P[i * LD + c] = s / H[i * LD + i];
-    }
-  }
-  __syncthreads();
-  // W = G P
-  for (int e = tid; e < M * M; e += 256) {
+  for (int e = tid; e < M * M; e += kFactorThreads) {
     const int r = e / M, c = e % M;
-    double s = 0.0;
-    for (int k = 0; k < M; ++k) s += Gm[r * LD + k] * P[k * LD + c];
-    W[r * LD + c] = s;
+    gram[r * kMaxSketch + c] = r == c ? s_rd[r] : R[r * LD + c];
   }
-  __syncthreads();
-  // S = tr(P G) = sum_r (P W')... tr(P G) = sum_{r,k} P_rk G_kr = sum_r (G P)_rr = sum_r W_rr
-  // q_i = (P G P)_ii = sum_k P_ki W_ki
-  if (tid < M) {
-    double q = 0.0;
-    for (int k = 0; k < M; ++k) q += P[k * LD + tid] * W[k * LD + tid];
-    double S = 0.0;
-    for (int r = 0; r < M; ++r) S += W[r * LD + r];
-    s_t[tid] = S + (1.0 - q) / P[tid * LD + tid];
-  }
-  __syncthreads();
   if (tid == 0) {
+    out[2] = bad ? 1.0 : 0.0;
+    *reinterpret_cast<unsigned long long*>(out + kCoreAux + 3 * kMaxSketch) = 0ull;  // nys_core's ticket
+  }
+}
+
+// CTA i: column i of P = L^{-T} D^{-1} L^{-1}, (G P)_ii and (P G P)_ii; the
+// last CTA forms t_i = tr(P G) + (1 - (P G P)_ii) / P_ii and its statistics
+__global__ void __launch_bounds__(kMaxSketch) nys_core(const double* gram, int M, double* out) {
+  __shared__ double s_p[kMaxSketch], s_v[kMaxSketch];
+  __shared__ int s_last;
+  const int i = blockIdx.x, k = threadIdx.x;
+  const double* G = gram + kMaxSketch * kMaxSketch;
+  // v_j = (L^{-1})_ji / D_j
+  if (k < M) s_v[k] = k < i ? 0.0 : (k == i ? 1.0 : gram[k * kMaxSketch + i]) * gram[k * kMaxSketch + k];
+  __syncthreads();
+  double p = 0.0;
+  if (k < M) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    const int j0 = max(k + 1, i);
+    int j = j0;
+    for (; j + 3 < M; j += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = fma(gram[(j + u) * kMaxSketch + k], s_v[j + u], a[u]);
+    for (; j < M; ++j) a[0] = fma(gram[j * kMaxSketch + k], s_v[j], a[0]);
+    p = (a[0] + a[1]) + (a[2] + a[3]) + s_v[k];
+    s_p[k] = p;
+  }
+  __syncthreads();
+  double g = 0.0;
+  if (k < M) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int j = 0;
+    for (; j + 3 < M; j += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        a[u] = fma(0.5 * (G[(j + u) * kMaxSketch + k] + G[k * kMaxSketch + j + u]), s_p[j + u], a[u]);
+    for (; j < M; ++j) a[0] = fma(0.5 * (G[j * kMaxSketch + k] + G[k * kMaxSketch + j]), s_p[j], a[0]);
+    g = (a[0] + a[1]) + (a[2] + a[3]);
+    s_v[k] = p * g;
+    if (k == i) {
+      out[kCoreAux + 3 * i] = g;
+      out[kCoreAux + 3 * i + 2] = p;
+    }
+  }
+  __syncthreads();
+  if (k == 0) {
+    double q = 0.0;
+    for (int j = 0; j < M; ++j) q += s_v[j];
+    out[kCoreAux + 3 * i + 1] = q;
+  }
+  __threadfence();
+  __syncthreads();
+  if (k == 0)
+    s_last = atomicAdd(reinterpret_cast<unsigned long long*>(out + kCoreAux + 3 * kMaxSketch), 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (k < M) s_p[k] = __ldcg(out + kCoreAux + 3 * k);
+  __syncthreads();
+  double t = 0.0;
+  if (k < M) {
+    double S = 0.0;
+    for (int j = 0; j < M; ++j) S += s_p[j];
+    t = S + (1.0 - __ldcg(out + kCoreAux + 3 * k + 1)) / __ldcg(out + kCoreAux + 3 * k + 2);
+    s_v[k] = t;
+    out[8 + k] = t;
+  }
+  __syncthreads();
+  if (k == 0) {
     double mean = 0.0;
-    for (int i = 0; i < M; ++i) mean += s_t[i];
+    for (int j = 0; j < M; ++j) mean += s_v[j];
     mean /= M;
     double var = 0.0;
-    for (int i = 0; i < M; ++i) var += (s_t[i] - mean) * (s_t[i] - mean);
+    for (int j = 0; j < M; ++j) var += (s_v[j] - mean) * (s_v[j] - mean);
     var /= (M - 1);
     out[0] = mean;
     out[1] = sqrt(var / M);
-    out[2] = s_bad ? 1.0 : 0.0;
   }
-  if (tid < M) out[8 + tid] = s_t[tid];
 }
 
 #endif  // WL_TRACE_KERNELS
