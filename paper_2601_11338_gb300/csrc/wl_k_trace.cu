@@ -20,7 +20,7 @@ static unsigned grid_cap(int64_t work, int64_t per, int cap) {
 
 cudaError_t launch_philox_sketch(uint16_t* omega, int64_t n, int M, uint64_t seed, cudaStream_t s) {
   const int64_t total = n * M;
-  philox_sketch<<<grid_cap((total + 3) / 4, 256, 152 * 32), 256, 0, s>>>(omega, total, seed);
+  philox_sketch<<<grid_cap((total + 3) / 4, kPhiloxBlock, 152 * 8), kPhiloxBlock, 0, s>>>(omega, total, seed);
   return cudaGetLastError();
 }
 
