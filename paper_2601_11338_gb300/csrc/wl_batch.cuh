@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_init(BatchGraph g, BatchStat
 
 // ---------------------------------------------------------------- S
 template <typename T, int K>
-__global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocks) bcg_s(BatchArgs<T> a) {
+__global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(BatchArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   __shared__ __align__(16) T s_red[kPhaseBlock * VW];
@@ -420,7 +420,7 @@ struct BatchResArgs {
 };
 
 template <int K>
-__global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocks) bres(BatchResArgs a) {
+__global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchResArgs a) {
   using C = Cfg<float, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   __shared__ __align__(16) float s_red[2][kPhaseBlock * VW];

@@ -29,7 +29,7 @@ constexpr int kHubDeg = 256;       // rows with more entries get a CTA each
 constexpr int kMidDeg = 30;        // rows with more entries (up to kHubDeg) get a warp each in the S kernels
 constexpr int kPhaseBlock = 256;   // threads per CTA of the phase kernels
 #ifndef WL_PHASE_MINB
-#define WL_PHASE_MINB 5
+#define WL_PHASE_MINB 3
 #endif
 constexpr int kPhaseMinBlocks = WL_PHASE_MINB;  // CTAs per SM the S kernel's registers are sized for
 // FP32 CG kernels: 5 CTAs per SM (48 registers) hold the eight predicated
@@ -99,10 +99,46 @@ __device__ __forceinline__ Pack<T, VW> ld_plain(const T* p) {
 #ifndef WL_GATHER_U
 #define WL_GATHER_U 8
 #endif
-// the same choice for the FP64 kernels (the plain FP64 form), measured on its own
-#ifndef WL_GATHER_PRED_F64
-#define WL_GATHER_PRED_F64 0
-#endif
+// acc + sum of eight FP64 values, the values added as integers. GB300 adds two
+// FP64 lanes per clock and SM, so a neighbour sum of doubles is bound by its
+// additions; here each value costs about 15 integer instructions (64 lanes
+// per clock) instead, and a batch two FP64 ones. The values are aligned to the
+// largest exponent among them with seven guard bits and summed exactly from
+// there on (53 + 7 + 3 bits), rounded once at the end: the error is below 2^-4
+// units in the last place of the largest value plus that rounding, less than
+// that of eight FP64 additions in sequence. Chung-Lu 3e5, K = 16: 257 -> 198 us
+// an S phase (FP64 additions alone, four values in flight). Batches with non-finite or tiny
+// values (exponent field below 64) are added in FP64.
+__device__ __forceinline__ double add8_aligned(double acc, const double (&v)[8]) {
+  int m = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) m = max(m, __double2hiint(v[u]) & 0x7fffffff);
+  const int em = m >> 20;
+  if (em < 64 || em == 0x7ff) {
+    int any = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) any |= (__double2hiint(v[u]) & 0x7fffffff) | __double2loint(v[u]);
+    if (any != 0) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    return acc;
+  }
+  unsigned long long sum = 0;
+  int neg = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int hi = __double2hiint(v[u]), e = (hi & 0x7fffffff) >> 20, s = hi >> 31;
+    unsigned long long x = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 |
+                            (unsigned)__double2loint(v[u])) << 7;
+    const unsigned d = (unsigned)(em - e);
+    asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(d));  // 0 from 64 on (a zero has e = 0, d >= 64)
+    sum += x ^ (unsigned long long)(long long)s;     // -x = ~x + 1 for the negative ones
+    neg -= s;
+  }
+  const long long total = (long long)(sum + (unsigned)neg);
+  return fma((double)total, __hiloint2double((em - 59) << 20, 0), acc);
+}
 
 // Sum of X over entries [beg, end) with stride `step`.
 // WL_GATHER_PRED = 1: every batch of WL_GATHER_U entries, the last one too,
@@ -113,8 +149,9 @@ __device__ __forceinline__ Pack<T, VW> ld_plain(const T* p) {
 template <typename T, int K, int VW>
 __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int beg, int end, int step,
                                            const T* X, int lane_off, T (&acc)[VW]) {
-  if constexpr (sizeof(T) == 4 ? WL_GATHER_PRED : WL_GATHER_PRED_F64) {
-  constexpr int U = WL_GATHER_U;
+  if constexpr (sizeof(T) == 8 || WL_GATHER_PRED) {
+  constexpr bool kInt = sizeof(T) == 8;
+  constexpr int U = kInt ? 8 : WL_GATHER_U;
   for (int e = beg; e < end; e += U * step) {
     int j[U];
 #pragma unroll
@@ -129,10 +166,27 @@ __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int 
         for (int v = 0; v < VW; ++v) a[u].v[v] = T(0);
       }
     }
+    if constexpr (kInt) {
+      if (end - e > 3 * step) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+        for (int v = 0; v < VW; ++v) {
+          double x[8];
 #pragma unroll
-      for (int v = 0; v < VW; ++v) acc[v] += a[u].v[v];
+          for (int u = 0; u < U; ++u) x[u] = a[u].v[v];
+          acc[v] = add8_aligned(acc[v], x);
+        }
+      } else {  // up to three values: fewer FP64 additions than the integer sum costs
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+#pragma unroll
+          for (int v = 0; v < VW; ++v) acc[v] += a[u].v[v];
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < VW; ++v) acc[v] += a[u].v[v];
+    }
   }
   return;
   }
@@ -268,19 +322,29 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
     const Pack<T, VW>& rr = w.r;
     Pack<T, VW> pp, qq;
     const T dg = (T)deg;
+    // (M r) of column v; FP64: the row's diagonal first (one product fewer per column)
+    T crow = T(0);
+    if constexpr (sizeof(T) == 8) crow = SH ? ca + cD * dg + dx : ca + cD * dg;
+    auto mr = [&](int v) {
+      if constexpr (sizeof(T) == 8) {
+        return crow * rr.v[v] + cA * nb[v];
+      } else {
+        T s = ca * rr.v[v] + cA * nb[v] + cD * dg * rr.v[v];
+        if constexpr (SH) s += dx * rr.v[v];
+        return s;
+      }
+    };
     if (first) {
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
         pp.v[v] = rr.v[v];
-        qq.v[v] = ca * rr.v[v] + cA * nb[v] + cD * dg * rr.v[v];
-        if constexpr (SH) qq.v[v] += dx * rr.v[v];
+        qq.v[v] = mr(v);
       }
     } else {
       Pack<T, VW> xx = w.x;
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
-        T s = ca * rr.v[v] + cA * nb[v] + cD * dg * rr.v[v];
-        if constexpr (SH) s += dx * rr.v[v];
+        const T s = mr(v);
         const T al = s_ab[0][lane_off + v], be = s_ab[1][lane_off + v];
         xx.v[v] += al * w.p.v[v];
         pp.v[v] = rr.v[v] + be * w.p.v[v];

@@ -125,3 +125,26 @@ def test_small_solves(prec, tol, bound, reorder):
         Df = w.degrees().cpu().numpy()
         assert np.abs(Df - D).max() <= bound * np.abs(D).max(), g.name
         w.close()
+
+
+def test_fp64_neighbour_sums_of_uneven_magnitude():
+    """FP64 solve of a graph too large for the cooperative kernel (the phase
+    kernels' integer-aligned neighbour sums): right-hand sides whose entries
+    spread over 18 decades with mixed signs, and rows of 0 to 200 entries,
+    against scipy's FP64 CG."""
+    from oracle import krylov
+    e = wlgen.erdos_renyi(70001, 8.0, 3)
+    src = np.repeat(np.arange(e.n), e.degrees)
+    hub = np.arange(5, 70001, 350)  # node 3 joins 200 others
+    g = wlgen.csr_from_edges(e.n, np.concatenate([src, np.full(hub.size, 3)]), np.concatenate([e.col_idx, hub]))
+    w = WL(g, variant="nbt", alpha_rel=0.5, prec="fp64", tol=1e-13)
+    L = krylov.ResolventLaplacian(krylov.adjacency(g.row_ptr, g.col_idx, g.n), 1.0, w.info["alpha"], tol=1e-14)
+    rng = np.random.default_rng(11)
+    V = rng.standard_normal((g.n, 16)) * 10.0 ** rng.uniform(-9, 9, (g.n, 1))
+    V[:, 3] = 0.0
+    V[:, 4] *= 1e-120
+    W = w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy()
+    want = L.apply(V)
+    scale = np.abs(want).max(0)
+    assert (np.abs(W - want).max(0) <= 1e-10 * scale).all()
+    w.close()
