@@ -351,6 +351,19 @@ int emit_iteration(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
   return WL_OK;
 }
 
+template <typename T>
+int emit_final(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
+  const dim3 gt(a.g.ntile, nslab);
+  switch (K) {
+#define C(k) case k: bcg_f<T, k><<<gt, kPhaseBlock, 0, s>>>(a); break;
+    BT_FOR_K(C)
+#undef C
+    default: return WL_ERR_INVALID_ARG;
+  }
+  BT_CU(cudaGetLastError());
+  return WL_OK;
+}
+
 int emit_res(int K, const BatchResArgs& a, int nslab, cudaStream_t s) {
   const dim3 gt(a.g.ntile, nslab);
   switch (K) {
@@ -392,7 +405,8 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
                         nullptr, nullptr, (double*)sb.part.p, st, b->prm.max_iter, tol2};
     BT_TRY(emit_init<double>(K, a, nullptr, nslab, s));
     BT_TRY(emit_red_init(K, g, st, a.part, nullptr, nullptr, nullptr, tol2, nslab, s));
-    return em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<double>(K, a, nslab, em.s()); });
+    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<double>(K, a, nslab, em.s()); }));
+    return emit_final<double>(K, a, nslab, em.s());
   }
   // refined: double-float residual / FP64 iterate around an FP32 CG whose
   // target is the inner tolerance relative to the current residual
@@ -418,7 +432,8 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
     BT_TRY(emit_init<float>(K, ia, o.outer_active, nslab, so));
     BT_TRY(emit_red_init(K, g, st, ia.part, o.rn2, o.skip, o.outer_active, tin * tin, nslab, so));
     // the correction d ends in sb.x; the next residual pass adds it to x64
-    return em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<float>(K, ia, nslab, em.s()); });
+    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<float>(K, ia, nslab, em.s()); }));
+    return emit_final<float>(K, ia, nslab, em.s());
   });
 }
 

@@ -13,13 +13,15 @@
 // for K columns. Tiles write per-column partial sums; one CTA per problem
 // then adds its tiles' partials in a fixed order (deterministic) and
 // updates that problem's scalars. One iteration is
-//   S: q = M r + beta q, p = r + beta p, delta partials
+//   S: x += alpha p, q = M r + beta q, p = r + beta p, delta partials
 //   RS: alpha = gamma / delta
-//   U: x += alpha p, r -= alpha q, gamma' partials
+//   U: r -= alpha q, gamma' partials
 //   RU: beta = gamma' / gamma, convergence, problem and global activity
-// A problem that has converged is skipped by every later launch.
+// and F makes the last x update. A problem that has converged is skipped by
+// every later launch.
 #pragma once
 #include "wl_cg2.cuh"
+#include "wl_coop.cuh"
 #include "wl_res.cuh"
 
 namespace wl {
@@ -79,30 +81,38 @@ struct BatchArgs {
 #ifdef WL_BATCH_KERNELS
 
 // CTA column sums of per-thread values (thread t owns columns (t % G) VW + v),
-// stored to out[0 .. K)
+// stored to out[0 .. K). FP32 values (or their double-float sums) are added in
+// double-float: the FP64 adds of a butterfly over 256 threads held a tile's
+// CTA for 1000 clocks.
 template <typename T, int K>
-__device__ __forceinline__ void block_colsum_store(const double (&val)[Cfg<T, K>::VW], double* out) {
+__device__ __forceinline__ void block_colsum_store(const typename CoopSum<T>::S (&val)[Cfg<T, K>::VW], double* out) {
   using C = Cfg<T, K>;
+  using SM = CoopSum<T>;
+  using S = typename SM::S;
   constexpr int VW = C::VW, G = C::G, NW = kPhaseBlock / 32;
-  __shared__ double s_w[NW * K];
+  __shared__ S s_w[NW * K];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double a[VW];
+  S a[VW];
 #pragma unroll
   for (int v = 0; v < VW; ++v) a[v] = val[v];
 #pragma unroll
   for (int off = G; off < 32; off <<= 1)
 #pragma unroll
-    for (int v = 0; v < VW; ++v) a[v] += __shfl_xor_sync(0xffffffffu, a[v], off);
+    for (int v = 0; v < VW; ++v) a[v] = SM::add(a[v], SM::shfl(a[v], off));
   if (lane < G)
 #pragma unroll
     for (int v = 0; v < VW; ++v) s_w[warp * K + lane * VW + v] = a[v];
   __syncthreads();
   if (tid < K) {
-    double t = 0.0;
-    for (int w = 0; w < NW; ++w) t += s_w[w * K + tid];
-    out[tid] = t;
+    S t = s_w[tid];
+    for (int w = 1; w < NW; ++w) t = SM::add(t, s_w[w * K + tid]);
+    out[tid] = SM::out(t);
   }
 }
+
+// s += x^2, exactly rounded to the sum's type
+__device__ __forceinline__ void acc_sq(float2& s, float x) { df_acc2(s.x, s.y, two_prod(x, x)); }
+__device__ __forceinline__ void acc_sq(double& s, double x) { s = fma(x, x, s); }
 
 // Sum over the tiles of one problem, fixed order: out[c] in shared memory
 template <int K>
@@ -136,18 +146,18 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_init(BatchArgs<T> a, const in
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   if (pmask && !pmask[pr]) {  // problem not refining any more: zero partials only
-    double z[Cfg<T, K>::VW];
+    typename CoopSum<T>::S z[Cfg<T, K>::VW];
 #pragma unroll
-    for (int v = 0; v < Cfg<T, K>::VW; ++v) z[v] = 0.0;
+    for (int v = 0; v < Cfg<T, K>::VW; ++v) z[v] = CoopSum<T>::zero();
     block_colsum_store<T, K>(z, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
     return;
   }
   const int tid = threadIdx.x, lane_off = (tid % G) * VW;
   const size_t slab = (size_t)s * a.g.n * K;
   const T sc = a.bscale ? (T)a.bscale[pr] : T(1);
-  double acc[VW];
+  typename CoopSum<T>::S acc[VW];
 #pragma unroll
-  for (int v = 0; v < VW; ++v) acc[v] = 0.0;
+  for (int v = 0; v < VW; ++v) acc[v] = CoopSum<T>::zero();
   for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
     if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
     const size_t o = slab + (size_t)row * K + lane_off;
@@ -164,7 +174,7 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_init(BatchArgs<T> a, const in
 #pragma unroll
     for (int v = 0; v < VW; ++v) {
       z.v[v] = T(0);
-      acc[v] += (double)rr.v[v] * (double)rr.v[v];
+      acc_sq(acc[v], rr.v[v]);
     }
     stp<T, VW>(a.x + o, z);
   }
@@ -221,13 +231,17 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
   const int tid = threadIdx.x, sl = tid % G, lane_off = sl * VW;
   const bool first = a.st.iters[pr] == 0;
   const T ca = (T)a.ca[pr], cA = (T)a.cA[pr], cD = (T)a.cD[pr];
-  T be[VW];
+  T al[VW], be[VW];
 #pragma unroll
-  for (int v = 0; v < VW; ++v) be[v] = first ? T(0) : (T)a.st.beta[pr * K + lane_off + v];
+  for (int v = 0; v < VW; ++v) {
+    al[v] = first ? T(0) : (T)a.st.alpha[pr * K + lane_off + v];
+    be[v] = first ? T(0) : (T)a.st.beta[pr * K + lane_off + v];
+  }
   const size_t slab = (size_t)s * a.g.n * K;
   const T* __restrict__ R = a.r + slab;
   T* __restrict__ P = a.p + slab;
   T* __restrict__ Q = a.q + slab;
+  T* __restrict__ X = a.x + slab;
   T dacc[VW];
 #pragma unroll
   for (int v = 0; v < VW; ++v) dacc[v] = T(0);
@@ -244,11 +258,14 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     } else {
       const Pack<T, VW> po = ld_plain<T, VW>(P + o);
       const Pack<T, VW> qo = ld_plain<T, VW>(Q + o);
+      Pack<T, VW> xx = ld_plain<T, VW>(X + o);
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
+        xx.v[v] += al[v] * po.v[v];
         pp.v[v] = rr.v[v] + be[v] * po.v[v];
         qq.v[v] = ca * rr.v[v] + cA * nb[v] + cD * (T)deg * rr.v[v] + be[v] * qo.v[v];
       }
+      stp<T, VW>(X + o, xx);
     }
 #pragma unroll
     for (int v = 0; v < VW; ++v) dacc[v] += pp.v[v] * qq.v[v];
@@ -282,9 +299,9 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
       fin(row, end - beg, acc);
     }
   }
-  double dd[VW];
+  typename CoopSum<T>::S dd[VW];
 #pragma unroll
-  for (int v = 0; v < VW; ++v) dd[v] = (double)dacc[v];
+  for (int v = 0; v < VW; ++v) dd[v] = CoopSum<T>::from(dacc[v]);
   block_colsum_store<T, K>(dd, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
 }
 
@@ -331,26 +348,49 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_u(BatchArgs<T> a) {
 #pragma unroll
   for (int v = 0; v < VW; ++v) al[v] = (T)a.st.alpha[pr * K + lane_off + v];
   const size_t slab = (size_t)s * a.g.n * K;
-  double acc[VW];
+  typename CoopSum<T>::S acc[VW];
 #pragma unroll
-  for (int v = 0; v < VW; ++v) acc[v] = 0.0;
+  for (int v = 0; v < VW; ++v) acc[v] = CoopSum<T>::zero();
+#pragma unroll 2
+  for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
+    if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
+    const size_t o = slab + (size_t)row * K + lane_off;
+    Pack<T, VW> rr = ld_plain<T, VW>(a.r + o);
+    const Pack<T, VW> qq = ld_plain<T, VW>(a.q + o);
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      rr.v[v] -= al[v] * qq.v[v];
+      acc_sq(acc[v], rr.v[v]);
+    }
+    stp<T, VW>(a.r + o, rr);
+  }
+  block_colsum_store<T, K>(acc, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
+}
+
+// x += alpha p: the update of each problem's last iteration (the S kernel
+// makes the others, where it reads p anyway)
+template <typename T, int K>
+__global__ void __launch_bounds__(kPhaseBlock) bcg_f(BatchArgs<T> a) {
+  using C = Cfg<T, K>;
+  constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
+  const BTile tl = a.g.tiles[blockIdx.x];
+  const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
+  if (a.st.iters[pr] == 0) return;
+  const int tid = threadIdx.x, lane_off = (tid % G) * VW;
+  T al[VW];
+#pragma unroll
+  for (int v = 0; v < VW; ++v) al[v] = (T)a.st.alpha[pr * K + lane_off + v];
+  const size_t slab = (size_t)s * a.g.n * K;
+#pragma unroll 2
   for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
     if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
     const size_t o = slab + (size_t)row * K + lane_off;
     Pack<T, VW> xx = ld_plain<T, VW>(a.x + o);
-    Pack<T, VW> rr = ld_plain<T, VW>(a.r + o);
     const Pack<T, VW> pp = ld_plain<T, VW>(a.p + o);
-    const Pack<T, VW> qq = ld_plain<T, VW>(a.q + o);
 #pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      xx.v[v] += al[v] * pp.v[v];
-      rr.v[v] -= al[v] * qq.v[v];
-      acc[v] += (double)rr.v[v] * (double)rr.v[v];
-    }
+    for (int v = 0; v < VW; ++v) xx.v[v] += al[v] * pp.v[v];
     stp<T, VW>(a.x + o, xx);
-    stp<T, VW>(a.r + o, rr);
   }
-  block_colsum_store<T, K>(acc, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
 }
 
 // beta, convergence, activity; grid (ngraph, nslab)
@@ -506,11 +546,11 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchRes
       fin(row, end - beg, sm, cm);
     }
   }
-  double pr_r[VW], pr_b[VW];
+  float2 pr_r[VW], pr_b[VW];
 #pragma unroll
   for (int v = 0; v < VW; ++v) {
-    pr_r[v] = (double)acc_r[v];
-    pr_b[v] = (double)acc_b[v];
+    pr_r[v] = make_float2(acc_r[v], 0.f);
+    pr_b[v] = make_float2(acc_b[v], 0.f);
   }
   double* out = a.part + ((size_t)s * a.g.ntile + blockIdx.x) * 2 * K;
   block_colsum_store<float, K>(pr_r, out);
