@@ -130,14 +130,44 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Column blocks used for k columns: powers of two up to 64, largest first.
-std::vector<int> column_blocks(int k) {
-  std::vector<int> out;
+// Column blocks used for k columns: powers of two K up to 64, the last one
+// with kr < K columns where padding it with zero columns (which take no part
+// in a solve) costs less than a further block. A block's iteration is taken
+// to cost a fixed time, as the bytes it could move in it, plus what it moves:
+// gathered rows of at least a 32-byte sector, ten vector streams and the
+// indices. Padding also stops where a block would pass kPadMaxElems elements:
+// the vectors of a solve and an outer basis grow with it, and what fitted in
+// memory without padding has to fit still. An apply of 13 columns, n = 20011:
+// 455 us as one block of 16, 947 us as 8 + 4 + 1.
+struct ColBlock {
+  int K, kr;
+};
+constexpr double kBlockFixedBytes = 4e7;  // about 10 us at 4 TB/s
+constexpr int64_t kPadMaxElems = (int64_t)1 << 26;
+
+std::vector<ColBlock> column_blocks(int k, int64_t n, int64_t nnz, int val_bytes) {
+  std::vector<ColBlock> out;
+  for (; k >= 64; k -= 64) out.push_back({64, 64});
+  double best[64];
+  int pick[64];
+  best[0] = 0.0;
+  for (int r = 1; r <= k; ++r) {
+    best[r] = 1e300;
+    for (int K = 1; K <= 64; K *= 2) {
+      if (K > r && n * K > kPadMaxElems) break;
+      const double c = kBlockFixedBytes + (double)nnz * (4 + std::max(32, K * val_bytes)) +
+                       10.0 * (double)n * K * val_bytes + (K < r ? best[r - K] : 0.0);
+      if (c < best[r]) {
+        best[r] = c;
+        pick[r] = K;
+      }
+      if (K >= r) break;
+    }
+  }
   while (k > 0) {
-    int b = 64;
-    while (b > k) b >>= 1;
-    out.push_back(b);
-    k -= b;
+    const int K = pick[k];
+    out.push_back({K, std::min(K, k)});
+    k -= std::min(K, k);
   }
   return out;
 }
@@ -1021,7 +1051,7 @@ int phi_apply(wl_handle* h, const double* Vp, double* X, int K, SolveInfo& info)
   WL_TRY(ensure(h->b64, nk * 8));
   // b = a V
   counted(h);
-  WL_CU(launch_pack(Vp, K, 0, K, h->n, h->a_scale, h->b64.p, false, S(h)));
+  WL_CU(launch_pack(Vp, K, 0, K, K, h->n, h->a_scale, h->b64.p, false, S(h)));
   return solve(h, (const double*)h->b64.p, X, K, true, info);
 }
 
@@ -1845,7 +1875,7 @@ int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& inf
 // U(tau) = |u0| V_m y(tau) for taus [t0, t0 + nt) of an outer run, nt <=
 // kMaxTau: block t at out + t * tstride, row perm[i] (or i), columns c0..c0+K.
 int outer_combine(wl_handle* h, const OuterRun& o, int t0, int nt, double* out, int64_t ld, int64_t tstride, int c0,
-                  const int32_t* perm) {
+                  int kr, const int32_t* perm) {
   const int K = o.K, ldT = kLdT;
   const int64_t n = h->n;
   double* Ta = (double*)h->Tab.p;
@@ -1881,11 +1911,11 @@ int outer_combine(wl_handle* h, const OuterRun& o, int t0, int nt, double* out, 
     counted(h, 2);
     e = launch_df_split((const double*)h->ybuf.p, ny, (float*)h->ydf.p, (float*)h->ydf.p + ny, S(h));
     DfCombineArgs ca{(const float*)h->basis.p, (const float*)h->ydf.p, (const float*)h->ydf.p + ny, o.m, nrm, out,
-                     n, ld, tstride, c0, ldT, nt, perm};
+                     n, ld, tstride, c0, kr, ldT, nt, perm};
     if (e == cudaSuccess) e = launch_df_combine(K, ca, S(h));
   } else {
-    CombineArgs ca{(const double*)h->basis.p, (const double*)h->ybuf.p, mcol, nrm, out, n, ld, tstride, c0, ldT, nt,
-                   perm};
+    CombineArgs ca{(const double*)h->basis.p, (const double*)h->ybuf.p, mcol, nrm, out, n, ld, tstride, c0, kr, ldT,
+                   nt, perm};
     counted(h);
     e = launch_combine(K, ca, S(h));
   }
@@ -2365,12 +2395,13 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
       if (ldw != k) cudaMemcpyAsync(Wd, W, (size_t)n * ldw * 8, cudaMemcpyHostToDevice, S(h));
     }
     int c0 = 0;
-    for (int K : column_blocks(k)) {
+    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+      const int K = cb.K;
       if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       counted(h);
-      cudaError_t e = h->perm ? launch_pack_perm(Vd, ldv, c0, K, n, 1.0, h->perm, (double*)h->packV.p, S(h))
-                              : launch_pack(Vd, ldv, c0, K, n, 1.0, h->packV.p, false, S(h));
+      cudaError_t e = h->perm ? launch_pack_perm(Vd, ldv, c0, cb.kr, K, n, 1.0, h->perm, (double*)h->packV.p, S(h))
+                              : launch_pack(Vd, ldv, c0, cb.kr, K, n, 1.0, h->packV.p, false, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "pack"); break; }
       if (h->prm.f == WL_F_IDENTITY) {
         PartDev* pd;
@@ -2378,19 +2409,19 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
         thresholds_f64(K, &Tw, &Tc);
         if ((rc = get_part(h, lanczos_step_grid(K), Tw, Tc, &pd, K, 8)) != WL_OK) break;
         counted(h);
-        e = launch_laplacian_apply(h->g, *pd, (const double*)h->packV.p, K, c0, h->perm, Wd, ldw, S(h));
+        e = launch_laplacian_apply(h->g, *pd, (const double*)h->packV.p, K, c0, cb.kr, h->perm, Wd, ldw, S(h));
         info.nnz_rhs += (double)h->nnz * K;
         info.iters += 1;
       } else {
         if ((rc = phi_apply(h, (const double*)h->packV.p, (double*)h->packX.p, K, info)) != WL_OK) break;
         counted(h);
         e = h->perm ? launch_apply_out_perm((const double*)h->packV.p, (const double*)h->packX.p,
-                                            (const double*)h->Df.p, n, K, c0, h->perm, Wd, ldw, S(h))
-                    : launch_apply_out(Vd, ldv, (const double*)h->packX.p, (const double*)h->Df.p, n, K, c0, Wd,
+                                            (const double*)h->Df.p, n, K, c0, cb.kr, h->perm, Wd, ldw, S(h))
+                    : launch_apply_out(Vd, ldv, (const double*)h->packX.p, (const double*)h->Df.p, n, K, c0, cb.kr, Wd,
                                        ldw, S(h));
       }
       if (e != cudaSuccess) { rc = set_cuda_error(e, "apply"); break; }
-      c0 += K;
+      c0 += cb.kr;
     }
     if (rc != WL_OK) break;
     if (!w_dev) {
@@ -2435,18 +2466,19 @@ int wl_expmv(wl_handle* h, const double* U0, int64_t ldu, int k, const double* t
     if ((rc = stage_taus(h, taus, ntau, &dtaus)) != WL_OK) break;
     int c0 = 0;
     bool capped = false;  // a column block reached max_outer: every block is still evaluated
-    for (int K : column_blocks(k)) {
+    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+      const int K = cb.K;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       counted(h);
-      cudaError_t e = h->perm ? launch_pack_perm(U0d, ldu, c0, K, n, 1.0, h->perm, (double*)h->packX.p, S(h))
-                              : launch_pack(U0d, ldu, c0, K, n, 1.0, h->packX.p, false, S(h));
+      cudaError_t e = h->perm ? launch_pack_perm(U0d, ldu, c0, cb.kr, K, n, 1.0, h->perm, (double*)h->packX.p, S(h))
+                              : launch_pack(U0d, ldu, c0, cb.kr, K, n, 1.0, h->packX.p, false, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "expmv pack"); break; }
       OuterRun o;
       if ((rc = outer_run(h, K, dtaus, ntau, info, o, outer_total)) != WL_OK) break;
       if (info.status != WL_OK) break;
-      if ((rc = outer_combine(h, o, 0, ntau, Ud, ldo, n * ldo, c0, h->perm)) != WL_OK) break;
+      if ((rc = outer_combine(h, o, 0, ntau, Ud, ldo, n * ldo, c0, cb.kr, h->perm)) != WL_OK) break;
       if (!o.converged) capped = true;
-      c0 += K;
+      c0 += cb.kr;
     }
     if (rc != WL_OK) break;
     if (capped && info.status == WL_OK) info.status = WL_ERR_NO_CONVERGENCE;
@@ -2490,14 +2522,15 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
       if (ldo != k) cudaMemcpyAsync(Od, out, (size_t)nsteps * n * ldo * 8, cudaMemcpyHostToDevice, S(h));
     }
     int c0 = 0;
-    for (int K : column_blocks(k)) {
+    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+      const int K = cb.K;
       if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       double* cur = (double*)h->packX.p;  // p_s of this block (internal node order)
       double* y = (double*)h->packV.p;    // p_s / D_f
       counted(h);
-      cudaError_t e = h->perm ? launch_pack_perm(P0d, ldp, c0, K, n, 1.0, h->perm, cur, S(h))
-                              : launch_pack(P0d, ldp, c0, K, n, 1.0, cur, false, S(h));
+      cudaError_t e = h->perm ? launch_pack_perm(P0d, ldp, c0, cb.kr, K, n, 1.0, h->perm, cur, S(h))
+                              : launch_pack(P0d, ldp, c0, cb.kr, K, n, 1.0, cur, false, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "markov pack"); break; }
       int s = 0;
       nstep = 0;
@@ -2524,11 +2557,11 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
         }
         if (rc != WL_OK || info.status != WL_OK) break;
         counted(h);
-        e = launch_unpack(cur, n, K, c0, h->perm, Od + (size_t)t * n * ldo, ldo, S(h));
+        e = launch_unpack(cur, n, K, c0, cb.kr, h->perm, Od + (size_t)t * n * ldo, ldo, S(h));
         if (e != cudaSuccess) { rc = set_cuda_error(e, "markov out"); break; }
       }
       if (rc != WL_OK || info.status != WL_OK) break;
-      c0 += K;
+      c0 += cb.kr;
     }
     if (rc != WL_OK) break;
     if (!o_dev) {
@@ -2717,7 +2750,7 @@ int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt,
     double* Y = (double*)h->ybig.p;
     for (int t0 = 0; t0 < nt && rc == WL_OK; t0 += kMaxTau) {
       const int nb = std::min(kMaxTau, nt - t0);
-      if ((rc = outer_combine(h, o, t0, nb, Y, K, (int64_t)nk, 0, nullptr)) != WL_OK) break;
+      if ((rc = outer_combine(h, o, t0, nb, Y, K, (int64_t)nk, 0, K, nullptr)) != WL_OK) break;
       for (int i = 0; i < nb; ++i) {
         // XNysTrace of exp(-t L) from Y(t) and Omega (Alg. 1, last step)
         counted(h, 3);

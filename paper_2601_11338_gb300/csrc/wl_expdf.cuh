@@ -70,7 +70,7 @@ struct DfCombineArgs {
   const double* nrm;
   double* out;
   int64_t n, ld, tstride;
-  int c0, ldT, ntau;
+  int c0, kr, ldT, ntau;  // kr: columns written (the rest are padding)
   const int32_t* perm;
 };
 
@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(kBlock) df_combine(DfCombineArgs a, int CS) {
       return df{__ldg(a.yh + src), __ldg(a.yl + src)};
     }
   };
+  if (c >= a.kr) return;
   const df sc = df_from_double(a.nrm[c]);
   const int rpb = kBlock / CS;
   for (int64_t i = (int64_t)blockIdx.x * rpb + tid / CS; i < a.n; i += (int64_t)gridDim.x * rpb) {

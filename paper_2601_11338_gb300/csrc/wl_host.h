@@ -46,12 +46,13 @@ cudaError_t launch_partition(const Graph& g, PartDev& p, cudaStream_t s);
 // flags[0] bit0: row_ptr not monotone / bounds; bit1: column out of range or
 // unsorted/duplicate; bit2: self loop; bit3: asymmetric
 cudaError_t launch_validate(const Graph& g, int* flags, cudaStream_t s);
-// dst (n x kb, contiguous, double or float) = scale * src[:, c0:c0+kb] (leading dim ld)
-cudaError_t launch_pack(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale, void* dst,
+// dst (n x kb, contiguous, double or float) = scale * src[:, c0:c0+kr] (leading dim ld), columns kr.. zero. Here and
+// below kr <= K is the number of a block's columns that the caller has.
+cudaError_t launch_pack(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale, void* dst,
                         bool to_f32, cudaStream_t s);
-// W[:, c0:c0+K] = Df (.) V[:, c0:c0+K] - X  (X contiguous n x K)
+// W[:, c0:c0+kr] = Df (.) V[:, c0:c0+kr] - X  (X contiguous n x K)
 cudaError_t launch_apply_out(const double* V, int64_t ldv, const double* X, const double* Df, int64_t n, int K,
-                             int c0, double* W, int64_t ldw, cudaStream_t s);
+                             int c0, int kr, double* W, int64_t ldw, cudaStream_t s);
 // W[:, c0:c0+K] = Df (.) V[:, c0:c0+K] - V[:, c0:c0+K] * 0 - X where Df = d (identity case uses gather)
 cudaError_t launch_fill(double* dst, double v, int64_t count, cudaStream_t s);
 cudaError_t launch_degree_vector(const Graph& g, double* out, cudaStream_t s);
@@ -64,10 +65,10 @@ cudaError_t launch_f2d_acc(const float* src, double* dst, int64_t count, cudaStr
 // discrete-time chain: Y = X / D_f per row; Y = A X; scatter a packed block into caller columns
 cudaError_t launch_row_div(const double* X, const double* Df, int64_t n, int K, double* Y, cudaStream_t s);
 cudaError_t launch_adj_apply(const Graph& g, const double* X, int K, double* Y, cudaStream_t s);
-cudaError_t launch_unpack(const double* src, int64_t n, int K, int c0, const int32_t* perm, double* dst, int64_t ld,
+cudaError_t launch_unpack(const double* src, int64_t n, int K, int c0, int kr, const int32_t* perm, double* dst, int64_t ld,
                           cudaStream_t s);
 // identity-function apply: W[:, c0:c0+K] = d (.) V - A V for V packed n x K
-cudaError_t launch_laplacian_apply(const Graph& g, const PartDev& p, const double* Vp, int K, int c0,
+cudaError_t launch_laplacian_apply(const Graph& g, const PartDev& p, const double* Vp, int K, int c0, int kr,
                                    const int32_t* perm, double* W, int64_t ldw, cudaStream_t s);
 
 // node relabelling by decreasing degree: perm[new] = old, iperm[old] = new,
@@ -84,10 +85,10 @@ int rcm_order(const int32_t* rp, const int32_t* col, int64_t n, int32_t* perm);
 cudaError_t launch_scan(const int64_t* in, int64_t n, int64_t* out, int64_t* tmp, cudaStream_t s);
 // partition by prefix of cost(row) = deg + kRowCost (hub rows weighted x3); tmp: 2 (n + 1) + n / 1024 + 4 int64
 cudaError_t launch_partition_weighted(const Graph& g, PartDev& p, int64_t* tmp, cudaStream_t s);
-cudaError_t launch_pack_perm(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale,
+cudaError_t launch_pack_perm(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale,
                              const int32_t* perm, double* dst, cudaStream_t s);
 cudaError_t launch_apply_out_perm(const double* Vp, const double* X, const double* Df, int64_t n, int K, int c0,
-                                  const int32_t* perm, double* W, int64_t ldw, cudaStream_t s);
+                                  int kr, const int32_t* perm, double* W, int64_t ldw, cudaStream_t s);
 cudaError_t launch_permute_vec(const double* in, int64_t n, const int32_t* perm, bool scatter, double* out,
                                cudaStream_t s);
 

@@ -141,12 +141,12 @@ cudaError_t launch_validate(const Graph& g, int* flags, cudaStream_t s) {
 }
 
 template <typename T>
-__global__ void k_pack(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale, T* dst) {
+__global__ void k_pack(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale, T* dst) {
   const int64_t total = n * kb;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / kb;
     const int c = (int)(e % kb);
-    dst[e] = (T)(scale * src[i * ld + c0 + c]);
+    dst[e] = c < kr ? (T)(scale * src[i * ld + c0 + c]) : T(0);
   }
 }
 
@@ -157,29 +157,29 @@ static unsigned grid_for(int64_t total) {
   return (unsigned)b;
 }
 
-cudaError_t launch_pack(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale, void* dst,
+cudaError_t launch_pack(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale, void* dst,
                         bool to_f32, cudaStream_t s) {
   const unsigned gb = grid_for(n * kb);
   if (to_f32)
-    k_pack<float><<<gb, 256, 0, s>>>(src, ld, c0, kb, n, scale, (float*)dst);
+    k_pack<float><<<gb, 256, 0, s>>>(src, ld, c0, kr, kb, n, scale, (float*)dst);
   else
-    k_pack<double><<<gb, 256, 0, s>>>(src, ld, c0, kb, n, scale, (double*)dst);
+    k_pack<double><<<gb, 256, 0, s>>>(src, ld, c0, kr, kb, n, scale, (double*)dst);
   return cudaGetLastError();
 }
 
 __global__ void k_apply_out(const double* V, int64_t ldv, const double* X, const double* Df, int64_t n, int K, int c0,
-                            double* W, int64_t ldw) {
+                            int kr, double* W, int64_t ldw) {
   const int64_t total = n * K;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / K;
     const int c = (int)(e % K);
-    W[i * ldw + c0 + c] = Df[i] * V[i * ldv + c0 + c] - X[e];
+    if (c < kr) W[i * ldw + c0 + c] = Df[i] * V[i * ldv + c0 + c] - X[e];
   }
 }
 
 cudaError_t launch_apply_out(const double* V, int64_t ldv, const double* X, const double* Df, int64_t n, int K,
-                             int c0, double* W, int64_t ldw, cudaStream_t s) {
-  k_apply_out<<<grid_for(n * K), 256, 0, s>>>(V, ldv, X, Df, n, K, c0, W, ldw);
+                             int c0, int kr, double* W, int64_t ldw, cudaStream_t s) {
+  k_apply_out<<<grid_for(n * K), 256, 0, s>>>(V, ldv, X, Df, n, K, c0, kr, W, ldw);
   return cudaGetLastError();
 }
 
@@ -307,24 +307,24 @@ cudaError_t launch_adj_apply(const Graph& g, const double* X, int K, double* Y, 
 }
 
 // dst[row(i) * ld + c0 + c] = src[i * K + c], row(i) = perm[i] (perm NULL: i)
-__global__ void k_unpack(const double* src, int64_t n, int K, int c0, const int32_t* perm, double* dst, int64_t ld) {
+__global__ void k_unpack(const double* src, int64_t n, int K, int c0, int kr, const int32_t* perm, double* dst, int64_t ld) {
   const int64_t total = n * K;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / K;
     const int c = (int)(e % K);
-    dst[(perm ? (int64_t)perm[i] : i) * ld + c0 + c] = src[e];
+    if (c < kr) dst[(perm ? (int64_t)perm[i] : i) * ld + c0 + c] = src[e];
   }
 }
 
-cudaError_t launch_unpack(const double* src, int64_t n, int K, int c0, const int32_t* perm, double* dst, int64_t ld,
+cudaError_t launch_unpack(const double* src, int64_t n, int K, int c0, int kr, const int32_t* perm, double* dst, int64_t ld,
                           cudaStream_t s) {
-  k_unpack<<<grid_for(n * K), 256, 0, s>>>(src, n, K, c0, perm, dst, ld);
+  k_unpack<<<grid_for(n * K), 256, 0, s>>>(src, n, K, c0, kr, perm, dst, ld);
   return cudaGetLastError();
 }
 
 // W[:, c0:c0+K] = d (.) V - A V (identity function: L = D - A, Sec. 3.1)
 template <int K>
-__global__ void __launch_bounds__(kBlock) k_laplacian_apply(Graph g, Part pt, const double* Vp, int c0,
+__global__ void __launch_bounds__(kBlock) k_laplacian_apply(Graph g, Part pt, const double* Vp, int c0, int kr,
                                                             const int32_t* perm, double* W, int64_t ldw) {
   using C = Cfg<double, K>;
   constexpr int VW = C::VW;
@@ -333,22 +333,23 @@ __global__ void __launch_bounds__(kBlock) k_laplacian_apply(Graph g, Part pt, co
   auto fin = [&](int row, int deg, int lane_off, const double (&nb)[VW], const Pack<double, VW>& vv) {
 #pragma unroll
     for (int v = 0; v < VW; ++v)
-      W[(size_t)(perm ? perm[row] : row) * ldw + c0 + lane_off + v] = (double)deg * vv.v[v] - nb[v];
+      if (lane_off + v < kr)
+        W[(size_t)(perm ? perm[row] : row) * ldw + c0 + lane_off + v] = (double)deg * vv.v[v] - nb[v];
   };
   for_rows_gather<double, K>(g, pt, Vp, s_gath, pre, fin);
 }
 
-cudaError_t launch_laplacian_apply(const Graph& g, const PartDev& p, const double* Vp, int K, int c0,
+cudaError_t launch_laplacian_apply(const Graph& g, const PartDev& p, const double* Vp, int K, int c0, int kr,
                                    const int32_t* perm, double* W, int64_t ldw, cudaStream_t s) {
   const Part pt = p.view();
   switch (K) {
-    case 1: k_laplacian_apply<1><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 2: k_laplacian_apply<2><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 4: k_laplacian_apply<4><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 8: k_laplacian_apply<8><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 16: k_laplacian_apply<16><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 32: k_laplacian_apply<32><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
-    case 64: k_laplacian_apply<64><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, perm, W, ldw); break;
+    case 1: k_laplacian_apply<1><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 2: k_laplacian_apply<2><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 4: k_laplacian_apply<4><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 8: k_laplacian_apply<8><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 16: k_laplacian_apply<16><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 32: k_laplacian_apply<32><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
+    case 64: k_laplacian_apply<64><<<p.G, kBlock, 0, s>>>(g, pt, Vp, c0, kr, perm, W, ldw); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -587,24 +588,24 @@ cudaError_t launch_partition_weighted(const Graph& g, PartDev& p, int64_t* tmp /
 
 // ---- permuted copies across the API boundary
 // dst[new * K + c] = scale * src[perm[new] * ld + c0 + c]
-__global__ void k_pack_perm(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale,
+__global__ void k_pack_perm(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale,
                             const int32_t* perm, double* dst) {
   const int64_t total = n * kb;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / kb;
     const int c = (int)(e % kb);
-    dst[e] = scale * src[(int64_t)perm[i] * ld + c0 + c];
+    dst[e] = c < kr ? scale * src[(int64_t)perm[i] * ld + c0 + c] : 0.0;
   }
 }
 
 // W[perm[i] * ldw + c0 + c] = Df[i] * Vp[i * K + c] - X[i * K + c]
 __global__ void k_apply_out_perm(const double* Vp, const double* X, const double* Df, int64_t n, int K, int c0,
-                                 const int32_t* perm, double* W, int64_t ldw) {
+                                 int kr, const int32_t* perm, double* W, int64_t ldw) {
   const int64_t total = n * K;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / K;
     const int c = (int)(e % K);
-    W[(int64_t)perm[i] * ldw + c0 + c] = Df[i] * Vp[e] - X[e];
+    if (c < kr) W[(int64_t)perm[i] * ldw + c0 + c] = Df[i] * Vp[e] - X[e];
   }
 }
 
@@ -615,15 +616,15 @@ __global__ void k_permute_vec(const double* in, int64_t n, const int32_t* perm, 
   }
 }
 
-cudaError_t launch_pack_perm(const double* src, int64_t ld, int c0, int kb, int64_t n, double scale,
+cudaError_t launch_pack_perm(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale,
                              const int32_t* perm, double* dst, cudaStream_t s) {
-  k_pack_perm<<<grid_for(n * kb), 256, 0, s>>>(src, ld, c0, kb, n, scale, perm, dst);
+  k_pack_perm<<<grid_for(n * kb), 256, 0, s>>>(src, ld, c0, kr, kb, n, scale, perm, dst);
   return cudaGetLastError();
 }
 
 cudaError_t launch_apply_out_perm(const double* Vp, const double* X, const double* Df, int64_t n, int K, int c0,
-                                  const int32_t* perm, double* W, int64_t ldw, cudaStream_t s) {
-  k_apply_out_perm<<<grid_for(n * K), 256, 0, s>>>(Vp, X, Df, n, K, c0, perm, W, ldw);
+                                  int kr, const int32_t* perm, double* W, int64_t ldw, cudaStream_t s) {
+  k_apply_out_perm<<<grid_for(n * K), 256, 0, s>>>(Vp, X, Df, n, K, c0, kr, perm, W, ldw);
   return cudaGetLastError();
 }
 

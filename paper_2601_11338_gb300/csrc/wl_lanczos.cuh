@@ -484,6 +484,7 @@ struct CombineArgs {
   int64_t ld;
   int64_t tstride;
   int c0;
+  int kr;               // columns written (the rest are padding)
   int ldT;
   int ntau;
   const int32_t* perm;  // internal row i goes to caller row perm[i] (NULL: identity)
@@ -496,6 +497,7 @@ __global__ void __launch_bounds__(kBlock) combine(CombineArgs a) {
   const size_t total = (size_t)a.n * K;
   for (size_t e = (size_t)blockIdx.x * kBlock + threadIdx.x; e < total; e += (size_t)gridDim.x * kBlock) {
     const int c = (int)(e % K);
+    if (c >= a.kr) continue;
     const size_t i = e / K;
     const int m = a.mcol[c];
     double acc[kMaxTau];

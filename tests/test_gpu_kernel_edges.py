@@ -148,3 +148,45 @@ def test_fp64_neighbour_sums_of_uneven_magnitude():
     scale = np.abs(want).max(0)
     assert (np.abs(W - want).max(0) <= 1e-10 * scale).all()
     w.close()
+
+
+# Column counts that end in a padded block, and leading dimensions beyond k:
+# the columns after the block's own keep what the caller has there
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)])
+@pytest.mark.parametrize("reorder", [0, 1])
+def test_padded_column_blocks(prec, tol, bound, reorder):
+    from paper_2601_11338_gb300 import wl
+    g = wlgen.erdos_renyi(411, 7.0, 9)
+    A = graph.dense_adjacency(g.row_ptr, g.col_idx, g.n)
+    w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=tol, outer_tol=tol, reorder=reorder)
+    phi = walks.phi_resolvent_closed(A, 1.0, w.info["alpha"])
+    L, D = walks.walk_laplacian(phi), walks.walk_degrees(phi)
+    for k in (3, 5, 13, 33, 63, 67, 100):
+        ld = k + 3
+        V = torch.as_tensor(np.random.default_rng(k).standard_normal((g.n, ld)), device="cuda")
+        W = torch.full((g.n, ld), 7.25, dtype=torch.float64, device="cuda")
+        assert wl.wl_apply(w.h, V, ld, k, W, ld) == wl.WL_OK
+        want = L @ V.cpu().numpy()[:, :k]
+        got = W.cpu().numpy()
+        assert (got[:, k:] == 7.25).all()
+        assert np.abs(got[:, :k] - want).max() <= bound * np.abs(want).max(), k
+    k = 5
+    U = torch.full((2, g.n, 8), 7.25, dtype=torch.float64, device="cuda")
+    for shift in ((0.0, 2.0) if prec == "refined" else (0.0,)):
+        w.set(shift=shift)
+        assert wl.wl_expmv(w.h, V, ld, k, [0.5, 2.0], U, 8) == wl.WL_OK
+        want = walks.diffusion(L, V.cpu().numpy()[:, :k], [0.5, 2.0])
+        got = U.cpu().numpy()
+        assert (got[:, :, k:] == 7.25).all()
+        for t in range(2):
+            assert np.abs(got[t, :, :k] - want[t]).max() <= bound * np.abs(want[t]).max()
+    w.set(shift=0.0)
+    P0 = torch.rand((g.n, ld), dtype=torch.float64, device="cuda")
+    assert wl.wl_markov(w.h, P0, ld, k, [1, 3], U, 8) == wl.WL_OK
+    got, p = U.cpu().numpy(), P0.cpu().numpy()[:, :k]
+    for t, steps in ((0, 1), (1, 2)):
+        for _ in range(steps):
+            p = phi @ (p / D[:, None])
+        assert np.abs(got[t, :, :k] - p).max() <= bound * np.abs(p).max()
+    assert (got[:, :, k:] == 7.25).all()
+    w.close()
