@@ -1136,8 +1136,13 @@ int sp_grid(wl_handle* h) {
 int sp_run(wl_handle* h, SpRun* r, double rtol, bool seeded) {
   const int cap = sp_cap(h), gu = sp_grid(h), gs = gu + h->nhub + h->nmid_blk;
   WL_TRY(sp_buffers(h, gs));
+  if (!t_sp_batch) WL_TRY(ensure_phase_buffers(h, std::max(gs, h->sms)));
   const SpArgs a = sp_args(h, r->c0, r->cD);
   SpState* st = (SpState*)h->spstate.p;
+  // a single graph's steps as cooperative kernels where its vectors fit; the
+  // batched build's searches share the GPU and run as kernels over all of them
+  const bool coop = !t_sp_batch && sp_coop_fits(a, h->nnz, h->sms);
+  if (coop) WL_CU(cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h)));
   for (int guard = 0; guard < 256; ++guard) {
     if (r->exact || (r->m > 0 && r->bound <= rtol * std::fabs(r->theta))) break;
     int mode = 2;
@@ -1174,11 +1179,24 @@ int sp_run(wl_handle* h, SpRun* r, double rtol, bool seeded) {
         WL_CU(launch_sp_ritz(a, gu, S(h)));
       }
       if (mode == 0) WL_CU(cudaMemsetAsync(st, 0, sizeof(SpState), S(h)));  // tickets and flags start at zero
-      counted(h, 1 + 2 * (j1 - j0) + (j1 - j0 + kSpCheck - 1) / kSpCheck);
       WL_CU(launch_sp_start(a, mode, gu, S(h)));
-      WL_CU(launch_sp_steps(a, j0, j1, cap, kSpCheck, rtol, gs, gu, S(h)));
+      const int chunks = (j1 - j0 + kSpCheck - 1) / kSpCheck;
+      if (coop) {
+        counted(h, 1 + 2 * chunks);
+        if (fault_mode() == kFaultTimeout) {
+          static const int gave_up = WL_ERR_TIMEOUT;
+          WL_CU(cudaMemcpyAsync(&h->cgbar()->err, &gave_up, sizeof(int), cudaMemcpyHostToDevice, S(h)));
+        }
+        WL_CU(launch_sp_steps_coop(a, h->nnz, h->sms, h->cgbar(), j0, j1, cap, kSpCheck, rtol, S(h)));
+        h->bar_clean = false;
+        WL_CU(cudaMemcpyAsync(h->h_pin + 16, &h->cgbar()->err, sizeof(int), cudaMemcpyDeviceToHost, S(h)));
+      } else {
+        counted(h, 1 + 2 * (j1 - j0) + chunks);
+        WL_CU(launch_sp_steps(a, j0, j1, cap, kSpCheck, rtol, gs, gu, S(h)));
+      }
       WL_CU(cudaMemcpyAsync(h->h_pin, &st->start_norm, 9 * 8 + 4 * 4, cudaMemcpyDeviceToHost, S(h)));
       WL_CU(cudaStreamSynchronize(S(h)));
+      if (coop && *(const int*)(h->h_pin + 16) != 0) return *(const int*)(h->h_pin + 16);
       for (int i = 0; i < 8; ++i) o[i] = h->h_pin[1 + i];
       const int* ints = (const int*)(h->h_pin + 9);
       m_eff = ints[0];

@@ -183,6 +183,10 @@ cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t 
 cudaError_t launch_sp_steps(const SpArgs& a, int j0, int j1, int cap, int check, double rtol, int grid_s,
                             int grid_u, cudaStream_t s);
 // Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
+// the same steps as cooperative kernels of `check` steps each; bar is cleared before each
+bool sp_coop_fits(const SpArgs& a, int64_t nnz, int sms);
+cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
+                                 int check, double rtol, cudaStream_t s);
 cudaError_t launch_sp_ritz(const SpArgs& a, int grid_u, cudaStream_t s);
 // One round of the batched spectral searches: the np jobs (device array) with
 // their CTA offsets in the S kernel (off_s, np + 1 entries, off_s[np] =

@@ -1,5 +1,7 @@
 // Spectral-scale Lanczos kernels (k = 1, double-float basis): launchers.
 #define WL_SPEC_KERNELS
+#include <algorithm>
+
 #include "wl_host.h"
 #include "wl_spec.cuh"
 
@@ -29,6 +31,51 @@ cudaError_t launch_sp_steps(const SpArgs& a0, int j0, int j1, int cap, int check
     sp_s<<<grid_s, kPhaseBlock, 0, s>>>(a);
     sp_u<<<grid_u, kPhaseBlock, 0, s>>>(a, j == cap - 1 ? 1 : 0);
     if ((j + 1) % check == 0 || j + 1 == j1) sp_eig<<<1, 2 * kSpEigT, 0, s>>>(a.st, rtol);
+  }
+  return cudaGetLastError();
+}
+
+// grid, threads and shared memory of the cooperative steps; false where a
+// run's vectors don't fit, or where they are so few that the row loops'
+// kernels cost no more
+static bool sp_coop_shape(const SpArgs& a, int64_t nnz, int sms, int* grid, int* threads, size_t* smem, int* nhead) {
+  const int64_t units = a.g.n * kSpCoopLpr;
+  *grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (units + 255) / 256));
+  const int64_t rows = coop_rows_local(a.g.n, *grid, kSpCoopCh);
+  const int64_t passes = (rows * kSpCoopLpr + kSpCoopThreads - 1) / kSpCoopThreads;
+  *threads = (int)std::max<int64_t>(256, (rows * kSpCoopLpr / passes + 31) / 32 * 32);
+  const int64_t nslot = rows + (a.nmid + *grid - 1) / *grid + (a.g.nhub + *grid - 1) / *grid;
+  const size_t vec = (size_t)nslot * 3 * sizeof(float2);
+  if (vec > kSpCoopSmem) return false;
+  *nhead = (int)std::min<int64_t>({a.g.n, nnz / (4 * *grid), (int64_t)((kSpCoopSmem - vec) / sizeof(float2))});
+  *smem = vec + (size_t)*nhead * sizeof(float2);
+  return true;
+}
+
+bool sp_coop_fits(const SpArgs& a, int64_t nnz, int sms) {
+  int grid, threads, nhead;
+  size_t smem;
+  return sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &nhead);
+}
+
+cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
+                                 int check, double rtol, cudaStream_t s) {
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(sp_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpCoopSmem);
+  if (attr != cudaSuccess) return attr;
+  SpCoopArgs ca{a, bar, 0, 0, cap, 0};
+  int grid, threads;
+  size_t smem;
+  if (!sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &ca.nhead)) return cudaErrorInvalidValue;
+  for (int j = j0; j < j1; j = ca.j1) {
+    ca.j0 = j;
+    ca.j1 = std::min(j1, (j / check + 1) * check);
+    cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+    void* args[] = {&ca};
+    e = cudaLaunchCooperativeKernel((const void*)sp_coop, dim3(grid), dim3(threads), args, smem, s);
+    if (e != cudaSuccess) return e;
+    sp_eig<<<1, 2 * kSpEigT, 0, s>>>(a.st, rtol);
   }
   return cudaGetLastError();
 }

@@ -20,6 +20,7 @@
 // the bound is below rtol |theta_1|.
 #pragma once
 #include "wl_cg2.cuh"
+#include "wl_coop.cuh"
 #include "wl_df.cuh"
 
 namespace wl {
@@ -51,6 +52,14 @@ struct SpArgs {
   SpState* st;
   int j;
   uint64_t seed;
+};
+
+// Steps j0 .. j1 - 1 of a run as one cooperative kernel
+struct SpCoopArgs {
+  SpArgs a;
+  CoopBar* bar;
+  int j0, j1, cap;
+  int nhead;  // leading entries of w kept in shared memory
 };
 
 // One problem's share of a round of the batched searches (many graphs'
@@ -304,6 +313,236 @@ __device__ __forceinline__ void sp_u_body(const SpArgs& a, int j, int last, int 
       st->stop = 1;
     }
     st->ticket = 0;
+  }
+}
+
+// ---------------------------------------------------------------- cooperative steps
+// The same steps with every row owned by one CTA for the launch (one CTA per
+// SM): w, v_j and v_{j-1} of its rows stay in shared memory, w_j and v_j are
+// also written to global memory (for the gathers, and the basis), and the two
+// column sums of a step end in grid barriers instead of kernels. Four lanes a
+// short row, a warp a mid or hub row, the CTA a longer hub row, as in the
+// cooperative CG kernel; the hubs' entries of w are gathered from shared
+// memory. Chung-Lu 4e5: 31 us a step (two kernels:
+// 44 us).
+constexpr int kSpCoopThreads = 1024;
+constexpr int kSpCoopLpr = 4;   // lanes of a short row
+constexpr int kSpCoopCh = 4;    // consecutive rows of a CTA (a 32-byte sector of w)
+constexpr int kSpCoopUnroll = 4;
+constexpr size_t kSpCoopSmem = 227 * 1024 - 2048;
+
+__global__ void __launch_bounds__(kSpCoopThreads, 1) sp_coop(SpCoopArgs ca) {
+  extern __shared__ __align__(16) float2 sp_smem[];
+  __shared__ float2 s_w[32];
+  __shared__ float s_l[32];
+  __shared__ double s_sum;
+  __shared__ df s_inv, s_al, s_bp;
+  const SpArgs& a = ca.a;
+  SpState* st = a.st;
+  if (*(volatile int*)&st->stop || *(volatile int*)&ca.bar->err) return;
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+  const int b = blockIdx.x, grid = gridDim.x;
+  const int nloc = (int)coop_rows_local(a.g.n, grid, kSpCoopCh);
+  const int lim = a.nmid > 0 ? kSpWarpDeg : kHubDeg;
+  const int nmid_l = a.nmid > b ? (a.nmid - b + grid - 1) / grid : 0;
+  const int nhub_l = a.g.nhub > b ? (a.g.nhub - b + grid - 1) / grid : 0;
+  const int mid0 = nloc, hub0 = mid0 + (a.nmid + grid - 1) / grid;
+  const int nslot = hub0 + (a.g.nhub + grid - 1) / grid;
+  float2* sw = sp_smem;
+  float2* sv = sw + nslot;
+  float2* sm = sv + nslot;
+  float2* s_head = sm + nslot;
+  const int32_t* __restrict__ rp = a.g.row_ptr;
+  const int32_t* __restrict__ col = a.g.col;
+  auto row_of = [&](int lr) -> int64_t {
+    return ((int64_t)(lr / kSpCoopCh) * grid + b) * kSpCoopCh + lr % kSpCoopCh;
+  };
+  auto for_slots = [&](auto f) {
+    for (int s = tid; s < nloc; s += nthr) {
+      const int64_t row = row_of(s);
+      if (row >= a.g.n || __ldg(rp + row + 1) - __ldg(rp + row) > lim) continue;
+      f(s, row);
+    }
+    for (int s = tid; s < nmid_l; s += nthr) f(mid0 + s, (int64_t)__ldg(a.mid + s * grid + b));
+    for (int s = tid; s < nhub_l; s += nthr) f(hub0 + s, (int64_t)__ldg(a.g.hubs + s * grid + b));
+  };
+  // sum over the grid of the threads' double-float values, in s_sum
+  float2* part = reinterpret_cast<float2*>(a.part);
+  unsigned target = 0;
+  int half = 0;
+  auto add2 = [](float2 x, float2 y) { return CoopSum<float>::add(x, y); };
+  auto grid_sum = [&](float aS, float aC) -> bool {
+    const df t0 = two_sum(aS, aC);
+    float2 t = make_float2(t0.hi, t0.lo);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) t = add2(t, CoopSum<float>::shfl(t, off));
+    if (lane == 0) s_w[warp] = t;
+    __syncthreads();
+    float2* p = part + (size_t)half * grid;
+    if (warp == 0) {
+      t = lane < nwarp ? s_w[lane] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) t = add2(t, CoopSum<float>::shfl(t, off));
+      if (lane == 0) p[b] = t;
+    }
+    target += grid;
+    if (!coop_sync(ca.bar, target)) return false;
+    if (warp == 0) {
+      t = make_float2(0.f, 0.f);
+      for (int g = lane; g < grid; g += 32) t = add2(t, __ldcg(p + g));
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) t = add2(t, CoopSum<float>::shfl(t, off));
+      if (lane == 0) s_sum = (double)t.x + (double)t.y;
+    }
+    half ^= 1;
+    __syncthreads();
+    return true;
+  };
+  const df c0 = df_from_double(a.c0), cA = df_from_double(a.cA), cD = df_from_double(a.cD);
+  {
+    const float2* w0 = (ca.j0 & 1) ? a.W[0] : a.W[1];
+    const float2* vm = a.V + (size_t)(ca.j0 > 0 ? ca.j0 - 1 : 0) * a.g.n;
+    for_slots([&](int s, int64_t row) {
+      sw[s] = __ldcg(w0 + row);
+      if (ca.j0 > 0) sm[s] = __ldcg(vm + row);
+    });
+  }
+  double bprev = ca.j0 == 0 ? st->start_norm : st->beta[ca.j0 - 1];
+  for (int j = ca.j0; j < ca.j1; ++j) {
+    const float2* Wp = (j & 1) ? a.W[0] : a.W[1];
+    float2* Wc = (j & 1) ? a.W[1] : a.W[0];
+    float2* Vj = a.V + (size_t)j * a.g.n;
+    if (tid == 0) s_inv = df_from_double(1.0 / bprev);
+    for (int i = tid; i < ca.nhead; i += nthr) s_head[i] = __ldcg(Wp + i);
+    __syncthreads();
+    const df inv = s_inv;
+    float aS = 0.f, aC = 0.f;
+    auto fin = [&](int s, int64_t row, int deg, float hs, float hc, float hl) {
+      const df nb = df_mul(two_sum(hs, hc + hl), inv);
+      const df v = df_mul(ld_df2(sw + s), inv);
+      const df crow = df_add(c0, df_mul_f(cD, (float)deg));
+      const df w = df_add(df_mul(crow, v), df_mul(cA, nb));
+      st_df2(sv + s, v);
+      st_df2(sw + s, w);
+      st_df2(Vj + row, v);
+      df_acc2(aS, aC, df_mul(v, w));
+    };
+    auto gather = [&](int beg, int end, int step, float& hs, float& hc, float& hl) {
+      constexpr int U = kSpCoopUnroll;
+      for (int e = beg; e < end; e += U * step) {
+        int q[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) q[u] = e + u * step < end ? __ldg(col + e + u * step) : -1;
+        float2 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if ((unsigned)q[u] < (unsigned)ca.nhead)
+            x[u] = s_head[q[u]];
+          else if (q[u] >= 0)
+            x[u] = *(Wp + q[u]);  // L1 allowed: ordered after the other SMs' writes by the barrier
+          else
+            x[u] = make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          df_acc(hs, hc, x[u].x);
+          hl += x[u].y;
+        }
+      }
+    };
+    auto fold = [&](float& hs, float& hc, float& hl, int off) {
+      const float so = __shfl_xor_sync(0xffffffffu, hs, off);
+      const float co = __shfl_xor_sync(0xffffffffu, hc, off);
+      const float lo = __shfl_xor_sync(0xffffffffu, hl, off);
+      const df u = two_sum(hs, so);
+      hs = u.hi;
+      hc += u.lo + co;
+      hl += lo;
+    };
+    for (int h = 0; h < nhub_l; ++h) {  // long hub rows by the whole CTA
+      const int64_t row = __ldg(a.g.hubs + h * grid + b);
+      const int beg = __ldg(rp + row), end = __ldg(rp + row + 1);
+      if (end - beg <= kCoopHubWarp) continue;
+      float hs = 0.f, hc = 0.f, hl = 0.f;
+      gather(beg + tid, end, nthr, hs, hc, hl);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) fold(hs, hc, hl, off);
+      __syncthreads();
+      if (lane == 0) {
+        s_w[warp] = make_float2(hs, hc);
+        s_l[warp] = hl;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        const float2 t = lane < nwarp ? s_w[lane] : make_float2(0.f, 0.f);
+        hs = t.x;
+        hc = t.y;
+        hl = lane < nwarp ? s_l[lane] : 0.f;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) fold(hs, hc, hl, off);
+        if (lane == 0) fin(hub0 + h, row, end - beg, hs, hc, hl);
+      }
+      __syncthreads();
+    }
+    for (int m = warp; m < nmid_l + nhub_l; m += nwarp) {  // a warp each
+      const bool hub = m >= nmid_l;
+      const int64_t row = hub ? __ldg(a.g.hubs + (m - nmid_l) * grid + b) : __ldg(a.mid + m * grid + b);
+      const int beg = __ldg(rp + row), end = __ldg(rp + row + 1);
+      if (hub && end - beg > kCoopHubWarp) continue;
+      float hs = 0.f, hc = 0.f, hl = 0.f;
+      gather(beg + lane, end, 32, hs, hc, hl);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) fold(hs, hc, hl, off);
+      if (lane == 0) fin(hub ? hub0 + m - nmid_l : mid0 + m, row, end - beg, hs, hc, hl);
+    }
+    for (int u0 = warp * 32; u0 < nloc * kSpCoopLpr; u0 += nthr) {
+      const int u = u0 + lane, lr = u / kSpCoopLpr, e = u % kSpCoopLpr;
+      const int64_t row = row_of(lr);
+      int beg = 0, end = 0;
+      bool live = lr < nloc && row < a.g.n;
+      if (live) {
+        beg = __ldg(rp + row);
+        end = __ldg(rp + row + 1);
+        live = end - beg <= lim;
+      }
+      float hs = 0.f, hc = 0.f, hl = 0.f;
+      if (live) gather(beg + e, end, kSpCoopLpr, hs, hc, hl);
+#pragma unroll
+      for (int off = 1; off < kSpCoopLpr; off <<= 1) fold(hs, hc, hl, off);
+      if (live && e == 0) fin(lr, row, end - beg, hs, hc, hl);
+    }
+    if (!grid_sum(aS, aC)) return;
+    const double al = s_sum, bp = j > 0 ? bprev : 0.0;
+    if (tid == 0) {
+      s_al = df_from_double(al);
+      s_bp = df_from_double(bp);
+    }
+    __syncthreads();
+    const df dal = s_al, dbp = s_bp;
+    aS = aC = 0.f;
+    for_slots([&](int s, int64_t row) {
+      df w = df_sub(ld_df2(sw + s), df_mul(dal, ld_df2(sv + s)));
+      if (j > 0) w = df_sub(w, df_mul(dbp, ld_df2(sm + s)));
+      st_df2(sw + s, w);
+      st_df2(Wc + row, w);
+      df_acc2(aS, aC, df_mul(w, w));
+    });
+    if (!grid_sum(aS, aC)) return;
+    const double bj = sqrt(fmax(s_sum, 0.0));
+    // invariant subspace reached: T_{j+1} is exact
+    const bool brk = !(bj > 1e-13 * (fabs(al) + bp + 1e-300));
+    if (b == 0 && tid == 0) {
+      st->alpha[j] = al;
+      st->beta[j] = bj;
+      st->m_eff = j + 1;
+      if (brk) st->brk = 1;
+      if (brk || j == ca.cap - 1) st->stop = 1;
+    }
+    if (brk) return;
+    bprev = bj;
+    float2* t = sm;  // v_j is the next step's v_{j-1}
+    sm = sv;
+    sv = t;
   }
 }
 
