@@ -634,7 +634,7 @@ struct CgStart {
 // fit in shared memory (nothing launched).
 template <typename T>
 bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& start, cudaError_t* e) {
-  CoopArgs<T> co{a, h->cgbar(), 0, start.r0 ? start.r0 : a.r, start.gamma0, start.add_x ? 1 : 0};
+  CoopArgs<T> co{a, h->cgbar(), start.r0 ? start.r0 : a.r, start.gamma0, start.add_x ? 1 : 0};
   if (!h->bar_clean) {
     *e = cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h));
     if (*e != cudaSuccess) return true;
@@ -715,7 +715,7 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, int grid_s, int grid_u
 }
 
 int ensure_phase_buffers(wl_handle* h, int grid) {
-  WL_TRY(ensure(h->part, (size_t)grid * 64 * 2 * 8 + 1024));
+  WL_TRY(ensure(h->part, ((size_t)grid + kCoopGroups) * 64 * 2 * 8 + 1024));
   if (!h->cgstate.p) {
     WL_TRY(ensure(h->cgstate, sizeof(CgBlock)));
     WL_CU(cudaMemsetAsync(h->cgstate.p, 0, sizeof(CgBlock), S(h)));

@@ -89,4 +89,48 @@ __host__ __device__ inline df df_from_double(double x) {
 
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 
+// sum type of the reductions: double-float for FP32 (error-free adds with
+// FP32 instructions; FP64 adds run at 1/64 of their rate), FP64 for FP64
+template <typename T>
+struct CoopSum;
+template <>
+struct CoopSum<float> {
+  using S = float2;
+  static __device__ __forceinline__ S from(float v) { return make_float2(v, 0.f); }
+  static __device__ __forceinline__ S add(S a, S b) {
+    const df t = df_add(df{a.x, a.y}, df{b.x, b.y});
+    return make_float2(t.hi, t.lo);
+  }
+  static __device__ __forceinline__ S shfl(S a, int off) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, off), __shfl_xor_sync(0xffffffffu, a.y, off));
+  }
+  static __device__ __forceinline__ S zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ double out(S a) { return (double)a.x + (double)a.y; }
+  static __device__ __forceinline__ S in(double v) {
+    const df t = df_from_double(v);
+    return make_float2(t.hi, t.lo);
+  }
+  static __device__ __forceinline__ float lead(S a) { return a.x; }
+  // a / b to FP32: the leading quotient and one correction (an FP64 division waits a microsecond here)
+  static __device__ __forceinline__ float quot(S a, S b) {
+    const float q = a.x / b.x;
+    const df r = df_sub(df{a.x, a.y}, df_mul_f(df{b.x, b.y}, q));
+    return q + r.hi / b.x;
+  }
+  static __device__ __forceinline__ bool le(S a, S b) { return a.x < b.x || (a.x == b.x && a.y <= b.y); }
+};
+template <>
+struct CoopSum<double> {
+  using S = double;
+  static __device__ __forceinline__ S from(double v) { return v; }
+  static __device__ __forceinline__ S add(S a, S b) { return a + b; }
+  static __device__ __forceinline__ S shfl(S a, int off) { return __shfl_xor_sync(0xffffffffu, a, off); }
+  static __device__ __forceinline__ S zero() { return 0.0; }
+  static __device__ __forceinline__ double out(S a) { return a; }
+  static __device__ __forceinline__ S in(double v) { return v; }
+  static __device__ __forceinline__ double lead(S a) { return a; }
+  static __device__ __forceinline__ double quot(S a, S b) { return a / b; }
+  static __device__ __forceinline__ bool le(S a, S b) { return a <= b; }
+};
+
 }  // namespace wl

@@ -329,6 +329,7 @@ constexpr int kSpCoopThreads = 1024;
 constexpr int kSpCoopLpr = 4;   // lanes of a short row
 constexpr int kSpCoopCh = 4;    // consecutive rows of a CTA (a 32-byte sector of w)
 constexpr int kSpCoopUnroll = 4;
+constexpr int kSpCoopHubWarp = 2048;  // hub rows of up to this many entries are taken by a warp
 constexpr size_t kSpCoopSmem = 227 * 1024 - 2048;
 
 __global__ void __launch_bounds__(kSpCoopThreads, 1) sp_coop(SpCoopArgs ca) {
@@ -462,7 +463,7 @@ __global__ void __launch_bounds__(kSpCoopThreads, 1) sp_coop(SpCoopArgs ca) {
     for (int h = 0; h < nhub_l; ++h) {  // long hub rows by the whole CTA
       const int64_t row = __ldg(a.g.hubs + h * grid + b);
       const int beg = __ldg(rp + row), end = __ldg(rp + row + 1);
-      if (end - beg <= kCoopHubWarp) continue;
+      if (end - beg <= kSpCoopHubWarp) continue;
       float hs = 0.f, hc = 0.f, hl = 0.f;
       gather(beg + tid, end, nthr, hs, hc, hl);
 #pragma unroll
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(kSpCoopThreads, 1) sp_coop(SpCoopArgs ca) {
       const bool hub = m >= nmid_l;
       const int64_t row = hub ? __ldg(a.g.hubs + (m - nmid_l) * grid + b) : __ldg(a.mid + m * grid + b);
       const int beg = __ldg(rp + row), end = __ldg(rp + row + 1);
-      if (hub && end - beg > kCoopHubWarp) continue;
+      if (hub && end - beg > kSpCoopHubWarp) continue;
       float hs = 0.f, hc = 0.f, hl = 0.f;
       gather(beg + lane, end, 32, hs, hc, hl);
 #pragma unroll

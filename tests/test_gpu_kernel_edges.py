@@ -190,3 +190,20 @@ def test_padded_column_blocks(prec, tol, bound, reorder):
         assert np.abs(got[t, :, :k] - p).max() <= bound * np.abs(p).max()
     assert (got[:, :, k:] == 7.25).all()
     w.close()
+
+
+def test_small_refined_solves_scale_with_their_columns():
+    """The cooperative FP32 corrections scale each column by a power of two:
+    columns of very different size give the same solutions, scaled (to the
+    parity tolerance; squares of 2^+-40 stay inside FP32's range)."""
+    for g in (wlgen.erdos_renyi(700, 8.0, 2), wlgen.barabasi_albert(9001, 10, 4)):
+        w = WL(g, variant="nbt", alpha_rel=0.5, prec="refined", tol=1e-12)
+        V = torch.as_tensor(np.random.default_rng(4).standard_normal((g.n, 8)), device="cuda")
+        e = torch.tensor([0, 40, -40, 13, -27, 1, 31, -38], device="cuda")
+        s = torch.pow(torch.tensor(2.0, dtype=torch.float64, device="cuda"), e)
+        want = w.apply(V)
+        got = w.apply(V * s) / s
+        assert (got - want).abs().max() <= 1e-8 * want.abs().max(), g.name
+        one = torch.stack([w.apply(V[:, :1] * c)[:, 0] / c for c in s], 1)
+        assert (one - want[:, :1]).abs().max() <= 1e-8 * want.abs().max(), g.name
+        w.close()
