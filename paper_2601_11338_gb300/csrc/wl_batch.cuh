@@ -80,54 +80,41 @@ struct BatchArgs {
 
 #ifdef WL_BATCH_KERNELS
 
-// CTA column sums of per-thread values (thread t owns columns (t % G) VW + v),
-// stored to out[0 .. K). FP32 values (or their double-float sums) are added in
-// double-float: the FP64 adds of a butterfly over 256 threads held a tile's
-// CTA for 1000 clocks.
-template <typename T, int K>
-__device__ __forceinline__ void block_colsum_store(const typename CoopSum<T>::S (&val)[Cfg<T, K>::VW], double* out) {
-  using C = Cfg<T, K>;
-  using SM = CoopSum<T>;
-  using S = typename SM::S;
-  constexpr int VW = C::VW, G = C::G, NW = kPhaseBlock / 32;
-  __shared__ S s_w[NW * K];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  S a[VW];
-#pragma unroll
-  for (int v = 0; v < VW; ++v) a[v] = val[v];
-#pragma unroll
-  for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-    for (int v = 0; v < VW; ++v) a[v] = SM::add(a[v], SM::shfl(a[v], off));
-  if (lane < G)
-#pragma unroll
-    for (int v = 0; v < VW; ++v) s_w[warp * K + lane * VW + v] = a[v];
-  __syncthreads();
-  if (tid < K) {
-    S t = s_w[tid];
-    for (int w = 1; w < NW; ++w) t = SM::add(t, s_w[w * K + tid]);
-    out[tid] = SM::out(t);
-  }
-}
-
 // s += x^2, exactly rounded to the sum's type
 __device__ __forceinline__ void acc_sq(float2& s, float x) { df_acc2(s.x, s.y, two_prod(x, x)); }
 __device__ __forceinline__ void acc_sq(double& s, double x) { s = fma(x, x, s); }
 
-// Sum over the tiles of one problem, fixed order: out[c] in shared memory
+// Sum over the tiles of one problem, fixed order: out[c] in shared memory.
+// Eight loads in flight per thread (one at a time, the sums of 312 tiles
+// waited 39 times for memory), and the threads' sums folded in a tree.
 template <int K>
 __device__ __forceinline__ void problem_sum(const double* part, int tb, int te, double* s_tmp, double* out) {
   constexpr int J = kPhaseBlock / K;
   const int tid = threadIdx.x, c = tid % K, j = tid / K;
   double s = 0.0;
-  for (int t = tb + j; t < te; t += J) s += __ldcg(part + (size_t)t * K + c);
+  int t = tb + j;
+  for (; t + 7 * J < te; t += 8 * J) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (size_t)(t + u * J) * K + c);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = t + u * J < te ? __ldcg(part + (size_t)(t + u * J) * K + c) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
   s_tmp[tid] = s;
   __syncthreads();
-  if (tid < K) {
-    double u = 0.0;
-    for (int jj = 0; jj < J; ++jj) u += s_tmp[jj * K + tid];
-    out[tid] = u;
+#pragma unroll
+  for (int h = J / 2; h >= 1; h >>= 1) {
+    if (j < h) s_tmp[tid] += s_tmp[tid + h * K];
+    __syncthreads();
   }
+  if (tid < K) out[tid] = s_tmp[tid];
   __syncthreads();
 }
 
@@ -224,7 +211,7 @@ template <typename T, int K>
 __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(BatchArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
-  __shared__ __align__(16) T s_red[kPhaseBlock * VW];
+  __shared__ T s_red[kPhaseBlock / 32 * K];
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   if (!a.st.active[pr]) return;
@@ -279,24 +266,45 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] = T(0);
     row_gather<T, K, VW>(a.g.col, beg + tid / G, end, RPB, R, lane_off, acc);
+    // the lane groups' sums: within each warp by shuffles, then the warps
 #pragma unroll
-    for (int v = 0; v < VW; ++v) s_red[tid * VW + v] = acc[v];
+    for (int off = G; off < 32; off <<= 1)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], off);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) s_red[(tid >> 5) * K + lane_off + v] = acc[v];
     __syncthreads();
     if (tid < G) {
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int w = 1; w < kPhaseBlock / 32; ++w)
 #pragma unroll
-        for (int v = 0; v < VW; ++v) acc[v] += s_red[(gr * G + sl) * VW + v];
+        for (int v = 0; v < VW; ++v) acc[v] += s_red[w * K + lane_off + v];
       fin(row, end - beg, acc);
     }
   } else {
-    for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
-      const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
-      if (end - beg > kHubDeg) continue;
+    // E lane groups per row where a row has few lanes (K <= 2)
+    constexpr int E = CoopCfg<T, K>::E, LPR = G * E, RPP = kPhaseBlock / LPR;
+    for (int64_t row0 = tl.row_beg; row0 < tl.row_end; row0 += RPP) {
+      const int64_t row = row0 + tid / LPR;
+      const int e = (tid / G) % E;
+      int beg = 0, end = 0;
+      bool live = row < tl.row_end;
+      if (live) {
+        beg = a.g.row_ptr[row];
+        end = a.g.row_ptr[row + 1];
+        live = end - beg <= kHubDeg;
+      }
       T acc[VW];
 #pragma unroll
       for (int v = 0; v < VW; ++v) acc[v] = T(0);
-      row_gather<T, K, VW>(a.g.col, beg, end, 1, R, lane_off, acc);
-      fin(row, end - beg, acc);
+      if (live) row_gather<T, K, VW>(a.g.col, beg + e, end, E, R, lane_off, acc);
+      if constexpr (E > 1) {
+#pragma unroll
+        for (int off = G; off < LPR; off <<= 1)
+#pragma unroll
+          for (int v = 0; v < VW; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], off);
+      }
+      if (live && e == 0) fin(row, end - beg, acc);
     }
   }
   typename CoopSum<T>::S dd[VW];
@@ -463,7 +471,7 @@ template <int K>
 __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchResArgs a) {
   using C = Cfg<float, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
-  __shared__ __align__(16) float s_red[2][kPhaseBlock * VW];
+  __shared__ float s_red[2][kPhaseBlock / 32 * K];
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   if (a.outer_active && !a.outer_active[pr]) return;
@@ -518,32 +526,62 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchRes
 #pragma unroll
     for (int v = 0; v < VW; ++v) sm[v] = cm[v] = lm[v] = 0.f;
     if (!first) df_row_gather<K, VW, false>(a.g.col, beg + tid / G, end, RPB, D, nullptr, lane_off, sm, cm, lm);
+    auto fold = [&](int off) {
 #pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      s_red[0][tid * VW + v] = sm[v];
-      s_red[1][tid * VW + v] = cm[v];
-    }
+      for (int v = 0; v < VW; ++v) {
+        const float so = __shfl_xor_sync(0xffffffffu, sm[v], off), co = __shfl_xor_sync(0xffffffffu, cm[v], off);
+        const df t = two_sum(sm[v], so);
+        sm[v] = t.hi;
+        cm[v] += t.lo + co;
+      }
+    };
+#pragma unroll
+    for (int off = G; off < 32; off <<= 1) fold(off);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        s_red[0][(tid >> 5) * K + lane_off + v] = sm[v];
+        s_red[1][(tid >> 5) * K + lane_off + v] = cm[v];
+      }
     __syncthreads();
     if (tid < G) {
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int w = 1; w < kPhaseBlock / 32; ++w)
 #pragma unroll
         for (int v = 0; v < VW; ++v) {
-          const int k = (gr * G + sl) * VW + v;
-          const df t = two_sum(sm[v], s_red[0][k]);
+          const df t = two_sum(sm[v], s_red[0][w * K + lane_off + v]);
           sm[v] = t.hi;
-          cm[v] += t.lo + s_red[1][k];
+          cm[v] += t.lo + s_red[1][w * K + lane_off + v];
         }
       fin(row, end - beg, sm, cm);
     }
   } else {
-    for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
-      const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
-      if (end - beg > kHubDeg) continue;
+    constexpr int E = CoopCfg<float, K>::E, LPR = G * E, RPP = kPhaseBlock / LPR;
+    for (int64_t row0 = tl.row_beg; row0 < tl.row_end; row0 += RPP) {
+      const int64_t row = row0 + tid / LPR;
+      const int e = (tid / G) % E;
+      int beg = 0, end = 0;
+      bool live = row < tl.row_end;
+      if (live) {
+        beg = a.g.row_ptr[row];
+        end = a.g.row_ptr[row + 1];
+        live = end - beg <= kHubDeg;
+      }
       float sm[VW], cm[VW], lm[VW];
 #pragma unroll
       for (int v = 0; v < VW; ++v) sm[v] = cm[v] = lm[v] = 0.f;
-      if (!first) df_row_gather<K, VW, false>(a.g.col, beg, end, 1, D, nullptr, lane_off, sm, cm, lm);
-      fin(row, end - beg, sm, cm);
+      if (live && !first) df_row_gather<K, VW, false>(a.g.col, beg + e, end, E, D, nullptr, lane_off, sm, cm, lm);
+      if constexpr (E > 1) {
+#pragma unroll
+        for (int off = G; off < LPR; off <<= 1)
+#pragma unroll
+          for (int v = 0; v < VW; ++v) {
+            const float so = __shfl_xor_sync(0xffffffffu, sm[v], off), co = __shfl_xor_sync(0xffffffffu, cm[v], off);
+            const df t = two_sum(sm[v], so);
+            sm[v] = t.hi;
+            cm[v] += t.lo + co;
+          }
+      }
+      if (live && e == 0) fin(row, end - beg, sm, cm);
     }
   }
   float2 pr_r[VW], pr_b[VW];

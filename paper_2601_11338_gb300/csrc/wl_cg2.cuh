@@ -22,6 +22,7 @@
 // Vector traffic per iteration: 10 n K s bytes + 4 nnz + 4 (n + 1).
 #pragma once
 #include "wl_common.cuh"
+#include "wl_df.cuh"
 
 namespace wl {
 
@@ -208,34 +209,82 @@ __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int 
   }
 }
 
-// CTA column sums of per-thread partials (thread t owns columns (t % G) VW + v)
-// written to part[blockIdx.x * K + c]; then the last CTA to finish returns
-// true (all partials visible to it).
-template <typename T, int K>
-__device__ __forceinline__ bool block_partials_last(const double (&val)[Cfg<T, K>::VW], double* part,
-                                                    unsigned* ticket) {
-  using C = Cfg<T, K>;
-  constexpr int VW = C::VW, G = C::G, NW = kPhaseBlock / 32;
-  __shared__ double s_w[NW * K];
-  __shared__ int s_last;
+// the same sums in FP64
+template <int K, int VW>
+__device__ __noinline__ void block_colsum_f64(const double* val, double* s_w, double* out) {
+  constexpr int G = K / VW, NW = kPhaseBlock / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double a[VW];
+  for (int v = 0; v < VW; ++v) {
+    double a = val[v];
+    for (int off = G; off < 32; off <<= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if (lane < G) s_w[warp * K + lane * VW + v] = a;
+  }
+  __syncthreads();
+  if (tid < K) {
+    double t = s_w[tid];
+    for (int w = 1; w < NW; ++w) t += s_w[w * K + tid];
+    out[tid] = t;
+  }
+}
+
+// CTA column sums of per-thread values (thread t owns columns (t % G) VW + v),
+// column c at out[c]. FP32 values (or their double-float sums) are added in
+// double-float, since the FP64 adds of a butterfly over 256 threads hold the
+// SM's FP64 pipe for a thousand clocks; in FP64 where one of them is so large
+// that the sum might leave FP32's range.
+template <typename T, int K>
+__device__ __forceinline__ void block_colsum_store(const typename CoopSum<T>::S (&val)[Cfg<T, K>::VW], double* out) {
+  using C = Cfg<T, K>;
+  using SM = CoopSum<T>;
+  using S = typename SM::S;
+  constexpr int VW = C::VW, G = C::G, NW = kPhaseBlock / 32;
+  static_assert(sizeof(S) == 8, "the FP64 sums reuse the array");
+  __shared__ __align__(8) S s_w[NW * K];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  S a[VW];
 #pragma unroll
   for (int v = 0; v < VW; ++v) a[v] = val[v];
 #pragma unroll
   for (int off = G; off < 32; off <<= 1)
 #pragma unroll
-    for (int v = 0; v < VW; ++v) a[v] += __shfl_xor_sync(0xffffffffu, a[v], off);
+    for (int v = 0; v < VW; ++v) a[v] = SM::add(a[v], SM::shfl(a[v], off));
   if (lane < G)
 #pragma unroll
     for (int v = 0; v < VW; ++v) s_w[warp * K + lane * VW + v] = a[v];
-  __syncthreads();
-  if (tid < K) {
-    double t = 0.0;
-    for (int w = 0; w < NW; ++w) t += s_w[w * K + tid];
-    part[(size_t)blockIdx.x * K + tid] = t;
-    __threadfence();
+  if constexpr (sizeof(T) == 4) {
+    bool big = false;
+#pragma unroll
+    for (int v = 0; v < VW; ++v) big |= !(fabsf(SM::lead(val[v])) < 1e35f);
+    if (__syncthreads_or(big)) {
+      double d[VW];
+#pragma unroll
+      for (int v = 0; v < VW; ++v) d[v] = SM::out(val[v]);
+      block_colsum_f64<K, VW>(d, reinterpret_cast<double*>(s_w), out);
+      return;
+    }
+  } else {
+    __syncthreads();
   }
+  if (tid < K) {
+    S t = s_w[tid];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) t = SM::add(t, s_w[w * K + tid]);
+    out[tid] = SM::out(t);
+  }
+}
+
+// CTA column sums of per-thread partials written to part[blockIdx.x * K + c];
+// then the last CTA to finish returns true (all partials visible to it).
+template <typename T, int K>
+__device__ __forceinline__ bool block_partials_last(const T (&val)[Cfg<T, K>::VW], double* part, unsigned* ticket) {
+  constexpr int VW = Cfg<T, K>::VW;
+  __shared__ int s_last;
+  const int tid = threadIdx.x;
+  typename CoopSum<T>::S a[VW];
+#pragma unroll
+  for (int v = 0; v < VW; ++v) a[v] = CoopSum<T>::from(val[v]);
+  block_colsum_store<T, K>(a, part + (size_t)blockIdx.x * K);
+  if (tid < K) __threadfence();
   __syncthreads();
   if (tid == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1 : 0;
   __syncthreads();
@@ -244,27 +293,31 @@ __device__ __forceinline__ bool block_partials_last(const double (&val)[Cfg<T, K
 }
 
 // Fixed-order sum over all CTAs' partials, by the last CTA: out[c] (shared).
+// 16 loads in flight per thread and added pairwise: this tail is waited for by
+// the whole grid (one dependent FP64 add takes some fifty clocks).
 template <int K>
 __device__ __forceinline__ void sum_partials(const double* part, int nblk, double* s_tmp, double* out) {
-  constexpr int J = kPhaseBlock / K;
+  constexpr int J = kPhaseBlock / K, W = 16;
   const int tid = threadIdx.x, c = tid % K, j = tid / K;
   double s = 0.0;
-  int b = j;
-  for (; b + 7 * J < nblk; b += 8 * J) {
-    double v[8];
+  for (int b = j; b < nblk; b += W * J) {
+    double v[W];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (size_t)(b + u * J) * K + c);
+    for (int u = 0; u < W; ++u) v[u] = b + u * J < nblk ? __ldcg(part + (size_t)(b + u * J) * K + c) : 0.0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) s += v[u];
+    for (int h = W / 2; h >= 1; h >>= 1)
+#pragma unroll
+      for (int u = 0; u < h; ++u) v[u] += v[u + h];
+    s += v[0];
   }
-  for (; b < nblk; b += J) s += __ldcg(part + (size_t)b * K + c);
   s_tmp[tid] = s;
   __syncthreads();
-  if (tid < K) {
-    double t = 0.0;
-    for (int jj = 0; jj < J; ++jj) t += s_tmp[jj * K + tid];
-    out[tid] = t;
+#pragma unroll
+  for (int h = J / 2; h >= 1; h >>= 1) {
+    if (j < h) s_tmp[tid] += s_tmp[tid + h * K];
+    __syncthreads();
   }
+  if (tid < K) out[tid] = s_tmp[tid];
   __syncthreads();
 }
 
@@ -275,7 +328,7 @@ template <typename T, int K, bool SH = false>
 __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase(PhaseArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;  // rows per CTA pass
-  __shared__ __align__(16) T s_red[kPhaseBlock * VW];
+  __shared__ T s_red[kPhaseBlock / 32 * K];
   __shared__ double s_tmp[kPhaseBlock];
   __shared__ double s_out[K];
   CgState* st = a.st;
@@ -366,14 +419,20 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] = T(0);
     row_gather<T, K, VW>(a.g.col, beg + tid / G, end, RPB, a.r, lane_off, acc);
+    // the lane groups' sums: within each warp by shuffles, then the warps
 #pragma unroll
-    for (int v = 0; v < VW; ++v) s_red[tid * VW + v] = acc[v];
+    for (int off = G; off < 32; off <<= 1)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], off);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) s_red[(tid >> 5) * K + lane_off + v] = acc[v];
     __syncthreads();
     if (tid < G) {
       const Own w = own(row);
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int wq = 1; wq < kPhaseBlock / 32; ++wq)
 #pragma unroll
-        for (int v = 0; v < VW; ++v) acc[v] += s_red[(gr * G + sl) * VW + v];
+        for (int v = 0; v < VW; ++v) acc[v] += s_red[wq * K + lane_off + v];
       fin(row, end - beg, acc, w);
     }
   } else if ((int)blockIdx.x < a.g.nhub + a.g.nmid_blk) {
@@ -400,21 +459,29 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
     const int nlist = a.g.nhub + a.g.nmid_blk;
     const int lim = a.g.nmid_blk > 0 ? kMidDeg : kHubDeg;  // longer rows: hub CTAs or mid warps
     const int64_t nblk = (int64_t)gridDim.x - nlist;
-    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPB + tid / G; row < a.g.n; row += nblk * RPB) {
+    // E lane groups per row where a row has few lanes (K <= 2)
+    constexpr int E = G >= 4 ? 1 : 4 / G, LPR = G * E, RPP = kPhaseBlock / LPR;
+    const int e = (tid / G) % E;
+    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPP + tid / LPR; row < a.g.n; row += nblk * RPP) {
       const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
       if (end - beg > lim) continue;
-      const Own w = own(row);
+      Own w;
+      if (e == 0) w = own(row);
       T acc[VW];
 #pragma unroll
       for (int v = 0; v < VW; ++v) acc[v] = T(0);
-      row_gather<T, K, VW>(a.g.col, beg, end, 1, a.r, lane_off, acc);
-      fin(row, end - beg, acc, w);
+      row_gather<T, K, VW>(a.g.col, beg + e, end, E, a.r, lane_off, acc);
+      if constexpr (E > 1) {
+        const unsigned m = ((1u << LPR) - 1u) << (tid & 31 & ~(LPR - 1));
+#pragma unroll
+        for (int off = G; off < LPR; off <<= 1)
+#pragma unroll
+          for (int v = 0; v < VW; ++v) acc[v] += __shfl_xor_sync(m, acc[v], off);
+      }
+      if (e == 0) fin(row, end - beg, acc, w);
     }
   }
-  double dd[VW];
-#pragma unroll
-  for (int v = 0; v < VW; ++v) dd[v] = (double)dacc[v];
-  if (!block_partials_last<T, K>(dd, a.part, &st->ticket)) return;
+  if (!block_partials_last<T, K>(dacc, a.part, &st->ticket)) return;
   // last CTA: delta -> alpha, breakdown checks
   sum_partials<K>(a.part, gridDim.x, s_tmp, s_out);
   if (tid < K) {
@@ -468,10 +535,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_u_phase
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] += rr.v[v] * rr.v[v];
   }
-  double dd[VW];
-#pragma unroll
-  for (int v = 0; v < VW; ++v) dd[v] = (double)acc[v];
-  if (!block_partials_last<T, K>(dd, a.part, &st->ticket)) return;
+  if (!block_partials_last<T, K>(acc, a.part, &st->ticket)) return;
   sum_partials<K>(a.part, gridDim.x, s_tmp, s_out);
   if (tid < K) {
     const double gn = s_out[tid];
@@ -546,7 +610,7 @@ template <int K>
 __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocks) res_phase(ResPhaseArgs a) {
   using C = Cfg<double, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
-  __shared__ __align__(16) double s_red[kPhaseBlock * VW];
+  __shared__ double s_red[kPhaseBlock / 32 * K];
   __shared__ double s_tmp[kPhaseBlock];
   __shared__ double s_out[K];
   const int tid = threadIdx.x, sl = tid % G, lane_off = sl * VW;
@@ -581,12 +645,17 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocks) res_phase(ResPha
     for (int v = 0; v < VW; ++v) acc[v] = 0.0;
     row_gather<double, K, VW>(a.g.col, beg + tid / G, end, RPB, a.x, lane_off, acc);
 #pragma unroll
-    for (int v = 0; v < VW; ++v) s_red[tid * VW + v] = acc[v];
+    for (int off = G; off < 32; off <<= 1)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], off);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) s_red[(tid >> 5) * K + lane_off + v] = acc[v];
     __syncthreads();
     if (tid < G) {
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int wq = 1; wq < kPhaseBlock / 32; ++wq)
 #pragma unroll
-        for (int v = 0; v < VW; ++v) acc[v] += s_red[(gr * G + sl) * VW + v];
+        for (int v = 0; v < VW; ++v) acc[v] += s_red[wq * K + lane_off + v];
       fin(row, end - beg, acc);
     }
   } else {

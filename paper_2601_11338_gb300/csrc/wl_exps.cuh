@@ -80,7 +80,7 @@ template <int K>
 __global__ void __launch_bounds__(kPhaseBlock, 4) exp_term(ExpArgs a) {
   using C = Cfg<float, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
-  __shared__ __align__(16) float s_red[3][kPhaseBlock * VW];
+  __shared__ float s_red[3][kPhaseBlock / 32 * K];
   __shared__ double s_tmp[kPhaseBlock];
   __shared__ double s_out[2 * K];
   CgState* st = a.st;
@@ -120,6 +120,18 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) exp_term(ExpArgs a) {
     stp<float, VW>(a.ah + o, ah);
     stp<float, VW>(a.al + o, al);
   };
+  auto fold = [](float (&s)[VW], float (&c)[VW], float (&l)[VW], int off, unsigned mask) {
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      const float so = __shfl_xor_sync(mask, s[v], off);
+      const float co = __shfl_xor_sync(mask, c[v], off);
+      const float lo = __shfl_xor_sync(mask, l[v], off);
+      const df t = two_sum(s[v], so);
+      s[v] = t.hi;
+      c[v] += t.lo + co;
+      l[v] += lo;
+    }
+  };
   if ((int)blockIdx.x < a.g.nhub) {
     const int64_t row = a.g.hubs[blockIdx.x];
     const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
@@ -127,18 +139,23 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) exp_term(ExpArgs a) {
 #pragma unroll
     for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
     exp_gather<K, VW>(a.g.col, beg + tid / G, end, RPB, a.wh, a.wl, lane_off, s, c, l);
+    // the lane groups' sums: within each warp by shuffles, then the warps
 #pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      s_red[0][tid * VW + v] = s[v];
-      s_red[1][tid * VW + v] = c[v];
-      s_red[2][tid * VW + v] = l[v];
-    }
+    for (int off = G; off < 32; off <<= 1) fold(s, c, l, off, 0xffffffffu);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        const int q = (tid >> 5) * K + lane_off + v;
+        s_red[0][q] = s[v];
+        s_red[1][q] = c[v];
+        s_red[2][q] = l[v];
+      }
     __syncthreads();
     if (tid < G) {
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int w = 1; w < kPhaseBlock / 32; ++w)
 #pragma unroll
         for (int v = 0; v < VW; ++v) {
-          const int q = (gr * G + sl) * VW + v;
+          const int q = w * K + lane_off + v;
           const df t = two_sum(s[v], s_red[0][q]);
           s[v] = t.hi;
           c[v] += t.lo + s_red[1][q];
@@ -157,31 +174,29 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) exp_term(ExpArgs a) {
       for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
       exp_gather<K, VW>(a.g.col, beg + lane / G, end, 32 / G, a.wh, a.wl, lane_off, s, c, l);
 #pragma unroll
-      for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-        for (int v = 0; v < VW; ++v) {
-          const float so = __shfl_xor_sync(0xffffffffu, s[v], off);
-          const float co = __shfl_xor_sync(0xffffffffu, c[v], off);
-          const float lo = __shfl_xor_sync(0xffffffffu, l[v], off);
-          const df t = two_sum(s[v], so);
-          s[v] = t.hi;
-          c[v] += t.lo + co;
-          l[v] += lo;
-        }
+      for (int off = G; off < 32; off <<= 1) fold(s, c, l, off, 0xffffffffu);
       if (lane < G) fin(row, end - beg, s, c, l);
     }
   } else {
     const int nlist = a.g.nhub + a.g.nmid_blk;
     const int lim = a.g.nmid_blk > 0 ? kMidDeg : kHubDeg;
     const int64_t nblk = (int64_t)gridDim.x - nlist;
-    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPB + tid / G; row < a.g.n; row += nblk * RPB) {
+    // E lane groups per row where a row has few lanes (K <= 2)
+    constexpr int E = G >= 4 ? 1 : 4 / G, LPR = G * E, RPP = kPhaseBlock / LPR;
+    const int e = (tid / G) % E;
+    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPP + tid / LPR; row < a.g.n; row += nblk * RPP) {
       const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
       if (end - beg > lim) continue;
       float s[VW], c[VW], l[VW];
 #pragma unroll
       for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
-      exp_gather<K, VW>(a.g.col, beg, end, 1, a.wh, a.wl, lane_off, s, c, l);
-      fin(row, end - beg, s, c, l);
+      exp_gather<K, VW>(a.g.col, beg + e, end, E, a.wh, a.wl, lane_off, s, c, l);
+      if constexpr (E > 1) {
+        const unsigned m = ((1u << LPR) - 1u) << (tid & 31 & ~(LPR - 1));
+#pragma unroll
+        for (int off = G; off < LPR; off <<= 1) fold(s, c, l, off, m);
+      }
+      if (e == 0) fin(row, end - beg, s, c, l);
     }
   }
   // |term|^2 in part[0 .. G K), |acc|^2 in part[G K .. 2 G K)

@@ -124,7 +124,7 @@ template <int K, bool FULL, bool SH = false>
 __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
   using C = Cfg<float, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
-  __shared__ __align__(16) float s_red[3][kPhaseBlock * VW];
+  __shared__ float s_red[3][kPhaseBlock / 32 * K];
   __shared__ double s_tmp[kPhaseBlock];
   __shared__ double s_out[K];
   const int tid = threadIdx.x, sl = tid % G, lane_off = sl * VW;
@@ -191,6 +191,18 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
     }
   };
 
+  auto fold = [](float (&s)[VW], float (&c)[VW], float (&l)[VW], int off, unsigned mask) {
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      const float so = __shfl_xor_sync(mask, s[v], off);
+      const float co = __shfl_xor_sync(mask, c[v], off);
+      const float lo = __shfl_xor_sync(mask, l[v], off);
+      const df t = two_sum(s[v], so);
+      s[v] = t.hi;
+      c[v] += t.lo + co;
+      l[v] += lo;
+    }
+  };
   if ((int)blockIdx.x < a.g.nhub) {
     // one hub row per CTA: RPB lane groups stride over the entries
     const int64_t row = a.g.hubs[blockIdx.x];
@@ -199,22 +211,27 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
 #pragma unroll
     for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
     df_row_gather<K, VW, FULL>(a.g.col, beg + tid / G, end, RPB, a.yh, a.yl, lane_off, s, c, l);
+    // the lane groups' sums: within each warp by shuffles, then the warps
 #pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      s_red[0][tid * VW + v] = s[v];
-      s_red[1][tid * VW + v] = c[v];
-      s_red[2][tid * VW + v] = l[v];
-    }
+    for (int off = G; off < 32; off <<= 1) fold(s, c, l, off, 0xffffffffu);
+    if ((tid & 31) < G)
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        const int q = (tid >> 5) * K + lane_off + v;
+        s_red[0][q] = s[v];
+        s_red[1][q] = c[v];
+        s_red[2][q] = l[v];
+      }
     __syncthreads();
     if (tid < G) {
-      for (int gr = 1; gr < RPB; ++gr)
+      for (int w = 1; w < kPhaseBlock / 32; ++w)
 #pragma unroll
         for (int v = 0; v < VW; ++v) {
-          const int k = (gr * G + sl) * VW + v;
-          const df t = two_sum(s[v], s_red[0][k]);
+          const int q = w * K + lane_off + v;
+          const df t = two_sum(s[v], s_red[0][q]);
           s[v] = t.hi;
-          c[v] += t.lo + s_red[1][k];
-          l[v] += s_red[2][k];
+          c[v] += t.lo + s_red[1][q];
+          l[v] += s_red[2][q];
         }
       fin(row, end - beg, s, c, l);
     }
@@ -230,37 +247,32 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
       for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
       df_row_gather<K, VW, FULL>(a.g.col, beg + lane / G, end, 32 / G, a.yh, a.yl, lane_off, s, c, l);
 #pragma unroll
-      for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-        for (int v = 0; v < VW; ++v) {
-          const float so = __shfl_xor_sync(0xffffffffu, s[v], off);
-          const float co = __shfl_xor_sync(0xffffffffu, c[v], off);
-          const float lo = __shfl_xor_sync(0xffffffffu, l[v], off);
-          const df t = two_sum(s[v], so);
-          s[v] = t.hi;
-          c[v] += t.lo + co;
-          l[v] += lo;
-        }
+      for (int off = G; off < 32; off <<= 1) fold(s, c, l, off, 0xffffffffu);
       if (lane < G) fin(row, end - beg, s, c, l);
     }
   } else {
     const int nlist = a.g.nhub + a.g.nmid_blk;
     const int lim = a.g.nmid_blk > 0 ? kMidDeg : kHubDeg;  // longer rows: hub CTAs or mid warps
     const int64_t nblk = (int64_t)gridDim.x - nlist;
-    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPB + tid / G; row < a.g.n; row += nblk * RPB) {
+    // E lane groups per row where a row has few lanes (K <= 2)
+    constexpr int E = G >= 4 ? 1 : 4 / G, LPR = G * E, RPP = kPhaseBlock / LPR;
+    const int e = (tid / G) % E;
+    for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPP + tid / LPR; row < a.g.n; row += nblk * RPP) {
       const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
       if (end - beg > lim) continue;
       float s[VW], c[VW], l[VW];
 #pragma unroll
       for (int v = 0; v < VW; ++v) s[v] = c[v] = l[v] = 0.f;
-      df_row_gather<K, VW, FULL>(a.g.col, beg, end, 1, a.yh, a.yl, lane_off, s, c, l);
-      fin(row, end - beg, s, c, l);
+      df_row_gather<K, VW, FULL>(a.g.col, beg + e, end, E, a.yh, a.yl, lane_off, s, c, l);
+      if constexpr (E > 1) {
+        const unsigned m = ((1u << LPR) - 1u) << (tid & 31 & ~(LPR - 1));
+#pragma unroll
+        for (int off = G; off < LPR; off <<= 1) fold(s, c, l, off, m);
+      }
+      if (e == 0) fin(row, end - beg, s, c, l);
     }
   }
-  double dd[VW];
-#pragma unroll
-  for (int v = 0; v < VW; ++v) dd[v] = (double)nacc[v];
-  if (!block_partials_last<float, K>(dd, a.part, &a.st->ticket)) return;
+  if (!block_partials_last<float, K>(nacc, a.part, &a.st->ticket)) return;
   sum_partials<K>(a.part, gridDim.x, s_tmp, s_out);
   if (tid < K) a.st->gamma[tid] = s_out[tid];
   if (tid == 0) a.st->ticket = 0;
@@ -295,10 +307,7 @@ __global__ void __launch_bounds__(kPhaseBlock) df_from_f64(const double* b, doub
     stp<float, VW>(bl + e * VW, ll);
     if (r32) stp<float, VW>(r32 + e * VW, hh);
   }
-  double dd[VW];
-#pragma unroll
-  for (int v = 0; v < VW; ++v) dd[v] = (double)acc[v];
-  if (!block_partials_last<float, K>(dd, part, &st->ticket)) return;
+  if (!block_partials_last<float, K>(acc, part, &st->ticket)) return;
   sum_partials<K>(part, gridDim.x, s_tmp, s_out);
   if (tid < K) b2[tid] = s_out[tid];
   if (tid == 0) st->ticket = 0;
