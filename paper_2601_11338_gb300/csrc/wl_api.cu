@@ -370,7 +370,9 @@ struct wl_handle {
   Buf csr_rp, csr_col;
   Buf x, r, p, q;         // CG vectors (FP64 or FP32), n * 64 doubles each at most
   Buf b64;                // FP64 right-hand sides (walk degrees, apply)
-  Buf d32, d32b, r32;     // refined form: FP32 corrections (two, alternating) and inner right-hand side
+  Buf hist;               // phase-kernel CG: CgHist and the kept residuals
+  const double* r_fin = nullptr;  // final residual of the last FP64 solve
+  Buf d32, r32;           // refined form: FP32 correction, residual scratch of its cooperative solve
   Buf xh, xl;             // refined form: the iterate as two FP32 terms (x = xh + xl)
   Buf bh, bl, rh, rl;     // refined form: right-hand side and residual as two FP32 terms
   Buf dfdf, ydf;          // refined form: D_f and the Lanczos coefficients y(tau) as two FP32 terms
@@ -634,7 +636,7 @@ struct CgStart {
 // fit in shared memory (nothing launched).
 template <typename T>
 bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& start, cudaError_t* e) {
-  CoopArgs<T> co{a, h->cgbar(), start.r0 ? start.r0 : a.r, start.gamma0, start.add_x ? 1 : 0};
+  CoopArgs<T> co{a, h->cgbar(), start.r0 ? start.r0 : a.rn, start.gamma0, start.add_x ? 1 : 0};
   if (!h->bar_clean) {
     *e = cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h));
     if (*e != cudaSuccess) return true;
@@ -667,50 +669,112 @@ bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& s
   return coop;
 }
 
-// Runs the CG iterations of an initialised solve state to completion (or the
-// iteration cap), reading back one flag per chunk, then the final x update.
+// bytes up to which the phase kernels keep kHist residuals
+constexpr double kHistBytes = 4.0e9;
+
+// A solve by the phase kernels: runs the CG iterations to completion (or the
+// iteration cap), reading back one flag per chunk, and forms x from the kept
+// residuals, every kHist iterations (fewer where they take more than
+// kHistBytes: two for vectors of 1.3 GB and more) and at the end. *r_fin: the
+// final residual.
 template <typename T>
-int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, int grid_s, int grid_u, SolveInfo& info, int cat_bytes,
-           bool init = true) {
+int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, const CgStart<T>& start, int grid_s, int grid_u, SolveInfo& info,
+           const T** r_fin = nullptr) {
   PhaseArgs<T> a = a_in;
   const int fault = fault_mode();
   if (fault == kFaultNoconv) a.max_iter = 1;
+  const T* r0 = start.r0 ? start.r0 : a.rn;
   if (fault == kFaultNan) {
     static const T nan_v = (T)NAN;
-    WL_CU(cudaMemcpyAsync(a.r, &nan_v, sizeof(T), cudaMemcpyHostToDevice, S(h)));
+    WL_CU(cudaMemcpyAsync(const_cast<T*>(r0), &nan_v, sizeof(T), cudaMemcpyHostToDevice, S(h)));
   }
-  auto launch = [&](int mode, int chunk) -> cudaError_t {
+  // r_j, j >= 1, takes the buffers in turn; keep + 1 of them
+  const size_t stride = ((size_t)h->n * K + 63) & ~(size_t)63, head = (sizeof(CgHist) + 255) & ~(size_t)255;
+  int keep = (int)std::max(2.0, std::min<double>(kHist, kHistBytes / (double)(stride * sizeof(T)) - 1.0));
+  for (;; keep /= 2) {  // less than that where memory is short
+    const int rc = ensure(h->hist, head + (size_t)(keep + 1) * stride * sizeof(T));
+    if (rc == WL_OK) break;
+    if (rc != WL_ERR_OOM || keep == 1) return rc;
+    cudaGetLastError();
+  }
+  a.hist = (CgHist*)h->hist.p;
+  T* ring = (T*)((char*)h->hist.p + head);
+  auto rj = [&](int j) -> const T* { return j == 0 ? r0 : ring + (size_t)((j - 1) % (keep + 1)) * stride; };
+  auto iterate = [&](int j) -> cudaError_t {
+    a.r = rj(j);
+    a.rn = const_cast<T*>(rj(j + 1));
+    a.slot = j % keep;
     if constexpr (sizeof(T) == 4)
-      return launch_cg_phases_f32(K, a, grid_s, grid_u, mode, chunk, S(h));
+      return launch_cg_phases_f32(K, a, grid_s, grid_u, false, S(h));
     else
-      return launch_cg_phases_f64(K, a, grid_s, grid_u, mode, chunk, S(h));
+      return launch_cg_phases_f64(K, a, grid_s, grid_u, false, S(h));
+  };
+  // x (and p, if the solve goes on) from r_{j-m} .. r_{j-1}
+  auto form_x = [&](int j, int m, bool flush) -> cudaError_t {
+    CgXArgs<T> xa{};
+    for (int i = 0; i < m; ++i) xa.r[i] = rj(j - m + i);
+    xa.x = a.x;
+    xa.p = a.p;
+    xa.hist = a.hist;
+    xa.st = a.st;
+    xa.n = h->n;
+    xa.m = m;
+    xa.has_p = j > m;
+    xa.add_x = start.add_x || j > m;
+    xa.flush = flush;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)h->n * K / 4 + kPhaseBlock - 1) / kPhaseBlock,
+                                                                 (int64_t)h->sms * 8));
+    if constexpr (sizeof(T) == 4)
+      return launch_cg_x_f32(K, xa, grid, S(h));
+    else
+      return launch_cg_x_f64(K, xa, grid, S(h));
   };
   const int pc = prof_begin(h, kCatCG);
-  if (init) {  // else the caller has set the state from known residual norms
-    counted(h, 1);
-    WL_CU(launch(0, 0));
+  counted(h, 1);
+  if (start.gamma0) {  // known residual norms: no pass over r to compute them
+    if (start.gamma0 != a.st->gamma)
+      WL_CU(cudaMemcpyAsync(a.st->gamma, start.gamma0, K * sizeof(double), cudaMemcpyDeviceToDevice, S(h)));
+    WL_CU(launch_cg_state_restart(a.st, a.skip, K, S(h)));
+  } else {
+    a.r = r0;
+    if constexpr (sizeof(T) == 4)
+      WL_CU(launch_cg_phases_f32(K, a, grid_s, grid_u, true, S(h)));
+    else
+      WL_CU(launch_cg_phases_f64(K, a, grid_s, grid_u, true, S(h)));
   }
   // the whole CG state comes back after every chunk: the check of the last
-  // chunk also carries the per-column results (the deferred x update launched
-  // after it changes none of them), so the solve ends without another wait
+  // chunk also carries the per-column results, so the solve ends without
+  // another wait
   CgState* hs = &reinterpret_cast<CgBlock*>(h->h_pin)->st;
   static_assert(sizeof(CgBlock) <= 4096 * sizeof(double), "pinned staging holds the CG state");
   // first chunk: one more iteration than the handle's previous solve took (a
   // launch that finds the solve finished returns at once, but still costs a
   // grid); later chunks of kChunkMore iterations
   int chunk = std::min(std::max(h->cg_hint + 1, 2), 2 * kChunk);
-  for (;;) {
-    counted(h, 2 * chunk);
-    WL_CU(launch(1, chunk));
+  for (int j = 0;;) {
+    for (const int end = j + chunk; j < end; ++j) {
+      if (j > 0 && j % keep == 0) {
+        counted(h, 1);
+        WL_CU(form_x(j, keep, true));
+      }
+      counted(h, 2);
+      WL_CU(iterate(j));
+    }
     WL_CU(cudaMemcpyAsync(hs, h->cgst(), sizeof(CgState), cudaMemcpyDeviceToHost, S(h)));
     WL_CU(cudaStreamSynchronize(S(h)));
     if (!hs->active) break;
     chunk = kChunkMore;
   }
-  counted(h, 1);
-  WL_CU(launch(2, 0));
+  const int it = hs->iters;
+  if (it > 0) {
+    counted(h, 1);
+    WL_CU(form_x(it, (it - 1) % keep + 1, false));
+  } else if (!start.add_x) {
+    WL_CU(cudaMemsetAsync(a.x, 0, (size_t)h->n * K * sizeof(T), S(h)));
+  }
+  if (r_fin) *r_fin = rj(it);
   prof_end(h, pc);
-  cg_outcome(h, K, cat_bytes, info);
+  cg_outcome(h, K, sizeof(T), info);
   return WL_OK;
 }
 
@@ -747,7 +811,7 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
     bn2 = st->b2;
     info.nnz_rhs += (double)h->nnz * K;
   }
-  PhaseArgs<double> a{phase_graph_mid(h, grid_u), x, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
+  PhaseArgs<double> a{phase_graph_mid(h, grid_u), x, (double*)h->r.p, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
                       bn2, nullptr, (double*)h->part.p, st, h->prm.max_iter, tol * tol};
   a.dshift = h->si_dsh64;  // shifted solve of the shift-and-invert Lanczos (else NULL)
   {
@@ -759,12 +823,9 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
       WL_CU(ce);
       WL_TRY(cg_block_to_host(h));
       cg_outcome(h, K, 8, info);
+      h->r_fin = (const double*)h->r.p;
     } else {
-      if (x_is_zero) {
-        WL_CU(cudaMemsetAsync(x, 0, nk * 8, S(h)));
-        WL_CU(cudaMemcpyAsync(h->r.p, b, nk * 8, cudaMemcpyDeviceToDevice, S(h)));
-      }
-      WL_TRY(run_cg<double>(h, K, a, grid_s, grid_u, info, 8));
+      WL_TRY(run_cg<double>(h, K, a, start, grid_s, grid_u, info, &h->r_fin));
     }
   }
   info.max_rel = std::max(info.max_rel, info.last_rel);
@@ -786,8 +847,6 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   WL_TRY(ensure(h->p, nk * 4));
   WL_TRY(ensure(h->q, nk * 4));
   WL_TRY(ensure(h->d32, nk * 4));
-  WL_TRY(ensure(h->d32b, nk * 4));
-  WL_TRY(ensure(h->r32, nk * 4));
   WL_TRY(ensure(h->rh, nk * 4));
   WL_TRY(ensure(h->rl, nk * 4));
   WL_TRY(ensure_phase_buffers(h, std::max({grid_s, grid_r, h->sms})));
@@ -795,7 +854,6 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   float* rh = (float*)h->rh.p;
   float* rl = (float*)h->rl.p;
   float* dcur = (float*)h->d32.p;
-  float* dnext = (float*)h->d32b.p;
   const df ca = df_from_double(h->ca), cA = df_from_double(h->cA), cD = df_from_double(h->cD);
   double* hp = h->h_pin;
   double* hbn2 = h->h_pin + 2048;  // beyond the solve's block
@@ -805,20 +863,22 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   const float* rch = bh;
   const float* rcl = bl;
   bool x_zero = (x0 == nullptr);
-  // Small solves run each correction as one cooperative kernel. It starts from
-  // B's or the residual's leading terms where they are and writes d whole, so
-  // nothing is staged for it, and the residual that follows it keeps its norms
-  // in a state of its own: both are launched before one wait for their outcome.
-  PhaseArgs<float> a{phase_graph_mid(h, grid_u), dcur, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
+  // A correction starts from B's or the residual's leading terms where they are
+  // and writes d whole, and the residual that follows it keeps its norms in a
+  // state of its own. Small solves run the correction as one cooperative kernel:
+  // both are launched before one wait for their outcome.
+  const PhaseGraph pg = phase_graph_mid(h, grid_u);
+  const bool coop = cg_coop_fits_f32(K, pg, h->nnz, h->sms);
+  if (coop) WL_TRY(ensure(h->r32, nk * 4));
+  PhaseArgs<float> a{pg, dcur, (float*)h->r32.p, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
                      h->ca, h->cA, h->cD, nullptr, dskip, (double*)h->part.p, st, h->prm.max_iter, 0.0};
   a.dshift = h->si_dsh_h;
-  const bool coop = cg_coop_fits_f32(K, a.g, h->nnz, h->sms);
-  CgState* rst = coop ? h->cgres() : st;  // the residual's norms
+  CgState* rst = h->cgres();  // the residual's norms
   if (!x_zero) {
     // r = B - M x0 (x0 split into two FP32 terms and gathered whole)
     counted(h, 2);
     WL_CU(launch_split_x(x0, (int64_t)nk, xh, xl, false, nullptr, S(h)));
-    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), xh, xl, bh, bl, rh, rl, (float*)h->r32.p, nullptr, nullptr, nullptr,
+    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), xh, xl, bh, bl, rh, rl, nullptr, nullptr,
                  ca, cA, cD, (double*)h->part.p, rst, 0};
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
@@ -835,18 +895,6 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // rel, with the same floor)
   const double inner0 = std::min(1e-3, std::max(h->inner_tol, kInner0C * std::sqrt(tol)));
   const int max_ref = 12;
-  // r32 (the next inner solve's right-hand side) and dcur (its zero start)
-  // are ready: the residual after the first correction writes them, later
-  // ones do not (the solve almost always ends there), and a further
-  // correction stages them itself
-  bool staged = true;
-  if (!coop) {
-    WL_CU(cudaMemsetAsync(dcur, 0, nk * 4, S(h)));
-    if (x_zero) {
-      WL_CU(cudaMemcpyAsync(h->r32.p, bh, nk * 4, cudaMemcpyDeviceToDevice, S(h)));
-      WL_CU(cudaMemcpyAsync(st->gamma, bn2, K * 8, cudaMemcpyDeviceToDevice, S(h)));
-    }
-  }
   const double* hgamma = nullptr;  // residual norms on the host, when the last wait brought them
   for (int ref = 0;; ++ref) {
     info.refinements++;
@@ -856,7 +904,6 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
       // the residual is B itself: every column with B != 0 still needs its
       // first correction (rel = 1), and the inner solve's start marks a zero
       // column done by itself, so no host check (and no wait) is needed
-      if (!coop) WL_CU(cudaMemsetAsync(dskip, 0, K * sizeof(int), S(h)));
     } else {
       if (!hgamma) {
         WL_CU(cudaMemcpyAsync(hp, rst->gamma, K * 8, cudaMemcpyDeviceToHost, S(h)));
@@ -882,46 +929,36 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
         break;
       }
       WL_CU(cudaMemcpyAsync(dskip, skip, K * sizeof(int), cudaMemcpyHostToDevice, S(h)));
-      if (!coop && !staged) {
-        WL_CU(cudaMemcpyAsync(h->r32.p, rh, nk * 4, cudaMemcpyDeviceToDevice, S(h)));
-        WL_CU(cudaMemsetAsync(dcur, 0, nk * 4, S(h)));
-        staged = true;
-      }
     }
     const double inner_tol = from_b ? inner0 : std::min(1e-3, std::max(h->inner_tol, 0.5 * tol / mx));
-    a.x = dcur;
     a.tol2 = inner_tol * inner_tol;
-    a.skip = coop && from_b ? nullptr : dskip;
+    a.skip = from_b ? nullptr : dskip;
     SolveInfo inner;
+    // the inner solve starts from the residual norms (from the double-float
+    // residual, or B's norms): no pass over r to recompute them
+    CgStart<float> start;
+    start.r0 = rch;
+    start.gamma0 = from_b ? bn2 : rst->gamma;
     if (coop) {
-      CgStart<float> start;
-      start.r0 = rch;
-      start.gamma0 = from_b ? bn2 : rst->gamma;
       cudaError_t ce = cudaSuccess;
       if (!cg_coop_try<float>(h, K, a, start, &ce)) return WL_ERR_UNSUPPORTED;  // fits: checked above
       WL_CU(ce);
     } else {
-      // the inner solve starts from the residual norms in st->gamma (from the
-      // double-float residual, or B's norms): no pass over r32 to recompute them
-      counted(h);
-      WL_CU(launch_cg_state_restart(st, dskip, K, S(h)));
       // the first correction and the later ones go to different depths: each
       // sizes its first launch chunk from the previous solve of its kind
       int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
       h->cg_hint = hint;
-      WL_TRY(run_cg<float>(h, K, a, grid_s, grid_u, inner, 4, false));
+      WL_TRY(run_cg<float>(h, K, a, start, grid_s, grid_u, inner));
       hint = h->cg_hint;
       if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
         info.status = inner.status;
         break;
       }
     }
-    // r <- r - M d, x <- x + d, next correction buffer zeroed
-    WL_CU(cudaMemsetAsync(rst, 0, coop ? sizeof(CgState) + sizeof(CoopBar) : sizeof(CgState), S(h)));
-    if (coop) h->bar_clean = true;
-    const bool stage_next = (ref == 0) && !coop;
-    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), dcur, nullptr, rch, rcl, rh, rl,
-                 stage_next ? (float*)h->r32.p : nullptr, xh, xl, stage_next ? dnext : nullptr,
+    // r <- r - M d, x <- x + d
+    WL_CU(cudaMemsetAsync(rst, 0, sizeof(CgState) + sizeof(CoopBar), S(h)));
+    h->bar_clean = true;
+    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), dcur, nullptr, rch, rcl, rh, rl, xh, xl,
                  ca, cA, cD, (double*)h->part.p, rst, x_zero ? 1 : 0};
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
@@ -945,10 +982,8 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     info.bytes += inner.bytes;
     info.nnz_rhs += (double)h->nnz * K;
     x_zero = false;
-    staged = stage_next;
     rch = rh;
     rcl = rl;
-    std::swap(dcur, dnext);
   }
   if (x_zero) {  // converged before any correction: X = 0
     WL_CU(cudaMemsetAsync(xh, 0, nk * 4, S(h)));
@@ -1603,9 +1638,9 @@ int si_apply(wl_handle* h, bool dfp, int K, int j, size_t blk, SolveInfo& info) 
       WL_TRY(solve_fp64(h, (const double*)h->b64.p, (double*)h->x.p, K, h->prm.tol, true, info));
     }
     if (info.status != WL_OK) return WL_OK;
-    // packX = -M z = -((B - r) + a Dt^{-1} z), r the CG's final residual in h->r
+    // packX = -M z = -((B - r) + a Dt^{-1} z), r the CG's final residual
     counted(h);
-    WL_CU(launch_si_mz64((const double*)h->b64.p, (const double*)h->r.p, (const double*)h->x.p, d64 + n,
+    WL_CU(launch_si_mz64((const double*)h->b64.p, h->r_fin, (const double*)h->x.p, d64 + n,
                          h->a_scale, n, K, (double*)h->packX.p, S(h)));
   }
   return WL_OK;
@@ -1970,7 +2005,7 @@ void free_handle(wl_handle* h) {
     pool_free(kv.second.meta);
   }
   Buf* bufs[] = {&h->csr_rp, &h->csr_col, &h->x, &h->r, &h->p, &h->q, &h->b64, &h->d32,
-                 &h->r32, &h->xh, &h->xl, &h->d32b, &h->bh, &h->bl, &h->rh, &h->rl, &h->dfdf, &h->ydf, &h->ew, &h->taus, &h->ybig, &h->part, &h->small, &h->Df, &h->warm, &h->basis, &h->Tab, &h->ybuf, &h->yprev,
+                 &h->r32, &h->xh, &h->xl, &h->hist, &h->bh, &h->bl, &h->rh, &h->rl, &h->dfdf, &h->ydf, &h->ew, &h->taus, &h->ybig, &h->part, &h->small, &h->Df, &h->warm, &h->basis, &h->Tab, &h->ybuf, &h->yprev,
                  &h->errb, &h->stage_a, &h->stage_b, &h->packV, &h->packX, &h->spV, &h->spW, &h->spstate, &h->mid, &h->omega, &h->gram,
                  &h->omega_int, &h->ptmp, &h->perm_b, &h->iperm_b, &h->hubs, &h->cgstate};
   for (Buf* b : bufs) release(*b);
@@ -2664,7 +2699,6 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       break;
     }
     if (e == cudaSuccess) e = launch_sketch_rhs(om_int, n, M, K, h->a_scale, (float*)h->r32.p, S(h));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->x.p, 0, nk * 4, S(h));
     if (e != cudaSuccess) { rc = set_cuda_error(e, "sketch"); break; }
     // Y = M^{-1} (a Omega) in FP32 lockstep CG
     const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4), grid_s = grid_u + h->nhub;
@@ -2673,14 +2707,14 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
     CgState* st = h->cgst();
     WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
     const double tol = std::max(h->prm.tol, 1e-7);
-    PhaseArgs<float> a{phase_graph_mid(h, grid_u), (float*)h->x.p, (float*)h->r32.p, (float*)h->p.p,
+    PhaseArgs<float> a{phase_graph_mid(h, grid_u), (float*)h->x.p, (float*)h->r32.p, (float*)h->r32.p, (float*)h->p.p,
                        (float*)h->q.p, h->ca, h->cA, h->cD, nullptr, nullptr, (double*)h->part.p, st,
                        h->prm.max_iter, tol * tol};
     if (cg_coop_try<float>(h, K, a, CgStart<float>{}, &e)) {
       if (e != cudaSuccess) { rc = set_cuda_error(e, "cooperative CG"); break; }
       if ((rc = cg_block_to_host(h)) != WL_OK) break;
       cg_outcome(h, K, 4, info);
-    } else if ((rc = run_cg<float>(h, K, a, grid_s, grid_u, info, 4)) != WL_OK) {
+    } else if ((rc = run_cg<float>(h, K, a, CgStart<float>{}, grid_s, grid_u, info)) != WL_OK) {
       break;
     }
     (void)sm;

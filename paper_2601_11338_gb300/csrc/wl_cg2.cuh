@@ -34,8 +34,8 @@ constexpr int kPhaseBlock = 256;   // threads per CTA of the phase kernels
 #endif
 constexpr int kPhaseMinBlocks = WL_PHASE_MINB;  // CTAs per SM the S kernel's registers are sized for
 // FP32 CG kernels: 5 CTAs per SM (48 registers) hold the eight predicated
-// gathers per lane; measured 236 us per K = 16 iteration on the Chung-Lu 1e6
-// graph (6 CTAs: 240 us; 4 CTAs: 248 us)
+// gathers per lane; measured 139 us per K = 16 S phase on the Chung-Lu 1e6
+// graph (6 CTAs: 147 us; 4 CTAs: the same, and U 3% slower)
 #ifndef WL_PHASE_MINB_F32
 #define WL_PHASE_MINB_F32 5
 #endif
@@ -65,11 +65,20 @@ struct PhaseGraph {
   int nmid_blk = 0;               // CTAs (after the hub CTAs) that walk the mid rows; 0: no mid path
 };
 
+constexpr int kHist = 16;  // residuals kept before p and x are formed from them, at most
+
+// Per column the step sizes of the kept iterations: x += sum alpha_i p_i with
+// p_i = r_i + beta_i p_{i-1}
+struct CgHist {
+  double alpha[kHist][64], beta[kHist][64];
+};
+
 template <typename T>
 struct PhaseArgs {
   PhaseGraph g;
   T* x;
-  T* r;
+  const T* r;  // r_j
+  T* rn;       // r_{j+1} (r_j itself where x and p are updated in each S phase)
   T* p;
   T* q;
   double ca, cA, cD;
@@ -82,12 +91,27 @@ struct PhaseArgs {
   // optional per-row diagonal added to M (the shifted solves of the
   // shift-and-invert Lanczos: M - a (D_f + sigma I)^{-1}); NULL: none
   const T* dshift = nullptr;
+  CgHist* hist = nullptr;  // where the iteration's alpha and beta go, at `slot`
+  int slot = 0;
 };
 
 // ---------------------------------------------------------------- helpers
 template <typename T, int VW>
 __device__ __forceinline__ Pack<T, VW> ld_plain(const T* p) {
   return *reinterpret_cast<const Pack<T, VW>*>(p);
+}
+// the last read of a value for a while: its line may leave L2 first
+template <typename T, int VW>
+__device__ __forceinline__ Pack<T, VW> ld_last(const T* p) {
+  Pack<T, VW> o;
+  if constexpr (sizeof(T) * VW == 16) {
+    const int4 t = __ldcs(reinterpret_cast<const int4*>(p));
+    o = *reinterpret_cast<const Pack<T, VW>*>(&t);
+  } else {
+#pragma unroll
+    for (int v = 0; v < VW; ++v) o.v[v] = __ldcs(p + v);
+  }
+  return o;
 }
 
 // Gathers per lane in flight in row_gather: predicated batches of 8 (1)
@@ -324,7 +348,17 @@ __device__ __forceinline__ void sum_partials(const double* part, int nblk, doubl
 // ---------------------------------------------------------------- S phase
 // SH: the solve carries the per-row diagonal a.dshift (a separate instance,
 // so that the unshifted kernel carries no trace of it)
-template <typename T, int K, bool SH = false>
+// X: x and p are updated here, in place (four vectors and no more: the entry
+// that allocates nothing). Otherwise the residuals r_j of up to kHist
+// iterations stay where they are, each in its own buffer, and x and p are formed
+// from them afterwards (cg_x_phase): the pass then reads r and q and writes q,
+// where it read and wrote x and p too (192 MB of vectors for 1e6 x 16 floats, not
+// 448). Chung-Lu 1e6 x 16, shifted: S 165 -> 134 us, and 85 us per solve of nine
+// iterations for x; what is left is the gathers, 24e6 sectors from L2 and L1.
+// 3e5 x 16 doubles: 198 -> 159 us; R-MAT scale 17 x 64 floats: 176 -> 162 us.
+// delta is (r, q) then, which is (p, q) as q = M p and p_{j-1} is M-orthogonal
+// to p_j: in FP32 simulations the same iterations (to one) up to condition 1e5.
+template <typename T, int K, bool SH = false, bool X = false>
 __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase(PhaseArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;  // rows per CTA pass
@@ -368,12 +402,14 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
     T dx = T(0);
     if constexpr (SH) dx = __ldg(a.dshift + row);
     if (!first) {
-      w.x = ld_plain<T, VW>(px + o);
-      w.p = ld_plain<T, VW>(pp_ + o);
-      w.q = ld_plain<T, VW>(pq + o);
+      if constexpr (X) {
+        w.x = ld_plain<T, VW>(px + o);
+        w.p = ld_plain<T, VW>(pp_ + o);
+      }
+      w.q = ld_last<T, VW>(pq + o);
     }
     const Pack<T, VW>& rr = w.r;
-    Pack<T, VW> pp, qq;
+    Pack<T, VW> pp, qq;  // p, or r where p is not formed
     const T dg = (T)deg;
     // (M r) of column v; FP64: the row's diagonal first (one product fewer per column)
     T crow = T(0);
@@ -394,20 +430,24 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
         qq.v[v] = mr(v);
       }
     } else {
-      Pack<T, VW> xx = w.x;
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
         const T s = mr(v);
-        const T al = s_ab[0][lane_off + v], be = s_ab[1][lane_off + v];
-        xx.v[v] += al * w.p.v[v];
-        pp.v[v] = rr.v[v] + be * w.p.v[v];
+        const T be = s_ab[1][lane_off + v];
+        pp.v[v] = rr.v[v];
+        if constexpr (X) pp.v[v] += be * w.p.v[v];
         qq.v[v] = s + be * w.q.v[v];
       }
-      stp<T, VW>(px + o, xx);
+      if constexpr (X) {
+        Pack<T, VW> xx = w.x;
+#pragma unroll
+        for (int v = 0; v < VW; ++v) xx.v[v] += s_ab[0][lane_off + v] * w.p.v[v];
+        stp<T, VW>(px + o, xx);
+      }
     }
 #pragma unroll
     for (int v = 0; v < VW; ++v) dacc[v] += pp.v[v] * qq.v[v];
-    stp<T, VW>(pp_ + o, pp);
+    if constexpr (X) stp<T, VW>(pp_ + o, pp);
     stp<T, VW>(pq + o, qq);
   };
 
@@ -497,6 +537,10 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
     } else {
       st->alpha[tid] = 0.0;
     }
+    if constexpr (!X) {
+      a.hist->alpha[a.slot][tid] = st->alpha[tid];
+      a.hist->beta[a.slot][tid] = st->beta[tid];
+    }
   }
   if (tid == 0) {
     st->iters += 1;
@@ -525,12 +569,15 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_u_phase
   const size_t nv = (size_t)a.g.n * K / VW;
 #pragma unroll 4
   for (size_t e = (size_t)blockIdx.x * kPhaseBlock + tid; e < nv; e += (size_t)gridDim.x * kPhaseBlock) {
-    Pack<T, VW> rr = ld_plain<T, VW>(a.r + e * VW);
-    if (!init) {
+    Pack<T, VW> rr;
+    if (init) {
+      rr = ld_plain<T, VW>(a.r + e * VW);
+    } else {
+      rr = ld_last<T, VW>(a.r + e * VW);
       const Pack<T, VW> qq = ld_plain<T, VW>(a.q + e * VW);
 #pragma unroll
       for (int v = 0; v < VW; ++v) rr.v[v] -= al[v] * qq.v[v];
-      stp<T, VW>(a.r + e * VW, rr);
+      stp<T, VW>(a.rn + e * VW, rr);
     }
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] += rr.v[v] * rr.v[v];
@@ -590,6 +637,80 @@ __global__ void __launch_bounds__(kPhaseBlock) cg_f_phase(PhaseArgs<T> a) {
 #pragma unroll
     for (int v = 0; v < VW; ++v) xx.v[v] += al[v] * pp.v[v];
     stp<T, VW>(a.x + e * VW, xx);
+  }
+}
+
+// x and p from the kept residuals r[0..m): with p_i = r_i + beta_i p_{i-1},
+//   sum_i alpha_i p_i = sum_i g_i r_i + beta_0 g_0 p_{-1},  g_i = alpha_i + beta_{i+1} g_{i+1}
+// and p_{m-1} likewise with h_i = beta_{i+1} h_{i+1}, h_{m-1} = 1. One pass over
+// them per kHist iterations or at the end of the solve, where x and p were read
+// and written in every iteration.
+template <typename T>
+struct CgXArgs {
+  const T* r[kHist];
+  T* x;
+  T* p;  // p_{-1} in (has_p), p_{m-1} out (flush)
+  const CgHist* hist;
+  const CgState* st;
+  int64_t n;
+  int m;
+  int has_p;  // 0: p_{-1} = 0
+  int add_x;  // 0: x is written, not read
+  int flush;  // the solve goes on: p too; nothing to do if it does not
+};
+
+template <typename T, int K>
+__global__ void __launch_bounds__(kPhaseBlock) cg_x_phase(CgXArgs<T> a) {
+  using C = Cfg<T, K>;
+  constexpr int VW = C::VW, G = C::G;
+  __shared__ T s_g[kHist + 1][K], s_h[kHist + 1][K];
+  if (a.flush && !*(volatile const int*)&a.st->active) return;
+  const int tid = threadIdx.x, m = a.m;
+  if (tid < K) {
+    T g = T(0), h = T(1), be = T(0);
+    for (int i = m - 1; i >= 0; --i) {
+      g = (T)a.hist->alpha[i][tid] + be * g;
+      if (i < m - 1) h *= be;
+      be = (T)a.hist->beta[i][tid];
+      s_g[i][tid] = g;
+      s_h[i][tid] = h;
+    }
+    s_g[kHist][tid] = be * g;
+    s_h[kHist][tid] = be * h;
+  }
+  __syncthreads();
+  const int mycol = (tid % G) * VW;
+  const size_t nv = (size_t)a.n * K / VW;
+  for (size_t e = (size_t)blockIdx.x * kPhaseBlock + tid; e < nv; e += (size_t)gridDim.x * kPhaseBlock) {
+    Pack<T, VW> xx, pp;
+#pragma unroll
+    for (int v = 0; v < VW; ++v) xx.v[v] = pp.v[v] = T(0);
+    if (a.add_x) xx = ld_last<T, VW>(a.x + e * VW);
+    if (a.has_p) {
+      const Pack<T, VW> p0 = ld_last<T, VW>(a.p + e * VW);
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        xx.v[v] += s_g[kHist][mycol + v] * p0.v[v];
+        pp.v[v] = s_h[kHist][mycol + v] * p0.v[v];
+      }
+    }
+    for (int i0 = 0; i0 < m; i0 += 4) {
+      Pack<T, VW> rr[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < m) rr[u] = ld_last<T, VW>(a.r[i0 + u] + e * VW);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < m) {
+#pragma unroll
+          for (int v = 0; v < VW; ++v) {
+            xx.v[v] += s_g[i0 + u][mycol + v] * rr[u].v[v];
+            if (a.flush) pp.v[v] += s_h[i0 + u][mycol + v] * rr[u].v[v];
+          }
+        }
+    }
+    stp<T, VW>(a.x + e * VW, xx);
+    if (a.flush) stp<T, VW>(a.p + e * VW, pp);
   }
 }
 

@@ -77,7 +77,7 @@ template <typename T>
 struct CoopArgs {
   PhaseArgs<T> a;  // a.g carries the mid list (nmid > 0: rows above kMidDeg are on it)
   CoopBar* bar;
-  const T* r0;           // the starting residual (a.r itself, or read only: a.r is then scratch; FP64: a.r is the
+  const T* r0;           // the starting residual (a.rn itself, or read only: a.rn is then scratch; FP64: a.rn is the
                          // final residual on return)
   const double* gamma0;  // its column norms |r0|^2; NULL: computed here
   int add_x;             // 1: x holds a start value, the correction is added to it; 0: x is written
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(CoopCfg<T, K>::TMAX, 1) cg_coop(CoopArgs<T> ca
   while (active) {
     // ---- S: s = M r, p, q, delta
     const bool first = iters == 0;
-    const T* rsrc = first ? ca_.r0 : a.r;
+    const T* rsrc = first ? ca_.r0 : a.rn;
     const bool l2 = ca_.cluster != 0;
     zero_acc();
     if (K == 1 && nhead > 0) {
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(CoopCfg<T, K>::TMAX, 1) cg_coop(CoopArgs<T> ca
       else
         sx[s] = xx;
       sr[s] = rr;
-      stp<T, VW>(a.r + (size_t)row * K + lane_off, rr);
+      stp<T, VW>(a.rn + (size_t)row * K + lane_off, rr);
     });
     if (!grid_sum(acc)) return;
     if (tid < K) {
@@ -676,8 +676,8 @@ __global__ void __launch_bounds__(CoopCfg<T, K>::TMAX, 1) cg_coop(CoopArgs<T> ca
       for (int w = 0; w < VW; ++w) z.v[w] = T(0);
       stp<T, VW>(px, z);
     }
-    // FP64: a.r ends as the solve's residual, also of one that took no iteration
-    if (sizeof(T) == 8 && iters == 0 && ca_.r0 != a.r) stp<T, VW>(a.r + (size_t)row * K + lane_off, sr[s]);
+    // FP64: a.rn ends as the solve's residual, also of one that took no iteration
+    if (sizeof(T) == 8 && iters == 0 && ca_.r0 != a.rn) stp<T, VW>(a.rn + (size_t)row * K + lane_off, sr[s]);
   });
   if (b == 0) {
     if (tid < K) {

@@ -96,10 +96,11 @@ cudaError_t launch_permute_vec(const double* in, int64_t n, const int32_t* perm,
 // mode 0: init (gamma_0, flags); 1: `chunk` iterations (S, U pairs); 2: final x += alpha p
 // a solve's start from the residual norms already in st->gamma (no pass over r)
 cudaError_t launch_cg_state_restart(CgState* st, const int* skip, int K, cudaStream_t s);
-cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, int grid_u, int mode, int chunk,
-                                 cudaStream_t s);
-cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, int mode, int chunk,
-                                 cudaStream_t s);
+// one iteration (S and U), or the start of a solve from r (init)
+cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, int grid_u, bool init, cudaStream_t s);
+cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, bool init, cudaStream_t s);
+cudaError_t launch_cg_x_f32(int K, const CgXArgs<float>& a, int grid, cudaStream_t s);
+cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStream_t s);
 // ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the
 // solve's vectors don't fit in shared memory
 bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
@@ -180,6 +181,8 @@ int sp_blocks();  // resident CTAs of the step kernels (all SMs)
 cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t s);
 // steps j0..j1-1 (the run stops by itself at cap - 1, on breakdown, or when the
 // error bound checked every `check` steps and at j1 is below rtol |theta_1|)
+// Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
+// the same steps as cooperative kernels of `check` steps each; bar is cleared before each
 cudaError_t launch_sp_steps(const SpArgs& a, int j0, int j1, int cap, int check, double rtol, int grid_s,
                             int grid_u, cudaStream_t s);
 // Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]

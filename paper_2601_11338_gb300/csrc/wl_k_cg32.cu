@@ -7,21 +7,16 @@ namespace wl {
 
 #define WL_FOR_K(X) X(1) X(2) X(4) X(8) X(16) X(32) X(64)
 
+// one CG iteration: S and U
 template <int K>
-static cudaError_t run_cg32(const PhaseArgs<float>& a, int grid_s, int grid_u, int mode, int chunk, cudaStream_t s) {
-  if (mode == 0) {
-    cg_u_phase<float, K><<<grid_u, kPhaseBlock, 0, s>>>(a, 1);
-  } else if (mode == 1) {
-    for (int i = 0; i < chunk; ++i) {
-      if (a.dshift)
-        cg_s_phase<float, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
-      else
-        cg_s_phase<float, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
-      cg_u_phase<float, K><<<grid_u, kPhaseBlock, 0, s>>>(a, 0);
-    }
-  } else {
-    cg_f_phase<float, K><<<grid_u, kPhaseBlock, 0, s>>>(a);
+static cudaError_t run_cg32(const PhaseArgs<float>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
+  if (!init) {
+    if (a.dshift)
+      cg_s_phase<float, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    else
+      cg_s_phase<float, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
   }
+  cg_u_phase<float, K><<<grid_u, kPhaseBlock, 0, s>>>(a, init ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -58,14 +53,25 @@ cudaError_t launch_cg_state_restart(CgState* st, const int* skip, int K, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, int grid_u, int mode, int chunk,
-                                 cudaStream_t s) {
+cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
   switch (K) {
 #define C32(k) \
   case k:      \
-    return run_cg32<k>(a, grid_s, grid_u, mode, chunk, s);
+    return run_cg32<k>(a, grid_s, grid_u, init, s);
     WL_FOR_K(C32)
 #undef C32
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_cg_x_f32(int K, const CgXArgs<float>& a, int grid, cudaStream_t s) {
+  switch (K) {
+#define X32(k)                                        \
+  case k:                                             \
+    cg_x_phase<float, k><<<grid, kPhaseBlock, 0, s>>>(a); \
+    return cudaGetLastError();
+    WL_FOR_K(X32)
+#undef X32
   }
   return cudaErrorInvalidValue;
 }

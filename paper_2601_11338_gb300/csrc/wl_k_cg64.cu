@@ -7,33 +7,38 @@ namespace wl {
 
 #define WL_FOR_K(X) X(1) X(2) X(4) X(8) X(16) X(32) X(64)
 
+// one CG iteration: S and U
 template <int K>
-static cudaError_t run_cg64(const PhaseArgs<double>& a, int grid_s, int grid_u, int mode, int chunk,
-                            cudaStream_t s) {
-  if (mode == 0) {
-    cg_u_phase<double, K><<<grid_u, kPhaseBlock, 0, s>>>(a, 1);
-  } else if (mode == 1) {
-    for (int i = 0; i < chunk; ++i) {
-      if (a.dshift)
-        cg_s_phase<double, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
-      else
-        cg_s_phase<double, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
-      cg_u_phase<double, K><<<grid_u, kPhaseBlock, 0, s>>>(a, 0);
-    }
-  } else {
-    cg_f_phase<double, K><<<grid_u, kPhaseBlock, 0, s>>>(a);
+static cudaError_t run_cg64(const PhaseArgs<double>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
+  if (!init) {
+    if (a.dshift)
+      cg_s_phase<double, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    else
+      cg_s_phase<double, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
   }
+  cg_u_phase<double, K><<<grid_u, kPhaseBlock, 0, s>>>(a, init ? 1 : 0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, int mode, int chunk,
-                                 cudaStream_t s) {
+cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
   switch (K) {
 #define C64(k) \
   case k:      \
-    return run_cg64<k>(a, grid_s, grid_u, mode, chunk, s);
+    return run_cg64<k>(a, grid_s, grid_u, init, s);
     WL_FOR_K(C64)
 #undef C64
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStream_t s) {
+  switch (K) {
+#define X64(k)                                        \
+  case k:                                             \
+    cg_x_phase<double, k><<<grid, kPhaseBlock, 0, s>>>(a); \
+    return cudaGetLastError();
+    WL_FOR_K(X64)
+#undef X64
   }
   return cudaErrorInvalidValue;
 }

@@ -109,7 +109,7 @@ int na_blocks() {
   int nb = 0, dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)cg_s_phase<double, 1>, kPhaseBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)cg_s_phase<double, 1, false, true>, kPhaseBlock, 0);
   const int g = (nb < 1 ? 1 : nb) * sms;
   return g > 2048 ? 2048 : g;
 }
@@ -184,13 +184,13 @@ extern "C" int wl_degrees_noalloc(const wl_csr* A, wl_variant v, double mu, doub
   na_fill<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(r, a, n);
   NA_CU(cudaGetLastError());
   NA_CU(cudaMemsetAsync(Df, 0, (size_t)n * sizeof(double), s));
-  PhaseArgs<double> pa{pg, Df, r, p, q, a, -alpha, alpha * alpha * m, nullptr, nullptr, part, state, max_iter,
+  PhaseArgs<double> pa{pg, Df, r, r, p, q, a, -alpha, alpha * alpha * m, nullptr, nullptr, part, state, max_iter,
                        tol * tol};
   cg_u_phase<double, 1><<<grid_u, kPhaseBlock, 0, s>>>(pa, 1);
   NA_CU(cudaGetLastError());
   for (;;) {
     for (int i = 0; i < 8; ++i) {
-      cg_s_phase<double, 1><<<grid_s, kPhaseBlock, 0, s>>>(pa);
+      cg_s_phase<double, 1, false, true><<<grid_s, kPhaseBlock, 0, s>>>(pa);
       cg_u_phase<double, 1><<<grid_u, kPhaseBlock, 0, s>>>(pa, 0);
     }
     NA_CU(cudaGetLastError());

@@ -29,10 +29,8 @@ struct DfResArgs {
   const float* bl;
   float* rh;        // r_out (may alias r_in)
   float* rl;
-  float* r32;       // copy of rh: right-hand side of the next FP32 inner solve (or NULL)
   float* xh;        // iterate, updated x += d in place (not FULL)
   float* xl;
-  float* dnext;     // zeroed here (start of the next inner solve), or NULL
   df ca, cA, cD;
   double* part;     // gridDim.x * K partials
   CgState* st;      // st->gamma[c] = |r_out[:, c]|^2
@@ -178,16 +176,9 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
     }
     stp<float, VW>(a.rh + o, rh);
     stp<float, VW>(a.rl + o, rl);
-    if (a.r32) stp<float, VW>(a.r32 + o, rh);
     if constexpr (!FULL) {
       stp<float, VW>(a.xh + o, xh);
       stp<float, VW>(a.xl + o, xl);
-      if (a.dnext) {
-        Pack<float, VW> z;
-#pragma unroll
-        for (int v = 0; v < VW; ++v) z.v[v] = 0.f;
-        stp<float, VW>(a.dnext + o, z);
-      }
     }
   };
 

@@ -207,3 +207,37 @@ def test_small_refined_solves_scale_with_their_columns():
         one = torch.stack([w.apply(V[:, :1] * c)[:, 0] / c for c in s], 1)
         assert (one - want[:, :1]).abs().max() <= 1e-8 * want.abs().max(), g.name
         w.close()
+
+
+# Phase kernels: x from the residuals kept over more iterations than are kept at
+# a time (near the pole), a warm start added to, several widths, and the final
+# residual that the FP64 shifted solves hand on; against scipy's FP64 CG
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)])
+def test_solves_by_kept_residuals(prec, tol, bound):
+    from oracle import krylov
+    g = wlgen.erdos_renyi(220001, 6.0, 8)
+    A = krylov.adjacency(g.row_ptr, g.col_idx, g.n)
+    for rel in (0.3, 0.97):
+        w = WL(g, variant="nbt", alpha_rel=rel, prec=prec, tol=tol)
+        L = krylov.ResolventLaplacian(A, 1.0, w.info["alpha"], tol=1e-14)
+        for k in (8, 16, 32) if rel < 0.5 else (16,):
+            V = np.random.default_rng(k).standard_normal((g.n, k))
+            V[:, 5] = 0.0
+            W = w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy()
+            want = L.apply(V[:, :4])
+            assert np.abs(W[:, :4] - want).max() <= bound * np.abs(want).max(), (rel, k)
+            assert (W[:, 5] == 0.0).all()
+        x0 = L.Df * (1.0 + 0.3 * np.cos(np.arange(g.n)))
+        w.warm_start(torch.as_tensor(x0, device="cuda"))
+        Df = w.degrees().cpu().numpy()
+        assert np.abs(Df - L.Df).max() <= bound * np.abs(L.Df).max()
+        if rel < 0.5:  # plain and shifted Lanczos on 16 sources agree
+            w.set(outer_tol=1e-11)
+            V = torch.zeros((g.n, 16), dtype=torch.float64, device="cuda")
+            V[torch.arange(16) * 999, torch.arange(16)] = 1.0
+            U = w.expmv(V, [0.5, 2.0])
+            w.set(shift=2.0)
+            S = w.expmv(V, [0.5, 2.0])
+            for t in range(2):
+                assert (S[t] - U[t]).abs().max() <= bound * U[t].abs().max()
+        w.close()
