@@ -632,6 +632,16 @@ struct CgStart {
   bool add_x = false;
 };
 
+// One column of more rows than this takes the kernels that stream the vectors
+// (wl_k1.cuh). CG, FP32, 5.2e5 rows (R-MAT) 1060 -> 975 us a call, 1e6 rows
+// 1529 -> 1354 (Chung-Lu) and 2392 -> 1981 us (R-MAT), but 645 -> 782 us at 4e5
+// rows (Chung-Lu), 306 -> 428 us at 8192; FP64, 1e6 rows 5186 -> 2193 us (R-MAT,
+// beyond shared memory otherwise), 5.2e5 rows 1244 -> 1322 us. The residual: 1e6
+// rows 257 -> 147 us (R-MAT), 4e5 rows 42 -> 39 us.
+template <typename T>
+constexpr int64_t k1_rows() { return sizeof(T) == 4 ? 500000 : 600000; }
+constexpr int64_t kResK1Rows = 250000;
+
 // Launches a solve as one cooperative kernel; false where its vectors don't
 // fit in shared memory (nothing launched).
 template <typename T>
@@ -656,7 +666,10 @@ bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& s
   }
   const int pc = prof_begin(h, kCatCG);
   bool coop;
-  if constexpr (sizeof(T) == 4)
+  if (K == 1 && h->n > k1_rows<T>()) {
+    *e = launch_cg_k1<T>(co, h->nnz, h->sms, S(h));
+    coop = true;
+  } else if constexpr (sizeof(T) == 4)
     coop = launch_cg_coop_f32(K, co, h->nnz, h->sms, S(h), e);
   else
     coop = launch_cg_coop_f64(K, co, h->nnz, h->sms, S(h), e);
@@ -868,7 +881,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // state of its own. Small solves run the correction as one cooperative kernel:
   // both are launched before one wait for their outcome.
   const PhaseGraph pg = phase_graph_mid(h, grid_u);
-  const bool coop = cg_coop_fits_f32(K, pg, h->nnz, h->sms);
+  const bool coop = (K == 1 && h->n > k1_rows<float>()) || cg_coop_fits_f32(K, pg, h->nnz, h->sms);
   if (coop) WL_TRY(ensure(h->r32, nk * 4));
   PhaseArgs<float> a{pg, dcur, (float*)h->r32.p, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
                      h->ca, h->cA, h->cD, nullptr, dskip, (double*)h->part.p, st, h->prm.max_iter, 0.0};
@@ -963,7 +976,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
     const int pi = prof_begin(h, kCatRes);
-    WL_CU(launch_df_res(K, ra, grid_r, false, S(h)));
+    WL_CU(K == 1 && h->n > kResK1Rows ? launch_df_res_k1(ra, h->nnz, h->sms, S(h)) : launch_df_res(K, ra, grid_r, false, S(h)));
     prof_end(h, pi);
     hgamma = nullptr;
     if (coop) {
@@ -1142,12 +1155,12 @@ int sp_cap(wl_handle* h) {
 SpArgs sp_args(wl_handle* h, double c0, double cD) {
   float2* W = (float2*)h->spW.p;
   return SpArgs{phase_graph(h), (const int32_t*)h->mid.p, h->nmid, h->nmid_blk, c0, 1.0, cD, (float2*)h->spV.p,
-                {W, W + h->n}, (double*)h->part.p, (SpState*)h->spstate.p, 0, 0x5EEDull};
+                {W, W + ((h->n + 1) & ~(int64_t)1)}, (double*)h->part.p, (SpState*)h->spstate.p, 0, 0x5EEDull};
 }
 
 int sp_buffers(wl_handle* h, int gs) {
   WL_TRY(ensure(h->spV, (size_t)sp_cap(h) * h->n * 8));
-  WL_TRY(ensure(h->spW, (size_t)2 * h->n * 8));
+  WL_TRY(ensure(h->spW, (size_t)2 * (h->n + 1) * 8));  // both on 16-byte boundaries
   WL_TRY(ensure(h->part, (size_t)gs * 64 * 2 * 8 + 1024));
   WL_TRY(ensure(h->spstate, sizeof(SpState)));
   return WL_OK;
@@ -1174,10 +1187,9 @@ int sp_run(wl_handle* h, SpRun* r, double rtol, bool seeded) {
   if (!t_sp_batch) WL_TRY(ensure_phase_buffers(h, std::max(gs, h->sms)));
   const SpArgs a = sp_args(h, r->c0, r->cD);
   SpState* st = (SpState*)h->spstate.p;
-  // a single graph's steps as cooperative kernels where its vectors fit; the
-  // batched build's searches share the GPU and run as kernels over all of them
-  const bool coop = !t_sp_batch && sp_coop_fits(a, h->nnz, h->sms);
-  if (coop) WL_CU(cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h)));
+  // a single graph's steps as cooperative kernels; the batched build's searches
+  // share the GPU and run as kernels over all of them
+  if (!t_sp_batch) WL_CU(cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h)));
   for (int guard = 0; guard < 256; ++guard) {
     if (r->exact || (r->m > 0 && r->bound <= rtol * std::fabs(r->theta))) break;
     int mode = 2;
@@ -1216,22 +1228,17 @@ int sp_run(wl_handle* h, SpRun* r, double rtol, bool seeded) {
       if (mode == 0) WL_CU(cudaMemsetAsync(st, 0, sizeof(SpState), S(h)));  // tickets and flags start at zero
       WL_CU(launch_sp_start(a, mode, gu, S(h)));
       const int chunks = (j1 - j0 + kSpCheck - 1) / kSpCheck;
-      if (coop) {
-        counted(h, 1 + 2 * chunks);
-        if (fault_mode() == kFaultTimeout) {
-          static const int gave_up = WL_ERR_TIMEOUT;
-          WL_CU(cudaMemcpyAsync(&h->cgbar()->err, &gave_up, sizeof(int), cudaMemcpyHostToDevice, S(h)));
-        }
-        WL_CU(launch_sp_steps_coop(a, h->nnz, h->sms, h->cgbar(), j0, j1, cap, kSpCheck, rtol, S(h)));
-        h->bar_clean = false;
-        WL_CU(cudaMemcpyAsync(h->h_pin + 16, &h->cgbar()->err, sizeof(int), cudaMemcpyDeviceToHost, S(h)));
-      } else {
-        counted(h, 1 + 2 * (j1 - j0) + chunks);
-        WL_CU(launch_sp_steps(a, j0, j1, cap, kSpCheck, rtol, gs, gu, S(h)));
+      counted(h, 1 + 2 * chunks);
+      if (fault_mode() == kFaultTimeout) {
+        static const int gave_up = WL_ERR_TIMEOUT;
+        WL_CU(cudaMemcpyAsync(&h->cgbar()->err, &gave_up, sizeof(int), cudaMemcpyHostToDevice, S(h)));
       }
+      WL_CU(launch_sp_steps_coop(a, h->nnz, h->sms, h->cgbar(), j0, j1, cap, kSpCheck, rtol, S(h)));
+      h->bar_clean = false;
+      WL_CU(cudaMemcpyAsync(h->h_pin + 16, &h->cgbar()->err, sizeof(int), cudaMemcpyDeviceToHost, S(h)));
       WL_CU(cudaMemcpyAsync(h->h_pin, &st->start_norm, 9 * 8 + 4 * 4, cudaMemcpyDeviceToHost, S(h)));
       WL_CU(cudaStreamSynchronize(S(h)));
-      if (coop && *(const int*)(h->h_pin + 16) != 0) return *(const int*)(h->h_pin + 16);
+      if (*(const int*)(h->h_pin + 16) != 0) return *(const int*)(h->h_pin + 16);
       for (int i = 0; i < 8; ++i) o[i] = h->h_pin[1 + i];
       const int* ints = (const int*)(h->h_pin + 9);
       m_eff = ints[0];
@@ -2903,7 +2910,7 @@ int sp_clone(wl_handle* h, wl_handle** out) {
   // the states back itself
   int rc = sp_buffers(c, sp_grid(c) + c->nhub + c->nmid_blk);
   if (rc != WL_OK) return fail(rc);
-  cudaError_t e = cudaMemcpyAsync(c->spW.p, h->spW.p, (size_t)2 * h->n * 8, cudaMemcpyDeviceToDevice, S(h));
+  cudaError_t e = cudaMemcpyAsync(c->spW.p, h->spW.p, (size_t)2 * (h->n + 1) * 8, cudaMemcpyDeviceToDevice, S(h));
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->spstate.p, h->spstate.p, sizeof(SpState), cudaMemcpyDeviceToDevice, S(h));
   if (e == cudaSuccess) e = cudaStreamSynchronize(S(h));
   if (e != cudaSuccess) return fail(set_cuda_error(e, "search context copy"));

@@ -104,6 +104,10 @@ cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStrea
 // ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the
 // solve's vectors don't fit in shared memory
 bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
+// ---- wl_k_k1.cu: the same for one column (any n), and its residual (df_res, not full)
+template <typename T>
+cudaError_t launch_cg_k1(const CoopArgs<T>& a, int64_t nnz, int sms, cudaStream_t s);
+cudaError_t launch_df_res_k1(const DfResArgs& a, int64_t nnz, int sms, cudaStream_t s);
 bool cg_coop_fits_f32(int K, const PhaseGraph& g, int64_t nnz, int sms);
 bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
 // one CTA waiting in the bounded grid barrier for nblocks CTAs (failure-detection self-test)
@@ -183,13 +187,8 @@ cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t 
 // error bound checked every `check` steps and at j1 is below rtol |theta_1|)
 // Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
 // the same steps as cooperative kernels of `check` steps each; bar is cleared before each
-cudaError_t launch_sp_steps(const SpArgs& a, int j0, int j1, int cap, int check, double rtol, int grid_s,
-                            int grid_u, cudaStream_t s);
-// Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
-// the same steps as cooperative kernels of `check` steps each; bar is cleared before each
-bool sp_coop_fits(const SpArgs& a, int64_t nnz, int sms);
-cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
-                                 int check, double rtol, cudaStream_t s);
+cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap, int check,
+                                 double rtol, cudaStream_t s);
 cudaError_t launch_sp_ritz(const SpArgs& a, int grid_u, cudaStream_t s);
 // One round of the batched spectral searches: the np jobs (device array) with
 // their CTA offsets in the S kernel (off_s, np + 1 entries, off_s[np] =

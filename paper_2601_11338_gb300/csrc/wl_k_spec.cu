@@ -11,7 +11,7 @@ int sp_blocks() {
   int nb = 0, dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)sp_s, kPhaseBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)sp_s_multi, kPhaseBlock, 0);
   return (nb < 1 ? 1 : nb) * sms;
 }
 
@@ -23,22 +23,13 @@ cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t 
   return cudaGetLastError();
 }
 
-cudaError_t launch_sp_steps(const SpArgs& a0, int j0, int j1, int cap, int check, double rtol, int grid_s,
-                            int grid_u, cudaStream_t s) {
-  SpArgs a = a0;
-  for (int j = j0; j < j1; ++j) {
-    a.j = j;
-    sp_s<<<grid_s, kPhaseBlock, 0, s>>>(a);
-    sp_u<<<grid_u, kPhaseBlock, 0, s>>>(a, j == cap - 1 ? 1 : 0);
-    if ((j + 1) % check == 0 || j + 1 == j1) sp_eig<<<1, 2 * kSpEigT, 0, s>>>(a.st, rtol);
-  }
-  return cudaGetLastError();
-}
+// Graphs of more rows take the steps that stream the vectors (eight of them:
+// Chung-Lu, 400003 nodes 250 -> 202 us, R-MAT scale 17 about a tenth less; the
+// others were 10% to 40% slower by it); up to it the vectors always fit.
+constexpr int64_t kSpStreamRows = 250000;
 
-// grid, threads and shared memory of the cooperative steps; false where a
-// run's vectors don't fit, or where they are so few that the row loops'
-// kernels cost no more
-static bool sp_coop_shape(const SpArgs& a, int64_t nnz, int sms, int* grid, int* threads, size_t* smem, int* nhead) {
+// grid, threads and shared memory of the cooperative steps
+static void sp_coop_shape(const SpArgs& a, int64_t nnz, int sms, int* grid, int* threads, size_t* smem, int* nhead) {
   const int64_t units = a.g.n * kSpCoopLpr;
   *grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (units + 255) / 256));
   const int64_t rows = coop_rows_local(a.g.n, *grid, kSpCoopCh);
@@ -46,34 +37,33 @@ static bool sp_coop_shape(const SpArgs& a, int64_t nnz, int sms, int* grid, int*
   *threads = (int)std::max<int64_t>(256, (rows * kSpCoopLpr / passes + 31) / 32 * 32);
   const int64_t nslot = rows + (a.nmid + *grid - 1) / *grid + (a.g.nhub + *grid - 1) / *grid;
   const size_t vec = (size_t)nslot * 3 * sizeof(float2);
-  if (vec > kSpCoopSmem) return false;
   *nhead = (int)std::min<int64_t>({a.g.n, nnz / (4 * *grid), (int64_t)((kSpCoopSmem - vec) / sizeof(float2))});
   *smem = vec + (size_t)*nhead * sizeof(float2);
-  return true;
 }
-
-bool sp_coop_fits(const SpArgs& a, int64_t nnz, int sms) {
-  int grid, threads, nhead;
-  size_t smem;
-  return sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &nhead);
-}
+// rows and listed rows of a CTA at that limit, three vectors each
+static_assert(2 * (kSpStreamRows / 128 + 2 * kSpCoopCh) * 3 * sizeof(float2) <= kSpCoopSmem, "a run's vectors fit");
 
 cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
                                  int check, double rtol, cudaStream_t s) {
+  const bool stream = a.g.n > kSpStreamRows;
   static const cudaError_t attr =
       cudaFuncSetAttribute(sp_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpCoopSmem);
   if (attr != cudaSuccess) return attr;
+  static const cudaError_t attr1 =
+      cudaFuncSetAttribute(sp_k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
+  if (attr1 != cudaSuccess) return attr1;
   SpCoopArgs ca{a, bar, 0, 0, cap, 0};
-  int grid, threads;
-  size_t smem;
-  if (!sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &ca.nhead)) return cudaErrorInvalidValue;
+  int grid = k1_grid(a.g.n, sms), threads = k1_threads<float2>();
+  ca.nhead = k1_head<float2>(a.g.n, nnz, grid);
+  size_t smem = k1_smem<float2>(ca.nhead);
+  if (!stream) sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &ca.nhead);
   for (int j = j0; j < j1; j = ca.j1) {
     ca.j0 = j;
     ca.j1 = std::min(j1, (j / check + 1) * check);
     cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     void* args[] = {&ca};
-    e = cudaLaunchCooperativeKernel((const void*)sp_coop, dim3(grid), dim3(threads), args, smem, s);
+    e = cudaLaunchCooperativeKernel(stream ? (const void*)sp_k1 : (const void*)sp_coop, dim3(grid), dim3(threads), args, smem, s);
     if (e != cudaSuccess) return e;
     sp_eig<<<1, 2 * kSpEigT, 0, s>>>(a.st, rtol);
   }

@@ -241,3 +241,34 @@ def test_solves_by_kept_residuals(prec, tol, bound):
             for t in range(2):
                 assert (S[t] - U[t]).abs().max() <= bound * U[t].abs().max()
         w.close()
+
+
+# One column, vectors streamed: rows by the CTA (one of 70000 entries), by a warp
+# and by eight lanes, groups of rows with and without one of them between, a
+# last group that isn't whole, with and without the nodes ordered; against
+# scipy's FP64 CG, and the spectral scale against its Lanczos solver
+@pytest.mark.parametrize("reorder", [0, 1])
+def test_one_column_of_many_rows(reorder):
+    from scipy.sparse.linalg import eigsh
+    from oracle import krylov
+    n = 600037
+    e = wlgen.erdos_renyi(n, 3.0, 12)
+    src = np.repeat(np.arange(n), e.degrees)
+    rng = np.random.default_rng(5)
+    deg = {17: 70000, 5000: 3000, 299999: 4096, 300000: 4097, 450001: 257, 450002: 256, 600036: 31}
+    hs = np.concatenate([np.full(d, v) for v, d in deg.items()])
+    hd = np.concatenate([rng.choice(n, d, replace=False) for d in deg.values()])
+    keep = hs != hd
+    g = wlgen.csr_from_edges(n, np.concatenate([src, hs[keep]]), np.concatenate([e.col_idx, hd[keep]]))
+    A = krylov.adjacency(g.row_ptr, g.col_idx, g.n)
+    lmax = eigsh(A, k=1, which="LA", return_eigenvectors=False)[0]
+    for prec, tol, bound in (("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)):
+        w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=tol, reorder=reorder)
+        assert abs(w.info["lambda_max"] - lmax) <= 1e-9 * lmax
+        D = krylov.ResolventLaplacian(A, 1.0, w.info["alpha"], tol=1e-14).Df
+        Df = w.degrees().cpu().numpy()
+        assert np.abs(Df - D).max() <= bound * np.abs(D).max()
+        w.warm_start(torch.as_tensor(D * (1.0 + 0.3 * np.cos(np.arange(n))), device="cuda"))
+        Df = w.degrees().cpu().numpy()
+        assert np.abs(Df - D).max() <= bound * np.abs(D).max()
+        w.close()
