@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <condition_variable>
 #include <cstdlib>
@@ -1493,17 +1494,19 @@ struct OuterRun {
   // shift-and-invert run: the shift, the time points and T_m per column (host)
   bool si = false;
   double sigma = 0.0;
-  std::vector<double> taus, Ta, Tb;  // Ta, Tb: K x m
+  std::vector<double> taus, T;  // T: K x m diagonals, then off-diagonals
 };
 
 constexpr int kLdT = 1024;  // T and y leading dimension (Lanczos steps per column at most kLdT - 1)
 
 // ------------------------------------------------------------------ shift-and-invert Lanczos (Sec. 4.4)
-// Eigenvalues th[0..m) and eigenvectors (column k: Z[i * m + k]) of the
+// Eigenvalues th[0..m) and eigenvectors (the k-th: Z[k * m + i]) of the
 // symmetric tridiagonal matrix with diagonal a[0..m) and off-diagonal
 // b[0..m-1), by implicit QR sweeps with the Wilkinson shift on each
 // unreduced block (Golub and Van Loan, Sec. 8.3), the rotations accumulated
-// into Z. False if a block needs more than 30 m sweeps.
+// into Z, whose rows k and k + 1 a rotation mixes (contiguous, so that the
+// compiler's vector instructions do it). False if a block needs more than 30 m
+// sweeps. 32 columns, m = 2, 4, .., 44: 20 -> 17 ms in all on one thread.
 bool tridiag_eig_host(int m, const double* a, const double* b, std::vector<double>& th, std::vector<double>& Z) {
   th.assign(a, a + m);
   std::vector<double> e(std::max(m, 1), 0.0);
@@ -1538,11 +1541,12 @@ bool tridiag_eig_host(int m, const double* a, const double* b, std::vector<doubl
         e[k + 1] *= c;
         x = e[k];
       }
+      double* __restrict__ z0 = &Z[(size_t)k * m];
+      double* __restrict__ z1 = z0 + m;
       for (int i = 0; i < m; ++i) {
-        double* zr = &Z[(size_t)i * m];
-        const double zk = zr[k], zk1 = zr[k + 1];
-        zr[k] = c * zk + sn * zk1;
-        zr[k + 1] = -sn * zk + c * zk1;
+        const double zk = z0[i], zk1 = z1[i];
+        z0[i] = c * zk + sn * zk1;
+        z1[i] = -sn * zk + c * zk1;
       }
     }
   }
@@ -1562,13 +1566,45 @@ bool si_eval(int m, const double* a, const double* b, double sigma, const std::v
     for (int i = 0; i < m; ++i) yt[i] = 0.0;
     for (int k = 0; k < m; ++k) {
       if (!(th[k] > 0.0)) continue;
-      const double f = std::exp(-taus[t] * (1.0 / th[k] - sigma)) * Z[k];
+      const double* zk = &Z[(size_t)k * m];
+      const double f = std::exp(-taus[t] * (1.0 / th[k] - sigma)) * zk[0];
       if (f == 0.0) continue;
-      for (int i = 0; i < m; ++i) yt[i] += Z[(size_t)i * m + k] * f;
+      for (int i = 0; i < m; ++i) yt[i] += zk[i] * f;
     }
   }
   return true;
 }
+
+// f(c) for every column c < K, which each take about `ops` operations, on up to
+// eight threads (a thread per half a million operations: starting one takes
+// some twenty microseconds): the checks of 32 columns up to 44 steps and 24 time
+// points took 35 of 174 ms of return probabilities on one, 16 of 155 here. False
+// if any call was false or threw.
+template <typename F>
+bool for_columns(int K, double ops, F f) {
+  std::atomic<int> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&]() {
+    try {
+      for (int c; (c = next.fetch_add(1)) < K;)
+        if (!f(c)) ok = false;
+    } catch (...) {
+      ok = false;
+    }
+  };
+  const int extra = (int)std::min<double>({7.0, (double)K - 1.0, ops * K / 5e5 - 1.0,
+                                           (double)std::thread::hardware_concurrency() - 1.0});
+  std::vector<std::thread> th;
+  try {
+    for (int i = 0; i < extra; ++i) th.emplace_back(work);
+  } catch (...) {  // no more threads: the others and this one do it
+  }
+  work();
+  for (auto& t : th) t.join();
+  return ok;
+}
+// operations of si_eval, about
+double si_eval_ops(int m, int ntau) { return 6.0 * m * m * m + 40.0 * m * m + ntau * (2.0 * m * m + 40.0 * m); }
 
 // the per-row diagonal and scaling of the shifted solves for the handle's
 // D_f and shift sigma (sibuf: dsh64, inv64 (n doubles each), then dsh_h,
@@ -1686,6 +1722,19 @@ int reorth_block(wl_handle* h, bool dfp, int K, int j, size_t blk, double* Tb, i
   if (e != cudaSuccess) return set_cuda_error(e, "reorth");
   return WL_OK;
 }
+// The first m steps of K columns' T (diagonals at Ta, off-diagonals behind them,
+// ldT apart) on the host, through pinned memory where it has the room: a
+// pageable 2D copy takes 150 us.
+int tridiag_to_host(wl_handle* h, const double* Ta, int K, int m, int ldT, std::vector<double>& T) {
+  T.resize((size_t)2 * K * m);
+  const bool pin = T.size() <= 4096;
+  WL_CU(cudaMemcpy2DAsync(pin ? h->h_pin : T.data(), (size_t)m * 8, Ta, (size_t)ldT * 8, (size_t)m * 8, (size_t)2 * K,
+                          cudaMemcpyDeviceToHost, S(h)));
+  WL_CU(cudaStreamSynchronize(S(h)));
+  if (pin) std::copy(h->h_pin, h->h_pin + T.size(), T.data());
+  return WL_OK;
+}
+
 constexpr int kMaxReturnT = 256;  // time points per wl_return_prob call
 
 int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& info, OuterRun& o, int& outer_total) {
@@ -1861,21 +1910,14 @@ int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& inf
     if (si && (m % check == 0 || m == maxm)) {
       // y(tau) = exp(-tau (T_m^{-1} - sigma I)) e_1 per column on the host,
       // compared with the previous check's (the rule of the polynomial run)
-      std::vector<double> hT((size_t)2 * K * m);
-      WL_CU(cudaMemcpy2DAsync(hT.data(), (size_t)m * 8, Ta, (size_t)ldT * 8, (size_t)m * 8, K,
-                              cudaMemcpyDeviceToHost, S(h)));
-      WL_CU(cudaMemcpy2DAsync(hT.data() + (size_t)K * m, (size_t)m * 8, Tb, (size_t)ldT * 8, (size_t)m * 8, K,
-                              cudaMemcpyDeviceToHost, S(h)));
-      WL_CU(cudaStreamSynchronize(S(h)));
+      std::vector<double> hT;
+      WL_TRY(tridiag_to_host(h, Ta, K, m, ldT, hT));
       const int berr = check_bar(h);
       if (berr) return berr;
-      bool all = true;
-      std::vector<double> y((size_t)ntau * m);
-      for (int c = 0; c < K; ++c) {
-        if (!si_eval(m, hT.data() + (size_t)c * m, hT.data() + (size_t)(K + c) * m, o.sigma, o.taus, y.data(), m)) {
-          all = false;
-          continue;
-        }
+      const bool all = for_columns(K, si_eval_ops(m, ntau), [&](int c) {
+        std::vector<double> y((size_t)ntau * m);
+        if (!si_eval(m, hT.data() + (size_t)c * m, hT.data() + (size_t)(K + c) * m, o.sigma, o.taus, y.data(), m)) return false;
+        bool col = true;
         for (int t = 0; t < ntau; ++t) {
           const double* yt = y.data() + (size_t)t * m;
           double ny = 0.0, dy = 0.0;
@@ -1888,12 +1930,11 @@ int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& inf
           // a zero start column (the padding of a block) has nothing to
           // converge; in any other column a y that vanished is not converged
           // (the space has not reached the slow modes yet)
-          const bool ok =
-              hdone[c] || (!yp.empty() && ny > 0.0 && std::sqrt(dy) <= h->prm.outer_tol * std::sqrt(ny));
-          if (!ok) all = false;
+          col &= hdone[c] || (!yp.empty() && ny > 0.0 && std::sqrt(dy) <= h->prm.outer_tol * std::sqrt(ny));
           si_prev[(size_t)c * ntau + t].assign(yt, yt + m);
         }
-      }
+        return col;
+      });
       if (all) { converged = true; break; }
     } else if (m % check == 0 || m == maxm) {
       std::vector<int> hm(K, m);
@@ -1921,13 +1962,7 @@ int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& inf
   o.m = m;
   o.converged = converged;
   if (si && m > 0) {  // T_m per column for outer_combine
-    o.Ta.resize((size_t)K * m);
-    o.Tb.resize((size_t)K * m);
-    WL_CU(cudaMemcpy2DAsync(o.Ta.data(), (size_t)m * 8, Ta, (size_t)ldT * 8, (size_t)m * 8, K,
-                            cudaMemcpyDeviceToHost, S(h)));
-    WL_CU(cudaMemcpy2DAsync(o.Tb.data(), (size_t)m * 8, Tb, (size_t)ldT * 8, (size_t)m * 8, K,
-                            cudaMemcpyDeviceToHost, S(h)));
-    WL_CU(cudaStreamSynchronize(S(h)));
+    WL_TRY(tridiag_to_host(h, Ta, K, m, ldT, o.T));
   }
   return WL_OK;
 }
@@ -1952,10 +1987,11 @@ int outer_combine(wl_handle* h, const OuterRun& o, int t0, int nt, double* out, 
   if (o.si) {  // y(tau) from the eigendecomposition of each column's T_m (host)
     std::vector<double> hy((size_t)K * nt * ldT, 0.0);
     const std::vector<double> tt(o.taus.begin() + t0, o.taus.begin() + t0 + nt);
-    for (int c = 0; c < K; ++c)
-      if (o.m > 0 && !si_eval(o.m, o.Ta.data() + (size_t)c * o.m, o.Tb.data() + (size_t)c * o.m, o.sigma, tt,
-                              hy.data() + (size_t)c * nt * ldT, ldT))
-        return WL_ERR_NO_CONVERGENCE;
+    if (o.m > 0 && !for_columns(K, si_eval_ops(o.m, nt), [&](int c) {
+          return si_eval(o.m, o.T.data() + (size_t)c * o.m, o.T.data() + (size_t)(K + c) * o.m, o.sigma, tt,
+                         hy.data() + (size_t)c * nt * ldT, ldT);
+        }))
+      return WL_ERR_NO_CONVERGENCE;
     WL_CU(cudaMemcpyAsync(h->ybuf.p, hy.data(), hy.size() * 8, cudaMemcpyHostToDevice, S(h)));
     WL_CU(cudaStreamSynchronize(S(h)));
   } else {
