@@ -174,14 +174,14 @@ int alloc_solve(wl_batch* b, SolveBufs& s, int K) {
   s.K = K;
   const size_t elems = (size_t)b->nslab * b->n * K;
   const size_t np = nprob(b), nc = np * K;
-  BT_CU(dalloc(s.x, elems * 8));
-  BT_CU(dalloc(s.r, elems * 8));
-  BT_CU(dalloc(s.p, elems * 8));
-  BT_CU(dalloc(s.q, elems * 8));
+  BT_CU(dalloc(s.x, elems * 8 + 64));
+  BT_CU(dalloc(s.r, elems * 8 + 64));
+  BT_CU(dalloc(s.p, elems * 8 + 64));
+  BT_CU(dalloc(s.q, elems * 8 + 64));
   BT_CU(dalloc(s.x64, elems * 8));
   if (b->prm.prec == WL_REFINED) BT_CU(dalloc(s.rdf, elems * 8));
   BT_CU(dalloc(s.part, (size_t)b->nslab * std::max(max_tiles(b), 1) * 2 * K * 8));
-  BT_CU(dalloc(s.colstate, nc * 6 * 8));
+  BT_CU(dalloc(s.colstate, nc * (6 + 2 * kBatchHist) * 8));
   BT_CU(dalloc(s.colint, nc * 4 * 4));
   BT_CU(dalloc(s.probint, np * 5 * 4));
   BT_CU(dalloc(s.flags, 64 * 4));
@@ -195,7 +195,9 @@ BatchState bstate(const wl_batch* b, SolveBufs& s) {
   int* ci = (int*)s.colint.p;
   int* pi = (int*)s.probint.p;
   int* fl = (int*)s.flags.p;
-  return BatchState{cs, cs + nc, cs + 2 * nc, cs + 3 * nc, ci, ci + nc, pi, pi + np, pi + 4 * np, fl + 0};
+  const bool refined = b->prm.prec == WL_REFINED;
+  return BatchState{cs, cs + nc, cs + 2 * nc, cs + 3 * nc, ci, ci + nc, pi, pi + np, pi + 4 * np, fl + 0,
+                    refined ? cs + 6 * nc : nullptr, refined ? cs + (6 + kBatchHist) * nc : nullptr};
 }
 
 BatchOuter bouter(const wl_batch* b, SolveBufs& s) {
@@ -307,10 +309,10 @@ unsigned grid1(int64_t work) {
 #define BT_FOR_K(X) X(1) X(2) X(4) X(8) X(16) X(32) X(64)
 
 template <typename T>
-int emit_init(int K, const BatchArgs<T>& a, const int* pmask, int nslab, cudaStream_t s) {
+int emit_init(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
   const dim3 grid(a.g.ntile, nslab);
   switch (K) {
-#define C(k) case k: bcg_init<T, k><<<grid, kPhaseBlock, 0, s>>>(a, pmask); break;
+#define C(k) case k: bcg_init<T, k><<<grid, kPhaseBlock, 0, s>>>(a); break;
     BT_FOR_K(C)
 #undef C
     default: return WL_ERR_INVALID_ARG;
@@ -400,10 +402,10 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
   BT_CU(cudaMemsetAsync(sb.flags.p, 0, sb.flags.bytes, s));
   BT_CU(cudaMemsetAsync(st.total, 0, sizeof(int) * np, s));
   if (b->prm.prec == WL_FP64) {
-    BatchArgs<double> a{g, (double*)sb.x.p, (double*)sb.r.p, (double*)sb.p.p, (double*)sb.q.p,
+    BatchArgs<double> a{g, (double*)sb.x.p, (double*)sb.r.p, (double*)sb.p.p, (double*)sb.q.p, nullptr, {},
                         (const double*)b->ca.p, (const double*)b->cA.p, (const double*)b->cD.p, rhs, bscale,
                         nullptr, nullptr, (double*)sb.part.p, st, b->prm.max_iter, tol2};
-    BT_TRY(emit_init<double>(K, a, nullptr, nslab, s));
+    BT_TRY(emit_init<double>(K, a, nslab, s));
     BT_TRY(emit_red_init(K, g, st, a.part, nullptr, nullptr, nullptr, tol2, nslab, s));
     BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<double>(K, a, nslab, em.s()); }));
     return emit_final<double>(K, a, nslab, em.s());
@@ -420,17 +422,21 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
   BT_CU(cudaGetLastError());
   const size_t elems = (size_t)nslab * b->n * K;
   BatchResArgs ra{g, (const float*)sb.x.p, rhs, bscale, (const double*)b->ca.p, (const double*)b->cA.p,
-                  (const double*)b->cD.p, (float*)sb.rdf.p, (float*)sb.rdf.p + elems, (float*)sb.r.p,
+                  (const double*)b->cD.p, (float*)sb.rdf.p, (float*)sb.rdf.p + elems,
                   (double*)sb.x64.p, (double*)sb.part.p, o.outer_active, o.outer_iters};
-  BatchArgs<float> ia{g, (float*)sb.x.p, (float*)sb.r.p, (float*)sb.p.p, (float*)sb.q.p, (const double*)b->ca.p,
-                      (const double*)b->cA.p, (const double*)b->cD.p, nullptr, nullptr, o.rn2, o.skip,
-                      (double*)sb.part.p, st, b->prm.max_iter, tin * tin};
+  // the inner solve starts from the residual's leading term and its norms; later
+  // residuals take the r buffer and the upper halves of it, x, p and q in turn
+  const size_t up = (elems + 3) & ~(size_t)3;
+  BatchArgs<float> ia{g, (float*)sb.x.p, nullptr, (float*)sb.p.p, (float*)sb.q.p, (const float*)sb.rdf.p,
+                      {(float*)sb.r.p, (float*)sb.r.p + up, (float*)sb.p.p + up, (float*)sb.q.p + up,
+                       (float*)sb.x.p + up},
+                      (const double*)b->ca.p, (const double*)b->cA.p, (const double*)b->cD.p, nullptr, nullptr, o.rn2,
+                      o.skip, (double*)sb.part.p, st, b->prm.max_iter, tin * tin};
   return em.loop(sb, o.any, b->prm.max_outer + 2, [&]() -> int {
     cudaStream_t so = em.s();
     BT_TRY(emit_res(K, ra, nslab, so));
     BT_TRY(emit_red_res(K, g, o, ra.part, tol2, b->prm.max_outer, nslab, so));
-    BT_TRY(emit_init<float>(K, ia, o.outer_active, nslab, so));
-    BT_TRY(emit_red_init(K, g, st, ia.part, o.rn2, o.skip, o.outer_active, tin * tin, nslab, so));
+    BT_TRY(emit_red_init(K, g, st, nullptr, o.rn2, o.skip, o.outer_active, tin * tin, nslab, so));
     // the correction d ends in sb.x; the next residual pass adds it to x64
     BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<float>(K, ia, nslab, em.s()); }));
     return emit_final<float>(K, ia, nslab, em.s());
@@ -469,8 +475,8 @@ int time_tiles(wl_batch* b, const TileSet& ts, int K, float* ms) {
   float best = 1e30f;
   for (int rep = 0; rep < 4; ++rep) {
     BT_CU(cudaEventRecord(e0, s));
-    BatchArgs<float> a{g, (float*)sb.x.p, (float*)sb.r.p, (float*)sb.p.p, (float*)sb.q.p, (const double*)b->ca.p,
-                       (const double*)b->cA.p, (const double*)b->cD.p, nullptr, nullptr, nullptr, nullptr,
+    BatchArgs<float> a{g, (float*)sb.x.p, nullptr, (float*)sb.p.p, (float*)sb.q.p, (const float*)sb.r.p, {},
+                       (const double*)b->ca.p, (const double*)b->cA.p, (const double*)b->cD.p, nullptr, nullptr, nullptr, nullptr,
                        (double*)sb.part.p, st, 1, 0.0};
     switch (K) {
 #define C(k) case k: bcg_s<float, k><<<dim3(g.ntile, b->nslab), kPhaseBlock, 0, s>>>(a); break;

@@ -56,15 +56,25 @@ struct BatchState {
   int* iters;    // per problem: iterations of the current solve
   int* total;    // per problem: iterations summed over the refinement steps
   int* any;      // one flag: some problem still iterates
+  double* ha;    // FP32: step sizes of the kept iterations, [kBatchHist][problem-columns]
+  double* hb;
 };
+
+// FP32 solves keep the residuals of this many iterations and form x and p from
+// them (as in wl_cg2.cuh): five buffers, the halves that FP32 vectors leave of the
+// FP64 form's five. A 24-graph batch, 32 columns:
+// 8.28 -> 7.99 ms (S phases 24 x 141 -> 124 us, x 3 x 36 -> 107 us, no start pass).
+constexpr int kBatchHist = 4;
 
 template <typename T>
 struct BatchArgs {
   BatchGraph g;
   T* x;
-  T* r;
+  T* r;                 // FP64: the residual, updated in place
   T* p;
   T* q;
+  const T* r0;          // FP32: the starting residual, and where later ones go in turn
+  T* ring[kBatchHist + 1];
   const double* ca;     // per problem
   const double* cA;
   const double* cD;
@@ -124,21 +134,83 @@ __device__ __forceinline__ bool plain_row(const int32_t* row_ptr, int64_t row) {
   return row_ptr[row + 1] - row_ptr[row] <= kHubDeg;
 }
 
-// ---------------------------------------------------------------- init
-// x = 0, r = bscale * b (or r as given), gamma_0 partials
+// r_j of an FP32 solve
+template <typename T>
+__device__ __forceinline__ T* batch_r(const BatchArgs<T>& a, int j) {
+  return j == 0 ? const_cast<T*>(a.r0) : a.ring[(j - 1) % (kBatchHist + 1)];
+}
+
+// x (and p, if the solve goes on) of a tile's rows from r_{j-m} .. r_{j-1}, as
+// cg_x_phase of wl_cg2.cuh
 template <typename T, int K>
-__global__ void __launch_bounds__(kPhaseBlock) bcg_init(BatchArgs<T> a, const int* pmask) {
+__device__ __forceinline__ void batch_form_x(const BatchArgs<T>& a, const BTile& tl, int s, int pr, int j, int m,
+                                             bool flush) {
+  using C = Cfg<T, K>;
+  constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
+  const int tid = threadIdx.x, lane_off = (tid % G) * VW;
+  const size_t slab = (size_t)s * a.g.n * K, nc = (size_t)gridDim.y * a.g.ngraph * K;
+  const bool more = j > m;  // x and p_{j-m-1} are there
+  T g[kBatchHist + 1][VW], h[kBatchHist + 1][VW];
+#pragma unroll
+  for (int v = 0; v < VW; ++v) {
+    const size_t i0 = (size_t)pr * K + lane_off + v;
+    T gg = T(0), hh = T(1), be = T(0);
+#pragma unroll
+    for (int i = kBatchHist - 1; i >= 0; --i) {
+      g[i][v] = h[i][v] = T(0);
+      if (i < m) {
+        gg = (T)a.st.ha[i * nc + i0] + be * gg;
+        if (i < m - 1) hh *= be;
+        be = (T)a.st.hb[i * nc + i0];
+        g[i][v] = gg;
+        h[i][v] = hh;
+      }
+    }
+    g[kBatchHist][v] = be * gg;
+    h[kBatchHist][v] = be * hh;
+  }
+  const T* R[kBatchHist];
+#pragma unroll
+  for (int i = 0; i < kBatchHist; ++i) R[i] = batch_r(a, i < m ? j - m + i : 0) + slab;
+  for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
+    if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
+    const size_t o = (size_t)row * K + lane_off;
+    Pack<T, VW> rr[kBatchHist], xx, pp;
+#pragma unroll
+    for (int v = 0; v < VW; ++v) xx.v[v] = pp.v[v] = T(0);
+    if (more) {
+      xx = ld_last<T, VW>(a.x + slab + o);
+      pp = ld_last<T, VW>(a.p + slab + o);
+    }
+#pragma unroll
+    for (int i = 0; i < kBatchHist; ++i)
+      if (i < m) rr[i] = ld_last<T, VW>(R[i] + o);
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      xx.v[v] += g[kBatchHist][v] * pp.v[v];
+      pp.v[v] *= h[kBatchHist][v];
+    }
+#pragma unroll
+    for (int i = 0; i < kBatchHist; ++i)
+      if (i < m)
+#pragma unroll
+        for (int v = 0; v < VW; ++v) {
+          xx.v[v] += g[i][v] * rr[i].v[v];
+          pp.v[v] += h[i][v] * rr[i].v[v];
+        }
+    stp<T, VW>(a.x + slab + o, xx);
+    if (flush) stp<T, VW>(a.p + slab + o, pp);
+  }
+}
+
+// ---------------------------------------------------------------- init
+// FP64: x = 0, r = bscale * b (or r as given), gamma_0 partials
+template <typename T, int K>
+__global__ void __launch_bounds__(kPhaseBlock) bcg_init(BatchArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
-  if (pmask && !pmask[pr]) {  // problem not refining any more: zero partials only
-    typename CoopSum<T>::S z[Cfg<T, K>::VW];
-#pragma unroll
-    for (int v = 0; v < Cfg<T, K>::VW; ++v) z[v] = CoopSum<T>::zero();
-    block_colsum_store<T, K>(z, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
-    return;
-  }
   const int tid = threadIdx.x, lane_off = (tid % G) * VW;
   const size_t slab = (size_t)s * a.g.n * K;
   const T sc = a.bscale ? (T)a.bscale[pr] : T(1);
@@ -168,7 +240,7 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_init(BatchArgs<T> a, const in
   block_colsum_store<T, K>(acc, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
 }
 
-// gamma_0, reference norms, flags; grid (ngraph, nslab)
+// gamma_0 (of the partials, or NULL: bnorm2), reference norms, flags; grid (ngraph, nslab)
 template <int K>
 __global__ void __launch_bounds__(kPhaseBlock) bred_init(BatchGraph g, BatchState st, const double* part,
                                                           const double* bnorm2, const int* skip, const int* pmask,
@@ -176,14 +248,15 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_init(BatchGraph g, BatchStat
   __shared__ double s_tmp[kPhaseBlock];
   __shared__ double s_out[K];
   const int s = blockIdx.y, pr = s * g.ngraph + blockIdx.x;
-  problem_sum<K>(part + (size_t)s * g.ntile * K, g.tile_beg[blockIdx.x], g.tile_beg[blockIdx.x + 1], s_tmp, s_out);
+  if (part)
+    problem_sum<K>(part + (size_t)s * g.ntile * K, g.tile_beg[blockIdx.x], g.tile_beg[blockIdx.x + 1], s_tmp, s_out);
   const int tid = threadIdx.x;
   __shared__ int s_any;
   if (tid == 0) s_any = 0;
   __syncthreads();
   if (tid < K) {
     const int i = pr * K + tid;
-    const double gn = s_out[tid];
+    const double gn = part ? s_out[tid] : bnorm2[i];
     const double b2 = bnorm2 ? bnorm2[i] : gn;
     st.gamma[i] = gn;
     st.b2[i] = b2;
@@ -216,7 +289,13 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   if (!a.st.active[pr]) return;
   const int tid = threadIdx.x, sl = tid % G, lane_off = sl * VW;
-  const bool first = a.st.iters[pr] == 0;
+  // FP32: the residuals are kept, x and p formed from them every kBatchHist iterations and at the end
+  constexpr bool kKept = sizeof(T) == 4;
+  const int it = a.st.iters[pr];
+  const bool first = it == 0;
+  if constexpr (kKept) {
+    if (!first && it % kBatchHist == 0) batch_form_x<T, K>(a, tl, s, pr, it, kBatchHist, true);
+  }
   const T ca = (T)a.ca[pr], cA = (T)a.cA[pr], cD = (T)a.cD[pr];
   T al[VW], be[VW];
 #pragma unroll
@@ -225,7 +304,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     be[v] = first ? T(0) : (T)a.st.beta[pr * K + lane_off + v];
   }
   const size_t slab = (size_t)s * a.g.n * K;
-  const T* __restrict__ R = a.r + slab;
+  const T* __restrict__ R = (kKept ? batch_r(a, it) : a.r) + slab;
   T* __restrict__ P = a.p + slab;
   T* __restrict__ Q = a.q + slab;
   T* __restrict__ X = a.x + slab;
@@ -242,6 +321,13 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
         pp.v[v] = rr.v[v];
         qq.v[v] = ca * rr.v[v] + cA * nb[v] + cD * (T)deg * rr.v[v];
       }
+    } else if constexpr (kKept) {
+      const Pack<T, VW> qo = ld_last<T, VW>(Q + o);
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        pp.v[v] = rr.v[v];  // (r, q) = (p, q)
+        qq.v[v] = ca * rr.v[v] + cA * nb[v] + cD * (T)deg * rr.v[v] + be[v] * qo.v[v];
+      }
     } else {
       const Pack<T, VW> po = ld_plain<T, VW>(P + o);
       const Pack<T, VW> qo = ld_plain<T, VW>(Q + o);
@@ -256,7 +342,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     }
 #pragma unroll
     for (int v = 0; v < VW; ++v) dacc[v] += pp.v[v] * qq.v[v];
-    stp<T, VW>(P + o, pp);
+    if constexpr (!kKept) stp<T, VW>(P + o, pp);
     stp<T, VW>(Q + o, qq);
   };
   if (tl.hub) {
@@ -320,6 +406,7 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_s(BatchGraph g, BatchState s
   __shared__ double s_out[K];
   const int s = blockIdx.y, pr = s * g.ngraph + blockIdx.x;
   if (!st.active[pr]) return;
+  const int it = st.iters[pr];
   problem_sum<K>(part + (size_t)s * g.ntile * K, g.tile_beg[blockIdx.x], g.tile_beg[blockIdx.x + 1], s_tmp, s_out);
   const int tid = threadIdx.x;
   if (tid < K) {
@@ -336,9 +423,14 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_s(BatchGraph g, BatchState s
     } else {
       st.alpha[i] = 0.0;
     }
+    if (st.ha) {
+      const size_t o = (size_t)(it % kBatchHist) * gridDim.x * gridDim.y * K + i;
+      st.ha[o] = st.alpha[i];
+      st.hb[o] = st.beta[i];
+    }
   }
   if (tid == 0) {
-    st.iters[pr] += 1;
+    st.iters[pr] = it + 1;
     st.total[pr] += 1;
   }
 }
@@ -356,6 +448,9 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_u(BatchArgs<T> a) {
 #pragma unroll
   for (int v = 0; v < VW; ++v) al[v] = (T)a.st.alpha[pr * K + lane_off + v];
   const size_t slab = (size_t)s * a.g.n * K;
+  const int it = a.st.iters[pr];  // of the S phase before, counted
+  const T* rin = sizeof(T) == 4 ? batch_r(a, it - 1) : a.r;
+  T* rout = sizeof(T) == 4 ? batch_r(a, it) : a.r;
   typename CoopSum<T>::S acc[VW];
 #pragma unroll
   for (int v = 0; v < VW; ++v) acc[v] = CoopSum<T>::zero();
@@ -363,27 +458,32 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_u(BatchArgs<T> a) {
   for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
     if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
     const size_t o = slab + (size_t)row * K + lane_off;
-    Pack<T, VW> rr = ld_plain<T, VW>(a.r + o);
+    Pack<T, VW> rr = ld_last<T, VW>(rin + o);
     const Pack<T, VW> qq = ld_plain<T, VW>(a.q + o);
 #pragma unroll
     for (int v = 0; v < VW; ++v) {
       rr.v[v] -= al[v] * qq.v[v];
       acc_sq(acc[v], rr.v[v]);
     }
-    stp<T, VW>(a.r + o, rr);
+    stp<T, VW>(rout + o, rr);
   }
   block_colsum_store<T, K>(acc, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
 }
 
-// x += alpha p: the update of each problem's last iteration (the S kernel
-// makes the others, where it reads p anyway)
+// FP64: x += alpha p, the update of each problem's last iteration (the S kernel
+// makes the others, where it reads p anyway). FP32: x from the kept residuals.
 template <typename T, int K>
 __global__ void __launch_bounds__(kPhaseBlock) bcg_f(BatchArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
-  if (a.st.iters[pr] == 0) return;
+  const int it = a.st.iters[pr];
+  if constexpr (sizeof(T) == 4) {
+    batch_form_x<T, K>(a, tl, s, pr, it, it == 0 ? 0 : (it - 1) % kBatchHist + 1, false);
+    return;
+  }
+  if (it == 0) return;
   const int tid = threadIdx.x, lane_off = (tid % G) * VW;
   T al[VW];
 #pragma unroll
@@ -447,8 +547,7 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_u(BatchGraph g, BatchState s
 // per neighbour entry) and r = rh + rl a double-float vector. The neighbour
 // sum A d is accumulated with the error-free two-sum, M d and the subtraction
 // in double-float, so r stays equal to bscale b - M x64 up to about 2^-46 of
-// |r| + |M d| per pass. r32 = rh is the next inner solve's right-hand side
-// (the inner init zeroes d). Partials per column: (r, r) from the leading
+// |r| + |M d| per pass. rh is the next inner solve's right-hand side. Partials per column: (r, r) from the leading
 // terms, and on the first pass (bscale b, bscale b).
 struct BatchResArgs {
   BatchGraph g;
@@ -460,7 +559,6 @@ struct BatchResArgs {
   const double* cD;
   float* rh;            // [nslab][n][K] residual, leading term
   float* rl;            // [nslab][n][K] residual, trailing term
-  float* r32;           // [nslab][n][K] inner right-hand side
   double* x64;          // [nslab][n][K] iterate
   double* part;         // [nslab][ntile][2K]
   const int* outer_active;  // per problem (NULL: all)
@@ -517,7 +615,6 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchRes
     for (int v = 0; v < VW; ++v) acc_r[v] = __fmaf_rn(rh.v[v], rh.v[v], acc_r[v]);
     stp<float, VW>(a.rh + slab + o, rh);
     stp<float, VW>(a.rl + slab + o, rl);
-    stp<float, VW>(a.r32 + slab + o, rh);
   };
   if (tl.hub) {
     const int64_t row = tl.row_beg;

@@ -272,3 +272,38 @@ def test_one_column_of_many_rows(reorder):
         Df = w.degrees().cpu().numpy()
         assert np.abs(Df - D).max() <= bound * np.abs(D).max()
         w.close()
+
+
+# Batched corrections whose residuals are kept: near the pole (tens of
+# iterations, so x and p are formed several times), far from it (fewer than are
+# kept), an odd number of rows (unaligned halves of the buffers, one column) and
+# a hub row, against the oracle's dense phi
+@pytest.mark.parametrize("rel", [0.02, 0.5, 0.97])
+@pytest.mark.parametrize("k", [1, 2, 4, 32])
+def test_batched_corrections_by_kept_residuals(rel, k):
+    from paper_2601_11338_gb300 import wl
+    gs = [wlgen.erdos_renyi(301, 6.0, 4), wlgen.path(3), wlgen.star(701), wlgen.grid2d(9, 11)]
+    mus = [0.25, 0.0]
+    n = sum(g.n for g in gs)
+    assert n % 2 == 1
+    p = wl.make_params(f=wl.WL_F_RESOLVENT, alpha_rel=rel, prec=wl.WL_REFINED, tol=1e-11,
+                       stream=torch.cuda.current_stream().cuda_stream)
+    b = wl.wl_batch_build([(g.row_ptr.astype(np.int32), g.col_idx, g.n, g.nnz) for g in gs], mus, p)
+    V = np.random.default_rng(k).standard_normal((n, k))
+    V[:301, k - 1] = 0.0 if k > 1 else V[:301, 0]  # a zero column of the first graph
+    Df = torch.empty((2, n), dtype=torch.float64, device="cuda")
+    W = torch.empty((2, n, k), dtype=torch.float64, device="cuda")
+    st = wl.wl_stats()
+    assert wl.wl_batch_run(b, torch.as_tensor(V, device="cuda"), k, Df, W, 0, st, ()) == wl.WL_OK
+    lo = 0
+    for i, g in enumerate(gs):
+        A = graph.dense_adjacency(g.row_ptr, g.col_idx, g.n)
+        for s, mu in enumerate(mus):
+            phi = walks.phi_resolvent_closed(A, mu, wl.wl_batch_info(b, i, s)["alpha"])
+            D, L = walks.walk_degrees(phi), walks.walk_laplacian(phi)
+            got, w = Df[s, lo:lo + g.n].cpu().numpy(), W[s, lo:lo + g.n].cpu().numpy()
+            want = L @ V[lo:lo + g.n]
+            assert np.abs(got - D).max() <= 1e-8 * np.abs(D).max(), (g.name, mu)
+            assert np.abs(w - want).max() <= 1e-8 * np.abs(want).max(), (g.name, mu)
+        lo += g.n
+    b.destroy()
