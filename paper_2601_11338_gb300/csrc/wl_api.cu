@@ -2157,7 +2157,7 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
   // validation
   Smalls sm = smalls(h);
   if (cudaMemsetAsync(sm.flags, 0, sizeof(int), S(h)) != cudaSuccess) return fail(WL_ERR_CUDA);
-  if (cudaError_t e = launch_validate(h->g, sm.flags, S(h)); e != cudaSuccess) return fail(set_cuda_error(e, "validate"));
+  if (cudaError_t e = launch_validate(h->g, sm.flags, (unsigned long long*)sm.misc, S(h)); e != cudaSuccess) return fail(set_cuda_error(e, "validate"));
   int flags = 0;
   if (cudaMemcpyAsync(&flags, sm.flags, sizeof(int), cudaMemcpyDeviceToHost, S(h)) != cudaSuccess ||
       cudaStreamSynchronize(S(h)) != cudaSuccess)

@@ -45,7 +45,7 @@ struct PartDev {
 cudaError_t launch_partition(const Graph& g, PartDev& p, cudaStream_t s);
 // flags[0] bit0: row_ptr not monotone / bounds; bit1: column out of range or
 // unsorted/duplicate; bit2: self loop; bit3: asymmetric
-cudaError_t launch_validate(const Graph& g, int* flags, cudaStream_t s);
+cudaError_t launch_validate(const Graph& g, int* flags, unsigned long long* diff, cudaStream_t s);
 // dst (n x kb, contiguous, double or float) = scale * src[:, c0:c0+kr] (leading dim ld), columns kr.. zero. Here and
 // below kr <= K is the number of a block's columns that the caller has.
 cudaError_t launch_pack(const double* src, int64_t ld, int c0, int kr, int kb, int64_t n, double scale, void* dst,

@@ -93,28 +93,77 @@ cudaError_t launch_partition(const Graph& g, PartDev& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// One warp per row: row_ptr monotone and within [0, nnz], columns strictly
-// increasing in range, no self-loop, and (i, j) stored implies (j, i) stored
-// (binary search in row j).
-__global__ void k_validate(const int32_t* row_ptr, const int32_t* col, int64_t n, int64_t nnz, int* flags) {
+// row_ptr from 0 to nnz and nowhere decreasing
+__global__ void __launch_bounds__(256) k_check_rows(const int32_t* row_ptr, int64_t n, int64_t nnz, int* flags) {
+  int f = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    f |= row_ptr[i + 1] < row_ptr[i];
+  if (blockIdx.x == 0 && threadIdx.x == 0) f |= row_ptr[0] != 0 || (int64_t)row_ptr[n] != nnz;
+  if (f) atomicOr(flags, 1);
+}
+
+// For sound row bounds: columns strictly increasing in range, no self-loop, and
+// (i, j) stored implies (j, i) stored. The last by binary search, for the entries
+// whose row i is the longer one (or, at equal length, has the larger index): i is
+// looked up in the shorter row j, so the hubs' long rows are never searched. Each
+// of these entries then has a mirror image among the others, and as no entry is
+// stored twice all others have one exactly when there are as many of the one kind
+// as of the other (*diff). A warp takes kValChunk entries, 32 at a time, whatever
+// rows they are of (a warp per row, or per 32 rows, waited for the hubs' warps).
+// Chung-Lu, 4e5 nodes, 4.8e6 entries: 74 us; a warp per row and
+// every entry searched: 335 us; 32 rows per warp: 273 us.
+constexpr int kValChunk = 512;
+__global__ void __launch_bounds__(256) k_validate(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                                                  int64_t n, int64_t nnz, int* flags, unsigned long long* diff) {
+  if (*(volatile int*)flags & 1) return;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    const int64_t beg = row_ptr[i], end = row_ptr[i + 1];
-    int f = 0;
-    if (beg < 0 || end < beg || end > nnz) {
-      if (lane == 0) atomicOr(flags, 1);
+  const int64_t e0 = warp * kValChunk, e1 = e0 + kValChunk < nnz ? e0 + kValChunk : nnz;
+  if (e0 >= nnz) return;  // whole warp
+  // the last row that starts at or before entry e
+  auto row_of = [&](int64_t e) {
+    int64_t lo = 0, hi = n;
+    while (hi - lo > 1) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (row_ptr[mid] <= e) lo = mid; else hi = mid;
+    }
+    return lo;
+  };
+  int f = 0;
+  long long d = 0;
+  int64_t r0 = row_of(e0), e = e0;
+  while (e < e1) {  // the rows r0 .. r0 + 31, a lane each
+    const int64_t row = r0 + lane < n ? r0 + lane : n;
+    const int64_t beg = row_ptr[row], end = row_ptr[row < n ? row + 1 : n];
+    const int64_t last = __shfl_sync(0xffffffffu, end, 31);
+    if (last <= e) {  // a run of empty rows
+      r0 = row_of(e);
       continue;
     }
-    for (int64_t e = beg + lane; e < end; e += 32) {
-      const int32_t j = col[e];
+    const int64_t stop = last < e1 ? last : e1;
+    for (; e < stop; e += 32) {
+      const int64_t t = e + lane;
+      int src = 0;  // the row of entry t: the last that starts at or before it
+#pragma unroll
+      for (int h = 16; h > 0; h >>= 1) {
+        const int64_t p = __shfl_sync(0xffffffffu, beg, src + h);
+        if (p <= t) src += h;
+      }
+      const int64_t bi = __shfl_sync(0xffffffffu, beg, src), li = __shfl_sync(0xffffffffu, end, src) - bi;
+      if (t >= stop) continue;
+      const int64_t i = r0 + src;
+      const int32_t j = col[t];
       if (j < 0 || j >= n) { f |= 2; continue; }
-      if (e > beg && col[e - 1] >= j) f |= 2;
+      if (t > bi && col[t - 1] >= j) f |= 2;
       if (j == i) { f |= 4; continue; }
-      int64_t lo = row_ptr[j], hi = row_ptr[j + 1] - 1;
+      int64_t lo = row_ptr[j], hi = (int64_t)row_ptr[j + 1] - 1;
+      const int64_t lj = hi - lo + 1;
+      if (lj > li || (lj == li && j > i)) {
+        --d;
+        continue;
+      }
+      ++d;
       bool found = false;
-      if (lo < 0 || hi >= nnz) { f |= 1; continue; }
       while (lo <= hi) {
         const int64_t mid = (lo + hi) >> 1;
         const int32_t v = col[mid];
@@ -123,19 +172,32 @@ __global__ void k_validate(const int32_t* row_ptr, const int32_t* col, int64_t n
       }
       if (!found) f |= 8;
     }
+    e = stop;
+    r0 += 32;
+  }
+  f = __reduce_or_sync(0xffffffffu, f);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+  if (lane == 0) {
     if (f) atomicOr(flags, f);
+    if (d != 0) atomicAdd(diff, (unsigned long long)d);
   }
 }
 
-__global__ void k_check_ends(const int32_t* row_ptr, int64_t n, int64_t nnz, int* flags) {
-  if (row_ptr[0] != 0 || (int64_t)row_ptr[n] != nnz) atomicOr(flags, 1);
+__global__ void k_check_counts(int* flags, const unsigned long long* diff) {
+  if (*diff != 0) atomicOr(flags, 8);
 }
 
-cudaError_t launch_validate(const Graph& g, int* flags, cudaStream_t s) {
-  k_check_ends<<<1, 1, 0, s>>>(g.row_ptr, g.n, g.nnz, flags);
-  if (g.n > 0) {
-    const int64_t warps = g.n < 152 * 64 ? g.n : 152 * 64;
-    k_validate<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(g.row_ptr, g.col, g.n, g.nnz, flags);
+// diff: 8 bytes of scratch
+cudaError_t launch_validate(const Graph& g, int* flags, unsigned long long* diff, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(diff, 0, sizeof(*diff), s);
+  if (e != cudaSuccess) return e;
+  k_check_rows<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((g.n + 255) / 256, 152 * 8)), 256, 0, s>>>(
+      g.row_ptr, g.n, g.nnz, flags);
+  if (g.n > 0 && g.nnz > 0) {
+    const int64_t warps = (g.nnz + kValChunk - 1) / kValChunk;
+    k_validate<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(g.row_ptr, g.col, g.n, g.nnz, flags, diff);
+    k_check_counts<<<1, 1, 0, s>>>(flags, diff);
   }
   return cudaGetLastError();
 }

@@ -165,7 +165,7 @@ extern "C" int wl_degrees_noalloc(const wl_csr* A, wl_variant v, double mu, doub
   NA_CU(cudaMemsetAsync(misc, 0, kNaMiscBytes, s));
   NA_CU(cudaMemsetAsync(state, 0, sizeof(CgState), s));
   const Graph g{A->row_ptr, A->col_idx, n, A->nnz};
-  NA_CU(launch_validate(g, misc, s));
+  NA_CU(launch_validate(g, misc, (unsigned long long*)(misc + 32), s));
   na_hub_list<<<1, 1024, 0, s>>>(A->row_ptr, n, hubs, misc + 1);
   NA_CU(cudaGetLastError());
   int hostv[2] = {0, 0};

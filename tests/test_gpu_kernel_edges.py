@@ -307,3 +307,39 @@ def test_batched_corrections_by_kept_residuals(rel, k):
             assert np.abs(w - want).max() <= 1e-8 * np.abs(want).max(), (g.name, mu)
         lo += g.n
     b.destroy()
+
+
+# Symmetry of the stored pattern: one entry without its mirror image at either
+# end of a hub row or between equal rows, two that keep the counts equal, in
+# groups of 32 rows with and without empty rows; and the sound graphs
+def test_every_one_sided_entry_is_found():
+    from paper_2601_11338_gb300 import wl
+    rng = np.random.default_rng(3)
+    n = 1301
+    e = wlgen.erdos_renyi(n, 3.0, 6)
+    src = np.repeat(np.arange(n), e.degrees)
+    hub = rng.choice(np.arange(200, n - 100), 700, replace=False)
+    g = wlgen.csr_from_edges(n, np.concatenate([src, np.full(700, 77)]), np.concatenate([e.col_idx, hub]))
+    rows = np.repeat(np.arange(n), np.diff(g.row_ptr))
+    cols = g.col_idx.astype(np.int64)
+
+    def built(drop):
+        keep = np.ones(cols.size, bool)
+        keep[list(drop)] = False
+        rp = np.concatenate([[0], np.cumsum(np.bincount(rows[keep], minlength=n))]).astype(np.int32)
+        try:
+            w = WL(wlgen.CSR(n, rp.astype(np.int64), cols[keep].astype(np.int32)), variant="nbt", alpha_rel=0.5)
+            w.close()
+            return wl.WL_OK
+        except wl.WLError as err:
+            return err.status
+
+    assert built(()) == wl.WL_OK
+    assert built(np.flatnonzero((rows == 77) | (cols == 77))) == wl.WL_OK  # row 77 empty, both sides gone
+    hubrow, hubcol = np.flatnonzero(rows == 77), np.flatnonzero(cols == 77)
+    small = np.flatnonzero((rows != 77) & (cols != 77))
+    for i in (hubrow[0], hubrow[-1], hubcol[0], hubcol[-1], *rng.choice(small, 6, replace=False)):
+        assert built((i,)) == wl.WL_ERR_NOT_SYMMETRIC, i
+    for a, b in ((hubrow[3], hubcol[5]), (hubrow[0], hubrow[1]), (small[0], small[-1]), (hubcol[0], small[5])):
+        if not (rows[a] == cols[b] and cols[a] == rows[b]):
+            assert built((a, b)) == wl.WL_ERR_NOT_SYMMETRIC, (a, b)
