@@ -731,11 +731,31 @@ __device__ __forceinline__ df df_rcp(df a) {
 // from the Gershgorin interval (129^7 > 1e14).
 constexpr int kSpEigT = 128;
 constexpr int kSpEigRounds = 7;
+constexpr double kSpEigStep = 1.0 / (kSpEigT + 1);
 constexpr int kSpEigCoarse = 3;     // 129^3 > 2e6: the FP32 bracket is below 1e-6 of the interval
 constexpr double kSpEigMargin = 1e-6;
 constexpr int kSpEigFine = 4;       // 129^4 > 2.7e8: from 2.9e-6 ||T|| to 1.1e-14 ||T||
 static_assert(kSpEigFine <= kSpEigRounds, "the narrow search ends within the full one");
 static_assert(2 * kSpEigT == kSpMax, "one row per thread in the eigen step");
+
+// The first point of the group whose count is above idx (kSpEigT: none), the
+// same in every thread of the group; all threads of the block call it. (One
+// thread walking the 128 counts took a third of the eigen step.)
+__device__ __forceinline__ int sp_first_above(int cnt, int idx, int grp) {
+  __shared__ int s_first[2 * kSpEigT / 32];
+  const int warp = threadIdx.x >> 5;
+  const unsigned above = __ballot_sync(0xffffffffu, cnt > idx);
+  if ((threadIdx.x & 31) == 0) s_first[warp] = above ? __ffs(above) - 1 : kSpEigT;
+  __syncthreads();
+  int k = kSpEigT;
+#pragma unroll
+  for (int w = kSpEigT / 32 - 1; w >= 0; --w) {
+    const int f = s_first[grp * (kSpEigT / 32) + w];
+    if (f < kSpEigT) k = 32 * w + f;
+  }
+  __syncthreads();
+  return k;
+}
 
 __device__ __forceinline__ void sp_eig_body(SpState* st, double rtol) {
   __shared__ double s_lo[2], s_hi[2];
@@ -803,13 +823,11 @@ __device__ __forceinline__ void sp_eig_body(SpState* st, double rtol) {
   // (1) FP32 multisection
   for (int round = 0; round < kSpEigCoarse; ++round) {
     const double lo = s_lo[grp], w = s_hi[grp] - lo;
-    s_cnt[grp][t] = sturm_count_f32(s_af, s_b2f, m, (float)(lo + w * (double)(t + 1) / (double)(kSpEigT + 1)));
-    __syncthreads();
+    const int cnt = sturm_count_f32(s_af, s_b2f, m, (float)(lo + w * ((double)(t + 1) * kSpEigStep)));
+    const int k = sp_first_above(cnt, idx, grp);
     if (t == 0) {
-      int k = 0;
-      while (k < kSpEigT && s_cnt[grp][k] <= idx) ++k;
-      s_lo[grp] = lo + w * (double)k / (double)(kSpEigT + 1);
-      s_hi[grp] = lo + w * (double)(k + 1) / (double)(kSpEigT + 1);
+      s_lo[grp] = lo + w * ((double)k * kSpEigStep);
+      s_hi[grp] = lo + w * ((double)(k + 1) * kSpEigStep);
     }
     __syncthreads();
   }
@@ -835,15 +853,14 @@ __device__ __forceinline__ void sp_eig_body(SpState* st, double rtol) {
     const bool nar = s_ok[grp] != 0;
     const bool act = nar ? round < kSpEigFine : true;
     const double lo = s_lo[grp], w = s_hi[grp] - lo;
-    const double x = lo + w * (double)(t + 1) / (double)(kSpEigT + 1);
-    if (act) s_cnt[grp][t] = nar ? sturm_count_df(s_ah, s_al, s_qh, s_ql, m, df_from_double(x))
-                                 : sturm_count_poly(s_a, s_b2, m, x);
-    __syncthreads();
+    const double x = lo + w * ((double)(t + 1) * kSpEigStep);
+    int cnt = 0;
+    if (act) cnt = nar ? sturm_count_df(s_ah, s_al, s_qh, s_ql, m, df_from_double(x))
+                       : sturm_count_poly(s_a, s_b2, m, x);
+    const int k = sp_first_above(cnt, idx, grp);
     if (act && t == 0) {
-      int k = 0;
-      while (k < kSpEigT && s_cnt[grp][k] <= idx) ++k;
-      s_lo[grp] = lo + w * (double)k / (double)(kSpEigT + 1);
-      s_hi[grp] = lo + w * (double)(k + 1) / (double)(kSpEigT + 1);
+      s_lo[grp] = lo + w * ((double)k * kSpEigStep);
+      s_hi[grp] = lo + w * ((double)(k + 1) * kSpEigStep);
     }
     __syncthreads();
   }
