@@ -1020,7 +1020,7 @@ int solve_refined(wl_handle* h, const double* b, double* x, int K, double tol, b
   double* bn2 = (double*)h->small.p + 600;
   WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
   counted(h);
-  WL_CU(launch_df_from_f64(K, b, 1.0, h->n, (float*)h->bh.p, (float*)h->bl.p, nullptr, (double*)h->part.p, st, bn2,
+  WL_CU(launch_df_from_f64(K, b, h->n, (float*)h->bh.p, (float*)h->bl.p, (double*)h->part.p, st, bn2,
                            grid_u, S(h)));
   WL_TRY(solve_refined_df(h, (const float*)h->bh.p, (const float*)h->bl.p, bn2, (float*)h->xh.p,
                           (float*)h->xl.p, x_is_zero ? nullptr : x, K, tol, info));

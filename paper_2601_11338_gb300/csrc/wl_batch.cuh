@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchRes
       const Pack<double, VW> bb = ld_plain<double, VW>(a.b + o);
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
-        const df r = df_from_double(sc * bb.v[v]);
+        const df r = split_f64(a.bscale ? sc * bb.v[v] : bb.v[v]);
         rh.v[v] = r.hi;
         rl.v[v] = r.lo;
         acc_b[v] = __fmaf_rn(r.hi, r.hi, acc_b[v]);
@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(kPhaseBlock, kPhaseMinBlocksF32) bres(BatchRes
         const df r = df_sub(df{ph.v[v], pl.v[v]}, Md);
         rh.v[v] = r.hi;
         rl.v[v] = r.lo;
-        xx.v[v] += (double)dd.v[v];
+        xx.v[v] += widen_f32(dd.v[v]);
       }
       stp<double, VW>(a.x64 + slab + o, xx);
     }

@@ -267,19 +267,18 @@ __global__ void __launch_bounds__(kBlock) df_scale_cols(const double* X, int64_t
   __syncthreads();
   const size_t total = (size_t)n * K;
   for (size_t e = (size_t)blockIdx.x * kBlock + threadIdx.x; e < total; e += (size_t)gridDim.x * kBlock) {
-    const double x = X[e] * inv[e & (size_t)(K - 1)];
-    const float h = (float)x;
-    hi[e] = h;
-    lo[e] = (float)(x - (double)h);
+    const df t = split_f64(X[e] * inv[e & (size_t)(K - 1)]);
+    hi[e] = t.hi;
+    lo[e] = t.lo;
   }
 }
 
 // FP64 vector -> (hi, lo)
 __global__ void __launch_bounds__(kBlock) df_split(const double* x, size_t total, float* hi, float* lo) {
   for (size_t e = (size_t)blockIdx.x * kBlock + threadIdx.x; e < total; e += (size_t)gridDim.x * kBlock) {
-    const float h = (float)x[e];
-    hi[e] = h;
-    lo[e] = (float)(x[e] - (double)h);
+    const df t = split_f64(x[e]);
+    hi[e] = t.hi;
+    lo[e] = t.lo;
   }
 }
 #endif  // WL_EXPDF_KERNELS

@@ -121,8 +121,8 @@ cudaError_t launch_split_x(const double* x, int64_t total, float* xh, float* xl,
 // r_out = r_in - M y (y gathered: the correction d; x += d) or, full, r_out = b - M x (x = yh + yl)
 cudaError_t launch_df_res(int K, const DfResArgs& a, int grid, bool full, cudaStream_t s);
 // (bh, bl) = scale * b (b: n x K FP64, contiguous), r32 = bh (if not NULL), |b|^2 per column -> b2
-cudaError_t launch_df_from_f64(int K, const double* b, double scale, int64_t n, float* bh, float* bl, float* r32,
-                               double* part, CgState* st, double* b2, int grid, cudaStream_t s);
+cudaError_t launch_df_from_f64(int K, const double* b, int64_t n, float* bh, float* bl, double* part, CgState* st,
+                               double* b2, int grid, cudaStream_t s);
 int df_res_blocks(int K);
 // outer Lanczos of the refined form on double-float vectors (cooperative launch)
 int df_lanczos_grid(int K);

@@ -52,15 +52,15 @@ static cudaError_t run_res(const ResPhaseArgs& a, int grid, cudaStream_t s) {
 // FP64 iterate <-> double-float terms (xh, xl)
 __global__ void __launch_bounds__(kPhaseBlock) split_x(const double* x, int64_t total, float* xh, float* xl) {
   for (int64_t e = (int64_t)blockIdx.x * kPhaseBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kPhaseBlock) {
-    const float h = (float)x[e];
-    xh[e] = h;
-    xl[e] = (float)(x[e] - (double)h);
+    const df t = split_f64(x[e]);
+    xh[e] = t.hi;
+    xl[e] = t.lo;
   }
 }
 
 __global__ void __launch_bounds__(kPhaseBlock) join_x(const float* xh, const float* xl, int64_t total, double* x) {
   for (int64_t e = (int64_t)blockIdx.x * kPhaseBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kPhaseBlock)
-    x[e] = (double)xh[e] + (double)xl[e];
+    x[e] = join_f64(xh[e], xl[e]);
 }
 
 cudaError_t launch_split_x(const double* x, int64_t total, float* xh, float* xl, bool join, double* xout,

@@ -32,12 +32,12 @@ cudaError_t launch_df_res(int K, const DfResArgs& a, int grid, bool full, cudaSt
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_df_from_f64(int K, const double* b, double scale, int64_t n, float* bh, float* bl, float* r32,
-                               double* part, CgState* st, double* b2, int grid, cudaStream_t s) {
+cudaError_t launch_df_from_f64(int K, const double* b, int64_t n, float* bh, float* bl, double* part,
+                               CgState* st, double* b2, int grid, cudaStream_t s) {
   switch (K) {
-#define DC(k)                                                                               \
-  case k:                                                                                   \
-    df_from_f64<k><<<grid, kPhaseBlock, 0, s>>>(b, scale, n, bh, bl, r32, part, st, b2);    \
+#define DC(k)                                                                 \
+  case k:                                                                     \
+    df_from_f64<k><<<grid, kPhaseBlock, 0, s>>>(b, n, bh, bl, part, st, b2);  \
     return cudaGetLastError();
     WL_FOR_K(DC)
 #undef DC

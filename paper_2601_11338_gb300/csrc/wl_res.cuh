@@ -269,11 +269,10 @@ __global__ void __launch_bounds__(kPhaseBlock, 4) df_res(DfResArgs a) {
   if (tid == 0) a.st->ticket = 0;
 }
 
-// b (n x K FP64, contiguous) * scale -> (bh, bl), r32 = bh, |b|^2 per column
-// (from bh) -> b2[c]; the conversion is the one FP64 pass of a refined solve.
+// b (n x K FP64, contiguous) -> (bh, bl), |b|^2 per column (from bh) -> b2[c]
 template <int K>
-__global__ void __launch_bounds__(kPhaseBlock) df_from_f64(const double* b, double scale, int64_t n, float* bh,
-                                                           float* bl, float* r32, double* part, CgState* st,
+__global__ void __launch_bounds__(kPhaseBlock) df_from_f64(const double* b, int64_t n, float* bh,
+                                                           float* bl, double* part, CgState* st,
                                                            double* b2) {
   using C = Cfg<float, K>;
   constexpr int VW = C::VW;
@@ -288,15 +287,13 @@ __global__ void __launch_bounds__(kPhaseBlock) df_from_f64(const double* b, doub
     Pack<float, VW> hh, ll;
 #pragma unroll
     for (int v = 0; v < VW; ++v) {
-      const double x = b[e * VW + v] * scale;
-      const float h = (float)x;
-      hh.v[v] = h;
-      ll.v[v] = (float)(x - (double)h);
-      acc[v] = __fmaf_rn(h, h, acc[v]);
+      const df x = split_f64(b[e * VW + v]);
+      hh.v[v] = x.hi;
+      ll.v[v] = x.lo;
+      acc[v] = __fmaf_rn(x.hi, x.hi, acc[v]);
     }
     stp<float, VW>(bh + e * VW, hh);
     stp<float, VW>(bl + e * VW, ll);
-    if (r32) stp<float, VW>(r32 + e * VW, hh);
   }
   if (!block_partials_last<float, K>(acc, part, &st->ticket)) return;
   sum_partials<K>(part, gridDim.x, s_tmp, s_out);

@@ -343,3 +343,22 @@ def test_every_one_sided_entry_is_found():
     for a, b in ((hubrow[3], hubcol[5]), (hubrow[0], hubrow[1]), (small[0], small[-1]), (hubcol[0], small[5])):
         if not (rows[a] == cols[b] and cols[a] == rows[b]):
             assert built((a, b)) == wl.WL_ERR_NOT_SYMMETRIC, (a, b)
+
+
+def test_right_hand_sides_outside_the_integer_split():
+    """Refined solves split their right-hand sides by integer instructions for
+    values from 2^-63 to 2^127, by conversions elsewhere: entries spread over 30
+    decades with both signs and zeros, values halfway between two FP32 ones,
+    against the FP64 form (at the refined form's parity tolerance)."""
+    g = wlgen.erdos_renyi(1500, 8.0, 2)
+    rng = np.random.default_rng(8)
+    V = rng.standard_normal((g.n, 4)) * 10.0 ** rng.uniform(-30, 0, (g.n, 4))
+    V[::7] = 0.0
+    V[1::7, 1] = np.float64(np.float32(V[1::7, 1])) * (1 + 2.0 ** -24)
+    V[3::7, 1] = np.nextafter(np.float32(2.0), np.float32(0)) * (1 + 2.0 ** -24.5)
+    out = []
+    for prec, tol in (("fp64", 1e-13), ("refined", 1e-12)):
+        w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=tol)
+        out.append(w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy())
+        w.close()
+    assert (np.abs(out[1] - out[0]).max(0) <= 1e-8 * np.abs(out[0]).max(0)).all()
