@@ -16,12 +16,30 @@
 //                                equally long
 // Elementwise phases walk the contiguous range, fully coalesced.
 #pragma once
+#include <atomic>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "wl.h"
 
 namespace wl {
+
+// Kernel attributes are kept per device: once(f) calls f until it has succeeded
+// on the current device
+struct PerDevice {
+  std::atomic<uint64_t> done{0};
+  template <typename F>
+  cudaError_t once(F f) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = f();
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 
 constexpr int kBlock = 256;        // threads per CTA of the persistent kernels
 #ifndef WL_MIN_BLOCKS

@@ -762,13 +762,14 @@ bool cgc_shape(const PhaseGraph& g, int64_t nnz, int sms, CoopShape* sh) {
 
 template <typename T, int K, bool SH>
 cudaError_t cgc_launch(CoopArgs<T> a, const CoopShape& sh, cudaStream_t s) {
-  static const cudaError_t attr = [] {
+  static PerDevice attr;
+  const cudaError_t ae = attr.once([] {
     cudaError_t e = cudaFuncSetAttribute(cg_coop<T, K, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)CoopCfg<T, K>::SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cg_coop<T, K, SH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
-  }();
-  if (attr != cudaSuccess) return attr;
+  });
+  if (ae != cudaSuccess) return ae;
   a.long_min = sh.long_min;
   a.nhead = sh.nhead;
   a.ch_log = sh.ch_log;

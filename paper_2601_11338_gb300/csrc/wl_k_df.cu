@@ -86,9 +86,12 @@ cudaError_t launch_df_lanczos_step(int K, const DfLanczosArgs& a, int G, cudaStr
 
 template <int K, int NT>
 static cudaError_t run_combine(const DfCombineArgs& a, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(df_combine<K, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCombSmemMax);
-  if (attr != cudaSuccess) return attr;
+  static PerDevice attr;
+  if (cudaError_t e = attr.once([] {
+        return cudaFuncSetAttribute(df_combine<K, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCombSmemMax);
+      });
+      e != cudaSuccess)
+    return e;
   const size_t per_col = (size_t)a.m * a.ntau * sizeof(float2);
   int CS = K;
   while (CS > 8 && per_col * CS > kCombSmem) CS /= 2;

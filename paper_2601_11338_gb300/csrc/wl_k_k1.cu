@@ -8,9 +8,12 @@ namespace wl {
 
 template <typename T, bool SH>
 static cudaError_t run_cg(CoopArgs<T> a, int64_t nnz, int sms, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(cg_k1<T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
-  if (attr != cudaSuccess) return attr;
+  static PerDevice attr;
+  if (cudaError_t e = attr.once([] {
+        return cudaFuncSetAttribute(cg_k1<T, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
+      });
+      e != cudaSuccess)
+    return e;
   const int grid = k1_grid(a.a.g.n, sms);
   a.nhead = k1_head<T>(a.a.g.n, nnz, grid);
   void* args[] = {&a};
@@ -27,9 +30,12 @@ template cudaError_t launch_cg_k1<double>(const CoopArgs<double>&, int64_t, int,
 
 template <bool SH>
 static cudaError_t run_res(const DfResArgs& a, int64_t nnz, int sms, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(df_res_k1<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
-  if (attr != cudaSuccess) return attr;
+  static PerDevice attr;
+  if (cudaError_t e = attr.once([] {
+        return cudaFuncSetAttribute(df_res_k1<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
+      });
+      e != cudaSuccess)
+    return e;
   const int grid = k1_grid(a.g.n, sms), nhead = k1_head<float>(a.g.n, nnz, grid);
   df_res_k1<SH><<<grid, k1_threads<float>(), k1_smem<float>(nhead), s>>>(a, nhead);
   return cudaGetLastError();

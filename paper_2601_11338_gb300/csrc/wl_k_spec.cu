@@ -46,12 +46,18 @@ static_assert(2 * (kSpStreamRows / 128 + 2 * kSpCoopCh) * 3 * sizeof(float2) <= 
 cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
                                  int check, double rtol, cudaStream_t s) {
   const bool stream = a.g.n > kSpStreamRows;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(sp_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpCoopSmem);
-  if (attr != cudaSuccess) return attr;
-  static const cudaError_t attr1 =
-      cudaFuncSetAttribute(sp_k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
-  if (attr1 != cudaSuccess) return attr1;
+  static PerDevice attr;
+  if (cudaError_t e = attr.once([] {
+        return cudaFuncSetAttribute(sp_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpCoopSmem);
+      });
+      e != cudaSuccess)
+    return e;
+  static PerDevice attr1;
+  if (cudaError_t e = attr1.once([] {
+        return cudaFuncSetAttribute(sp_k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kK1Smem);
+      });
+      e != cudaSuccess)
+    return e;
   SpCoopArgs ca{a, bar, 0, 0, cap, 0};
   int grid = k1_grid(a.g.n, sms), threads = k1_threads<float2>();
   ca.nhead = k1_head<float2>(a.g.n, nnz, grid);

@@ -104,13 +104,13 @@ cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, i
 }
 
 cudaError_t launch_nys_core(double* gram, int M, double* out, cudaStream_t s) {
-  const int smem = (2 * kMaxSketch * (kMaxSketch + 1) + 2 * kMaxSketch) * (int)sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(nys_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  constexpr int smem = (2 * kMaxSketch * (kMaxSketch + 1) + 2 * kMaxSketch) * (int)sizeof(double);
+  static PerDevice attr;
+  if (cudaError_t e = attr.once([] {
+        return cudaFuncSetAttribute(nys_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      });
+      e != cudaSuccess)
+    return e;
   nys_factor<<<1, kFactorThreads, smem, s>>>(gram, M, out);
   nys_core<<<M, kMaxSketch, 0, s>>>(gram, M, out);
   return cudaGetLastError();

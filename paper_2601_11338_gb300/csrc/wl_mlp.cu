@@ -747,14 +747,14 @@ __global__ void k_log_ratio(const double* __restrict__ Df, const double* __restr
 }
 
 cudaError_t mlp_setup() {
-  static const cudaError_t e = [] {
+  static PerDevice attr;
+  return attr.once([] {
     cudaError_t r = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(MlpGradSmem));
     if (r == cudaSuccess)
       r = cudaFuncSetAttribute(k_mlp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
     return r;
-  }();
-  return e;
+  });
 }
 
 // CTAs of a gradient pass: up to two per SM, each with at most kGradTiles tiles
