@@ -2725,7 +2725,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       double* part64 = (double*)h->gram.p;
       gout = part64 + gram_f64_partial_doubles(n, M);
       core = gout + 2 * kMaxSketch * kMaxSketch;
-      counted(h, 3);
+      counted(h, 4);
       e = launch_gram_f64(om_int, (const double*)h->packX.p, n, M, K, part64, gout, S(h));
       if (e == cudaSuccess) e = launch_nys_core(gout, M, core, S(h));
       if (e != cudaSuccess) { rc = set_cuda_error(e, "gram/core"); break; }
@@ -2761,7 +2761,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       break;
     }
     (void)sm;
-    counted(h, 3);
+    counted(h, 4);
     int* gerr = (int*)((double*)h->small.p + 1000);
     e = cudaMemsetAsync(gerr, 0, sizeof(int), S(h));
     if (e == cudaSuccess) e = launch_gram(om_int, (const float*)h->x.p, n, M, K, partial, Gg, gout, h->gram_tc, gerr, S(h));
@@ -2848,7 +2848,7 @@ int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt,
       if ((rc = outer_combine(h, o, t0, nb, Y, K, (int64_t)nk, 0, K, nullptr)) != WL_OK) break;
       for (int i = 0; i < nb; ++i) {
         // XNysTrace of exp(-t L) from Y(t) and Omega (Alg. 1, last step)
-        counted(h, 3);
+        counted(h, 4);
         e = cudaMemsetAsync(gerr, 0, sizeof(int), S(h));
         if (!sketch) {
           if (e == cudaSuccess)
