@@ -114,17 +114,10 @@ __device__ __forceinline__ Pack<T, VW> ld_last(const T* p) {
   return o;
 }
 
-// Gathers per lane in flight in row_gather: predicated batches of 8 (1)
-// measured 240 vs 252 us per K = 16 FP32 CG iteration against the unrolled
-// loop with a serial tail (0), and 236 us with the FP32 kernels at 5 CTAs per
-// SM (48 registers)
-#ifndef WL_GATHER_PRED
-#define WL_GATHER_PRED 1
-#endif
-#ifndef WL_GATHER_U
-#define WL_GATHER_U 8
-#endif
-// acc + sum of eight FP64 values, the values added as integers. GB300 adds two
+// Gathers per lane in flight in row_gather (unrolled batches of four with the tail
+// walked entry by entry: 252 us where these take 240, per K = 16 FP32 iteration)
+constexpr int kGatherU = 8;
+// acc + sum of N = 8 or 4 FP64 values, the values added as integers. GB300 adds two
 // FP64 lanes per clock and SM, so a neighbour sum of doubles is bound by its
 // additions; here each value costs about 15 integer instructions (64 lanes
 // per clock) instead, and a batch two FP64 ones. The values are aligned to the
@@ -132,27 +125,31 @@ __device__ __forceinline__ Pack<T, VW> ld_last(const T* p) {
 // there on (53 + 7 + 3 bits), rounded once at the end: the error is below 2^-4
 // units in the last place of the largest value plus that rounding, less than
 // that of eight FP64 additions in sequence. Chung-Lu 3e5, K = 16: 257 -> 198 us
-// an S phase (FP64 additions alone, four values in flight). Batches with non-finite or tiny
+// an S phase (FP64 additions alone, four values in flight), 159 -> 157 us with four
+// values summed so too where a row's last batch has no more (three FP64 additions
+// before; R-MAT scale 18, K = 8: 3% of a call). Batches with non-finite or tiny
 // values (exponent field below 64) are added in FP64.
-__device__ __forceinline__ double add8_aligned(double acc, const double (&v)[8]) {
+template <int N>
+__device__ __forceinline__ double add_aligned(double acc, const double (&v)[N]) {
+  static_assert(N <= 8, "three bits of headroom");
   int m = 0;
 #pragma unroll
-  for (int u = 0; u < 8; ++u) m = max(m, __double2hiint(v[u]) & 0x7fffffff);
+  for (int u = 0; u < N; ++u) m = max(m, __double2hiint(v[u]) & 0x7fffffff);
   const int em = m >> 20;
   if (em < 64 || em == 0x7ff) {
     int any = 0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) any |= (__double2hiint(v[u]) & 0x7fffffff) | __double2loint(v[u]);
+    for (int u = 0; u < N; ++u) any |= (__double2hiint(v[u]) & 0x7fffffff) | __double2loint(v[u]);
     if (any != 0) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc += v[u];
+      for (int u = 0; u < N; ++u) acc += v[u];
     }
     return acc;
   }
   unsigned long long sum = 0;
   int neg = 0;
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
+  for (int u = 0; u < N; ++u) {
     const int hi = __double2hiint(v[u]), e = (hi & 0x7fffffff) >> 20, s = hi >> 31;
     unsigned long long x = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 |
                             (unsigned)__double2loint(v[u])) << 7;
@@ -165,18 +162,15 @@ __device__ __forceinline__ double add8_aligned(double acc, const double (&v)[8])
   return fma((double)total, __hiloint2double((em - 59) << 20, 0), acc);
 }
 
-// Sum of X over entries [beg, end) with stride `step`.
-// WL_GATHER_PRED = 1: every batch of WL_GATHER_U entries, the last one too,
-// issues its index loads and then its gathers together (predicated on the
-// row end), so a short row costs one index latency and one gather latency
-// per batch instead of a dependent pair per entry of its tail. (0: batches of
-// four with the tail walked entry by entry.)
+// Sum of X over entries [beg, end) with stride `step`. Every batch of kGatherU
+// entries, the last one too, issues its index loads and then its gathers
+// together (predicated on the row end), so a short row costs one index latency
+// and one gather latency per batch instead of a dependent pair per entry of its
+// tail.
 template <typename T, int K, int VW>
 __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int beg, int end, int step,
                                            const T* X, int lane_off, T (&acc)[VW]) {
-  if constexpr (sizeof(T) == 8 || WL_GATHER_PRED) {
-  constexpr bool kInt = sizeof(T) == 8;
-  constexpr int U = kInt ? 8 : WL_GATHER_U;
+  constexpr int U = kGatherU;
   for (int e = beg; e < end; e += U * step) {
     int j[U];
 #pragma unroll
@@ -191,20 +185,19 @@ __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int 
         for (int v = 0; v < VW; ++v) a[u].v[v] = T(0);
       }
     }
-    if constexpr (kInt) {
-      if (end - e > 3 * step) {
+    if constexpr (sizeof(T) == 8) {
+      if (end - e > 4 * step) {
 #pragma unroll
         for (int v = 0; v < VW; ++v) {
-          double x[8];
-#pragma unroll
-          for (int u = 0; u < U; ++u) x[u] = a[u].v[v];
-          acc[v] = add8_aligned(acc[v], x);
+          const double x[8] = {a[0].v[v], a[1].v[v], a[2].v[v], a[3].v[v], a[4].v[v], a[5].v[v], a[6].v[v], a[7].v[v]};
+          acc[v] = add_aligned<8>(acc[v], x);
         }
-      } else {  // up to three values: fewer FP64 additions than the integer sum costs
+      } else {
 #pragma unroll
-        for (int u = 0; u < 3; ++u)
-#pragma unroll
-          for (int v = 0; v < VW; ++v) acc[v] += a[u].v[v];
+        for (int v = 0; v < VW; ++v) {
+          const double x[4] = {a[0].v[v], a[1].v[v], a[2].v[v], a[3].v[v]};
+          acc[v] = add_aligned<4>(acc[v], x);
+        }
       }
     } else {
 #pragma unroll
@@ -212,24 +205,6 @@ __device__ __forceinline__ void row_gather(const int32_t* __restrict__ col, int 
 #pragma unroll
         for (int v = 0; v < VW; ++v) acc[v] += a[u].v[v];
     }
-  }
-  return;
-  }
-  int e = beg;
-  for (; e + 3 * step < end; e += 4 * step) {
-    const int j0 = __ldg(col + e), j1 = __ldg(col + e + step);
-    const int j2 = __ldg(col + e + 2 * step), j3 = __ldg(col + e + 3 * step);
-    const Pack<T, VW> a0 = ld_plain<T, VW>(X + (size_t)j0 * K + lane_off);
-    const Pack<T, VW> a1 = ld_plain<T, VW>(X + (size_t)j1 * K + lane_off);
-    const Pack<T, VW> a2 = ld_plain<T, VW>(X + (size_t)j2 * K + lane_off);
-    const Pack<T, VW> a3 = ld_plain<T, VW>(X + (size_t)j3 * K + lane_off);
-#pragma unroll
-    for (int v = 0; v < VW; ++v) acc[v] += (a0.v[v] + a1.v[v]) + (a2.v[v] + a3.v[v]);
-  }
-  for (; e < end; e += step) {
-    const Pack<T, VW> a0 = ld_plain<T, VW>(X + (size_t)__ldg(col + e) * K + lane_off);
-#pragma unroll
-    for (int v = 0; v < VW; ++v) acc[v] += a0.v[v];
   }
 }
 

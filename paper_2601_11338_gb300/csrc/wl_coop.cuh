@@ -160,19 +160,22 @@ __device__ __forceinline__ void coop_gather(const int32_t* col, int (&beg)[N], c
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       if constexpr (sizeof(T) == 8 && U == 8) {
-        if (end[i] - beg[i] > 3 * step) {
+        if (end[i] - beg[i] > 4 * step) {
 #pragma unroll
           for (int w = 0; w < VW; ++w) {
             double x[8];
 #pragma unroll
-            for (int u = 0; u < U; ++u) x[u] = v[i][u].v[w];
-            acc[i][w] = add8_aligned(acc[i][w], x);
+            for (int u = 0; u < 8; ++u) x[u] = v[i][u].v[w];
+            acc[i][w] = add_aligned<8>(acc[i][w], x);
           }
         } else {
 #pragma unroll
-          for (int u = 0; u < 3; ++u)
+          for (int w = 0; w < VW; ++w) {
+            double x[4];
 #pragma unroll
-            for (int w = 0; w < VW; ++w) acc[i][w] += v[i][u].v[w];
+            for (int u = 0; u < 4; ++u) x[u] = v[i][u].v[w];
+            acc[i][w] = add_aligned<4>(acc[i][w], x);
+          }
         }
       } else {
 #pragma unroll

@@ -47,8 +47,7 @@ template <int K, int VW, bool FULL>
 __device__ __forceinline__ void df_row_gather(const int32_t* __restrict__ col, int beg, int end, int step,
                                               const float* YH, const float* YL, int lane_off, float (&s)[VW],
                                               float (&c)[VW], float (&l)[VW]) {
-#if WL_GATHER_PRED
-  constexpr int U = WL_GATHER_U;  // predicated batches, as in row_gather
+  constexpr int U = kGatherU;  // predicated batches, as in row_gather
   for (int e = beg; e < end; e += U * step) {
     int j[U];
 #pragma unroll
@@ -76,43 +75,6 @@ __device__ __forceinline__ void df_row_gather(const int32_t* __restrict__ col, i
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int v = 0; v < VW; ++v) df_acc(s[v], c[v], hh[u].v[v]);
-  }
-  return;
-#endif
-  int e = beg;
-  for (; e + 3 * step < end; e += 4 * step) {
-    const int j0 = __ldg(col + e), j1 = __ldg(col + e + step);
-    const int j2 = __ldg(col + e + 2 * step), j3 = __ldg(col + e + 3 * step);
-    const Pack<float, VW> h0 = ld_plain<float, VW>(YH + (size_t)j0 * K + lane_off);
-    const Pack<float, VW> h1 = ld_plain<float, VW>(YH + (size_t)j1 * K + lane_off);
-    const Pack<float, VW> h2 = ld_plain<float, VW>(YH + (size_t)j2 * K + lane_off);
-    const Pack<float, VW> h3 = ld_plain<float, VW>(YH + (size_t)j3 * K + lane_off);
-    if constexpr (FULL) {
-      const Pack<float, VW> l0 = ld_plain<float, VW>(YL + (size_t)j0 * K + lane_off);
-      const Pack<float, VW> l1 = ld_plain<float, VW>(YL + (size_t)j1 * K + lane_off);
-      const Pack<float, VW> l2 = ld_plain<float, VW>(YL + (size_t)j2 * K + lane_off);
-      const Pack<float, VW> l3 = ld_plain<float, VW>(YL + (size_t)j3 * K + lane_off);
-#pragma unroll
-      for (int v = 0; v < VW; ++v) l[v] += (l0.v[v] + l1.v[v]) + (l2.v[v] + l3.v[v]);
-    }
-#pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      df_acc(s[v], c[v], h0.v[v]);
-      df_acc(s[v], c[v], h1.v[v]);
-      df_acc(s[v], c[v], h2.v[v]);
-      df_acc(s[v], c[v], h3.v[v]);
-    }
-  }
-  for (; e < end; e += step) {
-    const int j0 = __ldg(col + e);
-    const Pack<float, VW> h0 = ld_plain<float, VW>(YH + (size_t)j0 * K + lane_off);
-    if constexpr (FULL) {
-      const Pack<float, VW> l0 = ld_plain<float, VW>(YL + (size_t)j0 * K + lane_off);
-#pragma unroll
-      for (int v = 0; v < VW; ++v) l[v] += l0.v[v];
-    }
-#pragma unroll
-    for (int v = 0; v < VW; ++v) df_acc(s[v], c[v], h0.v[v]);
   }
 }
 
