@@ -414,6 +414,12 @@ struct wl_handle {
   Buf mid;                // rows with kSpWarpDeg < deg <= kHubDeg (a warp each in the spectral Lanczos)
   int nmid = 0, nmid_blk = 0;
   double mid_share = 0.0; // share of the S kernels' CTAs that walk the mid rows
+  double e_low = 0.0;     // entries of the other (short) rows
+  // the same for the solves by phase kernels (phase_lists)
+  Buf hubs2, mid2;        // rows with more than kPhaseHubDeg entries; rows between the short ones and these
+  int nhub2 = 0, nmid2 = 0;
+  double mid_share2 = 0.0;
+  bool have_lists2 = false;
   double sp_c0 = 0.0, sp_cD = 0.0, sp_theta = 0.0;  // operator and Ritz value of the basis held in spV
   bool sp_ritz_ready = false;                        // W[1] holds that run's Ritz vector
   double sp_ritz_uu = 0.0, sp_ritz_udu = 0.0;        // its |u|^2 and u^T D u
@@ -579,6 +585,61 @@ PhaseGraph phase_graph_mid(wl_handle* h, int grid_u) {
     g.mids = (const int32_t*)h->mid.p;
     g.nmid = h->nmid;
     g.nmid_blk = (int)std::min<long>(grid_u - 1, std::max<long>(1, std::lround(h->mid_share * grid_u)));
+  }
+  return g;
+}
+
+// Rows with more entries than this get a CTA each in the phase kernels of a solve
+// (S and the double-float residual); from kMidDeg up to it a warp each. A CTA per
+// row of more than kHubDeg took its launch, its partial sums and a few waits for
+// little work: S of Chung-Lu 1e6 x 16 134 -> 114 us (2048: 127), of R-MAT scale
+// 17 x 64 165 -> 118 us (2048: 105), of Chung-Lu 3e5 x 16 doubles 157 -> 144 us.
+constexpr int kPhaseHubDeg = 1024;
+
+// weight of m rows with e entries that take a warp each, and of short rows: a
+// warp takes about 32 entries per round on either path, but a mid row pays the
+// fixed cost of a row (pointers, own-row vectors, finish: ~3 rounds) for a
+// whole warp, a short row for a lane group (1/8 of a warp at K = 16 FP32)
+double warp_rows_share(double e_mid, double n_mid, double e_low, double n_low) {
+  const double w_mid = e_mid / 32.0 + 3.0 * n_mid, w_low = e_low / 32.0 + 0.375 * n_low;
+  return w_mid / std::max(w_mid + w_low, 1e-300);
+}
+
+// Builds the lists on a handle's first such solve; without hub rows the others serve.
+int phase_lists(wl_handle* h) {
+  if (h->have_lists2 || h->nhub == 0) return WL_OK;
+  WL_TRY(ensure(h->hubs2, sizeof(int32_t) * (size_t)h->n));
+  WL_TRY(ensure(h->mid2, sizeof(int32_t) * (size_t)h->n));
+  WL_TRY(ensure(h->ptmp, sizeof(int64_t) * (3 * (size_t)(h->n + 1) + h->n / 1024 + 8)));
+  int64_t* cnt = (int64_t*)h->h_pin;
+  unsigned long long* dsum = (unsigned long long*)((double*)h->small.p + 900);
+  counted(h, 11);
+  WL_CU(launch_row_list(h->g.row_ptr, h->n, kPhaseHubDeg, INT32_MAX, (int32_t*)h->hubs2.p, (int64_t*)h->ptmp.p, cnt, S(h)));
+  WL_CU(launch_row_list(h->g.row_ptr, h->n, kMidDeg, kPhaseHubDeg, (int32_t*)h->mid2.p, (int64_t*)h->ptmp.p, cnt + 1, S(h)));
+  WL_CU(cudaStreamSynchronize(S(h)));
+  h->nhub2 = (int)cnt[0];
+  h->nmid2 = (int)cnt[1];
+  WL_CU(launch_list_entries(h->g.row_ptr, (const int32_t*)h->hubs2.p, h->nhub2, dsum, S(h)));
+  WL_CU(cudaMemcpyAsync(cnt, dsum, 8, cudaMemcpyDeviceToHost, S(h)));
+  WL_CU(cudaStreamSynchronize(S(h)));
+  h->mid_share2 = warp_rows_share((double)h->nnz - h->e_low - (double)cnt[0], h->nmid2, h->e_low,
+                                  (double)(h->n - h->nhub2 - h->nmid2));
+  h->have_lists2 = true;
+  return WL_OK;
+}
+
+int phase_hubs(const wl_handle* h) { return h->have_lists2 ? h->nhub2 : h->nhub; }
+
+// the graph as seen by a phase kernel of grid_u CTAs plus phase_hubs
+PhaseGraph phase_graph_wide(wl_handle* h, int grid_u) {
+  if (!h->have_lists2) return phase_graph_mid(h, grid_u);
+  PhaseGraph g = phase_graph(h);
+  g.hubs = (const int32_t*)h->hubs2.p;
+  g.nhub = h->nhub2;
+  if (h->nmid2 > 0) {
+    g.mids = (const int32_t*)h->mid2.p;
+    g.nmid = h->nmid2;
+    g.nmid_blk = (int)std::min<long>(grid_u - 1, std::max<long>(1, std::lround(h->mid_share2 * grid_u)));
   }
   return g;
 }
@@ -805,13 +866,13 @@ int ensure_phase_buffers(wl_handle* h, int grid) {
 // x holds the starting guess on entry, or, x_is_zero, nothing yet.
 int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool x_is_zero, SolveInfo& info) {
   NvtxRange nvtx__("fp64 solve");
-  const int grid_u = phase_grid(h, phase_blocks_f64(K), K, 8), grid_s = grid_u + h->nhub;
+  const int grid_u = phase_grid(h, phase_blocks_f64(K), K, 8);
   const int grid_w = phase_grid(h, res_blocks(K), K, 8) + h->nhub;
   const size_t nk = (size_t)h->n * K;
   WL_TRY(ensure(h->r, nk * 8));
   WL_TRY(ensure(h->p, nk * 8));
   WL_TRY(ensure(h->q, nk * 8));
-  WL_TRY(ensure_phase_buffers(h, std::max({grid_s, grid_w, h->sms})));
+  WL_TRY(ensure_phase_buffers(h, std::max({grid_u + h->nhub, grid_w, h->sms})));
   CgState* st = h->cgst();
   WL_CU(cudaMemsetAsync(st, 0, sizeof(CgBlock), S(h)));  // the cooperative kernel's barrier too
   h->bar_clean = true;
@@ -839,7 +900,11 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
       cg_outcome(h, K, 8, info);
       h->r_fin = (const double*)h->r.p;
     } else {
-      WL_TRY(run_cg<double>(h, K, a, start, grid_s, grid_u, info, &h->r_fin));
+      if (grid_u > 1) {
+        WL_TRY(phase_lists(h));
+        a.g = phase_graph_wide(h, grid_u);
+      }
+      WL_TRY(run_cg<double>(h, K, a, start, grid_u + a.g.nhub, grid_u, info, &h->r_fin));
     }
   }
   info.max_rel = std::max(info.max_rel, info.last_rel);
@@ -855,15 +920,15 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
 int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const double* bn2, float* xh, float* xl,
                      const double* x0, int K, double tol, SolveInfo& info) {
   NvtxRange nvtx__("refined solve");
-  const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4), grid_s = grid_u + h->nhub;
-  const int grid_r = phase_grid(h, df_res_blocks(K), K, 4) + h->nhub;
+  const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4);
+  const int grid_r = phase_grid(h, df_res_blocks(K), K, 4);
   const size_t nk = (size_t)h->n * K;
   WL_TRY(ensure(h->p, nk * 4));
   WL_TRY(ensure(h->q, nk * 4));
   WL_TRY(ensure(h->d32, nk * 4));
   WL_TRY(ensure(h->rh, nk * 4));
   WL_TRY(ensure(h->rl, nk * 4));
-  WL_TRY(ensure_phase_buffers(h, std::max({grid_s, grid_r, h->sms})));
+  WL_TRY(ensure_phase_buffers(h, std::max({grid_u + h->nhub, grid_r + h->nhub, h->sms})));
   CgState* st = h->cgst();
   float* rh = (float*)h->rh.p;
   float* rl = (float*)h->rl.p;
@@ -881,9 +946,15 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // and writes d whole, and the residual that follows it keeps its norms in a
   // state of its own. Small solves run the correction as one cooperative kernel:
   // both are launched before one wait for their outcome.
-  const PhaseGraph pg = phase_graph_mid(h, grid_u);
+  PhaseGraph pg = phase_graph_mid(h, grid_u);
   const bool coop = (K == 1 && h->n > k1_rows<float>()) || cg_coop_fits_f32(K, pg, h->nnz, h->sms);
   if (coop) WL_TRY(ensure(h->r32, nk * 4));
+  const bool wide = !coop && grid_u > 1 && grid_r > 1;
+  if (wide) {
+    WL_TRY(phase_lists(h));
+    pg = phase_graph_wide(h, grid_u);
+  }
+  const PhaseGraph rg = wide ? phase_graph_wide(h, grid_r) : phase_graph_mid(h, grid_r);
   PhaseArgs<float> a{pg, dcur, (float*)h->r32.p, (float*)h->r32.p, (float*)h->p.p, (float*)h->q.p,
                      h->ca, h->cA, h->cD, nullptr, dskip, (double*)h->part.p, st, h->prm.max_iter, 0.0};
   a.dshift = h->si_dsh_h;
@@ -892,12 +963,12 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     // r = B - M x0 (x0 split into two FP32 terms and gathered whole)
     counted(h, 2);
     WL_CU(launch_split_x(x0, (int64_t)nk, xh, xl, false, nullptr, S(h)));
-    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), xh, xl, bh, bl, rh, rl, nullptr, nullptr,
+    DfResArgs ra{rg, xh, xl, bh, bl, rh, rl, nullptr, nullptr,
                  ca, cA, cD, (double*)h->part.p, rst, 0};
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
     const int pi = prof_begin(h, kCatRes);
-    WL_CU(launch_df_res(K, ra, grid_r, true, S(h)));
+    WL_CU(launch_df_res(K, ra, grid_r + rg.nhub, true, S(h)));
     prof_end(h, pi);
     info.nnz_rhs += (double)h->nnz * K;
     rch = rh;
@@ -962,7 +1033,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
       // sizes its first launch chunk from the previous solve of its kind
       int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
       h->cg_hint = hint;
-      WL_TRY(run_cg<float>(h, K, a, start, grid_s, grid_u, inner));
+      WL_TRY(run_cg<float>(h, K, a, start, grid_u + pg.nhub, grid_u, inner));
       hint = h->cg_hint;
       if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
         info.status = inner.status;
@@ -972,12 +1043,12 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     // r <- r - M d, x <- x + d
     WL_CU(cudaMemsetAsync(rst, 0, sizeof(CgState) + sizeof(CoopBar), S(h)));
     h->bar_clean = true;
-    DfResArgs ra{phase_graph_mid(h, grid_r - h->nhub), dcur, nullptr, rch, rcl, rh, rl, xh, xl,
+    DfResArgs ra{rg, dcur, nullptr, rch, rcl, rh, rl, xh, xl,
                  ca, cA, cD, (double*)h->part.p, rst, x_zero ? 1 : 0};
     ra.dsh_h = h->si_dsh_h;
     ra.dsh_l = h->si_dsh_l;
     const int pi = prof_begin(h, kCatRes);
-    WL_CU(K == 1 && h->n > kResK1Rows ? launch_df_res_k1(ra, h->nnz, h->sms, S(h)) : launch_df_res(K, ra, grid_r, false, S(h)));
+    WL_CU(K == 1 && h->n > kResK1Rows ? launch_df_res_k1(ra, h->nnz, h->sms, S(h)) : launch_df_res(K, ra, grid_r + rg.nhub, false, S(h)));
     prof_end(h, pi);
     hgamma = nullptr;
     if (coop) {
@@ -2049,7 +2120,7 @@ void free_handle(wl_handle* h) {
   }
   Buf* bufs[] = {&h->csr_rp, &h->csr_col, &h->x, &h->r, &h->p, &h->q, &h->b64, &h->d32,
                  &h->r32, &h->xh, &h->xl, &h->hist, &h->bh, &h->bl, &h->rh, &h->rl, &h->dfdf, &h->ydf, &h->ew, &h->taus, &h->ybig, &h->part, &h->small, &h->Df, &h->warm, &h->basis, &h->Tab, &h->ybuf, &h->yprev,
-                 &h->errb, &h->stage_a, &h->stage_b, &h->packV, &h->packX, &h->spV, &h->spW, &h->spstate, &h->mid, &h->omega, &h->gram,
+                 &h->errb, &h->stage_a, &h->stage_b, &h->packV, &h->packX, &h->spV, &h->spW, &h->spstate, &h->mid, &h->hubs2, &h->mid2, &h->omega, &h->gram,
                  &h->omega_int, &h->ptmp, &h->perm_b, &h->iperm_b, &h->hubs, &h->cgstate};
   for (Buf* b : bufs) release(*b);
   for (void* p : h->retired) pool_free(p);
@@ -2251,12 +2322,8 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
     if (e != cudaSuccess) return fail(set_cuda_error(e, "mid-row list"));
     h->nmid = (int)*(int64_t*)h->h_pin;
     h->nmid_blk = h->nmid > 0 ? (int)std::min<int64_t>((h->nmid + 31) / 32, 2 * 152) : 0;
-    // share of the S kernels' CTAs for the mid rows: a warp takes about 32
-    // entries per round on either path, but a mid row pays the fixed cost of
-    // a row (pointers, own-row vectors, finish: ~3 rounds) for a whole warp,
-    // a short row for a lane group (1/8 of a warp at K = 16 FP32)
     h->mid_share = 0.0;
-    if (h->nmid > 0) {
+    if (h->nmid > 0 || h->nhub > 0) {
       unsigned long long* cnt = (unsigned long long*)h->h_pin;
       unsigned long long* dsum = (unsigned long long*)((double*)h->small.p + 900);
       double ent[2];
@@ -2270,10 +2337,8 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
         ent[li] = (double)*cnt;
       }
       counted(h, 4);
-      const double e_mid = ent[0], e_low = (double)h->nnz - ent[0] - ent[1];
-      const double n_low = (double)(h->n - h->nhub - h->nmid);
-      const double w_mid = e_mid / 32.0 + 3.0 * h->nmid, w_low = e_low / 32.0 + 0.375 * n_low;
-      h->mid_share = w_mid / std::max(w_mid + w_low, 1e-300);
+      h->e_low = (double)h->nnz - ent[0] - ent[1];
+      h->mid_share = warp_rows_share(ent[0], h->nmid, h->e_low, (double)(h->n - h->nhub - h->nmid));
     }
   }
 
@@ -2744,8 +2809,8 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
     if (e == cudaSuccess) e = launch_sketch_rhs(om_int, n, M, K, h->a_scale, (float*)h->r32.p, S(h));
     if (e != cudaSuccess) { rc = set_cuda_error(e, "sketch"); break; }
     // Y = M^{-1} (a Omega) in FP32 lockstep CG
-    const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4), grid_s = grid_u + h->nhub;
-    if ((rc = ensure_phase_buffers(h, std::max(grid_s, h->sms))) != WL_OK) break;
+    const int grid_u = phase_grid(h, phase_blocks_f32(K), K, 4);
+    if ((rc = ensure_phase_buffers(h, std::max(grid_u + h->nhub, h->sms))) != WL_OK) break;
     Smalls sm = smalls(h);
     CgState* st = h->cgst();
     WL_CU(cudaMemsetAsync(st, 0, sizeof(CgState), S(h)));
@@ -2757,8 +2822,12 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
       if (e != cudaSuccess) { rc = set_cuda_error(e, "cooperative CG"); break; }
       if ((rc = cg_block_to_host(h)) != WL_OK) break;
       cg_outcome(h, K, 4, info);
-    } else if ((rc = run_cg<float>(h, K, a, CgStart<float>{}, grid_s, grid_u, info)) != WL_OK) {
-      break;
+    } else {
+      if (grid_u > 1) {
+        if ((rc = phase_lists(h)) != WL_OK) break;
+        a.g = phase_graph_wide(h, grid_u);
+      }
+      if ((rc = run_cg<float>(h, K, a, CgStart<float>{}, grid_u + a.g.nhub, grid_u, info)) != WL_OK) break;
     }
     (void)sm;
     counted(h, 4);

@@ -362,3 +362,30 @@ def test_right_hand_sides_outside_the_integer_split():
         out.append(w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy())
         w.close()
     assert (np.abs(out[1] - out[0]).max(0) <= 1e-8 * np.abs(out[0]).max(0)).all()
+
+
+# Phase kernels with rows on both sides of every way a row is taken (a lane
+# group up to 30 entries, a warp up to 1024, a CTA beyond), and with no row between
+# 31 and 1024, against scipy's FP64 CG
+@pytest.mark.parametrize("degs", [{7: 31, 99: 256, 1000: 257, 70000: 1024, 150001: 1025, 220000: 5000},
+                                  {3: 1500, 219999: 3000}])
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)])
+def test_long_rows_of_the_phase_kernels(prec, tol, bound, degs):
+    from oracle import krylov
+    n = 220001
+    e = wlgen.erdos_renyi(n, 4.0, 8)
+    src = np.repeat(np.arange(n), e.degrees)
+    rng = np.random.default_rng(6)
+    hs = np.concatenate([np.full(d, v) for v, d in degs.items()])
+    hd = np.concatenate([rng.choice(n, d, replace=False) for d in degs.values()])
+    keep = hs != hd
+    g = wlgen.csr_from_edges(n, np.concatenate([src, hs[keep]]), np.concatenate([e.col_idx, hd[keep]]))
+    A = krylov.adjacency(g.row_ptr, g.col_idx, g.n)
+    w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=tol)
+    L = krylov.ResolventLaplacian(A, 1.0, w.info["alpha"], tol=1e-14)
+    for k in (8, 16, 64):
+        V = np.random.default_rng(k).standard_normal((n, k))
+        W = w.apply(torch.as_tensor(V, device="cuda")).cpu().numpy()
+        want = L.apply(V[:, :2])
+        assert np.abs(W[:, :2] - want).max() <= bound * np.abs(want).max(), k
+    w.close()
