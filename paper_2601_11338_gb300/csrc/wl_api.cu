@@ -592,9 +592,10 @@ PhaseGraph phase_graph_mid(wl_handle* h, int grid_u) {
 // Rows with more entries than this get a CTA each in the phase kernels of a solve
 // (S and the double-float residual); from kMidDeg up to it a warp each. A CTA per
 // row of more than kHubDeg took its launch, its partial sums and a few waits for
-// little work: S of Chung-Lu 1e6 x 16 134 -> 114 us (2048: 127), of R-MAT scale
-// 17 x 64 165 -> 118 us (2048: 105), of Chung-Lu 3e5 x 16 doubles 157 -> 144 us.
-constexpr int kPhaseHubDeg = 1024;
+// little work: S of Chung-Lu 1e6 x 16 134 -> 116 us (600: 118, 1024: 115, 2048: 127),
+// of R-MAT scale 17 x 64 165 -> 102 us (600: 118, 1024: 119, 2048: 105), of Chung-Lu
+// 3e5 x 16 doubles 157 -> 144 us (the same at the others).
+constexpr int kPhaseHubDeg = 1400;
 
 // weight of m rows with e entries that take a warp each, and of short rows: a
 // warp takes about 32 entries per round on either path, but a mid row pays the

@@ -331,8 +331,8 @@ __device__ __forceinline__ void sum_partials(const double* part, int nblk, doubl
 // 448). Chung-Lu 1e6 x 16, shifted: S 165 -> 134 us, and 85 us per solve of nine
 // iterations for x; what is left is the gathers, 24e6 sectors from L2 and L1.
 // 3e5 x 16 doubles: 198 -> 159 us; R-MAT scale 17 x 64 floats: 176 -> 162 us. (With
-// a CTA per row of more than 256 entries; with rows of up to 1024 by a warp each
-// the three take 114, 144 and 118 us.)
+// a CTA per row of more than 256 entries; with rows of up to 1400 by a warp each
+// the three take 116, 144 and 102 us.)
 // delta is (r, q) then, which is (p, q) as q = M p and p_{j-1} is M-orthogonal
 // to p_j: in FP32 simulations the same iterations (to one) up to condition 1e5.
 template <typename T, int K, bool SH = false, bool X = false>

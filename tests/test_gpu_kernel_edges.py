@@ -365,9 +365,9 @@ def test_right_hand_sides_outside_the_integer_split():
 
 
 # Phase kernels with rows on both sides of every way a row is taken (a lane
-# group up to 30 entries, a warp up to 1024, a CTA beyond), and with no row between
-# 31 and 1024, against scipy's FP64 CG
-@pytest.mark.parametrize("degs", [{7: 31, 99: 256, 1000: 257, 70000: 1024, 150001: 1025, 220000: 5000},
+# group up to 30 entries, a warp up to 1400, a CTA beyond), and with no row between
+# 31 and 1400, against scipy's FP64 CG
+@pytest.mark.parametrize("degs", [{7: 31, 99: 256, 1000: 257, 70000: 1400, 150001: 1401, 220000: 5000},
                                   {3: 1500, 219999: 3000}])
 @pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("refined", 1e-12, 1e-8)])
 def test_long_rows_of_the_phase_kernels(prec, tol, bound, degs):
