@@ -705,10 +705,20 @@ template <typename T>
 constexpr int64_t k1_rows() { return sizeof(T) == 4 ? 500000 : 600000; }
 constexpr int64_t kResK1Rows = 250000;
 
+// Two FP64 columns of more rows take the phase kernels though they would fit: a
+// CTA's 512 threads of the cooperative kernel hide the gathers worse (3e5 rows,
+// Erdos-Renyi 1680 -> 958 us a call, 4e5, Chung-Lu 2065 -> 1173, 5.2e5, R-MAT 3016 ->
+// 1961; but 564 -> 743 us at 6e4 rows and 744 -> 875 us at 1e5).
+constexpr int64_t kCoopF64K2Rows = 150000;
+
 // Launches a solve as one cooperative kernel; false where its vectors don't
 // fit in shared memory (nothing launched).
 template <typename T>
 bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& start, cudaError_t* e) {
+  if (sizeof(T) == 8 && K == 2 && h->n > kCoopF64K2Rows) return false;
+  // one FP64 column without long rows: no hubs to keep in shared memory (1e6 rows,
+  // Erdos-Renyi 2166 -> 1281 us a call, Chung-Lu 2226 -> 1776)
+  if (sizeof(T) == 8 && K == 1 && h->n > k1_rows<T>() && 2.0 * h->e_low > (double)h->nnz) return false;
   CoopArgs<T> co{a, h->cgbar(), start.r0 ? start.r0 : a.rn, start.gamma0, start.add_x ? 1 : 0};
   if (!h->bar_clean) {
     *e = cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h));
@@ -2324,6 +2334,7 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
     h->nmid = (int)*(int64_t*)h->h_pin;
     h->nmid_blk = h->nmid > 0 ? (int)std::min<int64_t>((h->nmid + 31) / 32, 2 * 152) : 0;
     h->mid_share = 0.0;
+    h->e_low = (double)h->nnz;
     if (h->nmid > 0 || h->nhub > 0) {
       unsigned long long* cnt = (unsigned long long*)h->h_pin;
       unsigned long long* dsum = (unsigned long long*)((double*)h->small.p + 900);

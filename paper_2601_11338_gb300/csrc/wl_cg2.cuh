@@ -476,8 +476,9 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase
     const int nlist = a.g.nhub + a.g.nmid_blk;
     const int lim = a.g.nmid_blk > 0 ? kMidDeg : kHubDeg;  // longer rows: hub CTAs or mid warps
     const int64_t nblk = (int64_t)gridDim.x - nlist;
-    // E lane groups per row where a row has few lanes (K <= 2)
-    constexpr int E = G >= 4 ? 1 : 4 / G, LPR = G * E, RPP = kPhaseBlock / LPR;
+    // E lane groups per row where a row has few lanes (K <= 2); not in FP64, where a
+    // warp's operations of the row's end cost the same for eight rows as for 32
+    constexpr int E = G >= 4 || sizeof(T) == 8 ? 1 : 4 / G, LPR = G * E, RPP = kPhaseBlock / LPR;
     const int e = (tid / G) % E;
     for (int64_t row = ((int64_t)blockIdx.x - nlist) * RPP + tid / LPR; row < a.g.n; row += nblk * RPP) {
       const int beg = a.g.row_ptr[row], end = a.g.row_ptr[row + 1];
