@@ -50,7 +50,9 @@ constexpr int kMinBlocks = WL_MIN_BLOCKS;  // CTAs per SM the register budget is
 #define WL_BATCH_ENTRIES 16  // neighbour entries per subgroup batch (gathers in flight per lane)
 #endif
 constexpr int kRowCost = 2;        // partition cost of a row beyond its entries
-constexpr uint64_t kWaitLimitNs = 2000000000ull;  // every device-side wait gives up after 2 s
+// every device-side spin wait gives up after 2 s (a cluster's hardware barrier is
+// no such wait: its CTAs are resident together, like the warps at __syncthreads)
+constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 // ------------------------------------------------------------------ grid barrier
 // Sense counter + generation word in global memory. Used only by kernels

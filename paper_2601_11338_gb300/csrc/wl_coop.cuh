@@ -189,8 +189,12 @@ __device__ __forceinline__ void coop_gather(const int32_t* col, int (&beg)[N], c
   }
 }
 
+// All threads of the cluster. Without .aligned: that form wants every warp
+// converged, and the callers' branches (four lanes a column, tid < K) leave
+// that to the compiler. The wait ends whatever the other CTAs do: a cluster's
+// CTAs start together, and a CTA that has exited counts as arrived.
 __device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // 8 bytes at the same shared-memory place of CTA `rank` of the cluster
