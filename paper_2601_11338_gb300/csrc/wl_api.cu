@@ -82,9 +82,11 @@ void retire(void* p) {
 //   timeout  every grid barrier starts in the gave-up state, so the
 //            cooperative kernels leave at their first barrier (WL_ERR_TIMEOUT)
 //   noconv   every CG solve is capped at one iteration (WL_ERR_NO_CONVERGENCE)
+//   nocluster  the device is taken to place no thread-block clusters: small
+//            solves run as grids (no error)
 // Nothing here faults, traps or hangs the GPU; each failure goes through the
 // library's normal status paths.
-enum FaultMode { kFaultNone = 0, kFaultAlloc, kFaultNan, kFaultTimeout, kFaultNoconv };
+enum FaultMode { kFaultNone = 0, kFaultAlloc, kFaultNan, kFaultTimeout, kFaultNoconv, kFaultNoCluster };
 
 int fault_mode() {
   const char* s = getenv("WL_FAULT");
@@ -93,8 +95,11 @@ int fault_mode() {
   if (!strcmp(s, "nan")) return kFaultNan;
   if (!strcmp(s, "timeout")) return kFaultTimeout;
   if (!strcmp(s, "noconv")) return kFaultNoconv;
+  if (!strcmp(s, "nocluster")) return kFaultNoCluster;
   return kFaultNone;
 }
+
+bool clusters_allowed() { return fault_mode() != kFaultNoCluster; }
 
 int ensure(Buf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
@@ -743,9 +748,9 @@ bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& s
     *e = launch_cg_k1<T>(co, h->nnz, h->sms, S(h));
     coop = true;
   } else if constexpr (sizeof(T) == 4)
-    coop = launch_cg_coop_f32(K, co, h->nnz, h->sms, S(h), e);
+    coop = launch_cg_coop_f32(K, co, h->nnz, h->sms, clusters_allowed(), S(h), e);
   else
-    coop = launch_cg_coop_f64(K, co, h->nnz, h->sms, S(h), e);
+    coop = launch_cg_coop_f64(K, co, h->nnz, h->sms, clusters_allowed(), S(h), e);
   if (coop) {
     prof_end(h, pc);
     h->bar_clean = false;
@@ -958,7 +963,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // state of its own. Small solves run the correction as one cooperative kernel:
   // both are launched before one wait for their outcome.
   PhaseGraph pg = phase_graph_mid(h, grid_u);
-  const bool coop = (K == 1 && h->n > k1_rows<float>()) || cg_coop_fits_f32(K, pg, h->nnz, h->sms);
+  const bool coop = (K == 1 && h->n > k1_rows<float>()) || cg_coop_fits_f32(K, pg, h->nnz, h->sms, h->si_dsh_h != nullptr, clusters_allowed());
   if (coop) WL_TRY(ensure(h->r32, nk * 4));
   const bool wide = !coop && grid_u > 1 && grid_r > 1;
   if (wide) {
@@ -2982,6 +2987,24 @@ int wl_selftest_bounded_wait(int missing, void* stream) {
     return WL_ERR_CUDA;
   }
   return err != 0 ? err : WL_OK;
+}
+
+// Launch shape of the cooperative CG kernel (FP32, or FP64 with fp64 != 0) for
+// K columns on a device of `sms` SMs: out = {grid, threads, dynamic shared bytes,
+// one cluster}. 1 where the solve fits, 0 where it takes the phase kernels.
+int wl_selftest_cg_shape(int fp64, int K, int64_t n, int64_t nnz, int nhub, int nmid, int sms, int clusters,
+                         int64_t* out) {
+  if (n < 1 || sms < 1 || !out) return WL_ERR_INVALID_ARG;
+  PhaseGraph g{nullptr, nullptr, n, nullptr, nhub};
+  g.nmid = nmid;
+  CoopShape sh;
+  if (!(fp64 ? cg_coop_shape_f64(K, g, nnz, sms, clusters != 0, &sh) : cg_coop_shape_f32(K, g, nnz, sms, clusters != 0, &sh)))
+    return 0;
+  out[0] = sh.grid;
+  out[1] = sh.threads;
+  out[2] = (int64_t)sh.smem;
+  out[3] = sh.cluster;
+  return 1;
 }
 
 }  // extern "C"

@@ -24,6 +24,7 @@
 // kernels' two launches took 43.
 #pragma once
 #include <algorithm>
+#include <atomic>
 
 #include "wl_cg2.cuh"
 #include "wl_df.cuh"
@@ -709,8 +710,9 @@ struct CoopShape {
 };
 
 // The launch of a solve with K columns, or false where its vectors don't fit.
+// clusters: the device can place the kernel's clusters.
 template <typename T, int K>
-bool cgc_shape(const PhaseGraph& g, int64_t nnz, int sms, CoopShape* sh) {
+bool cgc_shape(const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh) {
   using CC = CoopCfg<T, K>;
   // 256 lane units (rows x LPR) per CTA until every SM has one (each CTA adds
   // to the reductions), then more threads, evenly over the passes of the row
@@ -718,7 +720,7 @@ bool cgc_shape(const PhaseGraph& g, int64_t nnz, int sms, CoopShape* sh) {
   // barrier and sums don't leave the cluster (FP64 only up to 4096 elements: 16
   // SMs' FP64 pipes take longer over 8000 than the grid's barrier costs).
   const int64_t units = g.n * CC::LPR, ctas = std::max<int64_t>(1, (units + 255) / 256);
-  sh->cluster = ctas <= 2 * kCoopCluster && (sizeof(T) == 4 || g.n * K <= 4096);
+  sh->cluster = clusters && ctas <= 2 * kCoopCluster && (sizeof(T) == 4 || g.n * K <= 4096);
   if (sh->cluster) {
     sh->grid = 1;
     while (sh->grid < kCoopCluster && sh->grid < ctas) sh->grid *= 2;
@@ -768,14 +770,60 @@ bool cgc_shape(const PhaseGraph& g, int64_t nnz, int sms, CoopShape* sh) {
 }
 
 template <typename T, int K, bool SH>
-cudaError_t cgc_launch(CoopArgs<T> a, const CoopShape& sh, cudaStream_t s) {
+cudaError_t cgc_attributes() {
   static PerDevice attr;
-  const cudaError_t ae = attr.once([] {
+  return attr.once([] {
     cudaError_t e = cudaFuncSetAttribute(cg_coop<T, K, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)CoopCfg<T, K>::SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cg_coop<T, K, SH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
   });
+}
+
+// Whether the current device can place a cluster of the kernel at its largest
+// (16 CTAs, one per SM, is more than the portable size: a part of a GPU may have
+// no 16 free SMs that form one). Asked once per device.
+template <typename T, int K, bool SH>
+bool cgc_clusters() {
+  static PerDevice asked;
+  static std::atomic<uint64_t> yes{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return false;
+  const cudaError_t e = asked.once([dev] {
+    cudaError_t ce = cgc_attributes<T, K, SH>();
+    if (ce != cudaSuccess) return ce;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCoopCluster);
+    cfg.blockDim = dim3(CoopCfg<T, K>::TMAX);
+    cfg.dynamicSmemBytes = CoopCfg<T, K>::SMEM;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kCoopCluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int num = 0;
+    if (cudaOccupancyMaxActiveClusters(&num, cg_coop<T, K, SH>, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      num = 0;
+    }
+    if (num > 0) yes.fetch_or(uint64_t(1) << dev);
+    return cudaSuccess;
+  });
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return (yes.load() >> dev & 1) != 0;
+}
+
+// the shape of a solve on the current device
+template <typename T, int K>
+bool cgc_device_shape(const PhaseGraph& g, int64_t nnz, int sms, bool shifted, bool clusters, CoopShape* sh) {
+  clusters = clusters && (shifted ? cgc_clusters<T, K, true>() : cgc_clusters<T, K, false>());
+  return cgc_shape<T, K>(g, nnz, sms, clusters, sh);
+}
+
+template <typename T, int K, bool SH>
+cudaError_t cgc_launch(CoopArgs<T> a, const CoopShape& sh, cudaStream_t s) {
+  const cudaError_t ae = cgc_attributes<T, K, SH>();
   if (ae != cudaSuccess) return ae;
   a.long_min = sh.long_min;
   a.nhead = sh.nhead;

@@ -103,13 +103,17 @@ cudaError_t launch_cg_x_f32(int K, const CgXArgs<float>& a, int grid, cudaStream
 cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStream_t s);
 // ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the
 // solve's vectors don't fit in shared memory
-bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
+bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, bool clusters, cudaStream_t s,
+                        cudaError_t* e);
+bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, bool clusters, cudaStream_t s,
+                        cudaError_t* e);
+bool cg_coop_fits_f32(int K, const PhaseGraph& g, int64_t nnz, int sms, bool shifted, bool clusters);
+bool cg_coop_shape_f32(int K, const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh);
+bool cg_coop_shape_f64(int K, const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh);
 // ---- wl_k_k1.cu: the same for one column (any n), and its residual (df_res, not full)
 template <typename T>
 cudaError_t launch_cg_k1(const CoopArgs<T>& a, int64_t nnz, int sms, cudaStream_t s);
 cudaError_t launch_df_res_k1(const DfResArgs& a, int64_t nnz, int sms, cudaStream_t s);
-bool cg_coop_fits_f32(int K, const PhaseGraph& g, int64_t nnz, int sms);
-bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, cudaStream_t s, cudaError_t* e);
 // one CTA waiting in the bounded grid barrier for nblocks CTAs (failure-detection self-test)
 cudaError_t launch_selftest_wait(GridBar* bar, unsigned nblocks, cudaStream_t s);
 // FP64 residual r = b - M x of a warm start, norms into st->gamma / st->b2

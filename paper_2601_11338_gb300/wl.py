@@ -101,6 +101,8 @@ def lib():
         L.wl_rcm_order.restype = c_int
         L.wl_selftest_bounded_wait.argtypes = [c_int, vp]
         L.wl_selftest_bounded_wait.restype = c_int
+        L.wl_selftest_cg_shape.argtypes = [c_int, c_int, i64, i64, c_int, c_int, c_int, c_int, ctypes.POINTER(i64)]
+        L.wl_selftest_cg_shape.restype = c_int
         L.wl_batch_build.argtypes = [vp, c_int, vp, c_int, ctypes.POINTER(wl_params), ctypes.POINTER(vp),
                                      ctypes.POINTER(wl_stats)]
         L.wl_batch_build.restype = c_int
@@ -274,6 +276,13 @@ def wl_selftest_bounded_wait(missing, stream=None):
     WL_OK when missing = 0, WL_ERR_TIMEOUT after the wait limit otherwise
     (the kernel returns; the context stays usable). See include/wl.h."""
     return lib().wl_selftest_bounded_wait(int(missing), stream)
+
+
+def wl_selftest_cg_shape(fp64, K, n, nnz, nhub, nmid, sms, clusters):
+    """Launch shape (grid, threads, shared bytes, one cluster) of the cooperative
+    CG kernel on a device of `sms` SMs, or None where it takes the phase kernels."""
+    out = (ctypes.c_int64 * 4)()
+    return tuple(out) if lib().wl_selftest_cg_shape(int(fp64), K, n, nnz, nhub, nmid, sms, int(clusters), out) == 1 else None
 
 
 def wl_set_warm_start(h, x0):
