@@ -3007,6 +3007,18 @@ int wl_selftest_cg_shape(int fp64, int K, int64_t n, int64_t nnz, int nhub, int 
   return 1;
 }
 
+// The same for the spectral searches' steps: out = {grid, threads, dynamic shared
+// bytes, 1 where the vectors are streamed}.
+int wl_selftest_search_shape(int64_t n, int64_t nnz, int nhub, int nmid, int sms, int64_t* out) {
+  if (n < 1 || sms < 1 || !out) return WL_ERR_INVALID_ARG;
+  const SpShape sh = sp_coop_shape(n, nnz, nmid, nhub, sms);
+  out[0] = sh.grid;
+  out[1] = sh.threads;
+  out[2] = (int64_t)sh.smem;
+  out[3] = sh.stream;
+  return WL_OK;
+}
+
 }  // extern "C"
 
 namespace wl {

@@ -189,10 +189,16 @@ int sp_blocks();  // resident CTAs of the step kernels (all SMs)
 cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t s);
 // steps j0..j1-1 (the run stops by itself at cap - 1, on breakdown, or when the
 // error bound checked every `check` steps and at j1 is below rtol |theta_1|)
-// Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
-// the same steps as cooperative kernels of `check` steps each; bar is cleared before each
+// (as cooperative kernels of `check` steps each; bar is cleared before each)
 cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap, int check,
                                  double rtol, cudaStream_t s);
+struct SpShape {
+  int grid = 0, threads = 0, nhead = 0;
+  size_t smem = 0;
+  bool stream = false;  // the kernel that streams the vectors
+};
+SpShape sp_coop_shape(int64_t n, int64_t nnz, int nmid, int nhub, int sms);
+// Ritz vector of the run into W[1], |u|^2 and u^T D u into st->out[5], out[6]
 cudaError_t launch_sp_ritz(const SpArgs& a, int grid_u, cudaStream_t s);
 // One round of the batched spectral searches: the np jobs (device array) with
 // their CTA offsets in the S kernel (off_s, np + 1 entries, off_s[np] =

@@ -25,27 +25,35 @@ cudaError_t launch_sp_start(const SpArgs& a, int mode, int grid_u, cudaStream_t 
 
 // Graphs of more rows take the steps that stream the vectors (eight of them:
 // Chung-Lu, 400003 nodes 250 -> 202 us, R-MAT scale 17 about a tenth less; the
-// others were 10% to 40% slower by it); up to it the vectors always fit.
+// others were 10% to 40% slower by it), and any graph whose vectors don't fit
+// in the SMs there are (fewer than some 130).
 constexpr int64_t kSpStreamRows = 250000;
 
-// grid, threads and shared memory of the cooperative steps
-static void sp_coop_shape(const SpArgs& a, int64_t nnz, int sms, int* grid, int* threads, size_t* smem, int* nhead) {
-  const int64_t units = a.g.n * kSpCoopLpr;
-  *grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (units + 255) / 256));
-  const int64_t rows = coop_rows_local(a.g.n, *grid, kSpCoopCh);
-  const int64_t passes = (rows * kSpCoopLpr + kSpCoopThreads - 1) / kSpCoopThreads;
-  *threads = (int)std::max<int64_t>(256, (rows * kSpCoopLpr / passes + 31) / 32 * 32);
-  const int64_t nslot = rows + (a.nmid + *grid - 1) / *grid + (a.g.nhub + *grid - 1) / *grid;
+// grid, threads and shared memory of the cooperative steps on `sms` SMs
+SpShape sp_coop_shape(int64_t n, int64_t nnz, int nmid, int nhub, int sms) {
+  SpShape sh;
+  const int64_t units = n * kSpCoopLpr;
+  sh.grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (units + 255) / 256));
+  const int64_t rows = coop_rows_local(n, sh.grid, kSpCoopCh);
+  const int64_t nslot = rows + (nmid + sh.grid - 1) / sh.grid + (nhub + sh.grid - 1) / sh.grid;
   const size_t vec = (size_t)nslot * 3 * sizeof(float2);
-  *nhead = (int)std::min<int64_t>({a.g.n, nnz / (4 * *grid), (int64_t)((kSpCoopSmem - vec) / sizeof(float2))});
-  *smem = vec + (size_t)*nhead * sizeof(float2);
+  sh.stream = n > kSpStreamRows || vec > kSpCoopSmem;
+  if (sh.stream) {
+    sh.grid = k1_grid(n, sms);
+    sh.threads = k1_threads<float2>();
+    sh.nhead = k1_head<float2>(n, nnz, sh.grid);
+    sh.smem = k1_smem<float2>(sh.nhead);
+    return sh;
+  }
+  const int64_t passes = (rows * kSpCoopLpr + kSpCoopThreads - 1) / kSpCoopThreads;
+  sh.threads = (int)std::max<int64_t>(256, (rows * kSpCoopLpr / passes + 31) / 32 * 32);
+  sh.nhead = (int)std::min<int64_t>({n, nnz / (4 * sh.grid), (int64_t)((kSpCoopSmem - vec) / sizeof(float2))});
+  sh.smem = vec + (size_t)sh.nhead * sizeof(float2);
+  return sh;
 }
-// rows and listed rows of a CTA at that limit, three vectors each
-static_assert(2 * (kSpStreamRows / 128 + 2 * kSpCoopCh) * 3 * sizeof(float2) <= kSpCoopSmem, "a run's vectors fit");
 
 cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar* bar, int j0, int j1, int cap,
                                  int check, double rtol, cudaStream_t s) {
-  const bool stream = a.g.n > kSpStreamRows;
   static PerDevice attr;
   if (cudaError_t e = attr.once([] {
         return cudaFuncSetAttribute(sp_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpCoopSmem);
@@ -58,18 +66,16 @@ cudaError_t launch_sp_steps_coop(const SpArgs& a, int64_t nnz, int sms, CoopBar*
       });
       e != cudaSuccess)
     return e;
-  SpCoopArgs ca{a, bar, 0, 0, cap, 0};
-  int grid = k1_grid(a.g.n, sms), threads = k1_threads<float2>();
-  ca.nhead = k1_head<float2>(a.g.n, nnz, grid);
-  size_t smem = k1_smem<float2>(ca.nhead);
-  if (!stream) sp_coop_shape(a, nnz, sms, &grid, &threads, &smem, &ca.nhead);
+  const SpShape sh = sp_coop_shape(a.g.n, nnz, a.nmid, a.g.nhub, sms);
+  SpCoopArgs ca{a, bar, 0, 0, cap, sh.nhead};
   for (int j = j0; j < j1; j = ca.j1) {
     ca.j0 = j;
     ca.j1 = std::min(j1, (j / check + 1) * check);
     cudaError_t e = cudaMemsetAsync(&bar->count, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     void* args[] = {&ca};
-    e = cudaLaunchCooperativeKernel(stream ? (const void*)sp_k1 : (const void*)sp_coop, dim3(grid), dim3(threads), args, smem, s);
+    e = cudaLaunchCooperativeKernel(sh.stream ? (const void*)sp_k1 : (const void*)sp_coop, dim3(sh.grid),
+                                    dim3(sh.threads), args, sh.smem, s);
     if (e != cudaSuccess) return e;
     sp_eig<<<1, 2 * kSpEigT, 0, s>>>(a.st, rtol);
   }

@@ -103,6 +103,8 @@ def lib():
         L.wl_selftest_bounded_wait.restype = c_int
         L.wl_selftest_cg_shape.argtypes = [c_int, c_int, i64, i64, c_int, c_int, c_int, c_int, ctypes.POINTER(i64)]
         L.wl_selftest_cg_shape.restype = c_int
+        L.wl_selftest_search_shape.argtypes = [i64, i64, c_int, c_int, c_int, ctypes.POINTER(i64)]
+        L.wl_selftest_search_shape.restype = c_int
         L.wl_batch_build.argtypes = [vp, c_int, vp, c_int, ctypes.POINTER(wl_params), ctypes.POINTER(vp),
                                      ctypes.POINTER(wl_stats)]
         L.wl_batch_build.restype = c_int
@@ -283,6 +285,14 @@ def wl_selftest_cg_shape(fp64, K, n, nnz, nhub, nmid, sms, clusters):
     CG kernel on a device of `sms` SMs, or None where it takes the phase kernels."""
     out = (ctypes.c_int64 * 4)()
     return tuple(out) if lib().wl_selftest_cg_shape(int(fp64), K, n, nnz, nhub, nmid, sms, int(clusters), out) == 1 else None
+
+
+def wl_selftest_search_shape(n, nnz, nhub, nmid, sms):
+    """Launch shape (grid, threads, shared bytes, streamed) of the spectral
+    searches' steps on a device of `sms` SMs."""
+    out = (ctypes.c_int64 * 4)()
+    _check(lib().wl_selftest_search_shape(n, nnz, nhub, nmid, sms, out), "wl_selftest_search_shape")
+    return tuple(out)
 
 
 def wl_set_warm_start(h, x0):

@@ -22,3 +22,16 @@ def test_cg_shape_without_clusters(fp64, sms):
                 assert sms < 16, (K, n, with_c)
             if with_c is not None and with_c[3]:
                 assert with_c[0] <= 16 and with_c[2] <= SMEM
+
+
+@pytest.mark.parametrize("sms", [1, 8, 32, 76, 127, 132, 152])
+def test_search_shape_fits_on_fewer_sms(sms):
+    """The vectors of up to 250000 rows fit in a whole device's shared memory;
+    on fewer SMs the steps stream them."""
+    for n in (1, 5, 2000, 60000, 131072, 249999, 250000, 250001, 1000000):
+        for nhub, nmid in ((0, 0), (n // 100, n // 3), (n // 2, n - n // 2)):
+            grid, threads, smem, stream = wl.wl_selftest_search_shape(n, 8 * n, nhub, nmid, sms)
+            assert 1 <= grid <= sms and 0 < threads <= 1024 and threads % 32 == 0
+            assert 0 <= smem <= SMEM, (n, nhub, nmid, smem)
+            if sms == 152:
+                assert bool(stream) == (n > 250000)
