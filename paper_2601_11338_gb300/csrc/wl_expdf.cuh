@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kBlock) df_combine(DfCombineArgs a, int CS) {
     }
   };
   if (c >= a.kr) return;
-  const df sc = df_from_double(a.nrm[c]);
+  const double sc = a.nrm[c];  // beyond FP32's range too: the last product is in FP64
   const int rpb = kBlock / CS;
   for (int64_t i = (int64_t)blockIdx.x * rpb + tid / CS; i < a.n; i += (int64_t)gridDim.x * rpb) {
     const size_t e = (size_t)i * K + c;
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kBlock) df_combine(DfCombineArgs a, int CS) {
 #pragma unroll
     for (int t = 0; t < NT; ++t)
       if (t < a.ntau)
-        a.out[(size_t)t * a.tstride + io * a.ld + a.c0 + c] = df_to_double(df_mul(sc, two_sum(S[t], Cc[t])));
+        a.out[(size_t)t * a.tstride + io * a.ld + a.c0 + c] = sc * join_f64(S[t], Cc[t]);
   }
 }
 

@@ -1,0 +1,35 @@
+"""Calls at the limits of the number formats and of memory, against the oracle at
+the tolerance of the quantity's own parity test."""
+import numpy as np
+import pytest
+
+import wlgen
+from oracle import graph, walks
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def WL(g, **kw):
+    from paper_2601_11338_gb300.api import WalkLaplacian
+    return WalkLaplacian(g.row_ptr.astype(np.int32), g.col_idx, g.n, **kw)
+
+
+@pytest.mark.parametrize("shift", [0.0, 1.0])
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-9), ("refined", 1e-12, 1e-8)])
+def test_diffusion_does_not_depend_on_the_scale_of_its_columns(prec, tol, bound, shift):
+    """exp(-tau L) is linear and the basis is normalised in FP64: columns whose
+    norms FP32 cannot hold come out like any other, each to its own scale."""
+    g = wlgen.erdos_renyi(400, 6.0, 9)
+    A = graph.dense_adjacency(g.row_ptr, g.col_idx, g.n)
+    w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=tol, outer_tol=1e-11, shift=shift)
+    lam, Q = np.linalg.eigh(walks.walk_laplacian(walks.phi_resolvent_closed(A, 1.0, w.info["alpha"])))
+    U = np.random.default_rng(3).standard_normal((g.n, 6))
+    scale = np.array([1e-60, 1e-44, 1e-35, 1.0, 1e37, 1e60])
+    taus = [0.0, 0.3, 2.0]
+    got = w.expmv(torch.as_tensor(U * scale, device="cuda"), taus).cpu().numpy().reshape(3, g.n, 6) / scale
+    for t, tau in enumerate(taus):
+        want = Q @ (np.exp(-tau * lam)[:, None] * (Q.T @ U))
+        err = np.linalg.norm(got[t] - want, axis=0) / np.linalg.norm(want, axis=0)
+        assert (err <= bound).all(), (tau, err)
+    w.close()
