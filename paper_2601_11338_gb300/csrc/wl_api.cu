@@ -355,12 +355,16 @@ void sp_batch_free(SpBatch* b) {
 
 // State of a solve. The cooperative CG kernel's barrier follows the norms of
 // the refinement residual, so that clearing those before each residual also
-// readies it for the next solve.
+// readies it for the next solve. Its error word, the last member, is not cleared with
+// them (kResClear): the host reads it with the outcome, after the residual.
 struct CgBlock {
   CgState st;
   CgState res;  // norms of the refinement residual that follows a cooperative solve
   CoopBar bar;
 };
+constexpr size_t kResClear = sizeof(CgState) + offsetof(CoopBar, err);
+static_assert(offsetof(CgBlock, bar) == offsetof(CgBlock, res) + sizeof(CgState), "one range from res to the error word");
+static_assert(offsetof(CoopBar, err) + sizeof(int) == sizeof(CoopBar), "the error word is last");
 
 struct wl_handle {
   int64_t n = 0, nnz = 0;
@@ -1057,7 +1061,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
       }
     }
     // r <- r - M d, x <- x + d
-    WL_CU(cudaMemsetAsync(rst, 0, sizeof(CgState) + sizeof(CoopBar), S(h)));
+    WL_CU(cudaMemsetAsync(rst, 0, kResClear, S(h)));
     h->bar_clean = true;
     DfResArgs ra{rg, dcur, nullptr, rch, rcl, rh, rl, xh, xl,
                  ca, cA, cD, (double*)h->part.p, rst, x_zero ? 1 : 0};
