@@ -143,7 +143,9 @@ bool is_device_ptr(const void* p) {
 // gathered rows of at least a 32-byte sector, ten vector streams and the
 // indices. Padding also stops where a block would pass kPadMaxElems elements:
 // the vectors of a solve and an outer basis grow with it, and what fitted in
-// memory without padding has to fit still. An apply of 13 columns, n = 20011:
+// memory without padding has to fit still. The widest block comes first, so that
+// every workspace has its final size from the first block on (a buffer that grows
+// is kept beside its successor until the handle goes). An apply of 13 columns, n = 20011:
 // 455 us as one block of 16, 947 us as 8 + 4 + 1.
 struct ColBlock {
   int K, kr;
@@ -175,6 +177,9 @@ std::vector<ColBlock> column_blocks(int k, int64_t n, int64_t nnz, int val_bytes
     out.push_back({K, std::min(K, k)});
     k -= std::min(K, k);
   }
+  std::stable_sort(out.begin(), out.end(), [](const ColBlock& a, const ColBlock& b) {
+    return a.K != b.K ? a.K > b.K : a.kr > b.kr;
+  });
   return out;
 }
 
@@ -3021,6 +3026,18 @@ int wl_selftest_search_shape(int64_t n, int64_t nnz, int nhub, int nmid, int sms
   out[2] = (int64_t)sh.smem;
   out[3] = sh.stream;
   return WL_OK;
+}
+
+// The column blocks of k columns (FP64, or FP32 with fp64 = 0): widths in K, columns
+// in kr, at most `cap` of each written; their number is returned.
+int wl_selftest_column_blocks(int k, int64_t n, int64_t nnz, int fp64, int* K, int* kr, int cap) {
+  if (k < 0 || n < 1 || nnz < 0 || !K || !kr) return WL_ERR_INVALID_ARG;
+  const auto blocks = column_blocks(k, n, nnz, fp64 ? 8 : 4);
+  for (size_t i = 0; i < blocks.size() && (int)i < cap; ++i) {
+    K[i] = blocks[i].K;
+    kr[i] = blocks[i].kr;
+  }
+  return (int)blocks.size();
 }
 
 }  // extern "C"

@@ -105,6 +105,8 @@ def lib():
         L.wl_selftest_cg_shape.restype = c_int
         L.wl_selftest_search_shape.argtypes = [i64, i64, c_int, c_int, c_int, ctypes.POINTER(i64)]
         L.wl_selftest_search_shape.restype = c_int
+        L.wl_selftest_column_blocks.argtypes = [c_int, i64, i64, c_int, ctypes.POINTER(c_int), ctypes.POINTER(c_int), c_int]
+        L.wl_selftest_column_blocks.restype = c_int
         L.wl_batch_build.argtypes = [vp, c_int, vp, c_int, ctypes.POINTER(wl_params), ctypes.POINTER(vp),
                                      ctypes.POINTER(wl_stats)]
         L.wl_batch_build.restype = c_int
@@ -293,6 +295,15 @@ def wl_selftest_search_shape(n, nnz, nhub, nmid, sms):
     out = (ctypes.c_int64 * 4)()
     _check(lib().wl_selftest_search_shape(n, nnz, nhub, nmid, sms, out), "wl_selftest_search_shape")
     return tuple(out)
+
+
+def wl_selftest_column_blocks(k, n, nnz, fp64):
+    """The blocks [(width, columns)] in which a call works on k columns."""
+    K, kr = (ctypes.c_int * 64)(), (ctypes.c_int * 64)()
+    m = lib().wl_selftest_column_blocks(k, n, nnz, int(fp64), K, kr, 64)
+    if m < 0:
+        raise WLError(m, "wl_selftest_column_blocks")
+    return list(zip(K[:m], kr[:m]))
 
 
 def wl_set_warm_start(h, x0):

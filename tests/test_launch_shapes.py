@@ -35,3 +35,18 @@ def test_search_shape_fits_on_fewer_sms(sms):
             assert 0 <= smem <= SMEM, (n, nhub, nmid, smem)
             if sms == 152:
                 assert bool(stream) == (n > 250000)
+
+
+@pytest.mark.parametrize("fp64", [0, 1])
+@pytest.mark.parametrize("n,nnz", [(1, 0), (2000, 20000), (20011, 240000), (10 ** 6, 12 * 10 ** 6), (10 ** 8, 10 ** 9)])
+def test_column_blocks_widest_first(fp64, n, nnz):
+    """Every column once, widths powers of two up to 64, none wider than the one
+    before it (workspaces are sized by the first), a padded block last among its
+    width."""
+    for k in range(0, 200):
+        b = wl.wl_selftest_column_blocks(k, n, nnz, fp64)
+        assert sum(kr for _, kr in b) == k
+        assert all(K in (1, 2, 4, 8, 16, 32, 64) and 0 < kr <= K for K, kr in b)
+        assert all(b[i][0] >= b[i + 1][0] for i in range(len(b) - 1)), (k, b)
+        assert all(b[i][1] >= b[i + 1][1] for i in range(len(b) - 1) if b[i][0] == b[i + 1][0]), (k, b)
+        assert sum(kr < K for K, kr in b) <= 1
