@@ -193,6 +193,8 @@ struct SolveInfo {
   double nnz_rhs = 0.0;
   double bytes = 0.0;
   int reorth_blocks = 0;  // basis blocks reorthogonalised (outer Lanczos)
+  int kr = 64;            // columns of the caller's in the current block (the others of its K are padding)
+  int cols(int K) const { return std::min(K, kr); }
 };
 
 }  // namespace
@@ -678,8 +680,8 @@ void cg_outcome(wl_handle* h, int K, int val_bytes, SolveInfo& info) {
   }
   info.iters += it;
   info.cg_iters += it;
-  info.nnz_rhs += (double)it * h->nnz * K;
-  info.bytes += (double)it * alg_bytes_per_iter(h, K, val_bytes);
+  info.nnz_rhs += (double)it * h->nnz * info.cols(K);
+  info.bytes += (double)it * alg_bytes_per_iter(h, info.cols(K), val_bytes);
   info.last_rel = 0.0;
   for (int c = 0; c < K; ++c) {
     if (cs[c] != 0 && info.status == WL_OK) info.status = cs[c];
@@ -909,7 +911,7 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
     WL_CU(launch_res_phases(K, ra, grid_w, S(h)));
     prof_end(h, pi);
     bn2 = st->b2;
-    info.nnz_rhs += (double)h->nnz * K;
+    info.nnz_rhs += (double)h->nnz * info.cols(K);
   }
   PhaseArgs<double> a{phase_graph_mid(h, grid_u), x, (double*)h->r.p, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
                       bn2, nullptr, (double*)h->part.p, st, h->prm.max_iter, tol * tol};
@@ -995,7 +997,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     const int pi = prof_begin(h, kCatRes);
     WL_CU(launch_df_res(K, ra, grid_r + rg.nhub, true, S(h)));
     prof_end(h, pi);
-    info.nnz_rhs += (double)h->nnz * K;
+    info.nnz_rhs += (double)h->nnz * info.cols(K);
     rch = rh;
     rcl = rl;
   }
@@ -1044,6 +1046,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     a.tol2 = inner_tol * inner_tol;
     a.skip = from_b ? nullptr : dskip;
     SolveInfo inner;
+    inner.kr = info.kr;
     // the inner solve starts from the residual norms (from the double-float
     // residual, or B's norms): no pass over r to recompute them
     CgStart<float> start;
@@ -1090,7 +1093,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
     info.cg_iters += inner.cg_iters;
     info.nnz_rhs += inner.nnz_rhs;
     info.bytes += inner.bytes;
-    info.nnz_rhs += (double)h->nnz * K;
+    info.nnz_rhs += (double)h->nnz * info.cols(K);
     x_zero = false;
     rch = rh;
     rcl = rl;
@@ -1182,7 +1185,7 @@ int exp_series(wl_handle* h, const double* V, double* X, int K, SolveInfo& info)
     if (hp[c] != 0 && info.status == WL_OK) info.status = hp[c];
   if (hp[65] && info.status == WL_OK) info.status = WL_ERR_NO_CONVERGENCE;  // term cap reached
   info.iters += terms;
-  info.nnz_rhs += (double)terms * h->nnz * K;
+  info.nnz_rhs += (double)terms * h->nnz * info.cols(K);
   counted(h);
   WL_CU(launch_split_x(nullptr, (int64_t)nk, Ah, Al, true, X, S(h)));
   return WL_OK;
@@ -1987,7 +1990,7 @@ int outer_run(wl_handle* h, int K, const double* dtaus, int ntau, SolveInfo& inf
         la.c0 = 0.0;
         la.cA = -1.0;
         la.cD = 1.0;
-        info.nnz_rhs += (double)h->nnz * K;
+        info.nnz_rhs += (double)h->nnz * info.cols(K);
         info.iters += 1;
       } else {
         WL_TRY(phi_apply(h, vj, (double*)h->packX.p, K, info));
@@ -2584,6 +2587,7 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
     int c0 = 0;
     for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
       const int K = cb.K;
+      info.kr = cb.kr;
       if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       counted(h);
@@ -2597,7 +2601,7 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
         if ((rc = get_part(h, lanczos_step_grid(K), Tw, Tc, &pd, K, 8)) != WL_OK) break;
         counted(h);
         e = launch_laplacian_apply(h->g, *pd, (const double*)h->packV.p, K, c0, cb.kr, h->perm, Wd, ldw, S(h));
-        info.nnz_rhs += (double)h->nnz * K;
+        info.nnz_rhs += (double)h->nnz * info.cols(K);
         info.iters += 1;
       } else {
         if ((rc = phi_apply(h, (const double*)h->packV.p, (double*)h->packX.p, K, info)) != WL_OK) break;
@@ -2655,6 +2659,7 @@ int wl_expmv(wl_handle* h, const double* U0, int64_t ldu, int k, const double* t
     bool capped = false;  // a column block reached max_outer: every block is still evaluated
     for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
       const int K = cb.K;
+      info.kr = cb.kr;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       counted(h);
       cudaError_t e = h->perm ? launch_pack_perm(U0d, ldu, c0, cb.kr, K, n, 1.0, h->perm, (double*)h->packX.p, S(h))
@@ -2711,6 +2716,7 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
     int c0 = 0;
     for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
       const int K = cb.K;
+      info.kr = cb.kr;
       if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
       if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
       double* cur = (double*)h->packX.p;  // p_s of this block (internal node order)
@@ -2734,7 +2740,7 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
               rc = set_cuda_error(e, "markov step");
               break;
             }
-            info.nnz_rhs += (double)h->nnz * K;
+            info.nnz_rhs += (double)h->nnz * info.cols(K);
             info.iters += 1;
           } else {
             if ((rc = phi_apply(h, y, cur, K, info)) != WL_OK) break;

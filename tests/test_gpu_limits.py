@@ -33,3 +33,32 @@ def test_diffusion_does_not_depend_on_the_scale_of_its_columns(prec, tol, bound,
         err = np.linalg.norm(got[t] - want, axis=0) / np.linalg.norm(want, axis=0)
         assert (err <= bound).all(), (tau, err)
     w.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "refined"])
+@pytest.mark.parametrize("f", ["resolvent", "identity", "exp"])
+def test_statistics_count_the_columns_of_the_caller(prec, f):
+    """nnz_rhs_iters sums nnz times columns over the operator's applications, and
+    bytes_alg the bytes of these columns, also where a block of 13 is worked on as 16."""
+    g = wlgen.erdos_renyi(2000, 8.0, 5)
+    kw = dict(alpha_rel=0.5) if f == "resolvent" else {}
+    w = WL(g, variant="nbt", f=f, prec=prec, tol=1e-10, **kw)
+    w.degrees()
+    v = torch.as_tensor(np.random.default_rng(1).standard_normal((g.n, 1)), device="cuda")
+    calls = [lambda V: w.apply(V)]
+    if f != "exp":
+        calls.append(lambda V: w.expmv(V, [0.2]))
+    if f != "exp":
+        calls.append(lambda V: w.markov(V.abs(), [1, 3]))
+    for call in calls:
+        times = {}
+        for k in (16, 13, 1):
+            call(v.repeat(1, k).contiguous())
+            times[k] = w.last.nnz_rhs_iters / (g.nnz * k)  # applications to one column
+            assert times[k] == round(times[k]) > 0, (k, w.last.nnz_rhs_iters)
+            if f == "resolvent":
+                per = 4.0 * g.nnz + 4.0 * (g.n + 1) + 6.0 * g.n * k * (8 if prec == "fp64" else 4)
+                assert w.last.bytes_alg == w.last.k_cg_iters * per
+        # equal columns: the same work each, up to a step of the stopping rule in every solve
+        assert abs(times[13] - times[16]) <= 0.1 * times[16], times
+    w.close()
