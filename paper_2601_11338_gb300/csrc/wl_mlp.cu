@@ -489,6 +489,12 @@ __global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_predict(const float* __r
 // rows: 602 us and 224 us for the reduction of the partials).
 constexpr int kGradTiles = 16;
 
+// A running sum (s, c) as FP64. One that has left FP32's range is infinite, as in
+// a plain sum, though its error term is not a number then.
+__device__ __forceinline__ double df_sum_f64(float s, float c) {
+  return isfinite(s) ? (double)s + (double)c : (double)s;
+}
+
 struct alignas(16) MlpGradSmem {
   MlpTile t;
   float g2[kH * kMlpPitch];  // dL/dz2, [unit][row]
@@ -630,7 +636,7 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_grad(const float* __rest
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b)
-      out[kOffW2 - kOffW1 + (ty + 16 * a) * kH + tx + 16 * b] = (double)dw2h[a][b] + (double)dw2l[a][b];
+      out[kOffW2 - kOffW1 + (ty + 16 * a) * kH + tx + 16 * b] = df_sum_f64(dw2h[a][b], dw2l[a][b]);
   // the other gradients: 16 threads (ty) hold parts of each; red[v][ty][tx]
   float* red = s.g2;
   constexpr int NV = 29;
@@ -650,7 +656,7 @@ __global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_grad(const float* __rest
     const int v = e / 16, u = e % 16;  // u: tx
     float h = 0.f, l = 0.f;
     for (int g = 0; g < 16; ++g) df_acc(h, l, red[v * kMlpThreads + g * 16 + u]);
-    const double d = (double)h + (double)l;
+    const double d = df_sum_f64(h, l);
     if (v < 16)
       out[(4 * u + v / 4) * kIn + v % 4] = d;
     else if (v < 20)

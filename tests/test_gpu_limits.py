@@ -62,3 +62,21 @@ def test_statistics_count_the_columns_of_the_caller(prec, f):
         # equal columns: the same work each, up to a step of the stopping rule in every solve
         assert abs(times[13] - times[16]) <= 0.1 * times[16], times
     w.close()
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_an_overflowing_gradient_is_infinite(sign):
+    """One tile whose gradient of b3 and W3 passes FP32's range (6e38 and 4.6e38):
+    infinities, as plain FP32 sums give them, and no NaN. W3 = 0 keeps the other
+    gradients at zero."""
+    from paper_2601_11338_gb300 import wl
+    p = np.zeros(4553, dtype=np.float32)
+    p[4:8] = 1.0
+    p[4424:4488] = 1.0  # b2: h2 = tanh(1)
+    F = np.random.default_rng(2).normal(size=(128, 4)).astype(np.float32)
+    T = np.full(128, -3e38 * sign, dtype=np.float32)
+    grad = np.zeros(4553, dtype=np.float32)
+    loss = wl.wl_mlp_loss_grad(p, F, T, 128, grad)
+    assert loss == np.inf
+    assert (grad[4488:] == sign * np.inf).all(), grad[4488:]
+    assert not grad[:4488].any()
