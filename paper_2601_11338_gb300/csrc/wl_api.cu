@@ -373,6 +373,8 @@ constexpr size_t kResClear = sizeof(CgState) + offsetof(CoopBar, err);
 static_assert(offsetof(CgBlock, bar) == offsetof(CgBlock, res) + sizeof(CgState), "one range from res to the error word");
 static_assert(offsetof(CoopBar, err) + sizeof(int) == sizeof(CoopBar), "the error word is last");
 
+enum { kCgFp64 = 0, kCgFirst, kCgLater, kCgSketch, kCgKinds };  // solves; first and later corrections of a refined one
+
 struct wl_handle {
   int64_t n = 0, nnz = 0;
   Graph g{};
@@ -442,6 +444,7 @@ struct wl_handle {
   double inner_tol = 4e-6;  // floor of the FP32 correction target of the refined form
   int cg_hint = 7;          // CG iterations of the handle's last solve (sizes the first launch chunk)
   int cg_hint_ref[2] = {7, 7};  // the same for the first and the later corrections of a refined solve
+  bool stiff[kCgKinds][2] = {};  // the last solve of each kind (unshifted, shifted) was stiff (run_cg)
   bool gram_tc = false;     // XNysTrace Gram of the sketch form on the tensor cores (tcgen05); false: CUDA cores
   CgState* cgst() { return &((CgBlock*)cgstate.p)->st; }
   CgState* cgres() { return &((CgBlock*)cgstate.p)->res; }
@@ -774,14 +777,26 @@ bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& s
 // bytes up to which the phase kernels keep kHist residuals
 constexpr double kHistBytes = 4.0e9;
 
+// |p|^2 / |r|^2 from which a solve by the phase kernels forms p in every iteration
+// (the X form of wl_cg2.cuh, which says why). An X iteration takes a fifth longer.
+// FP32: with the line at 100 or 300 the diffusion at alpha = 1 / (1 + rho) on 1e6 nodes took
+// 392 ms where it takes 326, the iterations the same; at 1000 Erdos-Renyi, 2e5 x 16, alpha
+// rho = 0.994, shift 0.1, still gets what there is to get. FP64 loses nothing worth
+// an X iteration before 1e6 (849 iterations either way at 0.99, shift 0.1; 359 -> 271 at
+// 0.9999).
+template <typename T>
+constexpr double stiff_line() { return sizeof(T) == 4 ? 1e3 : 1e6; }
+
 // A solve by the phase kernels: runs the CG iterations to completion (or the
 // iteration cap), reading back one flag per chunk, and forms x from the kept
 // residuals, every kHist iterations (fewer where they take more than
-// kHistBytes: two for vectors of 1.3 GB and more) and at the end. *r_fin: the
+// kHistBytes: two for vectors of 1.3 GB and more) and at the end. Once it is
+// stiff, x and p are formed and then updated in every iteration, r in place; and
+// from the start where the handle's last solve of this kind was. *r_fin: the
 // final residual.
 template <typename T>
-int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, const CgStart<T>& start, int grid_s, int grid_u, SolveInfo& info,
-           const T** r_fin = nullptr) {
+int run_cg(wl_handle* h, int kind, int K, const PhaseArgs<T>& a_in, const CgStart<T>& start, int grid_s, int grid_u,
+           SolveInfo& info, const T** r_fin = nullptr) {
   PhaseArgs<T> a = a_in;
   const int fault = fault_mode();
   if (fault == kFaultNoconv) a.max_iter = 1;
@@ -801,7 +816,16 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, const CgStart<T>& star
   }
   a.hist = (CgHist*)h->hist.p;
   T* ring = (T*)((char*)h->hist.p + head);
-  auto rj = [&](int j) -> const T* { return j == 0 ? r0 : ring + (size_t)((j - 1) % (keep + 1)) * stride; };
+  bool& was_stiff = h->stiff[kind][h->si_dsh_h || h->si_dsh64];
+  T* r_own = was_stiff ? ring : nullptr;  // where r stays once x and p are updated in every iteration
+  if (r_own) {
+    a.hist = nullptr;
+    if (!start.add_x) WL_CU(cudaMemsetAsync(a.x, 0, (size_t)h->n * K * sizeof(T), S(h)));
+  }
+  auto rj = [&](int j) -> const T* {
+    return j == 0 ? r0 : r_own ? r_own : ring + (size_t)((j - 1) % (keep + 1)) * stride;
+  };
+  a.stiff = stiff_line<T>();
   auto iterate = [&](int j) -> cudaError_t {
     a.r = rj(j);
     a.rn = const_cast<T*>(rj(j + 1));
@@ -812,7 +836,7 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, const CgStart<T>& star
       return launch_cg_phases_f64(K, a, grid_s, grid_u, false, S(h));
   };
   // x (and p, if the solve goes on) from r_{j-m} .. r_{j-1}
-  auto form_x = [&](int j, int m, bool flush) -> cudaError_t {
+  auto form_x = [&](int j, int m, int flush) -> cudaError_t {
     CgXArgs<T> xa{};
     for (int i = 0; i < m; ++i) xa.r[i] = rj(j - m + i);
     xa.x = a.x;
@@ -851,26 +875,46 @@ int run_cg(wl_handle* h, int K, const PhaseArgs<T>& a_in, const CgStart<T>& star
   static_assert(sizeof(CgBlock) <= 4096 * sizeof(double), "pinned staging holds the CG state");
   // first chunk: one more iteration than the handle's previous solve took (a
   // launch that finds the solve finished returns at once, but still costs a
-  // grid); later chunks of kChunkMore iterations
+  // grid); later chunks of kChunkMore iterations, after a stop at a stiff iteration what
+  // the previous solve had left
   int chunk = std::min(std::max(h->cg_hint + 1, 2), 2 * kChunk);
   for (int j = 0;;) {
     for (const int end = j + chunk; j < end; ++j) {
-      if (j > 0 && j % keep == 0) {
+      if (!r_own && j > 0 && j % keep == 0) {
         counted(h, 1);
-        WL_CU(form_x(j, keep, true));
+        WL_CU(form_x(j, keep, 1));
       }
       counted(h, 2);
       WL_CU(iterate(j));
     }
     WL_CU(cudaMemcpyAsync(hs, h->cgst(), sizeof(CgState), cudaMemcpyDeviceToHost, S(h)));
     WL_CU(cudaStreamSynchronize(S(h)));
-    if (!hs->active) break;
     chunk = kChunkMore;
+    if (!hs->active) {
+      if (!hs->stiff || r_own || hs->iters >= a.max_iter) break;
+      // x and p_{j-1}, with no step left over (alpha = 0) for the S phase to add
+      j = hs->iters;
+      counted(h, 1);
+      WL_CU(form_x(j, (j - 1) % keep + 1, 2));
+      r_own = const_cast<T*>(rj(j));
+      a.hist = nullptr;
+      static const int on = 1;
+      WL_CU(cudaMemsetAsync(a.st->alpha, 0, sizeof(a.st->alpha), S(h)));
+      WL_CU(cudaMemcpyAsync(&a.st->active, &on, sizeof(int), cudaMemcpyHostToDevice, S(h)));
+      chunk = std::min(std::max(h->cg_hint + 1 - j, kChunkMore), 2 * kChunk);
+    }
   }
+  was_stiff = hs->stiff != 0;
   const int it = hs->iters;
-  if (it > 0) {
+  if (r_own) {
     counted(h, 1);
-    WL_CU(form_x(it, (it - 1) % keep + 1, false));
+    if constexpr (sizeof(T) == 4)
+      WL_CU(launch_cg_last_f32(K, a, grid_u, S(h)));
+    else
+      WL_CU(launch_cg_last_f64(K, a, grid_u, S(h)));
+  } else if (it > 0) {
+    counted(h, 1);
+    WL_CU(form_x(it, (it - 1) % keep + 1, 0));
   } else if (!start.add_x) {
     WL_CU(cudaMemsetAsync(a.x, 0, (size_t)h->n * K * sizeof(T), S(h)));
   }
@@ -931,7 +975,7 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
         WL_TRY(phase_lists(h));
         a.g = phase_graph_wide(h, grid_u);
       }
-      WL_TRY(run_cg<double>(h, K, a, start, grid_u + a.g.nhub, grid_u, info, &h->r_fin));
+      WL_TRY(run_cg<double>(h, kCgFp64, K, a, start, grid_u + a.g.nhub, grid_u, info, &h->r_fin));
     }
   }
   info.max_rel = std::max(info.max_rel, info.last_rel);
@@ -1061,7 +1105,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
       // sizes its first launch chunk from the previous solve of its kind
       int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
       h->cg_hint = hint;
-      WL_TRY(run_cg<float>(h, K, a, start, grid_u + pg.nhub, grid_u, inner));
+      WL_TRY(run_cg<float>(h, ref == 0 ? kCgFirst : kCgLater, K, a, start, grid_u + pg.nhub, grid_u, inner));
       hint = h->cg_hint;
       if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
         info.status = inner.status;
@@ -2859,7 +2903,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
         if ((rc = phase_lists(h)) != WL_OK) break;
         a.g = phase_graph_wide(h, grid_u);
       }
-      if ((rc = run_cg<float>(h, K, a, CgStart<float>{}, grid_u + a.g.nhub, grid_u, info)) != WL_OK) break;
+      if ((rc = run_cg<float>(h, kCgSketch, K, a, CgStart<float>{}, grid_u + a.g.nhub, grid_u, info)) != WL_OK) break;
     }
     (void)sm;
     counted(h, 4);

@@ -122,6 +122,7 @@ struct wl_batch {
   std::vector<TileSet> tilesets;       // candidate tile heights
   std::map<int, int> tuned;            // K * 2 + refined -> tileset index
   std::vector<double> mu, lmax, rho, alpha, phi;  // per graph / per problem
+  double pole = 1.0;  // the smallest 1 - alpha rho
   DBuf ca, cA, cD, phis;                           // per problem (device)
   DBuf ones;                                       // n doubles = 1
   DBuf Vin, Df, W;                                 // staged input and outputs
@@ -334,13 +335,13 @@ int emit_red_init(int K, const BatchGraph& g, const BatchState& st, const double
   return WL_OK;
 }
 
-template <typename T>
+template <typename T, bool KEPT>
 int emit_iteration(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
   const dim3 gt(a.g.ntile, nslab), gp(a.g.ngraph, nslab);
   switch (K) {
 #define C(k)                                                                      \
   case k:                                                                         \
-    bcg_s<T, k><<<gt, kPhaseBlock, 0, s>>>(a);                                    \
+    bcg_s<T, k, KEPT><<<gt, kPhaseBlock, 0, s>>>(a);                                    \
     bred_s<k><<<gp, kPhaseBlock, 0, s>>>(a.g, a.st, a.part);                       \
     bcg_u<T, k><<<gt, kPhaseBlock, 0, s>>>(a);                                    \
     bred_u<k><<<gp, kPhaseBlock, 0, s>>>(a.g, a.st, a.part, a.tol2, a.max_iter);   \
@@ -353,11 +354,11 @@ int emit_iteration(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
   return WL_OK;
 }
 
-template <typename T>
+template <typename T, bool KEPT>
 int emit_final(int K, const BatchArgs<T>& a, int nslab, cudaStream_t s) {
   const dim3 gt(a.g.ntile, nslab);
   switch (K) {
-#define C(k) case k: bcg_f<T, k><<<gt, kPhaseBlock, 0, s>>>(a); break;
+#define C(k) case k: bcg_f<T, k, KEPT><<<gt, kPhaseBlock, 0, s>>>(a); break;
     BT_FOR_K(C)
 #undef C
     default: return WL_ERR_INVALID_ARG;
@@ -391,6 +392,13 @@ int emit_red_res(int K, const BatchGraph& g, const BatchOuter& o, const double* 
   return WL_OK;
 }
 
+// 1 - alpha rho below which some problem's FP32 corrections would take more iterations
+// with kept residuals than they save (cg_s_phase says why; an iteration that forms p takes
+// a fifth longer). D_f's right-hand side is 1, close to the near-null vector: the same
+// iterations up to alpha rho = 0.94, 54 -> 68 on 20000-node graphs at 0.999. A Gaussian
+// right-hand side: the same up to 0.999.
+constexpr double kKeptPoleOnes = 0.06, kKeptPole = 0.002;
+
 // one batched solve M_{s,g} X = bscale b for all problems: X ends in
 // sb.x (FP64 form) or sb.x64 (refined form)
 int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const double* rhs, const double* bscale) {
@@ -407,12 +415,13 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
                         nullptr, nullptr, (double*)sb.part.p, st, b->prm.max_iter, tol2};
     BT_TRY(emit_init<double>(K, a, nslab, s));
     BT_TRY(emit_red_init(K, g, st, a.part, nullptr, nullptr, nullptr, tol2, nslab, s));
-    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<double>(K, a, nslab, em.s()); }));
-    return emit_final<double>(K, a, nslab, em.s());
+    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<double, false>(K, a, nslab, em.s()); }));
+    return emit_final<double, false>(K, a, nslab, em.s());
   }
   // refined: double-float residual / FP64 iterate around an FP32 CG whose
   // target is the inner tolerance relative to the current residual
   const BatchOuter o = bouter(b, sb);
+  const bool kept = b->pole >= (&sb == &b->sb1 ? kKeptPoleOnes : kKeptPole);
   const double tin = std::min(1e-3, std::max(4e-6, 0.5 * std::sqrt(b->prm.tol)));
   BT_CU(cudaMemsetAsync(sb.x64.p, 0, (size_t)nslab * b->n * K * 8, s));
   bfill_int<<<grid1(np), kPhaseBlock, 0, s>>>(o.outer_active, np, 1);
@@ -438,8 +447,10 @@ int emit_solve(wl_batch* b, Emitter& em, SolveBufs& sb, const TileSet& ts, const
     BT_TRY(emit_red_res(K, g, o, ra.part, tol2, b->prm.max_outer, nslab, so));
     BT_TRY(emit_red_init(K, g, st, nullptr, o.rn2, o.skip, o.outer_active, tin * tin, nslab, so));
     // the correction d ends in sb.x; the next residual pass adds it to x64
-    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() { return emit_iteration<float>(K, ia, nslab, em.s()); }));
-    return emit_final<float>(K, ia, nslab, em.s());
+    BT_TRY(em.loop(sb, st.any, b->prm.max_iter + 2, [&]() {
+      return kept ? emit_iteration<float, true>(K, ia, nslab, em.s()) : emit_iteration<float, false>(K, ia, nslab, em.s());
+    }));
+    return kept ? emit_final<float, true>(K, ia, nslab, em.s()) : emit_final<float, false>(K, ia, nslab, em.s());
   });
 }
 
@@ -503,7 +514,7 @@ int time_tiles(wl_batch* b, const TileSet& ts, int K, float* ms) {
                        (const double*)b->ca.p, (const double*)b->cA.p, (const double*)b->cD.p, nullptr, nullptr, nullptr, nullptr,
                        (double*)sb.part.p, st, 1, 0.0};
     switch (K) {
-#define C(k) case k: bcg_s<float, k><<<dim3(g.ntile, b->nslab), kPhaseBlock, 0, s>>>(a); break;
+#define C(k) case k: bcg_s<float, k, true><<<dim3(g.ntile, b->nslab), kPhaseBlock, 0, s>>>(a); break;
       BT_FOR_K(C)
 #undef C
     }
@@ -698,6 +709,7 @@ int wl_batch_build(const wl_csr* graphs, int ngraph, const double* mus, int nmu,
       if (p->alpha_rel > 0) a = rho > 0 ? p->alpha_rel / rho : 0.0;
       if (!(a >= 0.0) || !std::isfinite(a) || a * rho >= 1.0) return fail(WL_ERR_ALPHA_RANGE);
       b->alpha[pr] = a;
+      b->pole = std::min(b->pole, 1.0 - a * rho);
       b->phi[pr] = 1.0 - m * m * a * a;
       ca[pr] = b->phi[pr];
       cA[pr] = -a;

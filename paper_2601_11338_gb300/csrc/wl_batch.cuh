@@ -280,8 +280,12 @@ __global__ void __launch_bounds__(kPhaseBlock) bred_init(BatchGraph g, BatchStat
 }
 
 // ---------------------------------------------------------------- S
-template <typename T, int K>
+// KEPT (FP32 only): the residuals are kept, x and p formed from them every
+// kBatchHist iterations and at the end. Not near the pole, where that takes more
+// iterations (cg_s_phase): there x and p are updated here as in the FP64 form.
+template <typename T, int K, bool KEPT>
 __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(BatchArgs<T> a) {
+  static_assert(sizeof(T) == 4 || !KEPT, "the FP64 form has no room for kept residuals");
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   __shared__ T s_red[kPhaseBlock / 32 * K];
@@ -289,11 +293,9 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   if (!a.st.active[pr]) return;
   const int tid = threadIdx.x, sl = tid % G, lane_off = sl * VW;
-  // FP32: the residuals are kept, x and p formed from them every kBatchHist iterations and at the end
-  constexpr bool kKept = sizeof(T) == 4;
   const int it = a.st.iters[pr];
   const bool first = it == 0;
-  if constexpr (kKept) {
+  if constexpr (KEPT) {
     if (!first && it % kBatchHist == 0) batch_form_x<T, K>(a, tl, s, pr, it, kBatchHist, true);
   }
   const T ca = (T)a.ca[pr], cA = (T)a.cA[pr], cD = (T)a.cD[pr];
@@ -304,7 +306,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     be[v] = first ? T(0) : (T)a.st.beta[pr * K + lane_off + v];
   }
   const size_t slab = (size_t)s * a.g.n * K;
-  const T* __restrict__ R = (kKept ? batch_r(a, it) : a.r) + slab;
+  const T* __restrict__ R = (sizeof(T) == 4 ? batch_r(a, it) : a.r) + slab;
   T* __restrict__ P = a.p + slab;
   T* __restrict__ Q = a.q + slab;
   T* __restrict__ X = a.x + slab;
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
         pp.v[v] = rr.v[v];
         qq.v[v] = ca * rr.v[v] + cA * nb[v] + cD * (T)deg * rr.v[v];
       }
-    } else if constexpr (kKept) {
+    } else if constexpr (KEPT) {
       const Pack<T, VW> qo = ld_last<T, VW>(Q + o);
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
@@ -331,7 +333,13 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     } else {
       const Pack<T, VW> po = ld_plain<T, VW>(P + o);
       const Pack<T, VW> qo = ld_plain<T, VW>(Q + o);
-      Pack<T, VW> xx = ld_plain<T, VW>(X + o);
+      Pack<T, VW> xx;
+      if (sizeof(T) == 4 && it == 1) {  // FP32 starts at zero, which no pass has written
+#pragma unroll
+        for (int v = 0; v < VW; ++v) xx.v[v] = T(0);
+      } else {
+        xx = ld_plain<T, VW>(X + o);
+      }
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
         xx.v[v] += al[v] * po.v[v];
@@ -342,7 +350,7 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) bcg_s(Batc
     }
 #pragma unroll
     for (int v = 0; v < VW; ++v) dacc[v] += pp.v[v] * qq.v[v];
-    if constexpr (!kKept) stp<T, VW>(P + o, pp);
+    if constexpr (!KEPT) stp<T, VW>(P + o, pp);
     stp<T, VW>(Q + o, qq);
   };
   if (tl.hub) {
@@ -470,20 +478,20 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_u(BatchArgs<T> a) {
   block_colsum_store<T, K>(acc, a.part + ((size_t)s * a.g.ntile + blockIdx.x) * K);
 }
 
-// FP64: x += alpha p, the update of each problem's last iteration (the S kernel
-// makes the others, where it reads p anyway). FP32: x from the kept residuals.
-template <typename T, int K>
+// KEPT: x from the kept residuals. Otherwise x += alpha p, the update of each
+// problem's last iteration (the S kernel makes the others, where it reads p anyway).
+template <typename T, int K, bool KEPT>
 __global__ void __launch_bounds__(kPhaseBlock) bcg_f(BatchArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G, RPB = kPhaseBlock / G;
   const BTile tl = a.g.tiles[blockIdx.x];
   const int s = blockIdx.y, pr = s * a.g.ngraph + tl.graph;
   const int it = a.st.iters[pr];
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (KEPT) {
     batch_form_x<T, K>(a, tl, s, pr, it, it == 0 ? 0 : (it - 1) % kBatchHist + 1, false);
     return;
   }
-  if (it == 0) return;
+  if (sizeof(T) == 8 && it == 0) return;  // x is zero already
   const int tid = threadIdx.x, lane_off = (tid % G) * VW;
   T al[VW];
 #pragma unroll
@@ -493,8 +501,11 @@ __global__ void __launch_bounds__(kPhaseBlock) bcg_f(BatchArgs<T> a) {
   for (int64_t row = tl.row_beg + tid / G; row < tl.row_end; row += RPB) {
     if (!tl.hub && !plain_row(a.g.row_ptr, row)) continue;
     const size_t o = slab + (size_t)row * K + lane_off;
-    Pack<T, VW> xx = ld_plain<T, VW>(a.x + o);
-    const Pack<T, VW> pp = ld_plain<T, VW>(a.p + o);
+    Pack<T, VW> xx, pp;
+#pragma unroll
+    for (int v = 0; v < VW; ++v) xx.v[v] = pp.v[v] = T(0);
+    if (sizeof(T) == 8 || it > 1) xx = ld_plain<T, VW>(a.x + o);
+    if (it > 0) pp = ld_plain<T, VW>(a.p + o);
 #pragma unroll
     for (int v = 0; v < VW; ++v) xx.v[v] += al[v] * pp.v[v];
     stp<T, VW>(a.x + o, xx);

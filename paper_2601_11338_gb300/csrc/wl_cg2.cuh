@@ -51,7 +51,8 @@ struct CgState {
   int active;  // 1 while some column iterates and iters < max_iter
   int iters;   // S phases executed
   unsigned ticket;
-  int pad;
+  int stiff;   // some column's p has grown beyond PhaseArgs::stiff
+  double pi[64];  // |p|^2 by recurrence
 };
 
 struct PhaseGraph {
@@ -91,8 +92,12 @@ struct PhaseArgs {
   // optional per-row diagonal added to M (the shifted solves of the
   // shift-and-invert Lanczos: M - a (D_f + sigma I)^{-1}); NULL: none
   const T* dshift = nullptr;
-  CgHist* hist = nullptr;  // where the iteration's alpha and beta go, at `slot`
+  CgHist* hist = nullptr;  // where the iteration's alpha and beta go, at `slot` (NULL: x and p are updated in S)
   int slot = 0;
+  // > 0: CgState::stiff is set once some column's next p has |p|^2 > stiff |r|^2
+  // (|p_j|^2 = |r_j|^2 + beta^2 |p_{j-1}|^2, as r_j is orthogonal to p_{j-1}), and the solve
+  // stops there (active 0) unless x and p are updated in S
+  double stiff = 0.0;
 };
 
 // ---------------------------------------------------------------- helpers
@@ -324,7 +329,7 @@ __device__ __forceinline__ void sum_partials(const double* part, int nblk, doubl
 // SH: the solve carries the per-row diagonal a.dshift (a separate instance,
 // so that the unshifted kernel carries no trace of it)
 // X: x and p are updated here, in place (four vectors and no more: the entry
-// that allocates nothing). Otherwise the residuals r_j of up to kHist
+// that allocates nothing, and what is left of a stiff solve). Otherwise the residuals r_j of up to kHist
 // iterations stay where they are, each in its own buffer, and x and p are formed
 // from them afterwards (cg_x_phase): the pass then reads r and q and writes q,
 // where it read and wrote x and p too (192 MB of vectors for 1e6 x 16 floats, not
@@ -334,7 +339,14 @@ __device__ __forceinline__ void sum_partials(const double* part, int nblk, doubl
 // a CTA per row of more than 256 entries; with rows of up to 1400 by a warp each
 // the three take 116, 144 and 102 us.)
 // delta is (r, q) then, which is (p, q) as q = M p and p_{j-1} is M-orthogonal
-// to p_j: in FP32 simulations the same iterations (to one) up to condition 1e5.
+// to p_j. Rounding leaves them so only while p is not much longer than r. Where M is
+// close to singular (alpha rho near 1, a small shift) p grows, and (r, q) costs
+// iterations that (p, q) does not: simulated in FP32 to 4e-6 on four graph
+// families, at most a half more with |p|^2 below 1000 |r|^2 (11 -> 15, Chung-Lu, alpha rho =
+// 0.99, right-hand side 1), beyond it two to ten times as many or no end (78 -> 508, Chung-Lu,
+// 0.999, shift 0.01). So a solve that gets there goes on in the X form, and the next
+// of its kind begins so (PhaseArgs::stiff, run_cg). The shift-and-invert solves of
+// the 1e6-node graph at alpha = 1 / (1 + rho) stay below.
 template <typename T, int K, bool SH = false, bool X = false>
 __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_s_phase(PhaseArgs<T> a) {
   using C = Cfg<T, K>;
@@ -561,10 +573,13 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_u_phase
     for (int v = 0; v < VW; ++v) acc[v] += rr.v[v] * rr.v[v];
   }
   if (!block_partials_last<T, K>(acc, a.part, &st->ticket)) return;
+  __shared__ int s_stiff;
+  if (tid == 0) s_stiff = 0;
   sum_partials<K>(a.part, gridDim.x, s_tmp, s_out);
   if (tid < K) {
     const double gn = s_out[tid];
     if (init) {
+      st->pi[tid] = gn;
       const double b2 = a.bnorm2 ? a.bnorm2[tid] : gn;
       st->gamma[tid] = gn;
       st->b2[tid] = b2;
@@ -578,9 +593,16 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_u_phase
       if (!isfinite(gn)) {
         st->status[tid] = WL_ERR_NONFINITE; st->done[tid] = 1; st->beta[tid] = 0.0;
       } else {
-        st->beta[tid] = gn / st->gamma[tid];
+        const double be = gn / st->gamma[tid], pi = gn + be * be * st->pi[tid];
+        st->beta[tid] = be;
         st->gamma[tid] = gn;
-        if (gn <= a.tol2 * st->b2[tid]) { st->done[tid] = 1; st->beta[tid] = 0.0; }
+        st->pi[tid] = pi;
+        if (gn <= a.tol2 * st->b2[tid]) {
+          st->done[tid] = 1;
+          st->beta[tid] = 0.0;
+        } else if (a.stiff > 0.0 && pi > a.stiff * gn) {
+          s_stiff = 1;
+        }
       }
     } else {
       st->beta[tid] = 0.0;
@@ -591,7 +613,10 @@ __global__ void __launch_bounds__(kPhaseBlock, phase_min_blocks<T>()) cg_u_phase
     if (init) st->iters = 0;
     int any = 0;
     for (int c = 0; c < K; ++c) any |= !st->done[c];
-    st->active = (any && st->iters < a.max_iter) ? 1 : 0;
+    const int go = (any && st->iters < a.max_iter) ? 1 : 0;
+    if (init) st->stiff = 0;
+    if (go && s_stiff) st->stiff = 1;
+    st->active = go && !(s_stiff && a.hist);
     st->ticket = 0;
   }
 }
@@ -634,7 +659,7 @@ struct CgXArgs {
   int m;
   int has_p;  // 0: p_{-1} = 0
   int add_x;  // 0: x is written, not read
-  int flush;  // the solve goes on: p too; nothing to do if it does not
+  int flush;  // 1: the solve goes on: p too, nothing to do if it does not; 2: p too, without that look
 };
 
 template <typename T, int K>
@@ -642,7 +667,7 @@ __global__ void __launch_bounds__(kPhaseBlock) cg_x_phase(CgXArgs<T> a) {
   using C = Cfg<T, K>;
   constexpr int VW = C::VW, G = C::G;
   __shared__ T s_g[kHist + 1][K], s_h[kHist + 1][K];
-  if (a.flush && !*(volatile const int*)&a.st->active) return;
+  if (a.flush == 1 && !*(volatile const int*)&a.st->active) return;
   const int tid = threadIdx.x, m = a.m;
   if (tid < K) {
     T g = T(0), h = T(1), be = T(0);

@@ -96,9 +96,12 @@ cudaError_t launch_permute_vec(const double* in, int64_t n, const int32_t* perm,
 // mode 0: init (gamma_0, flags); 1: `chunk` iterations (S, U pairs); 2: final x += alpha p
 // a solve's start from the residual norms already in st->gamma (no pass over r)
 cudaError_t launch_cg_state_restart(CgState* st, const int* skip, int K, cudaStream_t s);
-// one iteration (S and U), or the start of a solve from r (init)
+// one iteration (S and U; a.hist NULL: x and p updated in S), or the start of a solve from r (init)
 cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, int grid_u, bool init, cudaStream_t s);
 cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, int grid_u, bool init, cudaStream_t s);
+// x += alpha p of the last iteration (a.hist NULL: S has made the others)
+cudaError_t launch_cg_last_f32(int K, const PhaseArgs<float>& a, int grid, cudaStream_t s);
+cudaError_t launch_cg_last_f64(int K, const PhaseArgs<double>& a, int grid, cudaStream_t s);
 cudaError_t launch_cg_x_f32(int K, const CgXArgs<float>& a, int grid, cudaStream_t s);
 cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStream_t s);
 // ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the

@@ -7,14 +7,20 @@ namespace wl {
 
 #define WL_FOR_K(X) X(1) X(2) X(4) X(8) X(16) X(32) X(64)
 
-// one CG iteration: S and U
+// one CG iteration: S and U (a.hist NULL: S updates x and p)
 template <int K>
 static cudaError_t run_cg32(const PhaseArgs<float>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
   if (!init) {
-    if (a.dshift)
-      cg_s_phase<float, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
-    else
-      cg_s_phase<float, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    if (a.hist) {
+      if (a.dshift)
+        cg_s_phase<float, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+      else
+        cg_s_phase<float, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    } else if (a.dshift) {
+      cg_s_phase<float, K, true, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    } else {
+      cg_s_phase<float, K, false, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    }
   }
   cg_u_phase<float, K><<<grid_u, kPhaseBlock, 0, s>>>(a, init ? 1 : 0);
   return cudaGetLastError();
@@ -34,6 +40,7 @@ __global__ void cg_state_restart(CgState* st, const int* skip, int K) {
     st->b2[c] = gn;
     st->alpha[c] = 0.0;
     st->beta[c] = 0.0;
+    st->pi[c] = gn;
     int status = 0, done = !(gn > 0.0) || (skip && skip[c]);
     if (!isfinite(gn)) { done = 1; status = WL_ERR_NONFINITE; }
     st->status[c] = status;
@@ -44,6 +51,7 @@ __global__ void cg_state_restart(CgState* st, const int* skip, int K) {
   if (c == 0) {
     st->iters = 0;
     st->ticket = 0;
+    st->stiff = 0;
     st->active = s_any;
   }
 }
@@ -60,6 +68,18 @@ cudaError_t launch_cg_phases_f32(int K, const PhaseArgs<float>& a, int grid_s, i
     return run_cg32<k>(a, grid_s, grid_u, init, s);
     WL_FOR_K(C32)
 #undef C32
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_cg_last_f32(int K, const PhaseArgs<float>& a, int grid, cudaStream_t s) {
+  switch (K) {
+#define F32(k)                                          \
+  case k:                                              \
+    cg_f_phase<float, k><<<grid, kPhaseBlock, 0, s>>>(a); \
+    return cudaGetLastError();
+    WL_FOR_K(F32)
+#undef F32
   }
   return cudaErrorInvalidValue;
 }

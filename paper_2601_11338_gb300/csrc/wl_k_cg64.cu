@@ -7,14 +7,20 @@ namespace wl {
 
 #define WL_FOR_K(X) X(1) X(2) X(4) X(8) X(16) X(32) X(64)
 
-// one CG iteration: S and U
+// one CG iteration: S and U (a.hist NULL: S updates x and p)
 template <int K>
 static cudaError_t run_cg64(const PhaseArgs<double>& a, int grid_s, int grid_u, bool init, cudaStream_t s) {
   if (!init) {
-    if (a.dshift)
-      cg_s_phase<double, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
-    else
-      cg_s_phase<double, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    if (a.hist) {
+      if (a.dshift)
+        cg_s_phase<double, K, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+      else
+        cg_s_phase<double, K><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    } else if (a.dshift) {
+      cg_s_phase<double, K, true, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    } else {
+      cg_s_phase<double, K, false, true><<<grid_s, kPhaseBlock, 0, s>>>(a);
+    }
   }
   cg_u_phase<double, K><<<grid_u, kPhaseBlock, 0, s>>>(a, init ? 1 : 0);
   return cudaGetLastError();
@@ -27,6 +33,18 @@ cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, 
     return run_cg64<k>(a, grid_s, grid_u, init, s);
     WL_FOR_K(C64)
 #undef C64
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_cg_last_f64(int K, const PhaseArgs<double>& a, int grid, cudaStream_t s) {
+  switch (K) {
+#define F64(k)                                          \
+  case k:                                              \
+    cg_f_phase<double, k><<<grid, kPhaseBlock, 0, s>>>(a); \
+    return cudaGetLastError();
+    WL_FOR_K(F64)
+#undef F64
   }
   return cudaErrorInvalidValue;
 }
