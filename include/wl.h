@@ -37,6 +37,11 @@
  *  - Ownership: the caller owns every buffer it passes; the handle owns its
  *    copy of the graph and all workspace, released by wl_destroy().
  *  - A handle must not be used from two host threads at once.
+ *  - Memory: a handle keeps its workspace between calls, the widest that a call
+ *    needed. Conjugate gradients on graphs beyond the SMs' shared memory keep the
+ *    residuals of up to 16 iterations (at most 4 GB; fewer, or none, where the
+ *    memory is not there); a handle gives these back when another of its
+ *    allocations fails.
  */
 #ifndef WL_H
 #define WL_H

@@ -58,12 +58,10 @@ int set_cuda_error(cudaError_t e, const char* where) {
 // (after its stream has been synchronised) instead of going back to the
 // allocator's cache, where another stream could pick them up.
 thread_local std::vector<void*>* t_retired = nullptr;
+thread_local wl_handle* t_call = nullptr;  // the handle of the running call
+thread_local size_t t_dead = 0;            // its blocks retired by earlier calls, which nothing reads any more
 
-struct CallScope {
-  std::vector<void*>* prev;
-  explicit CallScope(std::vector<void*>* r) : prev(t_retired) { t_retired = r; }
-  ~CallScope() { t_retired = prev; }
-};
+bool give_back();
 
 void retire(void* p) {
   if (!p) return;
@@ -82,6 +80,8 @@ void retire(void* p) {
 //   timeout  every grid barrier starts in the gave-up state, so the
 //            cooperative kernels leave at their first barrier (WL_ERR_TIMEOUT)
 //   noconv   every CG solve is capped at one iteration (WL_ERR_NO_CONVERGENCE)
+//   budget:N the library's device blocks may not pass N bytes in all: the
+//            allocation of a buffer that would is refused (WL_ERR_OOM)
 //   nocluster  the device is taken to place no thread-block clusters: small
 //            solves run as grids (no error)
 // Nothing here faults, traps or hangs the GPU; each failure goes through the
@@ -99,6 +99,12 @@ int fault_mode() {
   return kFaultNone;
 }
 
+// bytes of WL_FAULT=budget:N, or none
+bool over_budget(size_t bytes) {
+  const char* s = getenv("WL_FAULT");
+  return s && !strncmp(s, "budget:", 7) && pool_live_bytes() + bytes > strtoull(s + 7, nullptr, 10);
+}
+
 bool clusters_allowed() { return fault_mode() != kFaultNoCluster; }
 
 int ensure(Buf& b, size_t bytes) {
@@ -111,7 +117,12 @@ int ensure(Buf& b, size_t bytes) {
   retire(b.p);
   b.p = nullptr;
   b.bytes = 0;
-  cudaError_t e = pool_malloc(&b.p, bytes);
+  auto get = [&] { return over_budget(bytes) ? cudaErrorMemoryAllocation : pool_malloc(&b.p, bytes); };
+  cudaError_t e = get();
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    if (give_back()) e = get();  // the handle held memory that it can do without
+  }
   if (e != cudaSuccess) {
     b.p = nullptr;
     return set_cuda_error(e, "cudaMalloc");
@@ -390,6 +401,7 @@ struct wl_handle {
   Buf x, r, p, q;         // CG vectors (FP64 or FP32), n * 64 doubles each at most
   Buf b64;                // FP64 right-hand sides (walk degrees, apply)
   Buf hist;               // phase-kernel CG: CgHist and the kept residuals
+  bool hist_busy = false; // a solve is using them
   const double* r_fin = nullptr;  // final residual of the last FP64 solve
   Buf d32, r32;           // refined form: FP32 correction, residual scratch of its cooperative solve
   Buf xh, xl;             // refined form: the iterate as two FP32 terms (x = xh + xl)
@@ -466,6 +478,44 @@ struct wl_handle {
 namespace {
 
 cudaStream_t S(wl_handle* h) { return h->stream; }
+
+struct CallScope {
+  std::vector<void*>* retired;
+  wl_handle* call;
+  size_t dead;
+  explicit CallScope(wl_handle* h) : retired(t_retired), call(t_call), dead(t_dead) {
+    t_retired = h ? &h->retired : nullptr;
+    t_call = h;
+    t_dead = h ? h->retired.size() : 0;
+  }
+  ~CallScope() {
+    t_retired = retired;
+    t_call = call;
+    t_dead = dead;
+  }
+};
+
+// An allocation of the running call has failed: its handle gives back the blocks
+// that earlier calls retired and, between solves, the kept residuals. False where
+// there is nothing to give.
+bool give_back() {
+  wl_handle* h = t_call;
+  if (!h) return false;
+  const bool hist = h->hist.p && !h->hist_busy;
+  if (!hist && t_dead == 0) return false;
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (hist) {
+    pool_free(h->hist.p);
+    h->hist = Buf{};
+  }
+  for (size_t i = 0; i < t_dead; ++i) pool_free(h->retired[i]);
+  h->retired.erase(h->retired.begin(), h->retired.begin() + t_dead);
+  t_dead = 0;
+  return true;
+}
 
 enum { kCatCG = 0, kCatRes = 1, kCatLan = 2 };
 
@@ -730,14 +780,25 @@ constexpr int64_t kResK1Rows = 250000;
 // 1961; but 564 -> 743 us at 6e4 rows and 744 -> 875 us at 1e5).
 constexpr int64_t kCoopF64K2Rows = 150000;
 
+// Whether a solve of K columns runs as one cooperative kernel
+template <typename T>
+bool cg_coop_fits(const wl_handle* h, int K, const PhaseGraph& g) {
+  if (sizeof(T) == 4) {
+    return (K == 1 && h->n > k1_rows<T>()) ||
+           cg_coop_fits_f32(K, g, h->nnz, h->sms, h->si_dsh_h != nullptr, clusters_allowed());
+  }
+  if (K == 2 && h->n > kCoopF64K2Rows) return false;
+  // one FP64 column without long rows: no hubs to keep in shared memory (1e6 rows,
+  // Erdos-Renyi 2166 -> 1281 us a call, Chung-Lu 2226 -> 1776)
+  if (K == 1 && h->n > k1_rows<T>()) return 2.0 * h->e_low <= (double)h->nnz;
+  return cg_coop_fits_f64(K, g, h->nnz, h->sms, h->si_dsh64 != nullptr, clusters_allowed());
+}
+
 // Launches a solve as one cooperative kernel; false where its vectors don't
 // fit in shared memory (nothing launched).
 template <typename T>
 bool cg_coop_try(wl_handle* h, int K, const PhaseArgs<T>& a, const CgStart<T>& start, cudaError_t* e) {
-  if (sizeof(T) == 8 && K == 2 && h->n > kCoopF64K2Rows) return false;
-  // one FP64 column without long rows: no hubs to keep in shared memory (1e6 rows,
-  // Erdos-Renyi 2166 -> 1281 us a call, Chung-Lu 2226 -> 1776)
-  if (sizeof(T) == 8 && K == 1 && h->n > k1_rows<T>() && 2.0 * h->e_low > (double)h->nnz) return false;
+  if (!cg_coop_fits<T>(h, K, a.g)) return false;
   CoopArgs<T> co{a, h->cgbar(), start.r0 ? start.r0 : a.rn, start.gamma0, start.add_x ? 1 : 0};
   if (!h->bar_clean) {
     *e = cudaMemsetAsync(h->cgbar(), 0, sizeof(CoopBar), S(h));
@@ -792,11 +853,12 @@ constexpr double stiff_line() { return sizeof(T) == 4 ? 1e3 : 1e6; }
 // residuals, every kHist iterations (fewer where they take more than
 // kHistBytes: two for vectors of 1.3 GB and more) and at the end. Once it is
 // stiff, x and p are formed and then updated in every iteration, r in place; and
-// from the start where the handle's last solve of this kind was. *r_fin: the
-// final residual.
+// from the start where the handle's last solve of this kind was, or where there is
+// no memory for two residuals (r then in rbuf, whose memory a.rn is if it is there).
+// *r_fin: the final residual.
 template <typename T>
-int run_cg(wl_handle* h, int kind, int K, const PhaseArgs<T>& a_in, const CgStart<T>& start, int grid_s, int grid_u,
-           SolveInfo& info, const T** r_fin = nullptr) {
+int run_cg(wl_handle* h, int kind, int K, const PhaseArgs<T>& a_in, Buf& rbuf, const CgStart<T>& start, int grid_s,
+           int grid_u, SolveInfo& info, const T** r_fin = nullptr) {
   PhaseArgs<T> a = a_in;
   const int fault = fault_mode();
   if (fault == kFaultNoconv) a.max_iter = 1;
@@ -808,20 +870,32 @@ int run_cg(wl_handle* h, int kind, int K, const PhaseArgs<T>& a_in, const CgStar
   // r_j, j >= 1, takes the buffers in turn; keep + 1 of them
   const size_t stride = ((size_t)h->n * K + 63) & ~(size_t)63, head = (sizeof(CgHist) + 255) & ~(size_t)255;
   int keep = (int)std::max(2.0, std::min<double>(kHist, kHistBytes / (double)(stride * sizeof(T)) - 1.0));
-  for (;; keep /= 2) {  // less than that where memory is short
-    const int rc = ensure(h->hist, head + (size_t)(keep + 1) * stride * sizeof(T));
+  T* r_own = nullptr;  // where r stays once x and p are updated in every iteration
+  for (; !r_own; keep /= 2) {  // less than that where memory is short
+    const size_t need = head + (size_t)(keep + 1) * stride * sizeof(T);
+    if (h->hist.p && h->hist.bytes < need) {  // nothing in it is needed: not kept beside a larger one
+      WL_CU(cudaStreamSynchronize(S(h)));
+      pool_free(h->hist.p);
+      h->hist = Buf{};
+    }
+    const int rc = ensure(h->hist, need);
     if (rc == WL_OK) break;
-    if (rc != WL_ERR_OOM || keep == 1) return rc;
-    cudaGetLastError();
+    if (rc != WL_ERR_OOM) return rc;
+    if (keep < 4) {
+      WL_TRY(ensure(rbuf, (size_t)h->n * K * sizeof(T)));
+      r_own = (T*)rbuf.p;
+    }
   }
-  a.hist = (CgHist*)h->hist.p;
+  struct Busy {
+    bool& b;
+    explicit Busy(bool& f) : b(f) { b = true; }
+    ~Busy() { b = false; }
+  } busy(h->hist_busy);
   T* ring = (T*)((char*)h->hist.p + head);
   bool& was_stiff = h->stiff[kind][h->si_dsh_h || h->si_dsh64];
-  T* r_own = was_stiff ? ring : nullptr;  // where r stays once x and p are updated in every iteration
-  if (r_own) {
-    a.hist = nullptr;
-    if (!start.add_x) WL_CU(cudaMemsetAsync(a.x, 0, (size_t)h->n * K * sizeof(T), S(h)));
-  }
+  if (was_stiff && !r_own) r_own = ring;
+  a.hist = r_own ? nullptr : (CgHist*)h->hist.p;
+  if (r_own && !start.add_x) WL_CU(cudaMemsetAsync(a.x, 0, (size_t)h->n * K * sizeof(T), S(h)));
   auto rj = [&](int j) -> const T* {
     return j == 0 ? r0 : r_own ? r_own : ring + (size_t)((j - 1) % (keep + 1)) * stride;
   };
@@ -940,7 +1014,8 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
   const int grid_u = phase_grid(h, phase_blocks_f64(K), K, 8);
   const int grid_w = phase_grid(h, res_blocks(K), K, 8) + h->nhub;
   const size_t nk = (size_t)h->n * K;
-  WL_TRY(ensure(h->r, nk * 8));
+  const PhaseGraph pg = phase_graph_mid(h, grid_u);
+  if (!x_is_zero || cg_coop_fits<double>(h, K, pg)) WL_TRY(ensure(h->r, nk * 8));
   WL_TRY(ensure(h->p, nk * 8));
   WL_TRY(ensure(h->q, nk * 8));
   WL_TRY(ensure_phase_buffers(h, std::max({grid_u + h->nhub, grid_w, h->sms})));
@@ -957,7 +1032,7 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
     bn2 = st->b2;
     info.nnz_rhs += (double)h->nnz * info.cols(K);
   }
-  PhaseArgs<double> a{phase_graph_mid(h, grid_u), x, (double*)h->r.p, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
+  PhaseArgs<double> a{pg, x, (double*)h->r.p, (double*)h->r.p, (double*)h->p.p, (double*)h->q.p, h->ca, h->cA, h->cD,
                       bn2, nullptr, (double*)h->part.p, st, h->prm.max_iter, tol * tol};
   a.dshift = h->si_dsh64;  // shifted solve of the shift-and-invert Lanczos (else NULL)
   {
@@ -975,7 +1050,7 @@ int solve_fp64(wl_handle* h, const double* b, double* x, int K, double tol, bool
         WL_TRY(phase_lists(h));
         a.g = phase_graph_wide(h, grid_u);
       }
-      WL_TRY(run_cg<double>(h, kCgFp64, K, a, start, grid_u + a.g.nhub, grid_u, info, &h->r_fin));
+      WL_TRY(run_cg<double>(h, kCgFp64, K, a, h->r, start, grid_u + a.g.nhub, grid_u, info, &h->r_fin));
     }
   }
   info.max_rel = std::max(info.max_rel, info.last_rel);
@@ -1018,7 +1093,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
   // state of its own. Small solves run the correction as one cooperative kernel:
   // both are launched before one wait for their outcome.
   PhaseGraph pg = phase_graph_mid(h, grid_u);
-  const bool coop = (K == 1 && h->n > k1_rows<float>()) || cg_coop_fits_f32(K, pg, h->nnz, h->sms, h->si_dsh_h != nullptr, clusters_allowed());
+  const bool coop = cg_coop_fits<float>(h, K, pg);
   if (coop) WL_TRY(ensure(h->r32, nk * 4));
   const bool wide = !coop && grid_u > 1 && grid_r > 1;
   if (wide) {
@@ -1105,7 +1180,7 @@ int solve_refined_df(wl_handle* h, const float* bh, const float* bl, const doubl
       // sizes its first launch chunk from the previous solve of its kind
       int& hint = h->cg_hint_ref[ref == 0 ? 0 : 1];
       h->cg_hint = hint;
-      WL_TRY(run_cg<float>(h, ref == 0 ? kCgFirst : kCgLater, K, a, start, grid_u + pg.nhub, grid_u, inner));
+      WL_TRY(run_cg<float>(h, ref == 0 ? kCgFirst : kCgLater, K, a, h->r32, start, grid_u + pg.nhub, grid_u, inner));
       hint = h->cg_hint;
       if (inner.status == WL_ERR_NOT_SPD || inner.status == WL_ERR_NONFINITE) {
         info.status = inner.status;
@@ -1157,7 +1232,6 @@ int solve_refined(wl_handle* h, const double* b, double* x, int K, double tol, b
   WL_TRY(ensure(h->bl, nk * 4));
   WL_TRY(ensure(h->xh, nk * 4));
   WL_TRY(ensure(h->xl, nk * 4));
-  WL_TRY(ensure(h->r32, nk * 4));
   WL_TRY(ensure_phase_buffers(h, grid_u + h->nhub));
   CgState* st = h->cgst();
   double* bn2 = (double*)h->small.p + 600;
@@ -2256,7 +2330,7 @@ int wl_build(const wl_csr* A, wl_variant v, const wl_params* p, wl_handle** out,
   if (!(mu >= 0.0 && mu <= 1.0)) return WL_ERR_INVALID_ARG;
 
   wl_handle* h = new wl_handle();
-  CallScope cs__(&h->retired);
+  CallScope cs__(h);
   h->n = A->n;
   h->nnz = A->nnz;
   h->variant = v;
@@ -2493,7 +2567,7 @@ int wl_get_info(const wl_handle* h, wl_stats* info) {
 }
 
 int wl_set_warm_start(wl_handle* h, const double* x0) {
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h) return WL_ERR_INVALID_ARG;
   if (!x0) {
     h->have_warm = false;
@@ -2521,7 +2595,7 @@ int wl_set_warm_start(wl_handle* h, const double* x0) {
 // in the caller's node order.
 int wl_mlp_features(wl_handle* h, float* feats, double* xan, wl_stats* st) {
   NvtxRange nvtx__("wl_mlp_features");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (st) memset(st, 0, sizeof(*st));
   if (!h || (!feats && !xan)) return WL_ERR_INVALID_ARG;
   if (h->prm.f != WL_F_RESOLVENT) return WL_ERR_UNSUPPORTED;
@@ -2555,7 +2629,7 @@ int wl_mlp_features(wl_handle* h, float* feats, double* xan, wl_stats* st) {
 // x0 = x_an * exp(y) on the device, kept as the handle's starting guess.
 int wl_mlp_warm_start(wl_handle* h, const float* params, wl_stats* st) {
   NvtxRange nvtx__("wl_mlp_warm_start");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (st) memset(st, 0, sizeof(*st));
   if (!h || !params) return WL_ERR_INVALID_ARG;
   if (h->prm.f != WL_F_RESOLVENT) return WL_ERR_UNSUPPORTED;
@@ -2588,7 +2662,7 @@ int wl_mlp_warm_start(wl_handle* h, const float* params, wl_stats* st) {
 
 int wl_degrees(wl_handle* h, double* Df, wl_stats* st) {
   NvtxRange nvtx__("wl_degrees");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || (!Df && h->n > 0)) return WL_ERR_INVALID_ARG;
   SolveInfo info;
   begin_timer(h);
@@ -2607,7 +2681,7 @@ int wl_degrees(wl_handle* h, double* Df, wl_stats* st) {
 
 int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64_t ldw, wl_stats* st) {
   NvtxRange nvtx__("wl_apply");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || k < 0 || (k > 0 && h->n > 0 && (!V || !W || ldv < k || ldw < k))) return WL_ERR_INVALID_ARG;
   SolveInfo info;
   begin_timer(h);
@@ -2673,7 +2747,7 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
 int wl_expmv(wl_handle* h, const double* U0, int64_t ldu, int k, const double* taus, int ntau, double* U,
              int64_t ldo, wl_stats* st) {
   NvtxRange nvtx__("wl_expmv");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || k < 0 || ntau < 0 || ntau > kMaxTau) return WL_ERR_INVALID_ARG;
   if (k > 0 && h->n > 0 && (!U0 || !U || !taus || ldu < k || ldo < k)) return WL_ERR_INVALID_ARG;
   for (int t = 0; t < ntau; ++t)
@@ -2732,7 +2806,7 @@ int wl_expmv(wl_handle* h, const double* U0, int64_t ldu, int k, const double* t
 int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* steps, int nsteps, double* out,
               int64_t ldo, wl_stats* st) {
   NvtxRange nvtx__("wl_markov");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || k < 0 || nsteps < 1 || nsteps > 64 || !steps) return WL_ERR_INVALID_ARG;
   if (k > 0 && h->n > 0 && (!P0 || !out || ldp < k || ldo < k)) return WL_ERR_INVALID_ARG;
   for (int t = 0; t < nsteps; ++t)
@@ -2814,7 +2888,7 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
 
 int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, uint16_t* omega_out, wl_stats* st) {
   NvtxRange nvtx__("wl_trace");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || !est || !err_est || M < 2 || M > kMaxSketch) return WL_ERR_INVALID_ARG;
   if (h->prm.f != WL_F_RESOLVENT) return WL_ERR_UNSUPPORTED;
   SolveInfo info;
@@ -2903,7 +2977,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
         if ((rc = phase_lists(h)) != WL_OK) break;
         a.g = phase_graph_wide(h, grid_u);
       }
-      if ((rc = run_cg<float>(h, kCgSketch, K, a, CgStart<float>{}, grid_u + a.g.nhub, grid_u, info)) != WL_OK) break;
+      if ((rc = run_cg<float>(h, kCgSketch, K, a, h->r32, CgStart<float>{}, grid_u + a.g.nhub, grid_u, info)) != WL_OK) break;
     }
     (void)sm;
     counted(h, 4);
@@ -2937,7 +3011,7 @@ int wl_trace(wl_handle* h, int M, uint64_t seed, double* est, double* err_est, u
 int wl_return_prob(wl_handle* h, int M, uint64_t seed, const double* ts, int nt, double* p_est, double* p_err,
                    wl_stats* st) {
   NvtxRange nvtx__("wl_return_prob");
-  CallScope cs__(h ? &h->retired : nullptr);
+  CallScope cs__(h);
   if (!h || !ts || !p_est || !p_err || M < 2 || M > kMaxSketch || nt < 1 || nt > kMaxReturnT) return WL_ERR_INVALID_ARG;
   for (int t = 0; t < nt; ++t)
     if (!(ts[t] >= 0.0) || !std::isfinite(ts[t])) return WL_ERR_INVALID_ARG;

@@ -110,6 +110,7 @@ bool launch_cg_coop_f32(int K, const CoopArgs<float>& a, int64_t nnz, int sms, b
                         cudaError_t* e);
 bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, bool clusters, cudaStream_t s,
                         cudaError_t* e);
+bool cg_coop_fits_f64(int K, const PhaseGraph& g, int64_t nnz, int sms, bool shifted, bool clusters);
 bool cg_coop_fits_f32(int K, const PhaseGraph& g, int64_t nnz, int sms, bool shifted, bool clusters);
 bool cg_coop_shape_f32(int K, const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh);
 bool cg_coop_shape_f64(int K, const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh);
@@ -256,6 +257,7 @@ inline int coop_grid(const void* fn, int cap_per_sm) {
 // ---- wl_pool.cu: caching allocator (free only blocks no queued work can touch)
 cudaError_t pool_malloc(void** out, size_t bytes);
 void pool_free(void* p);
+size_t pool_live_bytes();  // device blocks handed out
 cudaError_t pool_malloc_host(void** out, size_t bytes);
 void pool_free_host(void* p);
 

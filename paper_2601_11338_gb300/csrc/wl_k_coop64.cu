@@ -28,6 +28,20 @@ bool launch_cg_coop_f64(int K, const CoopArgs<double>& a, int64_t nnz, int sms, 
   return false;
 }
 
+bool cg_coop_fits_f64(int K, const PhaseGraph& g, int64_t nnz, int sms, bool shifted, bool clusters) {
+  CoopShape sh;
+  switch (K) {
+    case 1: return cgc_device_shape<double, 1>(g, nnz, sms, shifted, clusters, &sh);
+    case 2: return cgc_device_shape<double, 2>(g, nnz, sms, shifted, clusters, &sh);
+    case 4: return cgc_device_shape<double, 4>(g, nnz, sms, shifted, clusters, &sh);
+    case 8: return cgc_device_shape<double, 8>(g, nnz, sms, shifted, clusters, &sh);
+    case 16: return cgc_device_shape<double, 16>(g, nnz, sms, shifted, clusters, &sh);
+    case 32: return cgc_device_shape<double, 32>(g, nnz, sms, shifted, clusters, &sh);
+    case 64: return cgc_device_shape<double, 64>(g, nnz, sms, shifted, clusters, &sh);
+  }
+  return false;
+}
+
 // the shape alone, for a device of `sms` SMs (no GPU needed)
 bool cg_coop_shape_f64(int K, const PhaseGraph& g, int64_t nnz, int sms, bool clusters, CoopShape* sh) {
   switch (K) {

@@ -103,6 +103,14 @@ cudaError_t pool_malloc(void** out, size_t bytes) {
   return cudaSuccess;
 }
 
+size_t pool_live_bytes() {
+  std::lock_guard<std::mutex> lk(g_mtx);
+  size_t t = 0;
+  for (const Cache& c : g_dev)
+    for (const auto& kv : c.live) t += kv.second;
+  return t;
+}
+
 void pool_free(void* p) {
   if (!p) return;
   std::lock_guard<std::mutex> lk(g_mtx);
@@ -164,6 +172,9 @@ void wl_pool_release(void) {
   cudaSetDevice(dev);
   wl::drop_all(wl::g_host, true);
 }
+
+// Device memory of live handles and batches.
+size_t wl_selftest_pool_live(void) { return wl::pool_live_bytes(); }
 
 size_t wl_pool_cached_bytes(void) {
   std::lock_guard<std::mutex> lk(wl::g_mtx);

@@ -107,6 +107,8 @@ def lib():
         L.wl_selftest_search_shape.restype = c_int
         L.wl_selftest_column_blocks.argtypes = [c_int, i64, i64, c_int, ctypes.POINTER(c_int), ctypes.POINTER(c_int), c_int]
         L.wl_selftest_column_blocks.restype = c_int
+        L.wl_selftest_pool_live.argtypes = []
+        L.wl_selftest_pool_live.restype = ctypes.c_size_t
         L.wl_batch_build.argtypes = [vp, c_int, vp, c_int, ctypes.POINTER(wl_params), ctypes.POINTER(vp),
                                      ctypes.POINTER(wl_stats)]
         L.wl_batch_build.restype = c_int
@@ -304,6 +306,11 @@ def wl_selftest_column_blocks(k, n, nnz, fp64):
     if m < 0:
         raise WLError(m, "wl_selftest_column_blocks")
     return list(zip(K[:m], kr[:m]))
+
+
+def wl_selftest_pool_live():
+    """Bytes of device memory that live handles and batches hold."""
+    return lib().wl_selftest_pool_live()
 
 
 def wl_set_warm_start(h, x0):

@@ -80,3 +80,65 @@ def test_an_overflowing_gradient_is_infinite(sign):
     assert loss == np.inf
     assert (grad[4488:] == sign * np.inf).all(), grad[4488:]
     assert not grad[:4488].any()
+
+
+# Rows beyond the SMs' shared memory for 16 columns: the phase kernels
+def _large(prec):
+    g = wlgen.erdos_renyi(200003, 6.0, 3)
+    return g, WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=1e-10)
+
+
+def _free():
+    from paper_2601_11338_gb300 import wl
+    import gc
+    gc.collect()
+    wl.wl_pool_release()
+    return wl.wl_selftest_pool_live()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "refined"])
+def test_a_solve_needs_no_kept_residuals(monkeypatch, prec):
+    """With room for the vectors of conjugate gradients in place and no more, an
+    apply gives the result that it gives with all the memory."""
+    from paper_2601_11338_gb300 import wl
+    k, MB = 16, 1 << 20
+    g, w = _large(prec)
+    V = torch.as_tensor(np.random.default_rng(5).standard_normal((g.n, k)), device="cuda")
+    want = w.apply(V)
+    w.close()
+    _free()
+    g, w = _large(prec)
+    w.degrees()
+    # V, X, b in FP64; then r, p, q (FP64), or b, x, r as two terms each, d, r, p, q (FP32); lists of long rows
+    # and 2 MB to round each of some twenty blocks up
+    need = (3 + 3) * 8 * g.n * k if prec == "fp64" else (3 * 8 + 10 * 4) * g.n * k
+    monkeypatch.setenv("WL_FAULT", f"budget:{wl.wl_selftest_pool_live() + need + 40 * g.n + 28 * MB}")
+    got = w.apply(V)
+    monkeypatch.delenv("WL_FAULT")
+    assert float((got - want).abs().max()) <= 1e-8 * float(want.abs().max())
+    w.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "refined"])
+def test_kept_residuals_are_given_back(monkeypatch, prec):
+    """An outer basis that fits only where the residuals of an earlier apply stood."""
+    from paper_2601_11338_gb300 import wl
+    k, MB = 16, 1 << 20
+    _free()
+    g, w = _large(prec)
+    V = torch.as_tensor(np.random.default_rng(6).standard_normal((g.n, k)), device="cuda")
+    w.set(max_outer=12)
+    want = w.expmv(V, [0.05], allow=(wl.WL_ERR_NO_CONVERGENCE,))
+    w.close()
+    _free()
+    g, w = _large(prec)
+    w.set(max_outer=12)
+    w.apply(V)
+    hist = 17 * (8 if prec == "fp64" else 4) * g.n * k
+    basis = 13 * 8 * g.n * k
+    # the basis, D_f as two terms, the coefficients; half of the residuals stay out
+    monkeypatch.setenv("WL_FAULT", f"budget:{wl.wl_selftest_pool_live() + basis + 16 * g.n + 40 * MB - hist // 2}")
+    got = w.expmv(V, [0.05], allow=(wl.WL_ERR_NO_CONVERGENCE,))
+    monkeypatch.delenv("WL_FAULT")
+    assert float((got - want).abs().max()) <= 1e-8 * float(want.abs().max())
+    w.close()
