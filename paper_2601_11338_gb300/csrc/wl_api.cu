@@ -154,7 +154,8 @@ bool is_device_ptr(const void* p) {
 // gathered rows of at least a 32-byte sector, ten vector streams and the
 // indices. Padding also stops where a block would pass kPadMaxElems elements:
 // the vectors of a solve and an outer basis grow with it, and what fitted in
-// memory without padding has to fit still. The widest block comes first, so that
+// memory without padding has to fit still (so a padded block that meets the end of
+// memory is done again in unpadded ones: for_blocks). The widest block comes first, so that
 // every workspace has its final size from the first block on (a buffer that grows
 // is kept beside its successor until the handle goes). An apply of 13 columns, n = 20011:
 // 455 us as one block of 16, 947 us as 8 + 4 + 1.
@@ -2254,6 +2255,53 @@ int copy_out_vec(wl_handle* h, const double* src, double* dst) {
   return WL_OK;
 }
 
+// The workspace of a call's column blocks back to the allocator (between blocks:
+// nothing in it is needed), with everything that was retired.
+int drop_block_workspace(wl_handle* h) {
+  WL_CU(cudaStreamSynchronize(S(h)));
+  for (Buf* b : {&h->x, &h->r, &h->p, &h->q, &h->b64, &h->hist, &h->d32, &h->r32, &h->xh, &h->xl, &h->bh, &h->bl, &h->rh,
+                 &h->rl, &h->ydf, &h->ew, &h->basis, &h->Tab, &h->ybuf, &h->yprev, &h->robuf, &h->packV, &h->packX}) {
+    pool_free(b->p);
+    *b = Buf{};
+  }
+  h->basis_blocks = 0;
+  for (void* p : h->retired) pool_free(p);
+  h->retired.clear();
+  t_dead = 0;
+  return WL_OK;
+}
+
+// f(block, first column) for the column blocks of k columns, until one fails or,
+// with stop_on_status, leaves a status that is not WL_OK
+template <typename F>
+int for_blocks(wl_handle* h, int k, SolveInfo& info, bool stop_on_status, F f) {
+  std::vector<ColBlock> blocks = column_blocks(k, h->n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4);
+  int c0 = 0;
+  for (size_t i = 0; i < blocks.size(); ++i) {
+    const ColBlock cb = blocks[i];
+    const SolveInfo before = info;
+    info.kr = cb.kr;
+    const int rc = f(cb, c0);
+    if (rc == WL_ERR_OOM && cb.kr < cb.K) {
+      WL_TRY(drop_block_workspace(h));
+      info = before;
+      blocks.erase(blocks.begin() + i);
+      size_t at = i;
+      for (int K = 32, left = cb.kr; left > 0; K /= 2)
+        if (K <= left) {
+          blocks.insert(blocks.begin() + at++, ColBlock{K, K});
+          left -= K;
+        }
+      --i;
+      continue;
+    }
+    WL_TRY(rc);
+    if (stop_on_status && info.status != WL_OK) break;
+    c0 += cb.kr;
+  }
+  return WL_OK;
+}
+
 void free_handle(wl_handle* h) {
   if (!h) return;
   cudaStreamSynchronize(h->stream);
@@ -2702,36 +2750,34 @@ int wl_apply(wl_handle* h, const double* V, int64_t ldv, int k, double* W, int64
       Wd = (double*)h->stage_b.p;
       if (ldw != k) cudaMemcpyAsync(Wd, W, (size_t)n * ldw * 8, cudaMemcpyHostToDevice, S(h));
     }
-    int c0 = 0;
-    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+    rc = for_blocks(h, k, info, false, [&](const ColBlock cb, int c0) -> int {
       const int K = cb.K;
-      info.kr = cb.kr;
-      if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
-      if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
+      WL_TRY(ensure(h->packV, (size_t)n * K * 8));
+      WL_TRY(ensure(h->packX, (size_t)n * K * 8));
       counted(h);
       cudaError_t e = h->perm ? launch_pack_perm(Vd, ldv, c0, cb.kr, K, n, 1.0, h->perm, (double*)h->packV.p, S(h))
                               : launch_pack(Vd, ldv, c0, cb.kr, K, n, 1.0, h->packV.p, false, S(h));
-      if (e != cudaSuccess) { rc = set_cuda_error(e, "pack"); break; }
+      if (e != cudaSuccess) return set_cuda_error(e, "pack");
       if (h->prm.f == WL_F_IDENTITY) {
         PartDev* pd;
         int Tw, Tc;
         thresholds_f64(K, &Tw, &Tc);
-        if ((rc = get_part(h, lanczos_step_grid(K), Tw, Tc, &pd, K, 8)) != WL_OK) break;
+        WL_TRY(get_part(h, lanczos_step_grid(K), Tw, Tc, &pd, K, 8));
         counted(h);
         e = launch_laplacian_apply(h->g, *pd, (const double*)h->packV.p, K, c0, cb.kr, h->perm, Wd, ldw, S(h));
         info.nnz_rhs += (double)h->nnz * info.cols(K);
         info.iters += 1;
       } else {
-        if ((rc = phi_apply(h, (const double*)h->packV.p, (double*)h->packX.p, K, info)) != WL_OK) break;
+        WL_TRY(phi_apply(h, (const double*)h->packV.p, (double*)h->packX.p, K, info));
         counted(h);
         e = h->perm ? launch_apply_out_perm((const double*)h->packV.p, (const double*)h->packX.p,
                                             (const double*)h->Df.p, n, K, c0, cb.kr, h->perm, Wd, ldw, S(h))
                     : launch_apply_out(Vd, ldv, (const double*)h->packX.p, (const double*)h->Df.p, n, K, c0, cb.kr, Wd,
                                        ldw, S(h));
       }
-      if (e != cudaSuccess) { rc = set_cuda_error(e, "apply"); break; }
-      c0 += cb.kr;
-    }
+      if (e != cudaSuccess) return set_cuda_error(e, "apply");
+      return WL_OK;
+    });
     if (rc != WL_OK) break;
     if (!w_dev) {
       cudaError_t e = cudaMemcpyAsync(W, Wd, (size_t)n * ldw * 8, cudaMemcpyDeviceToHost, S(h));
@@ -2773,23 +2819,21 @@ int wl_expmv(wl_handle* h, const double* U0, int64_t ldu, int k, const double* t
     }
     const double* dtaus = nullptr;
     if ((rc = stage_taus(h, taus, ntau, &dtaus)) != WL_OK) break;
-    int c0 = 0;
     bool capped = false;  // a column block reached max_outer: every block is still evaluated
-    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+    rc = for_blocks(h, k, info, true, [&](const ColBlock cb, int c0) -> int {
       const int K = cb.K;
-      info.kr = cb.kr;
-      if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
+      WL_TRY(ensure(h->packX, (size_t)n * K * 8));
       counted(h);
       cudaError_t e = h->perm ? launch_pack_perm(U0d, ldu, c0, cb.kr, K, n, 1.0, h->perm, (double*)h->packX.p, S(h))
                               : launch_pack(U0d, ldu, c0, cb.kr, K, n, 1.0, h->packX.p, false, S(h));
-      if (e != cudaSuccess) { rc = set_cuda_error(e, "expmv pack"); break; }
+      if (e != cudaSuccess) return set_cuda_error(e, "expmv pack");
       OuterRun o;
-      if ((rc = outer_run(h, K, dtaus, ntau, info, o, outer_total)) != WL_OK) break;
-      if (info.status != WL_OK) break;
-      if ((rc = outer_combine(h, o, 0, ntau, Ud, ldo, n * ldo, c0, cb.kr, h->perm)) != WL_OK) break;
+      WL_TRY(outer_run(h, K, dtaus, ntau, info, o, outer_total));
+      if (info.status != WL_OK) return WL_OK;
+      WL_TRY(outer_combine(h, o, 0, ntau, Ud, ldo, n * ldo, c0, cb.kr, h->perm));
       if (!o.converged) capped = true;
-      c0 += cb.kr;
-    }
+      return WL_OK;
+    });
     if (rc != WL_OK) break;
     if (capped && info.status == WL_OK) info.status = WL_ERR_NO_CONVERGENCE;
     if (!u_dev) {
@@ -2831,49 +2875,40 @@ int wl_markov(wl_handle* h, const double* P0, int64_t ldp, int k, const int* ste
       Od = (double*)h->stage_b.p;
       if (ldo != k) cudaMemcpyAsync(Od, out, (size_t)nsteps * n * ldo * 8, cudaMemcpyHostToDevice, S(h));
     }
-    int c0 = 0;
-    for (const ColBlock cb : column_blocks(k, n, h->nnz, h->prm.prec == WL_FP64 ? 8 : 4)) {
+    rc = for_blocks(h, k, info, true, [&](const ColBlock cb, int c0) -> int {
       const int K = cb.K;
-      info.kr = cb.kr;
-      if ((rc = ensure(h->packV, (size_t)n * K * 8)) != WL_OK) break;
-      if ((rc = ensure(h->packX, (size_t)n * K * 8)) != WL_OK) break;
+      WL_TRY(ensure(h->packV, (size_t)n * K * 8));
+      WL_TRY(ensure(h->packX, (size_t)n * K * 8));
       double* cur = (double*)h->packX.p;  // p_s of this block (internal node order)
       double* y = (double*)h->packV.p;    // p_s / D_f
       counted(h);
       cudaError_t e = h->perm ? launch_pack_perm(P0d, ldp, c0, cb.kr, K, n, 1.0, h->perm, cur, S(h))
                               : launch_pack(P0d, ldp, c0, cb.kr, K, n, 1.0, cur, false, S(h));
-      if (e != cudaSuccess) { rc = set_cuda_error(e, "markov pack"); break; }
+      if (e != cudaSuccess) return set_cuda_error(e, "markov pack");
       int s = 0;
       nstep = 0;
-      for (int t = 0; t < nsteps && rc == WL_OK; ++t) {
+      for (int t = 0; t < nsteps; ++t) {
         for (; s < steps[t]; ++s) {
           counted(h);
-          if ((e = launch_row_div(cur, (const double*)h->Df.p, n, K, y, S(h))) != cudaSuccess) {
-            rc = set_cuda_error(e, "markov scale");
-            break;
-          }
+          if ((e = launch_row_div(cur, (const double*)h->Df.p, n, K, y, S(h))) != cudaSuccess)
+            return set_cuda_error(e, "markov scale");
           if (h->prm.f == WL_F_IDENTITY) {
             counted(h);
-            if ((e = launch_adj_apply(h->g, y, K, cur, S(h))) != cudaSuccess) {
-              rc = set_cuda_error(e, "markov step");
-              break;
-            }
+            if ((e = launch_adj_apply(h->g, y, K, cur, S(h))) != cudaSuccess) return set_cuda_error(e, "markov step");
             info.nnz_rhs += (double)h->nnz * info.cols(K);
             info.iters += 1;
           } else {
-            if ((rc = phi_apply(h, y, cur, K, info)) != WL_OK) break;
-            if (info.status != WL_OK) break;
+            WL_TRY(phi_apply(h, y, cur, K, info));
+            if (info.status != WL_OK) return WL_OK;
           }
           ++nstep;
         }
-        if (rc != WL_OK || info.status != WL_OK) break;
         counted(h);
         e = launch_unpack(cur, n, K, c0, cb.kr, h->perm, Od + (size_t)t * n * ldo, ldo, S(h));
-        if (e != cudaSuccess) { rc = set_cuda_error(e, "markov out"); break; }
+        if (e != cudaSuccess) return set_cuda_error(e, "markov out");
       }
-      if (rc != WL_OK || info.status != WL_OK) break;
-      c0 += cb.kr;
-    }
+      return WL_OK;
+    });
     if (rc != WL_OK) break;
     if (!o_dev) {
       cudaError_t e = cudaMemcpyAsync(out, Od, (size_t)nsteps * n * ldo * 8, cudaMemcpyDeviceToHost, S(h));

@@ -142,3 +142,34 @@ def test_kept_residuals_are_given_back(monkeypatch, prec):
     monkeypatch.delenv("WL_FAULT")
     assert float((got - want).abs().max()) <= 1e-8 * float(want.abs().max())
     w.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "refined"])
+def test_a_padded_block_that_does_not_fit_is_done_unpadded(monkeypatch, prec):
+    """13 columns are worked on as 16 where there is room for the basis of 16, and
+    as 8, 4 and 1 where there is not."""
+    from paper_2601_11338_gb300 import wl
+    k, MB = 13, 1 << 20
+    g = wlgen.erdos_renyi(20011, 12.0, 3)
+    assert wl.wl_selftest_column_blocks(k, g.n, g.nnz, prec == "fp64") == [(16, 13)]
+
+    def make():
+        _free()
+        w = WL(g, variant="nbt", alpha_rel=0.5, prec=prec, tol=1e-11, outer_tol=1e-9, max_outer=150)
+        w.degrees()
+        return w
+    U = torch.as_tensor(np.random.default_rng(7).standard_normal((g.n, k)), device="cuda")
+    w = make()
+    want, W = w.expmv(U, [0.4]), w.apply(U)
+    w.close()
+    w = make()
+    basis = 151 * 8 * 8 * g.n  # of eight columns: 194 MB, of 16: 387 MB; some 20 vectors of 16 columns beside it
+    monkeypatch.setenv("WL_FAULT", f"budget:{wl.wl_selftest_pool_live() + basis + 20 * 8 * 16 * g.n + 40 * MB}")
+    got = w.expmv(U, [0.4])
+    work = w.last.nnz_rhs_iters
+    got_apply = w.apply(U)
+    monkeypatch.delenv("WL_FAULT")
+    assert work % g.nnz == 0
+    assert float((got - want).abs().max()) <= 1e-8 * float(want.abs().max())
+    assert float((got_apply - W).abs().max()) <= 1e-8 * float(W.abs().max())
+    w.close()
