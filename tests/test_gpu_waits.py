@@ -65,3 +65,79 @@ def test_refined_streamed_solve_of_one_column(fault):
     times_out(fault, w, lambda allow: w.degrees(allow=allow))
     assert torch.equal(w.degrees(), want)
     w.close()
+
+
+@pytest.mark.parametrize("n", [300, 20000])
+def test_fp64_cooperative_solve(fault, n):
+    g = wlgen.erdos_renyi(n, 6, 4)
+    w = WL(g, variant="nbt", alpha_rel=0.5, tol=1e-12, prec="fp64")
+    times_out(fault, w, lambda allow: w.degrees(allow=allow))
+    want = w.degrees().clone()
+    times_out(fault, w, lambda allow: w.degrees(allow=allow))
+    assert torch.equal(w.degrees(), want)
+    w.close()
+
+
+def test_fp64_streamed_solve_of_one_column(fault):
+    # more than half of the entries in long rows: hubs worth keeping in shared memory
+    g = wlgen.star(620000)
+    w = WL(g, variant="nbt", alpha=1e-4, tol=1e-12, prec="fp64")
+    times_out(fault, w, lambda allow: w.degrees(allow=allow))
+    want = w.degrees().clone()
+    assert torch.equal(w.degrees(), want)
+    w.close()
+
+
+def test_sketch_solve(fault):
+    from paper_2601_11338_gb300 import wl
+    g = wlgen.erdos_renyi(3000, 6, 4)
+    w = WL(g, variant="nbt", alpha_rel=0.5, prec="sketch")
+    want = w.trace(16, 5)
+    fault("timeout")
+    with pytest.raises(wl.WLError) as e:
+        w.trace(16, 5)
+    assert e.value.status == wl.WL_ERR_TIMEOUT
+    fault("")
+    assert w.trace(16, 5) == want
+    w.close()
+
+
+@pytest.mark.parametrize("n", [300, 260000])  # vectors in shared memory, and streamed
+def test_spectral_search(fault, n):
+    from paper_2601_11338_gb300 import wl
+    g = wlgen.erdos_renyi(n, 4, 4)
+    fault("timeout")
+    with pytest.raises(wl.WLError) as e:
+        WL(g, variant="nbt", alpha_rel=0.5)
+    assert e.value.status == wl.WL_ERR_TIMEOUT
+    fault("")
+    w = WL(g, variant="nbt", alpha_rel=0.5)
+    assert w.info["rho"] > 1.0
+    w.close()
+
+
+def test_outer_lanczos_step_fp64(fault):
+    """f = identity makes no solve: the first kernel that waits is the Lanczos step."""
+    g = wlgen.erdos_renyi(300, 6, 4)
+    w = WL(g, f="identity", prec="fp64")
+    U0 = torch.zeros((g.n, 2), dtype=torch.float64, device="cuda")
+    U0[0, 0] = U0[7, 1] = 1.0
+    want = w.expmv(U0, [1.0]).clone()
+    times_out(fault, w, lambda allow: w.expmv(U0, [1.0], allow=allow))
+    assert torch.equal(w.expmv(U0, [1.0]), want)
+    w.close()
+
+
+def test_outer_lanczos_step_refined(fault):
+    """Solves by the phase kernels (16 columns, more rows than the SMs hold) wait for
+    nothing; a Lanczos run of one step is checked after it."""
+    from paper_2601_11338_gb300 import wl
+    g = wlgen.erdos_renyi(200003, 6, 3)
+    w = WL(g, variant="nbt", alpha_rel=0.5, tol=1e-10, prec="refined", max_outer=1)
+    U0 = torch.as_tensor(np.random.default_rng(0).standard_normal((g.n, 16)), device="cuda")
+    w.degrees()
+    capped = (wl.WL_ERR_NO_CONVERGENCE,)
+    want = w.expmv(U0, [0.5], allow=capped).clone()
+    times_out(fault, w, lambda allow: w.expmv(U0, [0.5], allow=allow + capped))
+    assert torch.equal(w.expmv(U0, [0.5], allow=capped), want)
+    w.close()
