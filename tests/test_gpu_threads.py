@@ -1,6 +1,7 @@
 """Handles in different host threads: nearly every solve is one kernel over the
 whole chip whose CTAs wait for one another, so the handles' kernels take turns. Each
 gives the results that it gives alone."""
+import gc
 import threading
 
 import numpy as np
@@ -41,7 +42,13 @@ class Job:
             self.error = e
 
 
-def test_two_handles_in_two_threads():
+@pytest.fixture
+def collected():
+    yield
+    gc.collect()  # the jobs' tensors go here, and not during a later test that watches the memory in use
+
+
+def test_two_handles_in_two_threads(collected):
     """One cluster, one grid of few CTAs, and grids over all SMs, side by side."""
     jobs = [Job(wlgen.erdos_renyi(300, 6, 4), 1, 12, prec="fp64", tol=1e-11),
             Job(wlgen.erdos_renyi(20011, 10, 5), 13, 8, prec="refined", tol=1e-10),
