@@ -699,9 +699,7 @@ int phase_lists(wl_handle* h) {
   return WL_OK;
 }
 
-int phase_hubs(const wl_handle* h) { return h->have_lists2 ? h->nhub2 : h->nhub; }
-
-// the graph as seen by a phase kernel of grid_u CTAs plus phase_hubs
+// the graph as seen by a phase kernel of grid_u CTAs plus one per hub of the list
 PhaseGraph phase_graph_wide(wl_handle* h, int grid_u) {
   if (!h->have_lists2) return phase_graph_mid(h, grid_u);
   PhaseGraph g = phase_graph(h);

@@ -6,28 +6,35 @@
 // The gather of neighbour vectors is latency bound, so these kernels keep
 // the SMs full of warps (G lanes per row, one 16-byte slice each, rows
 // spread over a grid-stride loop) instead of persisting with few warps.
-// Rows with more than kHubDeg entries are gathered by one CTA each; when the
-// graph carries a list of mid rows (kMidDeg < deg <= kHubDeg), the S kernel
+// Hub rows (the graph's list of them) are gathered by one CTA each; when the
+// graph carries a list of mid rows (kMidDeg < deg, not hubs), the S kernel
 // spends a share of its CTAs (proportional to those rows' entries) on them,
 // one warp per row, so that no lane group walks a long row alone, and the
-// remaining CTAs take the short rows; the grid stays one wave.
+// remaining CTAs take the short rows; the grid stays one wave. Where the line
+// between mid rows and hubs lies is the caller's: kHubDeg entries in a handle's own
+// lists, kPhaseHubDeg (wl_api.cu) in those of its solves.
 //
 // One iteration = two kernels:
-//   S: s = M r ; x += alpha p ; p = r + beta p ; q = s + beta q ; delta = (p, q)
-//   U: r -= alpha q ; gamma' = (r, r)
+//   S: s = M r ; q = s + beta q ; delta = (r, q)
+//   U: r' = r - alpha q ; gamma' = (r', r')
+// with r' in a buffer of its own, and x (and p, every kHist iterations) formed
+// from the kept residuals by a third kernel (cg_x_phase). In the X form, which
+// keeps none, S also makes x += alpha p and p = r + beta p, and delta = (p, q).
 // Each kernel ends with a last-CTA reduction (fixed order, deterministic)
 // that derives the next scalars and the per-column convergence on the
 // device; a kernel finding the solve inactive returns at once, so the host
 // launches iterations in chunks and reads one flag between chunks.
-// Vector traffic per iteration: 10 n K s bytes + 4 nnz + 4 (n + 1).
+// Vector traffic per iteration, besides the gathers, 4 nnz and 4 (n + 1) bytes: 6 n K s
+// bytes (r, q read, q written; r, q read, r' written) and n K s for x at the end;
+// 10 n K s in the X form.
 #pragma once
 #include "wl_common.cuh"
 #include "wl_df.cuh"
 
 namespace wl {
 
-constexpr int kHubDeg = 256;       // rows with more entries get a CTA each
-constexpr int kMidDeg = 30;        // rows with more entries (up to kHubDeg) get a warp each in the S kernels
+constexpr int kHubDeg = 256;       // rows with more entries are on a handle's list of hubs
+constexpr int kMidDeg = 30;        // rows with more entries (not hubs) get a warp each in the S kernels
 constexpr int kPhaseBlock = 256;   // threads per CTA of the phase kernels
 #ifndef WL_PHASE_MINB
 #define WL_PHASE_MINB 3
@@ -59,9 +66,9 @@ struct PhaseGraph {
   const int32_t* row_ptr;
   const int32_t* col;
   int64_t n;
-  const int32_t* hubs;  // rows with deg > kHubDeg
+  const int32_t* hubs;  // rows with more entries than the line of the list (kHubDeg, kPhaseHubDeg)
   int nhub;
-  const int32_t* mids = nullptr;  // rows with kMidDeg < deg <= kHubDeg
+  const int32_t* mids = nullptr;  // rows with more than kMidDeg entries that are not hubs
   int nmid = 0;
   int nmid_blk = 0;               // CTAs (after the hub CTAs) that walk the mid rows; 0: no mid path
 };

@@ -93,7 +93,6 @@ cudaError_t launch_permute_vec(const double* in, int64_t n, const int32_t* perm,
                                cudaStream_t s);
 
 // ---- wl_k_cg64.cu / wl_k_cg32.cu: CG phase kernels
-// mode 0: init (gamma_0, flags); 1: `chunk` iterations (S, U pairs); 2: final x += alpha p
 // a solve's start from the residual norms already in st->gamma (no pass over r)
 cudaError_t launch_cg_state_restart(CgState* st, const int* skip, int K, cudaStream_t s);
 // one iteration (S and U; a.hist NULL: x and p updated in S), or the start of a solve from r (init)
@@ -102,6 +101,7 @@ cudaError_t launch_cg_phases_f64(int K, const PhaseArgs<double>& a, int grid_s, 
 // x += alpha p of the last iteration (a.hist NULL: S has made the others)
 cudaError_t launch_cg_last_f32(int K, const PhaseArgs<float>& a, int grid, cudaStream_t s);
 cudaError_t launch_cg_last_f64(int K, const PhaseArgs<double>& a, int grid, cudaStream_t s);
+// x (and p) from the kept residuals
 cudaError_t launch_cg_x_f32(int K, const CgXArgs<float>& a, int grid, cudaStream_t s);
 cudaError_t launch_cg_x_f64(int K, const CgXArgs<double>& a, int grid, cudaStream_t s);
 // ---- wl_k_coop{32,64}.cu: a whole solve as one cooperative kernel; false (nothing launched) where the
@@ -125,10 +125,10 @@ cudaError_t launch_res_phases(int K, const ResPhaseArgs& a, int grid, cudaStream
 // x (n K doubles) -> (xh, xl) FP32 terms, or (join) xh + xl -> xout
 cudaError_t launch_split_x(const double* x, int64_t total, float* xh, float* xl, bool join, double* xout,
                            cudaStream_t s);
-// ---- wl_k_res.cu: double-float residual of the refined form
+// ---- wl_k_df.cu: double-float residual of the refined form
 // r_out = r_in - M y (y gathered: the correction d; x += d) or, full, r_out = b - M x (x = yh + yl)
 cudaError_t launch_df_res(int K, const DfResArgs& a, int grid, bool full, cudaStream_t s);
-// (bh, bl) = scale * b (b: n x K FP64, contiguous), r32 = bh (if not NULL), |b|^2 per column -> b2
+// (bh, bl) = b (n x K FP64, contiguous), |b|^2 per column -> b2
 cudaError_t launch_df_from_f64(int K, const double* b, int64_t n, float* bh, float* bl, double* part, CgState* st,
                                double* b2, int grid, cudaStream_t s);
 int df_res_blocks(int K);
@@ -230,7 +230,8 @@ cudaError_t launch_gram(const uint16_t* omega, const float* Y, int64_t n, int M,
 // out[0] estimate, out[1] error estimate, out[2] status, out[8 + i] = t_i
 // gram (128 x 64) is used as scratch; out: kCoreDoubles
 cudaError_t launch_nys_core(double* gram, int M, double* out, cudaStream_t s);
-// [Omega Y]^T Y from an FP64 Y (n x K, first M columns), FP64 throughout; partial: G x 2 x 64 x 64 doubles
+// [Omega Y]^T Y from an FP64 Y (n x K, first M columns), FP64 throughout; partial: gram_f64_partial_doubles, the
+// output tiles of gram_grid_f64 CTAs
 int gram_grid_f64(int64_t n);
 size_t gram_f64_partial_doubles(int64_t n, int M);
 cudaError_t launch_gram_f64(const uint16_t* omega, const double* Y, int64_t n, int M, int K, double* partial,
